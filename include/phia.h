@@ -190,7 +190,7 @@ int phia_create_from_device(phia_t **out, const int8_t *J_k, const int32_t *h_k,
 /* Create a sparse instance in CSR form (host arrays): row_ptr[N+1], col[nnz]
  * (0 <= col < N, no self loops), val_k[nnz] int8; the pattern and values must be
  * symmetric.  Stored zeros are allowed.  Runs on the CSR path (a batch of one); its
- * replicas run in groups of 256, smaller counts padded with unreported replicas.  One
+ * replicas run in groups of 32, other counts padded with unreported replicas.  One
  * launch per iteration (opts->tc_kernel = 1: one persistent launch for the run instead;
  * that cooperative launch assumes no other persistent launch runs on the device at the
  * same time, and reports PHIA_ETIMEOUT rather than waiting without end if one does). */
@@ -360,14 +360,14 @@ int phia_run_noalloc(const int8_t *J_k, const int32_t *h_k, int32_t N, int32_t f
 
 /* ---------------------------------------------------------------- batches
  * Many independent instances of uneven N annealed together.  Dense descriptors with
- * N <= 384 and every |k| <= 16, or N <= 256, run on the resident tcgen05 kernel over a
- * table of CTAs (8 replicas each): every such instance, all iterations, one launch per
- * (operand, number of 128-spin tiles) group.  The other instances run on the sparse CSR
- * path (larger dense descriptors converted to CSR): by default one persistent cooperative
- * launch covers every iteration of every CSR instance (blocks take 64-row x 256-replica
- * work units from a counter, the grid meets at a bounded barrier between iterations);
- * phia_opts.tc_kernel = 2 at creation gives one launch per iteration instead (replayed as
- * CUDA graphs), and phia_batch_autotune picks the faster.  Each instance keeps its own
+ * N <= 256 run on the resident warp-level kernel, those with N <= 384 and every |k| <= 16 on
+ * the resident tcgen05 kernel, over a table of CTAs (8 replicas each): every such instance,
+ * all iterations, one launch per size class.  The other instances run on the sparse path
+ * (larger dense descriptors converted to CSR), in sets whose state fits in L2 together, by
+ * default with one launch per iteration and set (replayed as CUDA graphs);
+ * phia_opts.tc_kernel = 1 at creation gives one persistent cooperative launch for every
+ * iteration of every instance instead (blocks take work units from a counter, the grid meets
+ * at a bounded barrier between iterations), and phia_batch_autotune picks the faster.  Each instance keeps its own
  * couplings, replicas, records and Philox instance id, so its result does not depend on
  * the rest of the batch or on the path, and equals the same instance run alone on that
  * path. */
@@ -387,13 +387,13 @@ typedef struct phia_instance_desc {
 typedef struct phia_batch_s phia_batch_t;
 
 /* Validate and upload `count` instances (copied; the caller keeps its arrays).  opts
- * may be NULL; opts->path must be PHIA_PATH_AUTO or PHIA_PATH_CSR; opts->tc_kernel: 0 or
- * 1 = the CSR instances in one persistent launch, 2 = one launch per iteration. */
+ * may be NULL; opts->path must be PHIA_PATH_AUTO or PHIA_PATH_CSR; opts->tc_kernel: 1 = the
+ * CSR instances in one persistent launch, 0 or 2 = one launch per iteration. */
 int phia_batch_create(phia_batch_t **out, int32_t count, const phia_instance_desc *descs,
                       const phia_opts *opts);
 
 /* Anneal `replicas` replicas of every instance for `steps` iterations (as phia_anneal
- * per instance).  The sparse path runs replicas in groups of 256; other counts are
+ * per instance).  The sparse path runs replicas in groups of 32; other counts are
  * padded with extra replicas that are run but never reported.  Asynchronous. */
 int phia_batch_anneal(phia_batch_t *b, const phia_schedule *sched, int32_t replicas, int64_t steps,
                       uint64_t seed);

@@ -41,16 +41,24 @@ struct phia_batch_s {
     std::vector<SmallCta> small_host;
     std::vector<int64_t> bits_pub;      // per public instance: offset of its best states
     std::vector<long long> targets;     // per instance, LLONG_MIN = none
-    std::vector<CsrBlock> blocks;
-    int64_t total_rows = 0, total_nnz = 0;
-    int max_words = 0;
+    std::vector<CsrBlock> blocks;       // the block lists for 1, 2, 4 and 8 slices a block
+    std::vector<int32_t> first_block[4];   // per CSR member (and one past): its first block in each list
+    std::vector<CsrSet> sets;           // instances whose state fits in L2 together, for sets_R replicas
+    int sets_R = 0;
+    int32_t set_max[4] = {0, 0, 0, 0};
+    CsrSet *d_sets = nullptr;
+    int64_t total_slices = 0;
+    int max_words = 0, max_np = 0;
     CsrInst *d_inst = nullptr;
     CsrBlock *d_blocks = nullptr;
-    int32_t *d_rowptr = nullptr, *d_col = nullptr, *d_hk = nullptr;
-    int8_t *d_val = nullptr;
+    void *d_col = nullptr;              // uint16 offsets (col16) or uint32
+    bool col16 = false;
+    int32_t *d_slice = nullptr, *d_hk2 = nullptr, *d_rowof = nullptr, *d_posof = nullptr;
+    uint32_t *d_val = nullptr;
+    int32_t *d_hk = nullptr;            // fields of the small dense members
     long long *d_targets = nullptr;
     bool any_target = false;
-    // replica state (R padded to a multiple of 256)
+    // replica state (R padded to a multiple of 32)
     int Rcap = 0, R = 0, R_real = 0;
     float *d_X = nullptr, *d_V = nullptr;
     uint32_t *d_S = nullptr;
@@ -64,7 +72,7 @@ struct phia_batch_s {
     int32_t *d_err = nullptr;
     IterCtl *d_ctl = nullptr;               // iteration control of the step kernel
     unsigned *d_sync = nullptr;             // barrier and work counters of the persistent launch
-    int csr_mode = 1;                       // 1 persistent CSR launch, 2 one launch per iteration
+    int csr_mode = 2;                       // 1 persistent CSR launch, 2 one launch per iteration
     StepGraphCache *graphs = nullptr;       // its step launches as replayable graphs
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     bool ran = false;
@@ -130,17 +138,53 @@ void layout(phia_batch_s *b, int R) {
         in.x_off = x; in.xin_off = xin; in.s_off = s;
         in.rec_off = (int64_t)k * R;
         in.bits_off = b->bits_pub[(size_t)k];
-        x += (int64_t)in.N * R;
+        x += (int64_t)in.Np * R;
         xin += (int64_t)in.N * b->R_real;
-        s += (int64_t)in.N * (R / 32);
+        s += (int64_t)in.Np * (R / 32);
     }
+}
+
+// Sets of consecutive CSR members for R replicas: as few as keep a set's x and v within 0.4 of L2,
+// of about equal size.
+int make_sets(phia_batch_s *b, int R) {
+    int l2 = 0;
+    BCU(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, b->device));
+    const int n = (int)b->inst.size();
+    int64_t total = 0;
+    for (const CsrInst &in : b->inst) total += (int64_t)in.Np * R * 8;
+    const int64_t budget = std::max<int64_t>(1, (int64_t)(0.4 * l2));
+    const int64_t share = total / std::max<int64_t>(1, (total + budget - 1) / budget) + 1;
+    b->sets.clear();
+    std::fill(b->set_max, b->set_max + 4, 0);
+    int64_t seen = 0;
+    for (int c0 = 0, c = 0; c < n; ++c) {
+        seen += (int64_t)b->inst[(size_t)c].Np * R * 8;
+        if (c + 1 < n && seen < share * (int64_t)(b->sets.size() + 1)) continue;
+        CsrSet s;
+        for (int l = 0; l < 4; ++l) {
+            s.off[l] = b->first_block[l][(size_t)c0];
+            s.len[l] = b->first_block[l][(size_t)c + 1] - s.off[l];
+            b->set_max[l] = std::max(b->set_max[l], s.len[l]);
+        }
+        // the heaviest blocks first
+        for (int l = 0; l < 4; ++l)
+            std::stable_sort(b->blocks.begin() + s.off[l], b->blocks.begin() + s.off[l] + s.len[l],
+                             [&](const CsrBlock &x, const CsrBlock &y) { return x.work > y.work; });
+        b->sets.push_back(s);
+        c0 = c + 1;
+    }
+    BCU(cudaMemcpyAsync(b->d_blocks, b->blocks.data(), b->blocks.size() * sizeof(CsrBlock), cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaMemcpyAsync(b->d_sets, b->sets.data(), b->sets.size() * sizeof(CsrSet), cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaStreamSynchronize(b->stream));
+    b->sets_R = R;
+    return PHIA_OK;
 }
 
 int ensure_state(phia_batch_s *b, int R) {
     if (R <= b->Rcap) return PHIA_OK;
     BCU(cudaStreamSynchronize(b->stream));
     free_state(b);
-    const int64_t rows = b->total_rows;
+    const int64_t rows = b->total_slices * 32;
     int64_t bits = 0;
     for (int k = 0; k < b->count; ++k) bits += (int64_t)R * words_of(b->N[k]);
     const int64_t reps = (int64_t)R * b->count;
@@ -172,15 +216,15 @@ int ensure_state(phia_batch_s *b, int R) {
 
 namespace phia {
 
-// One instance of a batch, checked and converted to padded CSR (row offsets relative to
-// the instance), before concatenation; code/msg hold its first error.
+// One instance of a batch, checked and converted to slices of 32 rows (relative to the
+// instance), before concatenation; code/msg hold its first error.
 struct PackedInst {
     int code = PHIA_OK;
     std::string msg;
-    std::vector<int32_t> rp, col;
-    std::vector<int8_t> val;
-    int64_t nnz_real = 0;
-    int small_op = 0;       // small dense member: its tensor-core operand (no CSR built)
+    std::vector<int32_t> slice, col, hk2, row_of, pos_of;
+    std::vector<uint32_t> val;
+    int wide = 0;
+    int small_op = 0;       // small dense member: its tensor-core operand (no slices built)
 };
 
 void pack_error(PackedInst &out, int code, const char *fmt, ...) {
@@ -193,6 +237,48 @@ void pack_error(PackedInst &out, int code, const char *fmt, ...) {
     out.msg = buf;
 }
 
+// The slices of a checked instance: rows sorted by their number of couplings (descending,
+// ties in row order), 32 to a slice, every row padded to the slice's longest with k = 0.
+void pack_slices(int n, const int32_t *rp, const int32_t *col, const int8_t *val, const int32_t *h, PackedInst &out) {
+    const int np = round_up(n, 32), ns = np / 32;
+    std::vector<int32_t> order((size_t)n);
+    for (int i = 0; i < n; ++i) order[(size_t)i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return rp[a + 1] - rp[a] > rp[b + 1] - rp[b]; });
+    out.row_of.assign((size_t)np, -1);
+    out.pos_of.resize((size_t)n);
+    for (int p = 0; p < n; ++p) {
+        out.row_of[(size_t)p] = order[(size_t)p];
+        out.pos_of[(size_t)order[(size_t)p]] = p;
+    }
+    out.slice.assign((size_t)ns + 1, 0);
+    for (int s = 0; s < ns; ++s) {
+        const int first = order[(size_t)s * 32];       // the slice's longest row
+        out.slice[(size_t)s + 1] = out.slice[(size_t)s] + (rp[first + 1] - rp[first] + 3) / 4;
+    }
+    out.col.assign((size_t)out.slice[(size_t)ns] * 128, 0);
+    out.val.assign((size_t)out.slice[(size_t)ns] * 32, 0u);
+    out.hk2.assign((size_t)np * 2, 0);
+    int64_t bound = 0;
+    for (int p = 0; p < n; ++p) {
+        const int i = order[(size_t)p], lane = p & 31;
+        const size_t e0 = (size_t)out.slice[(size_t)p / 32];
+        int64_t mag = 2 * std::abs((int64_t)h[i]);
+        int32_t ksum = 0;
+        for (int32_t c = rp[i]; c < rp[i + 1]; ++c) {
+            const size_t m = (size_t)(c - rp[i]), e = e0 + m / 4;
+            out.col[(e * 32 + (size_t)lane) * 4 + m % 4] = out.pos_of[(size_t)col[c]] * 4;
+            out.val[e * 32 + (size_t)lane] |= (uint32_t)(uint8_t)val[c] << (8 * (m % 4));
+            ksum += val[c];
+            mag += std::abs((int)val[c]);
+        }
+        out.hk2[(size_t)p * 2] = h[i];
+        out.hk2[(size_t)p * 2 + 1] = h[i] - ksum;
+        bound = std::max(bound, mag);
+    }
+    // |I + h| <= bound: 128 rows' terms and a sum scaled by 2^7 stay in 32 bits up to 2^23.
+    out.wide = bound > ((int64_t)1 << 23);
+}
+
 void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
     const int n = x.N;
     if (n < 1) return pack_error(out, PHIA_EINVAL, "instance %d: N must be >= 1", k);
@@ -201,20 +287,9 @@ void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
     for (int i = 0; i < n; ++i)
         if (x.h_k[i] >= (1 << 24) || x.h_k[i] <= -(1 << 24))
             return pack_error(out, PHIA_ERANGE, "instance %d: |h_k[%d]| >= 2^24", k, i);
-    std::vector<int32_t> &col = out.col;
-    std::vector<int8_t> &val = out.val;
-    // Every row is padded to a multiple of 8 entries with k = 0 (column 0): rows start
-    // 32-byte aligned in col and 8-byte aligned in val (instances are concatenated in
-    // whole padded rows), so the step kernel reads a row's entries 8 at a time with
-    // aligned vector loads and no tail.
-    auto pad_row = [&]() {
-        while (col.size() % 8) {
-            col.push_back(0);
-            val.push_back(0);
-        }
-    };
-    std::vector<int32_t> &rp = out.rp;
-    rp.assign((size_t)n + 1, 0);
+    // Rows as lists of (column, coupling), in CSR order.
+    std::vector<int32_t> rp((size_t)n + 1, 0), col;
+    std::vector<int8_t> val;
     if (x.J_k) {
         // Small enough for the resident tensor-core kernel: checked here, kept dense.
         int maxk = 0;
@@ -240,13 +315,11 @@ void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
                 if (x.J_k[(size_t)i * n + j] != 0) {
                     col.push_back(j);
                     val.push_back(x.J_k[(size_t)i * n + j]);
-                    ++out.nnz_real;
                 }
             }
-            pad_row();
             rp[i + 1] = (int32_t)col.size();
         }
-        return;
+        return pack_slices(n, rp.data(), col.data(), val.data(), x.h_k, out);
     }
     if (!x.row_ptr || !x.col || !x.val_k) return pack_error(out, PHIA_EINVAL, "instance %d: CSR arrays missing", k);
     if (x.row_ptr[0] != 0) return pack_error(out, PHIA_EINVAL, "instance %d: row_ptr[0] != 0", k);
@@ -255,8 +328,6 @@ void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
     // Rows with ascending columns are searched by bisection in the symmetry check.
     std::vector<uint8_t> row_sorted(n);
     for (int i = 0; i < n; ++i) row_sorted[i] = std::is_sorted(x.col + x.row_ptr[i], x.col + x.row_ptr[i + 1]);
-    col.reserve((size_t)x.row_ptr[n] + 8 * (size_t)n);
-    val.reserve((size_t)x.row_ptr[n] + 8 * (size_t)n);
     for (int i = 0; i < n; ++i) {
         for (int32_t p = x.row_ptr[i]; p < x.row_ptr[i + 1]; ++p) {
             const int j = x.col[p];
@@ -268,13 +339,9 @@ void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
             if (f != ce && *f != i) f = ce;
             if (f == ce || x.val_k[x.row_ptr[j] + (f - cb)] != x.val_k[p])
                 return pack_error(out, PHIA_EINVAL, "instance %d: CSR is not symmetric at (%d, %d)", k, i, j);
-            col.push_back(j);
-            val.push_back(x.val_k[p]);
-            ++out.nnz_real;
         }
-        pad_row();
-        rp[i + 1] = (int32_t)col.size();
     }
+    pack_slices(n, x.row_ptr, x.col, x.val_k, x.h_k, out);
 }
 
 int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d, const phia_opts *opts) {
@@ -287,7 +354,7 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         return bfail(PHIA_ENOTSUP, "batches run on the CSR path");
     if (o.tc_kernel < 0 || o.tc_kernel > 2) return bfail(PHIA_EINVAL, "batches: tc_kernel must be 0, 1 or 2");
     phia_batch_s *b = new phia_batch_s();
-    b->csr_mode = o.tc_kernel == 2 ? 2 : 1;
+    b->csr_mode = o.tc_kernel == 1 ? 1 : 2;
     auto cleanup = [&](int code) { phia_batch_destroy(b); return code; };
     b->count = count;
     // Instances are checked and converted independently, on every host core (a batch of
@@ -305,19 +372,25 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         work();
         for (std::thread &t : workers) t.join();
     }
-    size_t tot_rp = 0, tot_nz = 0, tot_h = 0, tot_dj = 0;
+    size_t tot_sl = 0, tot_ent = 0, tot_pos = 0, tot_inv = 0, tot_h = 0, tot_dj = 0;
     for (int k = 0; k < count; ++k) {
         if (packed[(size_t)k].code != PHIA_OK)
             return cleanup(bfail(packed[(size_t)k].code, "%s", packed[(size_t)k].msg.c_str()));
-        tot_rp += packed[(size_t)k].rp.size();
-        tot_nz += packed[(size_t)k].col.size();
-        tot_h += (size_t)d[k].N;
-        if (packed[(size_t)k].small_op) tot_dj += (size_t)d[k].N * d[k].N;
+        tot_sl += packed[(size_t)k].slice.size();
+        tot_ent += packed[(size_t)k].val.size();
+        tot_pos += packed[(size_t)k].row_of.size();
+        tot_inv += packed[(size_t)k].pos_of.size();
+        if (packed[(size_t)k].small_op) {
+            tot_h += (size_t)d[k].N;
+            tot_dj += (size_t)d[k].N * d[k].N;
+        }
     }
-    std::vector<int32_t> rowptr, col, hk;
-    std::vector<int8_t> val, dj;
-    rowptr.reserve(tot_rp); col.reserve(tot_nz); val.reserve(tot_nz); hk.reserve(tot_h); dj.reserve(tot_dj);
-    int64_t row_base = 0, nnz_real = 0;
+    if (tot_ent / 32 > (size_t)INT32_MAX) return cleanup(bfail(PHIA_ERANGE, "too many couplings in one batch"));
+    std::vector<int32_t> slice, col, hk2, row_of, pos_of, hk;
+    std::vector<uint32_t> val;
+    std::vector<int8_t> dj;
+    slice.reserve(tot_sl); col.reserve(4 * tot_ent); val.reserve(tot_ent); hk2.reserve(2 * tot_pos);
+    row_of.reserve(tot_pos); pos_of.reserve(tot_inv); hk.reserve(tot_h); dj.reserve(tot_dj);
     for (int k = 0; k < count; ++k) {
         const phia_instance_desc &x = d[k];
         PackedInst &pk = packed[(size_t)k];
@@ -340,26 +413,35 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         b->csr_pub.push_back(k);
         CsrInst in{};
         in.N = n;
+        in.Np = round_up(n, 32);
         in.inst_id = x.instance_id;
         in.q = ldexpf(1.0f, -x.frac_bits);
-        in.rp_off = (int64_t)rowptr.size();
-        in.nz_off = (int64_t)col.size();
-        in.h_off = (int64_t)hk.size();
-        in.row_base = row_base;
-        rowptr.insert(rowptr.end(), pk.rp.begin(), pk.rp.end());
+        in.wide = pk.wide;
+        in.slice_base = b->total_slices;
+        in.slice_off = (int64_t)slice.size();
+        in.pos_off = (int64_t)row_of.size();
+        in.inv_off = (int64_t)pos_of.size();
+        const int32_t ent0 = (int32_t)(val.size() / 32);
+        for (int32_t e : pk.slice) slice.push_back(ent0 + e);
         col.insert(col.end(), pk.col.begin(), pk.col.end());
         val.insert(val.end(), pk.val.begin(), pk.val.end());
-        nnz_real += pk.nnz_real;
-        std::vector<int32_t>().swap(pk.rp);
-        std::vector<int32_t>().swap(pk.col);
-        std::vector<int8_t>().swap(pk.val);
-        hk.insert(hk.end(), x.h_k, x.h_k + n);
+        hk2.insert(hk2.end(), pk.hk2.begin(), pk.hk2.end());
+        row_of.insert(row_of.end(), pk.row_of.begin(), pk.row_of.end());
+        pos_of.insert(pos_of.end(), pk.pos_of.begin(), pk.pos_of.end());
+        pk = PackedInst();
+        b->max_np = std::max(b->max_np, in.Np);
+        b->total_slices += in.Np / 32;
         b->inst.push_back(in);
-        for (int i0 = 0; i0 < n; i0 += 64) b->blocks.push_back(CsrBlock{(int32_t)(b->inst.size() - 1), i0});
-        row_base += n;
     }
-    b->total_rows = row_base;
-    b->total_nnz = nnz_real;
+    for (int l = 0; l < 4; ++l)
+        for (size_t c = 0; c <= b->inst.size(); ++c) {
+            b->first_block[l].push_back((int32_t)b->blocks.size());
+            if (c < b->inst.size())
+                for (int ns = b->inst[c].Np / 32, s0 = 0; s0 < ns; s0 += 1 << l) {
+                    const int32_t *e = slice.data() + b->inst[c].slice_off;
+                    b->blocks.push_back(CsrBlock{(int32_t)c, s0, e[std::min(ns, s0 + (1 << l))] - e[s0]});
+                }
+        }
     int dev_count = 0;
     if (cudaGetDeviceCount(&dev_count) != cudaSuccess || dev_count == 0)
         return cleanup(bfail(PHIA_ECUDA, "no CUDA device available"));
@@ -373,14 +455,23 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         if (cudaMalloc(dst, std::max<size_t>(bytes, 16)) != cudaSuccess) { ok = false; return; }
         if (bytes && cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
     };
-    up((void **)&b->d_rowptr, rowptr.data(), rowptr.size() * 4);
-    up((void **)&b->d_col, col.data(), col.size() * 4);
-    up((void **)&b->d_val, val.data(), val.size());
+    up((void **)&b->d_slice, slice.data(), slice.size() * 4);
+    b->col16 = b->max_np <= 16384;
+    std::vector<uint16_t> col16;
+    if (b->col16) col16.assign(col.begin(), col.end());
+    if (b->col16) up(&b->d_col, col16.data(), col16.size() * 2);
+    else up(&b->d_col, col.data(), col.size() * 4);
+    up((void **)&b->d_val, val.data(), val.size() * 4);
+    up((void **)&b->d_hk2, hk2.data(), hk2.size() * 4);
+    up((void **)&b->d_rowof, row_of.data(), row_of.size() * 4);
+    up((void **)&b->d_posof, pos_of.data(), pos_of.size() * 4);
     up((void **)&b->d_hk, hk.data(), hk.size() * 4);
     up((void **)&b->d_blocks, b->blocks.data(), b->blocks.size() * sizeof(CsrBlock));
     up((void **)&b->d_targets, b->targets.data(), b->targets.size() * sizeof(long long));
     up((void **)&b->d_dJ, dj.data(), dj.size());
     if (ok && cudaMalloc((void **)&b->d_inst, sizeof(CsrInst) * std::max<size_t>(b->inst.size(), 1)) != cudaSuccess)
+        ok = false;
+    if (ok && cudaMalloc((void **)&b->d_sets, sizeof(CsrSet) * std::max<size_t>(b->inst.size(), 1)) != cudaSuccess)
         ok = false;
     if (ok && cudaMalloc((void **)&b->d_min_hit, 8) != cudaSuccess) ok = false;
     if (ok && cudaMalloc((void **)&b->d_start_ns, 8) != cudaSuccess) ok = false;
@@ -415,7 +506,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         if (total > ((int64_t)1 << 31)) return bfail(PHIA_ERANGE, "total_steps must be < 2^31");
     }
     if (R_real < 1) return bfail(PHIA_EINVAL, "replicas must be >= 1");
-    const int R = round_up(R_real, 256);
+    const int R = round_up(R_real, 32);
     BCU(cudaSetDevice(b->device));
     if (!field_mode && !reset && (!b->ran || b->R_real != R_real))
         return bfail(PHIA_ESTATE, "reset_best = 0 needs a previous run with the same replica count");
@@ -463,12 +554,20 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     a.hit_ns = b->d_hit_ns;
     a.min_hit = b->d_min_hit; a.replica_iters = b->d_iters; a.err = b->d_err;
     C.inst = b->d_inst; C.count = ncsr;
-    C.blocks = b->d_blocks; C.nblocks = (int32_t)b->blocks.size();
-    C.row_ptr = b->d_rowptr; C.col = b->d_col; C.val = b->d_val; C.hk = b->d_hk;
+    C.blocks = b->d_blocks;
+    if (ncsr > 0 && b->sets_R != R) {
+        rc = make_sets(b, R);
+        if (rc) return rc;
+    }
+    C.sets = b->d_sets;
+    C.nsets = (int32_t)b->sets.size();
+    C.max_np = b->max_np;
+    C.slice = b->d_slice; C.col = b->d_col; C.col16 = b->col16 ? 1 : 0; C.val = b->d_val; C.hk = b->d_hk2;
+    C.row_of = b->d_rowof; C.pos_of = b->d_posof;
     C.X = b->d_X; C.V = b->d_V;
     C.x_in = x_in; C.v_in = v_in; C.x_out = x_out; C.v_out = v_out;
     C.S = b->d_S;
-    C.total_swords = b->total_rows * (R / 32);
+    C.total_swords = b->total_slices * 32 * (R / 32);
     C.Esum = b->d_Esum; C.flags = b->d_flags; C.total_reps = reps;
     C.best_bits = b->d_bits;
     // per-instance targets: the instance's own, else the schedule's (CSR members, by CSR index)
@@ -485,7 +584,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     }
     C.R = R; C.R_real = R_real;
     C.max_words = b->max_words;
-    C.total_rows = b->total_rows;
+    C.total_slices = b->total_slices;
     // Small dense members: a table of CTAs (8 replicas each) per (operand, spin tiles)
     // group, every instance's own couplings, field, scale, Philox id, target and records.
     std::vector<std::pair<size_t, size_t>> groups;   // [begin, end) in small_host
@@ -537,7 +636,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     C.sync = b->d_sync;
     C.persistent = (b->csr_mode == 1 && !field_mode) ? 1 : 0;
     if (ncsr > 0) {
-        cudaError_t e = launch_csr(C, b->graphs, b->stream, &launches);
+        cudaError_t e = launch_csr(C, b->set_max, b->graphs, b->stream, &launches);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
     }
     for (size_t gi = 0; gi < groups.size(); ++gi) {
@@ -748,7 +847,8 @@ void phia_batch_destroy(phia_batch_t *b) {
     cudaSetDevice(b->device);
     cudaStreamSynchronize(b->stream);
     free_state(b);
-    cudaFree(b->d_inst); cudaFree(b->d_blocks); cudaFree(b->d_rowptr); cudaFree(b->d_col); cudaFree(b->d_val);
+    cudaFree(b->d_inst); cudaFree(b->d_blocks); cudaFree(b->d_slice); cudaFree(b->d_col); cudaFree(b->d_val);
+    cudaFree(b->d_sets); cudaFree(b->d_hk2); cudaFree(b->d_rowof); cudaFree(b->d_posof);
     cudaFree(b->d_hk); cudaFree(b->d_targets); cudaFree(b->d_min_hit); cudaFree(b->d_start_ns); cudaFree(b->d_iters); cudaFree(b->d_err);
     cudaFree(b->d_dJ); cudaFree(b->d_small); cudaFree(b->d_sync);
     cudaFree(b->d_ctl);

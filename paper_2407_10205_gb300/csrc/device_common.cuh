@@ -102,6 +102,35 @@ __device__ __forceinline__ float momentum_quad(float v, float x, float I, float 
     return __fmaf_rn(eps, __fmaf_rn(f, I, -x), v);
 }
 
+// All ones when s = sgn x is -1 (x < 0 or NaN), 0 when it is +1 (x >= 0, both zeros).
+__device__ __forceinline__ uint32_t minus_mask(float x) {
+    uint32_t m;
+    asm("set.ltu.u32.f32 %0, %1, 0f00000000;" : "=r"(m) : "f"(x));
+    return m;
+}
+
+// The momentum update in two parts, v' = fma(eps, fma(f, I, -x), v) with the derivative factor
+// f = beta gamma q (1 - tanh^2(gamma x)) or its stand-in: f depends on the position alone, so
+// it is at hand before the field is.  The same operations in the same order as momentum_exact
+// and momentum_quad, so the same bits.
+__device__ __forceinline__ float factor_exact(float x, float bgq4, float gamma) {
+    const float e = ex2_approx(-fabsf(__fmul_rn(2.8853900817779268f, __fmul_rn(gamma, x))));
+    const float d = __fadd_rn(1.0f, e);
+    return __fmul_rn(bgq4, __fmul_rn(e, rcp_approx(__fmul_rn(d, d))));
+}
+__device__ __forceinline__ float factor_quad(float x, float bgq, float gamma) {
+    const float u = __fmul_rn(__fmul_rn(gamma, x), 0.6666667f);
+    return __fmul_rn(bgq, fmaxf(0.0f, __fmaf_rn(-u, u, 1.0f)));
+}
+__device__ __forceinline__ float momentum_of(float v, float x, float I, float f, float eps) {
+    return __fmaf_rn(eps, __fmaf_rn(f, I, -x), v);
+}
+
+// Spins of two elements as a bf16 pair (+1 / -1 from their minus masks).
+__device__ __forceinline__ uint32_t spins2_bf16(uint32_t m0, uint32_t m1) {
+    return 0x3F803F80u ^ (__byte_perm(m0, m1, 0x5410) & 0x80008000u);
+}
+
 __device__ __forceinline__ float momentum_update(float v, float x, float I, float eps, float bgq, float gamma,
                                                  int deriv) {
     return deriv == 1 ? momentum_quad(v, x, I, eps, bgq, gamma) : momentum_exact(v, x, I, eps, bgq, gamma);
@@ -342,6 +371,11 @@ __device__ __forceinline__ void cp_async_4(void *dst, const void *src, bool vali
 __device__ __forceinline__ uint64_t l2_evict_last_policy() {
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ uint64_t l2_evict_normal_policy() {
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
 // 16-byte global store (16-byte aligned) under an L2 policy from createpolicy.

@@ -1,20 +1,39 @@
-// k_csr.cu -- sparse PHIA path: many instances of uneven N in one launch per iteration,
-// the field I = J s + h (Eq. 6) gathered warp-per-row from CSR couplings over
-// bit-packed spins, fused with the update of Eqs. 5, 8 and A7.
+// k_csr.cu -- sparse PHIA path: many instances of uneven N, the field I = J s + h (Eq. 6)
+// gathered from bit-packed spins with a row to a lane, fused with the update of Eqs. 5, 8 and
+// A7; one launch per iteration, or one cooperative launch per run.
 //
-// Layout per instance b (N_b spins, R replicas, R a multiple of 256):
-//   spins   4 rotating buffers of uint32 [N_b][R/32]: bit r%32 of word r/32 of row j is
-//           (s_j of replica r = +1); iteration t reads buffer t%4, writes t+1%4.
-//   x, v    float32 [N_b][R] (spin-major, so a row's 256 replicas are 1 KB contiguous)
-//   best    uint32 [R][ceil(N_b/32)] bit-packed over spins (as on every path)
-// Work unit: a block of 64 consecutive rows of one instance and 256 replicas; a warp
-// takes 8 rows, a lane 8 replicas (one byte of each spin row).
-// For a row i and its entries (j, k): acc_r = sum k [s_j^r = +1], ksum = sum k, so
-// I_r = 2 acc_r - ksum + kh_i (exact integers).  Energy partials s_i (I_i + h_i) are
-// reduced per block in shared memory and added to a per-(instance, replica) int64 sum.
-// Records are lagged as in the dense per-iteration kernel: the launch for iteration t
-// settles t-1 (block 0 of each instance) and copies the spins of t-2 for the replicas
-// that improved then (every block, its 64 rows).
+// Layout per instance b.  Rows (spins) are held in positions: sorted by their number of
+// couplings, descending, so that the 32 rows of a slice have about equally many; Np = N
+// rounded up to 32, positions past N are empty.  Replicas go in groups of 32.
+//   spins     4 rotating buffers of uint32 [group][Np]: bit r of word p = (the spin at position
+//             p of replica 32 group + r is +1); iteration t reads buffer t % 4, writes t+1 % 4
+//   x, v      float32 [group][8][Np][4]: 4 replicas of one row sit together, so that a lane
+//             moves them as one vector and a warp's vector covers 512 contiguous bytes
+//   couplings per slice, for every 4 neighbours of its rows: 4 byte offsets of their positions in
+//             a spin buffer (16 bits each while every Np <= 16384, else 32) and 4 x int8, one
+//             entry per lane
+//   best      uint32 [R][ceil(N/32)] bit-packed over spins in their own order
+//
+// A warp takes a slice (32 rows, one per lane) and a group of 32 replicas.  For 4 neighbours a
+// lane reads 4 words (32 replicas each) from the block's shared-memory copy of the group's
+// spins, turns them into 8-replica bytes (a 4 x 4 byte transpose) and adds, for each replica,
+// (bytes & 2^b) . (4 couplings) with one 4-way dot product: acc_r = 2^b sum k [s = +1], b = r
+// % 8.  With ksum the row's sum of couplings, I_r = 2 sum k [s = +1] - ksum + kh, exactly.
+//
+// What bounds it: the instructions of the gather (per 4 neighbours and 32 rows x 32 replicas
+// 32 dot products, 32 masks, 8 byte permutes, 4 shared loads) and of the update, with the x, v
+// stream (16 bytes per spin update) behind them.  The earlier form took a row to a warp and 8
+// replicas to a lane: every neighbour cost the warp a load of 32 bytes, its address and its
+// share of the byte permutes for 8 replicas a lane instead of 32.  Per iteration (us), that
+// form and this one: 48 Erdos-Renyi instances of 100 .. 3000 spins x 256 replicas 166 / 139, 12
+// of them x 256 44 / 26, one of 5000 spins x 256 27 / 15, where the longest slice sets the time.
+//
+// The instances go through their iterations in sets whose state fits in L2 together: a set runs
+// all of its iterations before the next begins (the instances are independent), so x and v are
+// read from L2 instead of the memory they would fall out to between two iterations of a batch.
+//
+// Records are lagged: the launch for iteration t settles t - 1 (the instance's first unit)
+// and copies the best spins of t - 2 for the replicas that improved then.
 #include <algorithm>
 
 #include "device_common.cuh"
@@ -24,17 +43,15 @@ namespace phia {
 
 namespace {
 
-constexpr int kRowsPerBlock = 64;
 constexpr int kWarps = 8;
-constexpr int kRowsPerWarp = kRowsPerBlock / kWarps;
-constexpr int kGroup = 256;          // replicas per block (8 per lane)
+constexpr int kBlk = 32 * kWarps;
 
 __device__ __forceinline__ void settle_csr(const CsrArgs &C, const CsrInst &in, int b, int r, int64_t tt) {
     const RunArgs &a = C.a;
     const size_t rec = (size_t)in.rec_off + r;
     unsigned long long *slot =
         reinterpret_cast<unsigned long long *>(C.Esum) + (size_t)(tt & 1) * C.total_reps + rec;
-    const long long twice = (long long)*slot;
+    const long long twice = (long long)__ldcg(slot);
     *slot = 0ull;
     const long long E = -twice / 2;
     int imp = 0;
@@ -50,167 +67,248 @@ __device__ __forceinline__ void settle_csr(const CsrArgs &C, const CsrInst &in, 
         if (a.hit_ns) a.hit_ns[rec] = globaltimer_ns();
     }
     C.flags[(size_t)(tt & 1) * C.total_reps + rec] = (int8_t)imp;
-    (void)b;
 }
 
-__device__ __forceinline__ const uint32_t *spin_buf(const CsrArgs &C, const CsrInst &in, int64_t tt) {
+__device__ __forceinline__ uint32_t *spin_buf(const CsrArgs &C, const CsrInst &in, int64_t tt) {
     return C.S + (size_t)(tt & 3) * C.total_swords + in.s_off;
 }
 
-// One work unit of iteration t: 64 rows (block `bi` of the list) x 256 replicas (group g).
-// Uses the block's shared arrays; every thread of the block calls it.
-__device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int g, int64_t t, int64_t t_first, int64_t t_end,
-                                         int32_t (*part)[kGroup], uint32_t (*sbits)[kGroup / 32]) {
+// 4 x 4 byte transpose: byte b of word k of the result is byte k of word b of the input, i.e.
+// word k holds the four neighbours' bytes of replicas 8k .. 8k + 7.
+__device__ __forceinline__ void transpose4(const uint32_t (&w)[4], uint32_t (&B)[4]) {
+    const uint32_t a = __byte_perm(w[0], w[1], 0x5140), b = __byte_perm(w[2], w[3], 0x5140);
+    const uint32_t c = __byte_perm(w[0], w[1], 0x7362), d = __byte_perm(w[2], w[3], 0x7362);
+    B[0] = __byte_perm(a, b, 0x5410);
+    B[1] = __byte_perm(a, b, 0x7632);
+    B[2] = __byte_perm(c, d, 0x5410);
+    B[3] = __byte_perm(c, d, 0x7632);
+}
+
+// d + sum over 4 bytes of (unsigned byte of a) x (signed byte of b).
+__device__ __forceinline__ int32_t dp4a_us(uint32_t a, uint32_t b, int32_t d) {
+    asm("dp4a.u32.s32 %0, %1, %2, %0;" : "+r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// One entry of a lane's row: the byte offsets of 4 neighbours' spin words (16 or 32 bits each)
+// and their couplings.
+template <bool C16>
+struct Entry {
+    uint2 c;
+    uint32_t k;
+    __device__ __forceinline__ void load(const CsrArgs &C, int e, int lane) {
+        c = __ldg(reinterpret_cast<const uint2 *>(C.col) + (size_t)e * 32 + lane);
+        k = __ldg(C.val + (size_t)e * 32 + lane);
+    }
+    __device__ __forceinline__ uint32_t at(int n) const { return n & 1 ? (n & 2 ? c.y : c.x) >> 16 : (n & 2 ? c.y : c.x) & 0xffffu; }
+};
+template <>
+struct Entry<false> {
+    uint4 c;
+    uint32_t k;
+    __device__ __forceinline__ void load(const CsrArgs &C, int e, int lane) {
+        c = __ldg(reinterpret_cast<const uint4 *>(C.col) + (size_t)e * 32 + lane);
+        k = __ldg(C.val + (size_t)e * 32 + lane);
+    }
+    __device__ __forceinline__ uint32_t at(int n) const { return n == 0 ? c.x : n == 1 ? c.y : n == 2 ? c.z : c.w; }
+};
+
+// acc[r] of the lane's row over its couplings: entries [e, e_end) of the slice, 4 neighbours
+// each; the next entries load meanwhile (three ahead with 16-bit offsets, whose registers allow
+// it: an entry's L2 latency is several times its arithmetic).  SCALED: acc_r carries the factor
+// 2^(r % 8) of its bit's place (one instruction less per replica); rows of over 2^16 couplings
+// take the bit down to place 0 instead, as the factor could leave 32 bits.
+template <bool SMEM, bool C16, bool SCALED>
+__device__ __forceinline__ void gather_row(const CsrArgs &C, const char *spins, int e, int e_end, int lane,
+                                           int32_t (&acc)[32]) {
+    constexpr int D = C16 ? 3 : 1;
+    Entry<C16> nx[D];
+#pragma unroll
+    for (int u = 0; u < D; ++u)
+        if (e + u < e_end) nx[u].load(C, e + u, lane);
+#pragma unroll 1
+    for (; e < e_end; e += D) {
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            if (u > 0 && e + u >= e_end) break;
+            const Entry<C16> en = nx[u];
+            if (e + u + D < e_end) nx[u].load(C, e + u + D, lane);
+            uint32_t w[4], B[4];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                if constexpr (SMEM) w[n] = *reinterpret_cast<const uint32_t *>(spins + en.at(n));
+                else w[n] = __ldcg(reinterpret_cast<const uint32_t *>(spins + en.at(n)));
+            }
+            transpose4(w, B);
+#pragma unroll
+            for (int r = 0; r < 32; ++r) {
+                const int bit = r & 7;
+                if constexpr (SCALED) acc[r] = dp4a_us(B[r >> 3] & (0x01010101u << bit), en.k, acc[r]);
+                else acc[r] = dp4a_us((B[r >> 3] >> bit) & 0x01010101u, en.k, acc[r]);
+            }
+        }
+    }
+}
+
+// One work unit of iteration t: C.slices slices of an instance (block `bi` of the list) x
+// C.gblock groups of 32 replicas (the y-th such set).  Uses the block's shared memory; every
+// thread of the block calls it.
+template <bool SMEM, bool C16>
+__device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_t t, int64_t t_first, int64_t t_end,
+                                         char *smem) {
     const RunArgs &a = C.a;
     const CsrBlock blk = C.blocks[bi];
     const CsrInst in = C.inst[blk.inst];
     const int b = blk.inst;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int N = in.N, R = C.R, RW = R / 32;
+    const int G = C.gblock, groups = C.R / 32;
+    const int gi = warp % G, sp = warp / G, spar = kWarps / G;     // group and slice lane of this warp
+    const int g = y * G + gi;
+    const bool active = g < groups;
+    const int nsl = in.Np / 32;
+    const int s_end = min(nsl, blk.s0 + C.slices);
 
-    // (a) records of iteration t-1 (block 0 of each instance).
-    if (blk.i0 == 0 && t - 1 >= t_first) settle_csr(C, in, b, g * kGroup + tid, t - 1);
-    // (b) best spins of iteration t-2 for the replicas that improved then: this block's
-    //     64 rows of spin bits go through shared memory, one thread per replica.
-    if (t - 2 >= t_first) {
-        const int rows = min(kRowsPerBlock, N - blk.i0);
-        const uint32_t *Sb = spin_buf(C, in, t - 2);
-        for (int e = tid; e < kRowsPerBlock * 8; e += 32 * kWarps) {
-            const int row = e >> 3, w = e & 7;
-            sbits[row][w] = row < rows ? Sb[(size_t)(blk.i0 + row) * RW + g * 8 + w] : 0u;
+    // The spins of this iteration of the block's groups into shared memory.
+    const uint32_t *Sg = spin_buf(C, in, t);
+    if constexpr (SMEM) {
+        const int words = min(G, groups - y * G) * in.Np;          // consecutive in the buffer
+        const uint32_t *src = Sg + (size_t)y * G * in.Np;
+        for (int e = tid * 4; e < words; e += kBlk * 4) cp_async_16(smem + (size_t)e * 4, src + e);
+        cp_async_commit();
+    }
+    // (a) records of iteration t-1 (the first block of each instance).
+    if (blk.s0 == 0 && t - 1 >= t_first) {
+        for (int e = tid; e < G * 32; e += kBlk)
+            if (y * G * 32 + e < C.R) settle_csr(C, in, b, y * G * 32 + e, t - 1);
+    }
+    // (b) best spins of iteration t-2 for the replicas that improved then: this block's share
+    //     of the words of the best state, a spin to a lane.
+    if (active && t - 2 >= t_first) {
+        const bool imp = __ldcg(C.flags + (size_t)((t - 2) & 1) * C.total_reps + in.rec_off + g * 32 + lane) != 0;
+        const uint32_t mask = __ballot_sync(0xffffffffu, imp);
+        if (mask) {
+            const uint32_t *Sb = spin_buf(C, in, t - 2) + (size_t)g * in.Np;
+            const int W = (in.N + 31) / 32;
+            for (int w = blk.s0 + sp; w < s_end; w += spar) {
+                const int i = w * 32 + lane;
+                const uint32_t word = i < in.N ? __ldcg(Sb + C.pos_of[in.inv_off + i]) : 0u;
+                for (uint32_t m = mask; m; m &= m - 1) {
+                    const int r = __ffs(m) - 1;
+                    const uint32_t bits = __ballot_sync(0xffffffffu, (word >> r) & 1u);
+                    if (lane == 0) C.best_bits[in.bits_off + (size_t)(g * 32 + r) * W + w] = bits;
+                }
+            }
         }
+    }
+    if constexpr (SMEM) {
+        cp_async_wait<0>();
         __syncthreads();
-        const int r = g * kGroup + tid;
-        if (C.flags[(size_t)((t - 2) & 1) * C.total_reps + in.rec_off + r]) {
-            const int W = (N + 31) / 32;
-            uint32_t w0 = 0, w1 = 0;
-            for (int row = 0; row < 32; ++row) w0 |= ((sbits[row][tid >> 5] >> (tid & 31)) & 1u) << row;
-            for (int row = 32; row < 64; ++row) w1 |= ((sbits[row][tid >> 5] >> (tid & 31)) & 1u) << (row - 32);
-            uint32_t *dst = C.best_bits + in.bits_off + (size_t)r * W;
-            const int word = blk.i0 / 32;
-            dst[word] = w0;
-            if (word + 1 < W) dst[word + 1] = w1;
-        }
     }
-
-    // (c) field and update, 8 rows per warp, 8 replicas per lane.
-    const uint8_t *Scur = reinterpret_cast<const uint8_t *>(spin_buf(C, in, t));
-    uint32_t *Snext = const_cast<uint32_t *>(spin_buf(C, in, t + 1));
-    const float bgq = beta_at(t, inv_tm1_of(a.T_total), a.beta0, a.beta1) * (a.gamma * in.q);
-    const float eps = a.eps, gamma = a.gamma;
-    const bool more = t + 1 < t_end;
-    const bool refresh_next = more && refresh_at(t + 1, a.refresh);
-    const int r0 = g * kGroup + lane * 8;          // first replica of this lane
-    int32_t epart[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int q = 0; q < kRowsPerWarp; ++q) {
-        const int i = blk.i0 + warp * kRowsPerWarp + q;
-        if (i >= N) break;
-        const int p_beg = C.row_ptr[in.rp_off + i], p_end = C.row_ptr[in.rp_off + i + 1];
-        // acc_r = sum_j k_j [s_j^r = +1] for this lane's 8 replicas r.  Rows are padded to
-        // multiples of 8 entries (k = 0), so the warp reads 8 columns and 8 couplings at
-        // a time with broadcast vector loads.  The spin bytes of 4 neighbours form one
-        // word B; (B >> r) & 0x01010101 holds replica r's four bits, one per byte, and a
-        // 4-way int8 dot product with the four couplings adds k [s = +1] for all four.
-        const int32_t *colp = C.col + in.nz_off;
-        const int8_t *valp = C.val + in.nz_off;
-        const uint8_t *Sl = Scur + g * 32 + lane;     // this lane's byte of spin row 0
-        const size_t rowb = (size_t)RW * 4;           // bytes per spin row
-        int32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        int32_t ksum = 0;
-        // The next round's columns and couplings load while this round's spins do.
-        int4 c0n = make_int4(0, 0, 0, 0), c1n = c0n;
-        int2 kkn = make_int2(0, 0);
-        if (p_beg < p_end) {
-            c0n = *reinterpret_cast<const int4 *>(colp + p_beg);
-            c1n = *reinterpret_cast<const int4 *>(colp + p_beg + 4);
-            kkn = *reinterpret_cast<const int2 *>(valp + p_beg);
-        }
-        for (int p = p_beg; p < p_end; p += 8) {
-            const int4 c0 = c0n, c1 = c1n;
-            const int2 kk = kkn;
-            if (p + 8 < p_end) {
-                c0n = *reinterpret_cast<const int4 *>(colp + p + 8);
-                c1n = *reinterpret_cast<const int4 *>(colp + p + 12);
-                kkn = *reinterpret_cast<const int2 *>(valp + p + 8);
+    // (c) field and update.
+    if (active) {
+        const char *spins = SMEM ? smem + (size_t)gi * in.Np * 4 : reinterpret_cast<const char *>(Sg + (size_t)g * in.Np);
+        uint32_t *Snext = spin_buf(C, in, t + 1) + (size_t)g * in.Np;
+        const float bgq = beta_at(t, inv_tm1_of(a.T_total), a.beta0, a.beta1) * (a.gamma * in.q);
+        const float eps = a.eps, gamma = a.gamma, bgq4 = 4.0f * bgq;
+        const bool more = t + 1 < t_end;
+        const bool refresh_next = more && refresh_at(t + 1, a.refresh);
+        long long esum = 0;                            // replica `lane` of the group
+        for (int s = blk.s0 + sp; s < s_end; s += spar) {
+            const int p = s * 32 + lane;
+            float *X = C.X + in.x_off + ((size_t)g * 8 * in.Np + p) * 4;
+            float *V = C.V + in.x_off + ((size_t)g * 8 * in.Np + p) * 4;
+            const size_t qs = (size_t)in.Np * 4;       // floats between quads of replicas
+            // x and v of the group's first 8 replicas load while the gather runs, the others two quads
+            // ahead of their use.
+            float4 xq[2], vq[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                xq[k] = *reinterpret_cast<const float4 *>(X + k * qs);
+                vq[k] = *reinterpret_cast<const float4 *>(V + k * qs);
             }
-            const uint32_t s0 = Sl[(size_t)c0.x * rowb], s1 = Sl[(size_t)c0.y * rowb];
-            const uint32_t s2 = Sl[(size_t)c0.z * rowb], s3 = Sl[(size_t)c0.w * rowb];
-            const uint32_t s4 = Sl[(size_t)c1.x * rowb], s5 = Sl[(size_t)c1.y * rowb];
-            const uint32_t s6 = Sl[(size_t)c1.z * rowb], s7 = Sl[(size_t)c1.w * rowb];
-            const uint32_t B0 = __byte_perm(__byte_perm(s0, s1, 0x0040), __byte_perm(s2, s3, 0x0040), 0x5410);
-            const uint32_t B1 = __byte_perm(__byte_perm(s4, s5, 0x0040), __byte_perm(s6, s7, 0x0040), 0x5410);
-            ksum = __dp4a(kk.x, 0x01010101, ksum);
-            ksum = __dp4a(kk.y, 0x01010101, ksum);
+            int32_t acc[32];
 #pragma unroll
-            for (int rr = 0; rr < 8; ++rr) {
-                acc[rr] = __dp4a((int)((B0 >> rr) & 0x01010101u), kk.x, acc[rr]);
-                acc[rr] = __dp4a((int)((B1 >> rr) & 0x01010101u), kk.y, acc[rr]);
+            for (int r = 0; r < 32; ++r) acc[r] = 0;
+            const int e0 = C.slice[in.slice_off + s], e1 = C.slice[in.slice_off + s + 1];
+            if (in.wide) gather_row<SMEM, C16, false>(C, spins, e0, e1, lane, acc);
+            else gather_row<SMEM, C16, true>(C, spins, e0, e1, lane, acc);
+            const int2 hh = __ldg(reinterpret_cast<const int2 *>(C.hk) + in.pos_off + p);    // h, h - ksum
+            const int row = refresh_next ? C.row_of[in.pos_off + p] : 0;
+            uint32_t bits = 0;
+#pragma unroll
+            for (int qd = 0; qd < 8; ++qd) {
+                const float4 x4 = xq[qd & 1], v4 = vq[qd & 1];
+                if (qd < 6) {
+                    xq[qd & 1] = *reinterpret_cast<const float4 *>(X + (qd + 2) * qs);
+                    vq[qd & 1] = *reinterpret_cast<const float4 *>(V + (qd + 2) * qs);
+                }
+                int32_t e4[4];
+                float xs[4] = {x4.x, x4.y, x4.z, x4.w}, If[4];
+                float vn[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int r = qd * 4 + k, bit = r & 7;
+                    const int32_t twice = (in.wide || bit == 0) ? acc[r] << 1 : acc[r] >> (bit - 1);
+                    const int32_t I = twice + hh.y;                                   // Eq. 6, exact
+                    const int32_t m = (int32_t)minus_mask(xs[k]);
+                    const int32_t e = ((I + hh.x) ^ m) - m;                           // s (I + h)
+                    if (in.wide) {      // sums of such terms may leave 32 bits: halves apart, at once
+                        const long long es = (long long)__reduce_add_sync(0xffffffffu, e & 0xffff) +
+                                             ((long long)__reduce_add_sync(0xffffffffu, e >> 16) << 16);
+                        if (lane == r) esum += es;
+                    } else {
+                        e4[k] = e;
+                    }
+                    If[k] = (float)I;
+                }
+                if (!in.wide) {
+                    // Sums over the rows of 4 replicas: two halving exchanges leave replica lane % 4 in
+                    // a lane, three more sum it over the warp (32 warp sums would take 8 cycles each).
+                    const bool h2 = lane & 2, h1 = lane & 1;
+                    const int32_t a0 = (h2 ? e4[2] : e4[0]) + __shfl_xor_sync(0xffffffffu, h2 ? e4[0] : e4[2], 2);
+                    const int32_t a1 = (h2 ? e4[3] : e4[1]) + __shfl_xor_sync(0xffffffffu, h2 ? e4[1] : e4[3], 2);
+                    int32_t es = (h1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h1 ? a0 : a1, 1);
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
+                    if ((lane >> 2) == qd) esum += es;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float f = a.deriv == 1 ? factor_quad(xs[k], bgq, gamma) : factor_exact(xs[k], bgq4, gamma);
+                    vn[k] = momentum_of(vn[k], xs[k], If[k], f, eps);
+                }
+                if (refresh_next && row >= 0) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        vn[k] = draw_v(a.seed, in.inst_id, (uint32_t)(g * 32 + qd * 4 + k), (uint32_t)row, (uint32_t)(t + 1));
+                }
+                if (more) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        xs[k] = __fmaf_rn(eps, vn[k], xs[k]);
+                        bits |= ~minus_mask(xs[k]) & (1u << (qd * 4 + k));
+                    }
+                    *reinterpret_cast<float4 *>(X + qd * qs) = make_float4(xs[0], xs[1], xs[2], xs[3]);
+                }
+                *reinterpret_cast<float4 *>(V + qd * qs) = make_float4(vn[0], vn[1], vn[2], vn[3]);
             }
+            if (more) Snext[p] = bits;
         }
-        const int32_t hk = C.hk[in.h_off + i];
-        const size_t xo = in.x_off + (size_t)i * R + r0;
-        float4 xa = *reinterpret_cast<const float4 *>(C.X + xo);
-        float4 xb = *reinterpret_cast<const float4 *>(C.X + xo + 4);
-        float4 va = *reinterpret_cast<const float4 *>(C.V + xo);
-        float4 vb = *reinterpret_cast<const float4 *>(C.V + xo + 4);
-        float xs[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-        float vs[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
-        uint32_t nbyte = 0;
-        float If[8];
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-            const int32_t I = 2 * acc[rr] - ksum + hk;                    // Eq. 6, exact
-            epart[rr] += (xs[rr] >= 0.0f ? 1 : -1) * (I + hk);
-            If[rr] = (float)I;
-        }
-        float vn[8];
-        if (a.deriv == 1) {
-#pragma unroll
-            for (int rr = 0; rr < 8; ++rr) vn[rr] = momentum_quad(vs[rr], xs[rr], If[rr], eps, bgq, gamma);
-        } else {
-#pragma unroll
-            for (int rr = 0; rr < 8; ++rr) vn[rr] = momentum_exact(vs[rr], xs[rr], If[rr], eps, bgq, gamma);
-        }
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-            float v = vn[rr];
-            float x = xs[rr];
-            if (more) {
-                if (refresh_next) v = draw_v(a.seed, in.inst_id, (uint32_t)(r0 + rr), (uint32_t)i, (uint32_t)(t + 1));
-                x = x + eps * v;
-            }
-            xs[rr] = x;
-            vs[rr] = v;
-            nbyte |= (uint32_t)(x >= 0.0f) << rr;
-        }
-        if (more) {
-            *reinterpret_cast<float4 *>(C.X + xo) = make_float4(xs[0], xs[1], xs[2], xs[3]);
-            *reinterpret_cast<float4 *>(C.X + xo + 4) = make_float4(xs[4], xs[5], xs[6], xs[7]);
-            reinterpret_cast<uint8_t *>(Snext)[(size_t)i * (RW * 4) + g * 32 + lane] = (uint8_t)nbyte;
-        }
-        *reinterpret_cast<float4 *>(C.V + xo) = make_float4(vs[0], vs[1], vs[2], vs[3]);
-        *reinterpret_cast<float4 *>(C.V + xo + 4) = make_float4(vs[4], vs[5], vs[6], vs[7]);
+        atomicAdd(reinterpret_cast<unsigned long long *>(C.Esum) + (size_t)(t & 1) * C.total_reps + in.rec_off + g * 32 + lane,
+                  (unsigned long long)esum);
     }
-#pragma unroll
-    for (int rr = 0; rr < 8; ++rr) part[warp][lane * 8 + rr] = epart[rr];
-    __syncthreads();
-    {
-        long long s = 0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) s += part[w][tid];
-        atomicAdd(reinterpret_cast<unsigned long long *>(C.Esum) + (size_t)(t & 1) * C.total_reps + in.rec_off +
-                      g * kGroup + tid,
-                  (unsigned long long)s);
-    }
-    __syncthreads();   // the shared arrays are free for the next unit
+    if constexpr (SMEM) __syncthreads();   // the shared spins are free for the next unit
 }
 
-// One launch per iteration: a block per work unit; the iteration comes from C.ctl.
-__global__ void __launch_bounds__(32 * kWarps, 4) csr_step(const CsrArgs C) {
-    __shared__ int32_t part[kWarps][kGroup];
-    __shared__ uint32_t sbits[kRowsPerBlock][kGroup / 32];
+// One launch per iteration of a set of instances: a block per work unit (the grid is that of
+// the largest set); the iteration and the set come from C.ctl.
+template <bool SMEM, bool C16>
+__global__ void __launch_bounds__(kBlk, 2) csr_step(const CsrArgs C) {
+    extern __shared__ __align__(16) char smem[];
     const int64_t t = C.ctl->t, t_first = C.ctl->t_first, t_end = C.ctl->t_end;
-    csr_unit(C, blockIdx.x, blockIdx.y, t, t_first, t_end, part, sbits);
+    const CsrSet set = C.sets[C.ctl->set];
+    if ((int)blockIdx.x < set.len[C.list]) csr_unit<SMEM, C16>(C, set.off[C.list] + blockIdx.x, blockIdx.y, t, t_first, t_end, smem);
+    __syncthreads();
     if (threadIdx.x == 0) iter_ctl_finish(C.ctl);
 }
 
@@ -239,92 +337,121 @@ __device__ bool grid_barrier(unsigned *bar, uint64_t timeout_ns) {
     return __syncthreads_and(ok) != 0;
 }
 
-// All iterations of the run in one cooperative launch: per iteration every block takes
-// work units from a counter (units of uneven cost balance themselves), then the grid
-// meets at a barrier.  ctr[t & 1] hands out iteration t's units; the last block to reach
-// the barrier after iteration t clears it for t + 2.
-__global__ void __launch_bounds__(32 * kWarps, 4) csr_persistent(const CsrArgs C, unsigned *bar, unsigned *ctr) {
-    __shared__ int32_t part[kWarps][kGroup];
-    __shared__ uint32_t sbits[kRowsPerBlock][kGroup / 32];
+// All iterations of the run in one cooperative launch, set after set: per iteration every block
+// takes work units from a counter (units of uneven cost balance themselves), then the grid
+// meets at a barrier.  ctr[k & 1] hands out the units of the launch's k-th iteration; block 0
+// clears it after that iteration's barrier, before it is used again.
+template <bool SMEM, bool C16>
+__global__ void __launch_bounds__(kBlk, 2) csr_persistent(const CsrArgs C, unsigned *bar, unsigned *ctr) {
+    extern __shared__ __align__(16) char smem[];
     __shared__ int unit;
     const int64_t t_first = C.a.t0, t_end = C.a.t0 + C.a.nsteps;
-    const int groups = C.R / kGroup, units = C.nblocks * groups;
-    for (int64_t t = t_first; t < t_end; ++t) {
-        for (;;) {
-            if (threadIdx.x == 0) unit = (int)atomicAdd(&ctr[t & 1], 1u);
-            __syncthreads();
-            const int u = unit;
-            __syncthreads();
-            if (u >= units) break;
-            csr_unit(C, u % C.nblocks, u / C.nblocks, t, t_first, t_end, part, sbits);
+    const int ny = (C.R / 32 + C.gblock - 1) / C.gblock;
+    int k = 0;
+    for (int sidx = 0; sidx < C.nsets; ++sidx) {
+        const CsrSet set = C.sets[sidx];
+        const int nb = set.len[C.list], units = nb * ny;
+        for (int64_t t = t_first; t < t_end; ++t, k ^= 1) {
+            for (;;) {
+                if (threadIdx.x == 0) unit = (int)atomicAdd(&ctr[k], 1u);
+                __syncthreads();
+                const int u = unit;
+                __syncthreads();
+                if (u >= units) break;
+                csr_unit<SMEM, C16>(C, set.off[C.list] + u % nb, u / nb, t, t_first, t_end, smem);
+            }
+            if (!grid_barrier(bar, kWaitTimeoutNs)) {
+                if (threadIdx.x == 0) atomicExch(C.a.err, 1);
+                return;
+            }
+            if (blockIdx.x == 0 && threadIdx.x == 0) ctr[k] = 0u;
         }
-        // The counter of iteration t is cleared once every block has left it: the barrier
-        // below waits for all; block 0 clears it after the barrier, before iteration t + 2.
-        if (!grid_barrier(bar, kWaitTimeoutNs)) {
-            if (threadIdx.x == 0) atomicExch(C.a.err, 1);
-            return;
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) ctr[t & 1] = 0u;
     }
 }
 
-// Initial state (or given, [R][N] per instance), refresh at t0, first position update,
-// spins of iteration t0.  One thread per (instance-spin row, lane of 8 replicas).
-__global__ void csr_prologue(const CsrArgs C) {
-    const RunArgs &a = C.a;
-    const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over total_rows * R / 8
-    if (gidx == 0) iter_ctl_start(C.ctl, a.t0, a.nsteps);
-    const int R = C.R, per_row = R / 8;
-    const int64_t row = gidx / per_row;
-    if (row >= C.total_rows) return;
-    const int l8 = (int)(gidx - row * per_row);
-    // find the instance of this global row (rows are stored instance after instance)
+// Iteration control back to the run's start, for the next set of instances.
+__global__ void csr_next_set(IterCtl *ctl, int64_t t0, int64_t nsteps, int32_t set) {
+    iter_ctl_start(ctl, t0, nsteps);
+    ctl->set = set;
+}
+
+// The instance that holds global slice gs (slices are numbered instance after instance).
+__device__ __forceinline__ int instance_of(const CsrArgs &C, int64_t gs) {
     int lo = 0, hi = C.count - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (C.inst[mid].row_base <= row) lo = mid; else hi = mid - 1;
+        if (C.inst[mid].slice_base <= gs) lo = mid; else hi = mid - 1;
     }
-    const CsrInst in = C.inst[lo];
-    const int i = (int)(row - in.row_base);
-    uint32_t byte = 0;
-    for (int rr = 0; rr < 8; ++rr) {
-        const int r = l8 * 8 + rr;
-        float x, v;
-        if (C.x_in && r < C.R_real) {
-            x = C.x_in[in.xin_off + (size_t)r * in.N + i];
-            v = C.v_in[in.xin_off + (size_t)r * in.N + i];
-        } else {
-            const U4 o = draw_raw(a.seed, in.inst_id, (uint32_t)r, (uint32_t)i, 0u);
-            x = box_muller(o.x, o.y);
-            v = box_muller(o.z, o.w);
+    return lo;
+}
+
+// Initial state (or given, [R][N] per instance), refresh at t0, first position update, spins
+// of iteration t0.  A block per (slice, group): a warp per 4 replicas, a lane per row.
+__global__ void __launch_bounds__(kBlk) csr_prologue(const CsrArgs C) {
+    __shared__ uint32_t part[8][32];
+    const RunArgs &a = C.a;
+    const int groups = C.R / 32;
+    const int64_t gs = blockIdx.x / groups;
+    const int g = (int)(blockIdx.x % groups);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        iter_ctl_start(C.ctl, a.t0, a.nsteps);
+        C.ctl->set = 0;
+    }
+    const CsrInst in = C.inst[instance_of(C, gs)];
+    const int qd = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int p = (int)(gs - in.slice_base) * 32 + lane;
+    const int row = C.row_of[in.pos_off + p];
+    float x[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
+    uint32_t bits = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = g * 32 + qd * 4 + k;
+        if (row >= 0) {
+            if (C.x_in && r < C.R_real) {
+                x[k] = C.x_in[in.xin_off + (size_t)r * in.N + row];
+                v[k] = C.v_in[in.xin_off + (size_t)r * in.N + row];
+            } else {
+                const U4 o = draw_raw(a.seed, in.inst_id, (uint32_t)r, (uint32_t)row, 0u);
+                x[k] = box_muller(o.x, o.y);
+                v[k] = box_muller(o.z, o.w);
+            }
+            if (refresh_at(a.t0, a.refresh)) v[k] = draw_v(a.seed, in.inst_id, (uint32_t)r, (uint32_t)row, (uint32_t)a.t0);
+            x[k] = x[k] + a.eps * v[k];
         }
-        if (refresh_at(a.t0, a.refresh)) v = draw_v(a.seed, in.inst_id, (uint32_t)r, (uint32_t)i, (uint32_t)a.t0);
-        x = x + a.eps * v;
-        C.X[in.x_off + (size_t)i * R + r] = x;
-        C.V[in.x_off + (size_t)i * R + r] = v;
-        byte |= (uint32_t)(x >= 0.0f) << rr;
+        bits |= ~minus_mask(x[k]) & (1u << (qd * 4 + k));
     }
-    uint8_t *S = reinterpret_cast<uint8_t *>(const_cast<uint32_t *>(spin_buf(C, in, a.t0)));
-    S[(size_t)i * (R / 8) + l8] = (uint8_t)byte;
+    const size_t off = in.x_off + ((size_t)(g * 8 + qd) * in.Np + p) * 4;
+    *reinterpret_cast<float4 *>(C.X + off) = make_float4(x[0], x[1], x[2], x[3]);
+    *reinterpret_cast<float4 *>(C.V + off) = make_float4(v[0], v[1], v[2], v[3]);
+    part[qd][lane] = bits;
+    __syncthreads();
+    if (qd == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) bits |= part[w][lane];
+        spin_buf(C, in, a.t0)[(size_t)g * in.Np + p] = bits;
+    }
 }
 
 // Final state back to [R][N] per instance (caller layout).
-__global__ void csr_export(const CsrArgs C) {
-    const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over total_rows * R
-    const int R = C.R;
-    const int64_t row = gidx / R;
-    if (row >= C.total_rows) return;
-    const int r = (int)(gidx - row * R);
-    int lo = 0, hi = C.count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (C.inst[mid].row_base <= row) lo = mid; else hi = mid - 1;
+__global__ void __launch_bounds__(kBlk) csr_export(const CsrArgs C) {
+    const int groups = C.R / 32;
+    const int64_t gs = blockIdx.x / groups;
+    const int g = (int)(blockIdx.x % groups);
+    const CsrInst in = C.inst[instance_of(C, gs)];
+    const int qd = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int p = (int)(gs - in.slice_base) * 32 + lane;
+    const int row = C.row_of[in.pos_off + p];
+    if (row < 0) return;
+    const size_t off = in.x_off + ((size_t)(g * 8 + qd) * in.Np + p) * 4;
+    const float4 x4 = *reinterpret_cast<const float4 *>(C.X + off), v4 = *reinterpret_cast<const float4 *>(C.V + off);
+    const float x[4] = {x4.x, x4.y, x4.z, x4.w}, v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = g * 32 + qd * 4 + k;
+        if (r >= C.R_real) continue;
+        C.x_out[in.xin_off + (size_t)r * in.N + row] = x[k];
+        C.v_out[in.xin_off + (size_t)r * in.N + row] = v[k];
     }
-    const CsrInst in = C.inst[lo];
-    const int i = (int)(row - in.row_base);
-    if (r >= C.R_real) return;
-    C.x_out[in.xin_off + (size_t)r * in.N + i] = C.X[in.x_off + (size_t)i * R + r];
-    C.v_out[in.xin_off + (size_t)r * in.N + i] = C.V[in.x_off + (size_t)i * R + r];
 }
 
 __global__ void csr_settle_all(const CsrArgs C, int64_t tt) {
@@ -333,49 +460,55 @@ __global__ void csr_settle_all(const CsrArgs C, int64_t tt) {
     for (int r = threadIdx.x; r < C.R; r += blockDim.x) settle_csr(C, in, b, r, tt);
 }
 
-// Copies for iterations not handled by a later launch; one thread per (replica, word).
-__global__ void csr_copy_all(const CsrArgs C, int64_t t_from, int64_t t_last) {
-    const int b = blockIdx.y;
-    const CsrInst in = C.inst[b];
-    const int W = (in.N + 31) / 32;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)C.R * W) return;
-    const int r = (int)(idx / W), w = (int)(idx - (int64_t)r * W);
+// Copies for iterations not handled by a later launch; a warp per (word of the best state, group).
+__global__ void __launch_bounds__(kBlk) csr_copy_all(const CsrArgs C, int64_t t_from, int64_t t_last) {
+    const CsrInst in = C.inst[blockIdx.y];
+    const int W = (in.N + 31) / 32, groups = C.R / 32, lane = threadIdx.x & 31;
+    const int64_t u = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    if (u >= (int64_t)W * groups) return;
+    const int w = (int)(u / groups), g = (int)(u - (int64_t)w * groups), i = w * 32 + lane;
     for (int64_t tt = t_from; tt <= t_last; ++tt) {
-        if (!C.flags[(size_t)(tt & 1) * C.total_reps + in.rec_off + r]) continue;
-        const uint32_t *Sb = spin_buf(C, in, tt);
-        uint32_t bits = 0;
-        for (int q = 0; q < 32; ++q) {
-            const int i = w * 32 + q;
-            if (i < in.N && ((Sb[(size_t)i * (C.R / 32) + (r >> 5)] >> (r & 31)) & 1u)) bits |= 1u << q;
+        const uint32_t mask = __ballot_sync(
+            0xffffffffu, C.flags[(size_t)(tt & 1) * C.total_reps + in.rec_off + g * 32 + lane] != 0);
+        if (!mask) continue;
+        const uint32_t word = i < in.N ? spin_buf(C, in, tt)[(size_t)g * in.Np + C.pos_of[in.inv_off + i]] : 0u;
+        for (uint32_t m = mask; m; m &= m - 1) {
+            const int r = __ffs(m) - 1;
+            const uint32_t bits = __ballot_sync(0xffffffffu, (word >> r) & 1u);
+            if (lane == 0) C.best_bits[in.bits_off + (size_t)(g * 32 + r) * W + w] = bits;
         }
-        C.best_bits[in.bits_off + (size_t)r * W + w] = bits;
     }
 }
 
 // Field only: spins given as int8 [R][N] per instance -> field int32 [R][N], energy [R].
 __global__ void csr_field_only(const CsrArgs C) {
     const RunArgs &a = C.a;
-    const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over total_rows * R
+    const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // over (slice, row, replica)
     const int R = C.R;
-    const int64_t row = gidx / R;
-    if (row >= C.total_rows) return;
-    const int r = (int)(gidx - row * R);
-    int lo = 0, hi = C.count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (C.inst[mid].row_base <= row) lo = mid; else hi = mid - 1;
-    }
-    const CsrInst in = C.inst[lo];
-    const int i = (int)(row - in.row_base);
-    if (r >= C.R_real) return;
+    const int64_t gp = gidx / R;
+    if (gp >= C.total_slices * 32) return;
+    const int r = (int)(gidx - gp * R);
+    const CsrInst in = C.inst[instance_of(C, gp / 32)];
+    const int p = (int)(gp - in.slice_base * 32), lane = p & 31;
+    const int row = C.row_of[in.pos_off + p];
+    if (row < 0 || r >= C.R_real) return;
     const int8_t *s = a.spins_in + in.xin_off + (size_t)r * in.N;
-    int32_t I = C.hk[in.h_off + i];
-    for (int p = C.row_ptr[in.rp_off + i]; p < C.row_ptr[in.rp_off + i + 1]; ++p)
-        I += (int32_t)C.val[in.nz_off + p] * s[C.col[in.nz_off + p]];
-    if (a.field_out) a.field_out[in.xin_off + (size_t)r * in.N + i] = I;
+    const int32_t h = C.hk[2 * (in.pos_off + p)];
+    int32_t I = h;
+    for (int e = C.slice[in.slice_off + p / 32]; e < C.slice[in.slice_off + p / 32 + 1]; ++e) {
+        Entry<true> e16;
+        Entry<false> e32;
+        if (C.col16) e16.load(C, e, lane);
+        else e32.load(C, e, lane);
+        const uint32_t kk = C.col16 ? e16.k : e32.k;
+        for (int n = 0; n < 4; ++n) {
+            const int kv = (int8_t)(kk >> (8 * n));
+            if (kv) I += kv * s[C.row_of[in.pos_off + (C.col16 ? e16.at(n) : e32.at(n)) / 4]];
+        }
+    }
+    if (a.field_out) a.field_out[in.xin_off + (size_t)r * in.N + row] = I;
     atomicAdd(reinterpret_cast<unsigned long long *>(C.Esum) + in.rec_off + r,
-              (unsigned long long)(long long)(s[i] * (I + C.hk[in.h_off + i])));
+              (unsigned long long)((long long)s[row] * (I + h)));
 }
 
 __global__ void csr_field_energy(const CsrArgs C) {
@@ -392,67 +525,102 @@ __global__ void csr_count(const CsrArgs C) {
         atomicAdd(C.a.replica_iters, (unsigned long long)((long long)C.total_reps * C.a.nsteps));
 }
 
+template <bool SMEM, bool C16>
+cudaError_t launch_iterations(const CsrArgs &C, size_t smem, StepGraphCache *graphs, cudaStream_t st, int sms,
+                              int max_blocks, int *launches) {
+    const int ny = (C.R / 32 + C.gblock - 1) / C.gblock;
+    CsrArgs Cs = C;
+    Cs.x_in = Cs.v_in = nullptr;
+    Cs.x_out = Cs.v_out = nullptr;
+    if (C.persistent) {
+        // Every iteration in one cooperative launch: as many blocks as can be resident.
+        auto k = csr_persistent<SMEM, C16>;
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int per_sm = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kBlk, smem);
+        if (e != cudaSuccess) return e;
+        const int64_t units = (int64_t)max_blocks * ny;
+        const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(units, (int64_t)per_sm * sms));
+        e = cudaMemsetAsync(C.sync, 0, 4 * sizeof(unsigned), st);
+        if (e != cudaSuccess) return e;
+        unsigned *bar = C.sync, *ctr = C.sync + 2;
+        void *args[3] = {&Cs, &bar, &ctr};
+        e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k), dim3(blocks), dim3(kBlk), args, smem, st);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+        return cudaSuccess;
+    }
+    // The step kernel reads its iteration from C.ctl: every launch is the same, and the
+    // arguments leave out what only the prologue and the export read.
+    Cs.a.t0 = 0;
+    Cs.a.nsteps = 0;
+    auto k = csr_step<SMEM, C16>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    void *args[1] = {&Cs};
+    for (int set = 0; set < C.nsets; ++set) {
+        if (set > 0) {
+            csr_next_set<<<1, 1, 0, st>>>(C.ctl, C.a.t0, C.a.nsteps, set);
+            ++*launches;
+        }
+        e = launch_steps(graphs, reinterpret_cast<const void *>(k), dim3(max_blocks, ny), dim3(kBlk), smem, args, &Cs,
+                         sizeof Cs, C.a.nsteps, st);
+        if (e != cudaSuccess) return e;
+        *launches += (int)C.a.nsteps;
+    }
+    return cudaSuccess;
+}
+
 }  // namespace
 
-cudaError_t launch_csr(const CsrArgs &Cin, StepGraphCache *graphs, cudaStream_t st, int *launches) {
-    const CsrArgs &C = Cin;
-    int n = 0;
+cudaError_t launch_csr(const CsrArgs &Cin, const int32_t *max_len, StepGraphCache *graphs, cudaStream_t st, int *launches) {
+    CsrArgs C = Cin;
+    int n = 0, dev = 0, sms = 0;
     cudaError_t e = cudaMemsetAsync(C.Esum, 0, 2 * (size_t)C.total_reps * sizeof(int64_t), st);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     if (C.a.field_mode) {
-        const int64_t work = C.total_rows * C.R;
+        const int64_t work = C.total_slices * 32 * C.R;
         csr_field_only<<<(unsigned)((work + 255) / 256), 256, 0, st>>>(C);
         csr_field_energy<<<(unsigned)((C.total_reps + 255) / 256), 256, 0, st>>>(C);
         if (launches) *launches += 2;
         return cudaGetLastError();
     }
-    const int64_t pw = C.total_rows * (C.R / 8);
-    csr_prologue<<<(unsigned)((pw + 255) / 256), 256, 0, st>>>(C);
+    const int groups = C.R / 32;
+    const unsigned conv = (unsigned)(C.total_slices * groups);
+    csr_prologue<<<conv, kBlk, 0, st>>>(C);
     ++n;
-    const dim3 grid(C.nblocks, C.R / kGroup);
-    if (C.persistent) {
-        // Every iteration in one cooperative launch: as many blocks as can be resident.
-        int per_sm = 0, dev = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, csr_persistent, 32 * kWarps, 0);
-        if (e == cudaSuccess) e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        const int units = C.nblocks * (C.R / kGroup);
-        const unsigned blocks = (unsigned)std::max(1, std::min(units, per_sm * sms));
-        e = cudaMemsetAsync(C.sync, 0, 4 * sizeof(unsigned), st);
-        if (e != cudaSuccess) return e;
-        CsrArgs Cp = C;
-        Cp.x_in = Cp.v_in = nullptr;
-        Cp.x_out = Cp.v_out = nullptr;
-        unsigned *bar = C.sync, *ctr = C.sync + 2;
-        void *args[3] = {&Cp, &bar, &ctr};
-        e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(csr_persistent), dim3(blocks),
-                                        dim3(32 * kWarps), args, 0, st);
-        if (e != cudaSuccess) return e;
-        ++n;
-    } else {
-        // The step kernel reads its iteration from C.ctl: every launch is the same, and
-        // the arguments leave out what only the prologue and the export read.
-        CsrArgs Cs = C;
-        Cs.a.t0 = 0;
-        Cs.a.nsteps = 0;
-        Cs.x_in = Cs.v_in = nullptr;
-        Cs.x_out = Cs.v_out = nullptr;
-        void *args[1] = {&Cs};
-        e = launch_steps(graphs, reinterpret_cast<const void *>(csr_step), grid, dim3(32 * kWarps), 0, args, &Cs,
-                         sizeof Cs, C.a.nsteps, st);
-        if (e != cudaSuccess) return e;
-        n += (int)C.a.nsteps;
-    }
+    // Groups per block: up to 8 share one reading of the couplings (through L1) and of the
+    // shared memory that two blocks an SM have; spins of an instance too large for it are read
+    // from L2.  Slices per block: 4, fewer while the units do not fill the GPU twice over (a
+    // set's time is that of its heaviest blocks).
+    int G = 1;
+    while (G < 8 && G < groups) G *= 2;
+    constexpr size_t kTwo = 113 * 1024, kOne = 226 * 1024;
+    while (G > 1 && (size_t)G * C.max_np * 4 > kTwo) G /= 2;
+    const size_t bytes = (size_t)G * C.max_np * 4;
+    const bool in_smem = bytes <= kOne;
+    if (!in_smem)
+        for (G = 1; G < 8 && G < groups;) G *= 2;
+    C.gblock = G;
+    const int spar = kWarps / G, ny = (groups + G - 1) / G;
+    int li = spar >= 8 ? 3 : 2;                 // block lists of 1, 2, 4, 8 slices
+    while ((1 << li) > spar && (int64_t)max_len[li] * ny < 4 * (int64_t)sms) --li;
+    C.slices = 1 << li;
+    C.list = li;
+    if (in_smem && C.col16) e = launch_iterations<true, true>(C, bytes, graphs, st, sms, max_len[li], &n);
+    else if (in_smem) e = launch_iterations<true, false>(C, bytes, graphs, st, sms, max_len[li], &n);
+    else e = launch_iterations<false, false>(C, 0, graphs, st, sms, max_len[li], &n);
+    if (e != cudaSuccess) return e;
     const int64_t t_last = C.a.t0 + C.a.nsteps - 1;
     csr_settle_all<<<C.count, 256, 0, st>>>(C, t_last);
-    const dim3 cg((unsigned)(((int64_t)C.R * C.max_words + 255) / 256), C.count);
-    csr_copy_all<<<cg, 256, 0, st>>>(C, t_last - 1 >= C.a.t0 ? t_last - 1 : t_last, t_last);
+    const dim3 cg((unsigned)(((int64_t)groups * C.max_words + kWarps - 1) / kWarps), C.count);
+    csr_copy_all<<<cg, kBlk, 0, st>>>(C, t_last - 1 >= C.a.t0 ? t_last - 1 : t_last, t_last);
     csr_count<<<1, 32, 0, st>>>(C);
     n += 3;
     if (C.x_out) {
-        const int64_t work = C.total_rows * C.R;
-        csr_export<<<(unsigned)((work + 255) / 256), 256, 0, st>>>(C);
+        csr_export<<<conv, kBlk, 0, st>>>(C);
         ++n;
     }
     if (launches) *launches += n;

@@ -80,7 +80,7 @@ struct IterCtl {
     int64_t t_first;    // first iteration of the run
     int64_t t_end;      // one past the run's last iteration
     uint32_t done;      // CTAs of the current launch that have finished
-    uint32_t pad;
+    int32_t set;        // sparse path: the set of instances that the launch works on
 };
 
 #ifdef __CUDACC__
@@ -156,33 +156,49 @@ inline int large_rpad(int R) { return round_up(R, 256); }
 // replicas into 224-wide tiles (ceil(R / 224) * 224 <= this).
 inline int large_rpad_handle(int R) { return round_up(R, 256) + 256; }
 
-// Sparse batched path: many CSR instances, one launch per iteration over all of them.
+// Sparse batched path: many instances in slices of 32 rows (see k_csr.cu for the layout).
 struct CsrInst {
-    int32_t N;
+    int32_t N, Np;          // spins; positions (N rounded up to 32)
     uint32_t inst_id;       // fourth Philox counter word
     float q;                // 2^-frac_bits
+    int32_t wide;           // energy terms or scaled sums of a row may leave 32 bits
     int32_t pad;
-    int64_t rp_off;         // into row_ptr (N + 1 entries, values relative to nz_off)
-    int64_t nz_off;         // into col / val
-    int64_t h_off;          // into hk
-    int64_t row_base;       // global index of row 0 (rows are stored instance after instance)
-    int64_t x_off;          // into X, V ([N][R] per instance)
+    int64_t slice_base;     // global index of slice 0 (slices are numbered instance after instance)
+    int64_t slice_off;      // into slice (Np/32 + 1 entries)
+    int64_t pos_off;        // into hk (pairs) and row_of, per position
+    int64_t inv_off;        // into pos_of, per spin
+    int64_t x_off;          // into X, V ([R/32][8][Np][4] per instance)
     int64_t xin_off;        // into caller arrays ([R][N] per instance)
-    int64_t s_off;          // into each spin buffer, in uint32 words ([N][R/32] per instance)
+    int64_t s_off;          // into each spin buffer, in uint32 words ([R/32][Np] per instance)
     int64_t rec_off;        // into per-replica records (R per instance)
     int64_t bits_off;       // into best_bits (R * ceil(N/32) per instance)
 };
 struct CsrBlock {
     int32_t inst;
-    int32_t i0;             // first of up to 64 rows
+    int32_t s0;             // first slice
+    int32_t work;           // its entries
+};
+struct CsrSet {             // a set's blocks in each of the lists
+    int32_t off[4], len[4];
 };
 struct CsrArgs {
     RunArgs a;              // run parameters; record pointers indexed by rec_off + r
     const CsrInst *inst;
     int32_t count;
-    const CsrBlock *blocks;
-    int32_t nblocks;
-    const int32_t *row_ptr; const int32_t *col; const int8_t *val; const int32_t *hk;
+    const CsrBlock *blocks; // the block lists for 1, 2, 4 and 8 slices a block
+    const CsrSet *sets;     // instances that go through their iterations together
+    int32_t nsets;
+    int32_t list;           // the list in use
+    int32_t slices;         // slices per block of that list
+    int32_t gblock;         // groups of 32 replicas per block
+    int32_t max_np;         // largest Np
+    const int32_t *slice;   // first entry of each slice (an entry: 4 neighbours of 32 rows)
+    const void *col;        // [entries][32][4] byte offsets of the neighbours' positions, uint16 or uint32
+    int32_t col16;          // 1: uint16
+    const uint32_t *val;    // [entries][32] their couplings, 4 x int8
+    const int32_t *hk;      // [positions][2] field h and h - (sum of the row's couplings)
+    const int32_t *row_of;  // [positions] spin at a position, -1 past N
+    const int32_t *pos_of;  // [spins] position of a spin
     float *X, *V;
     const float *x_in, *v_in;
     float *x_out, *v_out;
@@ -193,16 +209,17 @@ struct CsrArgs {
     int64_t total_reps;
     uint32_t *best_bits;
     const long long *targets;   // per instance, or null (then a.target)
-    int32_t R;              // replicas per instance as run (multiple of 256)
+    int32_t R;              // replicas per instance as run (multiple of 32)
     int32_t R_real;         // replicas the caller asked for (<= R); the rest pad the groups
     int32_t max_words;      // max ceil(N/32)
-    int64_t total_rows;
+    int64_t total_slices;
     IterCtl *ctl;           // iteration control
     int32_t persistent;     // 1: every iteration in one cooperative launch (grid barrier per iteration)
     int32_t pad1;
     unsigned *sync;         // 4 words of device memory for that launch's barrier and work counters
 };
-cudaError_t launch_csr(const CsrArgs &C, StepGraphCache *graphs, cudaStream_t st, int *launches);
+// max_len: the most blocks that a set has in each list.
+cudaError_t launch_csr(const CsrArgs &C, const int32_t *max_len, StepGraphCache *graphs, cudaStream_t st, int *launches);
 
 }  // namespace phia
 struct phia_batch_s;
