@@ -80,9 +80,9 @@ typedef struct phia_opts {
                               2 = tensor memory; 0 = automatic */
     int32_t tc_kernel;     /* tensor-core path: 1 = resident tcgen05 kernel (all iterations in one
                               launch, J on chip; N <= 384 e4m3 / 256 bf16), 2 = one launch per
-                              iteration (J streamed by TMA; any N), 3 = resident int8 kernel
-                              (warp-level mma.sync s8 x s8 -> s32, J in registers; N <= 256;
-                              tile_replicas 8 or 16), 4 = resident incremental-field kernel
+                              iteration (J streamed by TMA; any N), 3 = resident warp-level
+                              kernel (mma.sync with bf16 operands, J in registers; N <= 256;
+                              8 replicas per CTA whatever tile_replicas says), 4 = resident incremental-field kernel
                               (CUDA cores: the exact integer field is updated by the columns of
                               the spins that changed sign, Eq. 6 being linear in s; N <= 384
                               e4m3 / 256 bf16; tile_replicas 4, 8 or 16); 0 = automatic */
@@ -157,8 +157,9 @@ typedef struct phia_stats {
     int32_t path;          /* path actually used (PHIA_PATH_TC / _FP32 / _CSR) */
     int32_t operand;       /* operand actually used (PHIA_OP_E4M3 / _BF16), 0 for other paths */
     int32_t kernel_launches; /* kernels launched by the last run */
-    int32_t tc_kernel;     /* dense kernel used (1 resident tcgen05, 2 per iteration, 3 resident
-                              int8 mma.sync, 4 resident incremental field), 0 for other paths */
+    int32_t tc_kernel;     /* dense kernel used (1 resident tcgen05, 2 per iteration, overlapped or
+                              over clusters, 3 resident warp-level, 4 resident incremental field),
+                              0 for other paths */
     int32_t reserved0;     /* 0 */
     int64_t hit_ns;        /* device time to target: %globaltimer nanoseconds from the start of
                               the run (its record reset, the first call of a resumed run) to
@@ -208,7 +209,7 @@ int phia_anneal(phia_t *p, const phia_schedule *sched, int32_t replicas, int64_t
 /* Autotuner.  Times short probe runs (probe_iters iterations of `replicas` replicas) of
  * every tensor-core kernel variant that applies to this handle -- the resident tcgen05
  * kernel with 4, 8 or 16 replicas per CTA and J in shared or tensor memory, the
- * resident int8 mma.sync kernel with 8 or 16 replicas per CTA (N small enough), the
+ * resident warp-level kernel (two candidates, alike; N small enough), the
  * resident incremental-field kernel with 4, 8 or 16 replicas per CTA (N small enough),
  * and the per-iteration kernel in its thirteen variants (phia_opts.large_variant) -- keeps
  * the fastest for the handle and caches it,
@@ -216,7 +217,7 @@ int phia_anneal(phia_t *p, const phia_schedule *sched, int32_t replicas, int64_t
  * automatic use the cached choice for runs with that replica count.  The probes
  * overwrite the handle's last-run records.  Tensor-core path only (else PHIA_ENOTSUP). */
 typedef struct phia_tune_result {
-    int32_t tc_kernel;         /* 1 resident tcgen05, 2 per iteration, 3 resident int8 mma.sync,
+    int32_t tc_kernel;         /* 1 resident tcgen05, 2 per iteration, 3 resident warp-level,
                                   4 resident incremental field; the per-iteration kernel's variant
                                   (phia_opts.large_variant) is reported in large_variant */
     int32_t tile_replicas;     /* resident kernel: replicas per CTA */

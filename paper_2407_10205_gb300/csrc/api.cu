@@ -66,6 +66,15 @@ namespace phia {
 int set_last_error(int code, const char *msg) { return fail(code, "%s", msg); }
 }  // namespace phia
 
+// A kernel choice of a handle (the autotuner's, or the automatic one).
+struct TuneChoice {
+    bool large;
+    int tile_rl, coupling_mem;
+    bool warpk;
+    bool inc;
+    int lvar;        // per-iteration kernel variant (large only)
+};
+
 struct phia_s {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -75,7 +84,8 @@ struct phia_s {
     int tile_rl = 0, coupling_mem = 0;
     phia_batch_s *batch = nullptr;      // CSR instances: a batch of one
     bool large = false;                 // tensor-core path through the per-iteration kernel
-    bool imma = false;                  // tensor-core path through the int8 mma.sync resident kernel
+    bool warpk = false;                 // tensor-core path through the warp-level resident kernel
+    int last_kernel = 0;                // stats.tc_kernel of the last run
     bool inc = false;                   // dense path through the incremental-field resident kernel
     void *d_Jop = nullptr;              // couplings in the operand encoding (per-iteration kernel)
     int Mpad = 0, Kbytes = 0;
@@ -123,7 +133,9 @@ struct phia_s {
     int last_stop = 0;
     int large_variant = 0;              // per-iteration kernel variant requested (0 = automatic)
     int tuned_variant = 0;              // the autotuner's choice for it
-    bool tuned_coop = false;            // this handle's own autotune chose the cooperative variant
+    bool tuned = false;                 // the kernel is the autotuner's choice for this replica count
+    bool accept_moved = false;          // an automatic handle runs the acceptance test on the resident kernel
+    TuneChoice before_accept{};         // ... and the choice that it had before
     int64_t wait_ns = 0;                // testing aid (phia_debug_wait): device wait bound, 0 = default
     int stall_producer = 0;             // testing aid: the per-iteration kernel's TMA producer issues nothing
 };
@@ -287,15 +299,6 @@ struct TuneKey {
         return N != o.N ? N < o.N : (R != o.R ? R < o.R : op < o.op);
     }
 };
-struct TuneChoice {
-    bool large;
-    int tile_rl, coupling_mem;
-    bool imma;
-    bool inc;
-    int lvar;        // per-iteration kernel variant (large only)
-    int lvar_alt;    // when lvar is a cooperative variant (7..13): the fastest of 1..6, which
-                     // other handles with the same key take (they may run concurrently)
-};
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneChoice> g_tune;
 
@@ -317,7 +320,8 @@ int apply_tuned(phia_t *p, int R) {
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tune.find(TuneKey{p->N, R, p->op});
-        if (it == g_tune.end()) return PHIA_OK;
+        p->tuned = it != g_tune.end();
+        if (!p->tuned) return PHIA_OK;
         c = it->second;
     }
     if (c.large) {
@@ -325,15 +329,28 @@ int apply_tuned(phia_t *p, int R) {
         if (rc) return rc;
     }
     p->large = c.large;
-    p->imma = c.imma;
+    p->warpk = c.warpk;
     p->inc = c.inc;
     p->tile_rl = c.tile_rl;
     p->coupling_mem = c.coupling_mem;
-    p->tuned_variant = c.large ? (c.lvar >= 7 && !p->tuned_coop ? c.lvar_alt : c.lvar) : 0;
+    p->tuned_variant = c.lvar;
     return PHIA_OK;
 }
 
+// Whether this run takes the warp-level resident kernel.  Automatic handles up to 208 spins
+// always do; up to 240 unless the e4m3 tcgen05 kernel fills the GPU with 16 replicas a CTA,
+// where it is the faster one (N = 230 x 4096: 3.30 against 3.34 us an iteration, 16384: 11.49
+// against 11.64; N = 200 x 4096: 3.24 both; bf16 at 200 x 4096: 3.62 against 3.20).
+bool takes_warp(const phia_t *p, const RunArgs &a) {
+    if (p->path != PHIA_PATH_TC || !p->warpk || a.field_mode) return false;
+    if (!p->auto_tile || p->tuned || p->op != kOpE4M3 || p->N <= 208) return true;
+    return tc_small_tile_replicas(a.R, 0) < 16;
+}
+
 cudaError_t launch_path(phia_t *p, const RunArgs &a, int *launches) {
+    const bool warp = takes_warp(p, a);
+    if (!a.field_mode)
+        p->last_kernel = p->path != PHIA_PATH_TC ? 0 : p->large ? 2 : warp ? 3 : p->inc ? 4 : 1;
     if (p->path == PHIA_PATH_TC && p->large) {
         LargeBuffers B;
         B.Jop = p->d_Jop; B.S = p->d_S; B.Epart = p->d_Epart; B.flags = p->d_flags; B.ready = p->d_ready;
@@ -342,9 +359,9 @@ cudaError_t launch_path(phia_t *p, const RunArgs &a, int *launches) {
         B.ctl = p->d_ctl; B.graphs = p->graphs;
         return launch_tc_large(B, a, p->op, p->stream, launches);
     }
-    if (p->path == PHIA_PATH_TC && p->imma) return launch_imma_small(a, p->stream, launches);
-    // The incremental kernel has no field-only mode: the resident tensor-core kernel
-    // covers the same sizes.
+    // The warp-level and the incremental kernel have no field-only mode: the resident tcgen05
+    // kernel covers the same sizes.
+    if (warp) return launch_warp_small(a, p->stream, launches);
     if (p->path == PHIA_PATH_TC && p->inc && !a.field_mode) return launch_inc_small(a, p->stream, launches);
     if (p->path == PHIA_PATH_TC) return launch_tc_small(a, p->op, p->stream, launches);
     if (p->path == PHIA_PATH_FP32) {
@@ -532,8 +549,8 @@ int create_dense(phia_t **out, const int8_t *J_k, const int32_t *h_k, int32_t N,
         if (N > nmax)
             return fail(PHIA_ENOTSUP, "the incremental kernel handles N <= %d with this operand (N = %d)", nmax, N);
     }
-    if (o.tc_kernel == 3 && N > imma_small_max_n())
-        return fail(PHIA_ENOTSUP, "the int8 mma.sync kernel handles N <= %d (N = %d)", imma_small_max_n(), N);
+    if (o.tc_kernel == 3 && N > warp_small_max_n())
+        return fail(PHIA_ENOTSUP, "the warp-level kernel handles N <= %d (N = %d)", warp_small_max_n(), N);
     if (o.large_variant < 0 || o.large_variant > 13) return fail(PHIA_EINVAL, "large_variant must be 0..13");
     int dev_count = 0;
     if (cudaGetDeviceCount(&dev_count) != cudaSuccess || dev_count == 0)
@@ -556,7 +573,7 @@ int create_dense(phia_t **out, const int8_t *J_k, const int32_t *h_k, int32_t N,
     p->max_abs_k = max_abs;
     if (path == PHIA_PATH_TC) {
         p->large = o.tc_kernel == 2 || (o.tc_kernel == 0 && N > tc_small_max_n(p->op));
-        p->imma = o.tc_kernel == 3;
+        p->warpk = o.tc_kernel == 3 || (p->auto_tile && N <= warp_small_auto_n());
         p->inc = o.tc_kernel == 4;
     }
     const size_t NN = (size_t)N * N;
@@ -655,13 +672,26 @@ static int run_impl(phia_t *p, const phia_schedule *sched, int32_t R, int64_t t0
     if (sched->accept_test == 1 && p->path == PHIA_PATH_TC) {
         // The acceptance test runs in the resident tcgen05 kernel with J in shared memory.
         if (p->auto_tile && p->N <= tc_small_max_n(p->op)) {
-            p->large = p->imma = p->inc = false;
+            if (!p->accept_moved)
+                p->before_accept = TuneChoice{p->large, p->tile_rl, p->coupling_mem, p->warpk, p->inc, p->tuned_variant};
+            p->accept_moved = true;
+            p->large = p->warpk = p->inc = false;
             p->coupling_mem = 1;
-        } else if (p->large || p->imma || p->inc || p->coupling_mem == 2) {
+        } else if (p->large || p->warpk || p->inc || p->coupling_mem == 2) {
             return fail(PHIA_ENOTSUP, "schedule.accept_test = 1 runs on the resident tcgen05 kernel with J in shared "
                                       "memory (tc_kernel 1, N <= %d with this operand) or the FP32 path",
                         tc_small_max_n(p->op));
         }
+    }
+    if (sched->accept_test == 0 && p->accept_moved) {   // back to the kernel of ordinary runs
+        const TuneChoice &c = p->before_accept;
+        p->accept_moved = false;
+        p->large = c.large;
+        p->warpk = c.warpk;
+        p->inc = c.inc;
+        p->tile_rl = c.tile_rl;
+        p->coupling_mem = c.coupling_mem;
+        p->tuned_variant = c.lvar;
     }
     if (steps < 1) return fail(PHIA_EINVAL, "steps must be >= 1");
     if (t0 < 0 || total < t0 + steps) return fail(PHIA_EINVAL, "need 0 <= t0 and t0 + steps <= total_steps");
@@ -716,30 +746,29 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
     std::vector<TuneChoice> cands;
     if (p->N <= tc_small_max_n(p->op)) {
         for (int tile : {4, 8, 16})
-            for (int mem : {1, 2}) cands.push_back(TuneChoice{false, tile, mem, false, false, 0, 0});
+            for (int mem : {1, 2}) cands.push_back(TuneChoice{false, tile, mem, false, false, 0});
     }
-    if (p->N <= imma_small_max_n()) {
-        cands.push_back(TuneChoice{false, 8, 0, true, false, 0, 0});
-        cands.push_back(TuneChoice{false, 16, 0, true, false, 0, 0});
+    if (p->N <= warp_small_max_n()) {
+        cands.push_back(TuneChoice{false, 8, 0, true, false, 0});
+        cands.push_back(TuneChoice{false, 16, 0, true, false, 0});
     }
     if (p->N <= std::min(inc_small_max_n(), tc_small_max_n(p->op))) {
         for (int tile : {4, 8, 16})
             if (inc_small_tile_replicas(p->N, tile) == tile)
-                cands.push_back(TuneChoice{false, tile, 0, false, true, 0, 0});
+                cands.push_back(TuneChoice{false, tile, 0, false, true, 0});
     }
-    for (int lv = 1; lv <= 13; ++lv) cands.push_back(TuneChoice{true, 0, 0, false, false, lv, 0});
+    for (int lv = 1; lv <= 13; ++lv) cands.push_back(TuneChoice{true, 0, 0, false, false, lv});
     const bool saved_auto = p->auto_tile;
     p->auto_tile = false;
-    float best_ms = 1e30f, worst_ms = 0.f, alt_ms = 1e30f;
+    float best_ms = 1e30f, worst_ms = 0.f;
     TuneChoice best = cands[0];
-    int best_alt = 1;   // fastest non-cooperative per-iteration variant
     for (const TuneChoice &c : cands) {
         if (c.large) {
             int rc = ensure_operand(p);
             if (rc) { p->auto_tile = saved_auto; return rc; }
         }
         p->large = c.large;
-        p->imma = c.imma;
+        p->warpk = c.warpk;
         p->inc = c.inc;
         p->tile_rl = c.tile_rl;
         p->coupling_mem = c.coupling_mem;
@@ -752,28 +781,26 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
             CU(cudaEventElapsedTime(&ms, p->ev0, p->ev1));
         }
         if (ms < best_ms) { best_ms = ms; best = c; }
-        if (c.large && c.lvar < 7 && ms < alt_ms) { alt_ms = ms; best_alt = c.lvar; }
         worst_ms = std::max(worst_ms, ms);
     }
     p->large = best.large;
-    p->imma = best.imma;
+    p->warpk = best.warpk;
     p->inc = best.inc;
     p->tile_rl = best.tile_rl;
     p->coupling_mem = best.coupling_mem;
     p->tuned_variant = best.lvar;
-    p->tuned_coop = best.large && best.lvar >= 7;
+    p->tuned = true;
     p->auto_tile = saved_auto;
-    best.lvar_alt = best_alt;
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         g_tune[TuneKey{p->N, replicas, p->op}] = best;
     }
     if (out) {
         memset(out, 0, sizeof *out);
-        out->tc_kernel = best.large ? 2 : (best.imma ? 3 : (best.inc ? 4 : 1));
+        out->tc_kernel = best.large ? 2 : (best.warpk ? 3 : (best.inc ? 4 : 1));
         out->tile_replicas = best.large ? 0
-                             : (best.imma || best.inc ? best.tile_rl : tc_small_tile_replicas(replicas, best.tile_rl));
-        out->coupling_mem = best.large || best.imma || best.inc ? 0 : best.coupling_mem;
+                             : (best.warpk || best.inc ? best.tile_rl : tc_small_tile_replicas(replicas, best.tile_rl));
+        out->coupling_mem = best.large || best.warpk || best.inc ? 0 : best.coupling_mem;
         out->candidates = (int32_t)cands.size();
         out->best_us_per_iter = 1000.f * best_ms / probe_iters;
         out->worst_us_per_iter = 1000.f * worst_ms / probe_iters;
@@ -920,6 +947,7 @@ int phia_gahmc(phia_t *p, const phia_gahmc_schedule *sched, int32_t R, int64_t K
     a.x_in = x; a.v_in = v; a.x_out = x; a.v_out = v;
     a.has_target = sched->has_target; a.target = sched->target_k;
     CU(cudaEventRecord(p->ev0, p->stream));
+    p->last_kernel = p->large ? 2 : p->inc ? 4 : p->warpk && !p->auto_tile ? 3 : 1;
     cudaError_t e = launch_gahmc(a, sched->travel, K, counts, events, events_cap, p->stream);
     if (e != cudaSuccess) return fail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
     CU(cudaEventRecord(p->ev1, p->stream));
@@ -991,7 +1019,7 @@ int phia_stats_get(phia_t *p, phia_stats *out) {
     out->path = p->path;
     out->operand = p->op == kOpE4M3 ? PHIA_OP_E4M3 : (p->op == kOpBF16 ? PHIA_OP_BF16 : 0);
     out->kernel_launches = p->last_launches;
-    out->tc_kernel = p->path == PHIA_PATH_TC ? (p->large ? 2 : (p->imma ? 3 : (p->inc ? 4 : 1))) : 0;
+    out->tc_kernel = p->last_kernel;
     return PHIA_OK;
 }
 

@@ -31,10 +31,9 @@ struct phia_batch_s {
     std::vector<int> N, frac;           // per public instance
     std::vector<uint32_t> inst_id;
     std::vector<int64_t> h_off;         // into d_hk
-    // small dense members: resident tcgen05 kernel over a table of CTAs
+    // small dense members: a resident kernel over a table of CTAs
     std::vector<int> dense_pub;         // public indices
     std::vector<int64_t> dense_joff;    // offset of each member's J in d_dJ
-    std::vector<int> dense_op;          // kOpE4M3 / kOpBF16
     int8_t *d_dJ = nullptr;
     SmallCta *d_small = nullptr;
     size_t small_cap = 0;
@@ -405,7 +404,6 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         if (pk.small_op) {
             b->dense_pub.push_back(k);
             b->dense_joff.push_back((int64_t)dj.size());
-            b->dense_op.push_back(pk.small_op);
             dj.insert(dj.end(), x.J_k, x.J_k + (size_t)n * n);
             hk.insert(hk.end(), x.h_k, x.h_k + n);
             continue;
@@ -585,42 +583,42 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     C.R = R; C.R_real = R_real;
     C.max_words = b->max_words;
     C.total_slices = b->total_slices;
-    // Small dense members: a table of CTAs (8 replicas each) per (operand, spin tiles)
-    // group, every instance's own couplings, field, scale, Philox id, target and records.
-    std::vector<std::pair<size_t, size_t>> groups;   // [begin, end) in small_host
-    std::vector<std::pair<int, int>> group_key;      // (operand, spin tiles)
-    std::vector<int> group_kpad;
+    // Small dense members: a table of CTAs (8 replicas each) per size class, every instance's
+    // own couplings, field, scale, Philox id, target and records.  Up to 256 spins they run on
+    // the warp-level kernel (classes of at most 64, 128 and 256 spins, as its register use
+    // grows with the size it is built for), above on the resident tcgen05 kernel.
+    struct SmallGroup {
+        size_t begin, end;       // in small_host
+        int nmax;
+    };
+    std::vector<SmallGroup> groups;
     if (!b->dense_pub.empty()) {
         b->small_host.clear();
-        for (int op : {kOpE4M3, kOpBF16})
-            for (int mt = 1; mt <= 3; ++mt) {
-                const size_t beg = b->small_host.size();
-                int nmax = 0;
-                for (size_t m = 0; m < b->dense_pub.size(); ++m) {
-                    const int k = b->dense_pub[m], n = b->N[(size_t)k];
-                    if (b->dense_op[m] != op || (n + 127) / 128 != mt) continue;
-                    nmax = std::max(nmax, n);
-                    for (int r0 = 0; r0 < R_real; r0 += 8) {
-                        SmallCta c{};
-                        c.Jk = b->d_dJ + b->dense_joff[m];
-                        c.hk = b->d_hk + b->h_off[(size_t)k];
-                        c.N = n;
-                        c.W = (int32_t)words_of(n);
-                        c.inst = b->inst_id[(size_t)k];
-                        c.q = ldexpf(1.0f, -b->frac[(size_t)k]);
-                        c.rbase = r0;
-                        c.rec_off = (int64_t)k * R;
-                        c.bits_off = b->bits_pub[(size_t)k];
-                        c.target = target_of(k);
-                        b->small_host.push_back(c);
-                    }
-                }
-                if (b->small_host.size() > beg) {
-                    groups.emplace_back(beg, b->small_host.size());
-                    group_key.emplace_back(op, mt);
-                    group_kpad.push_back(op == kOpE4M3 ? (nmax + 31) / 32 * 32 : (nmax + 15) / 16 * 16);
+        const int bounds[5] = {0, 64, 128, warp_small_max_n(), INT_MAX};
+        for (int cls = 0; cls < 4; ++cls) {
+            const size_t beg = b->small_host.size();
+            int nmax = 0;
+            for (size_t m = 0; m < b->dense_pub.size(); ++m) {
+                const int k = b->dense_pub[m], n = b->N[(size_t)k];
+                if (n <= bounds[cls] || n > bounds[cls + 1]) continue;
+                nmax = std::max(nmax, n);
+                for (int r0 = 0; r0 < R_real; r0 += 8) {
+                    SmallCta c{};
+                    c.Jk = b->d_dJ + b->dense_joff[m];
+                    c.hk = b->d_hk + b->h_off[(size_t)k];
+                    c.N = n;
+                    c.W = (int32_t)words_of(n);
+                    c.inst = b->inst_id[(size_t)k];
+                    c.q = ldexpf(1.0f, -b->frac[(size_t)k]);
+                    c.rbase = r0;
+                    c.rec_off = (int64_t)k * R;
+                    c.bits_off = b->bits_pub[(size_t)k];
+                    c.target = target_of(k);
+                    b->small_host.push_back(c);
                 }
             }
+            if (b->small_host.size() > beg) groups.push_back(SmallGroup{beg, b->small_host.size(), nmax});
+        }
         if (b->small_host.size() > b->small_cap) {
             cudaFree(b->d_small);
             b->d_small = nullptr;
@@ -639,16 +637,17 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         cudaError_t e = launch_csr(C, b->set_max, b->graphs, b->stream, &launches);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
     }
-    for (size_t gi = 0; gi < groups.size(); ++gi) {
+    for (const SmallGroup &grp : groups) {
         RunArgs ad = a;
         ad.R = R_real;
         ad.best_bits = b->d_bits;        // the CSR path keeps its best states in C.best_bits
         if (!ad.best_e || !ad.best_step || !ad.hit_step || !ad.hit_ns || !ad.best_bits || !ad.replica_iters || !ad.err)
             return bfail(PHIA_ECUDA, "internal: a record array of the dense launch is missing");
-        ad.small_cta = b->d_small + groups[gi].first;
-        ad.small_ctas = (int32_t)(groups[gi].second - groups[gi].first);
+        ad.small_cta = b->d_small + grp.begin;
+        ad.small_ctas = (int32_t)(grp.end - grp.begin);
         ad.has_target = b->any_target || sched->has_target;
-        cudaError_t e = launch_tc_small_batch(ad, group_key[gi].first, group_key[gi].second, group_kpad[gi], b->stream);
+        cudaError_t e = grp.nmax <= warp_small_max_n() ? launch_warp_small_batch(ad, grp.nmax, b->stream)
+                                                       : launch_tc_small_batch(ad, grp.nmax, b->stream);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
         ++launches;
     }

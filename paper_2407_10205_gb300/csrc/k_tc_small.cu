@@ -662,36 +662,20 @@ cudaError_t launch_mt(const RunArgs &a, int Kpad, cudaStream_t st) {
 
 int tc_small_max_n(int op) { return op == kOpE4M3 ? 384 : 256; }
 
-namespace {
-
-template <int MT, int OP>
-cudaError_t launch_batch_mt(const RunArgs &a, int Kpad, cudaStream_t st) {
-    // Every instance of the launch shares MT and the operand; K is padded for the group's
-    // largest N (Kpad), so that one shared-memory layout serves all of them (the couplings
-    // and spins past an instance's N are zero).
-    constexpr int ESZ = OP == kOpE4M3 ? 1 : 2;
-    const size_t smem = (size_t)(MT * 128 + kNB) * Kpad * ESZ + sizeof(SmallShared) + 16;
-    auto kern = a.deriv == 1 ? tc_small_kernel<MT, OP, 2, 4, false, 1, false, true>
-                             : tc_small_kernel<MT, OP, 2, 4, false, 0, false, true>;
+cudaError_t launch_tc_small_batch(const RunArgs &a, int nmax, cudaStream_t st) {
+    // Members of 257 .. 384 spins (e4m3, three 128-spin tiles).  K is padded for the largest
+    // (nmax), so that one shared-memory layout serves all of them (the couplings and spins
+    // past an instance's N are zero).
+    if (a.small_ctas < 1) return cudaSuccess;
+    if (nmax > tc_small_max_n(kOpE4M3)) return cudaErrorInvalidValue;
+    const int Kpad = (nmax + 31) / 32 * 32;
+    const size_t smem = (size_t)(3 * 128 + kNB) * Kpad + sizeof(SmallShared) + 16;
+    auto kern = a.deriv == 1 ? tc_small_kernel<3, kOpE4M3, 2, 4, false, 1, false, true>
+                             : tc_small_kernel<3, kOpE4M3, 2, 4, false, 0, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<a.small_ctas, 128 * MT * 2 + 64 * MT, smem, st>>>(a, Kpad);
+    kern<<<a.small_ctas, 128 * 3 * 2 + 64 * 3, smem, st>>>(a, Kpad);
     return cudaGetLastError();
-}
-
-}  // namespace
-
-cudaError_t launch_tc_small_batch(const RunArgs &a, int op, int mt, int kpad, cudaStream_t st) {
-    if (a.small_ctas < 1) return cudaSuccess;
-    if (op == kOpE4M3) {
-        if (mt == 1) return launch_batch_mt<1, kOpE4M3>(a, kpad, st);
-        if (mt == 2) return launch_batch_mt<2, kOpE4M3>(a, kpad, st);
-        if (mt == 3) return launch_batch_mt<3, kOpE4M3>(a, kpad, st);
-    } else {
-        if (mt == 1) return launch_batch_mt<1, kOpBF16>(a, kpad, st);
-        if (mt == 2) return launch_batch_mt<2, kOpBF16>(a, kpad, st);
-    }
-    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_tc_small(const RunArgs &a, int op, cudaStream_t st, int *launches) {

@@ -123,9 +123,9 @@ int tc_small_max_n(int op);
 int tc_small_tile_replicas(int R, int requested);
 cudaError_t launch_tc_small(const RunArgs &a, int op, cudaStream_t st, int *launches);
 // The same kernel over a table of CTAs (a.small_cta, a.small_ctas entries, 8 live replicas
-// each) of small dense instances of one operand and one number of 128-spin tiles (mt):
-// all iterations of every instance in one launch; no early stop at a target.
-cudaError_t launch_tc_small_batch(const RunArgs &a, int op, int mt, int kpad, cudaStream_t st);
+// each) of e4m3 instances of 257 .. nmax spins: all iterations of every instance in one
+// launch; no early stop at a target.
+cudaError_t launch_tc_small_batch(const RunArgs &a, int nmax, cudaStream_t st);
 
 // tcgen05 per-iteration kernel for dense instances of any size (TMA-staged J and spins).
 struct LargeBuffers {
@@ -239,9 +239,17 @@ int batch_stats(phia_batch_s *b, int inst, phia_stats *out);
 // Thread-local error message of the C ABI.
 int set_last_error(int code, const char *msg);
 
-// int8 tensor-core resident kernel (mma.sync s8 x s8 -> s32) for small dense instances.
-int imma_small_max_n();
-cudaError_t launch_imma_small(const RunArgs &a, cudaStream_t st, int *launches);
+// Warp-level tensor-core resident kernel (mma.sync bf16, J in registers) for small dense
+// instances, 8 replicas per CTA (no field mode), and over a table of CTAs (a.small_cta) of
+// instances with at most nmax spins.
+int warp_small_max_n();
+// Automatic handles take it up to here: with 17 warps the registers run short (N = 256: 1.3 to
+// 1.8 us an iteration, against 1.18 for the tcgen05 one).
+int warp_small_auto_n();
+cudaError_t launch_warp_small(const RunArgs &a, cudaStream_t st, int *launches);
+cudaError_t launch_warp_small_batch(const RunArgs &a, int nmax, cudaStream_t st);
+// Its estimated time per iteration (us).
+double warp_small_estimate(int N, int R, int sms);
 
 // Incremental-field resident kernel for small dense instances (CUDA cores, exact
 // integer field updated by the columns whose spin changed sign; no field mode).
