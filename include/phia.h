@@ -96,15 +96,19 @@ typedef struct phia_opts {
                               iteration and start a replica tile's next iteration as soon as
                               all of its spins are written (per-replica-tile counters instead
                               of a launch boundary; a records warp settles the energies); its
-                              CTAs wait on each other, so it wants the GPU's SMs to itself;
+                              CTAs wait on each other, so they have to be resident together,
+                              which the launch guarantees;
                               its tile width (256, 224, 160 or 128 replicas; 160-wide tiles
                               with three tensor-memory accumulators) is the one whose
-                              estimated iteration time is least; 8 / 9 = as 7 with 256- or
+                              estimated iteration time is least, and runs whose estimate is
+                              less take one of two kernels for few replicas instead: the whole
+                              run over thread-block clusters with J in registers (N <= 1024
+                              e4m3, 512 bf16) or overlapped tiles of 128 replicas x 32 or 64
+                              spins with x, v in registers; 8 / 9 = as 7 with 256- or
                               128-wide tiles and the spin-operand multicast over clusters of
                               2 / 4 CTAs; 10 / 11 / 12 / 13 = as 7 with 256- / 224- / 128- /
                               160-wide tiles; 0 = automatic (the autotuner's choice where it
-                              has one; a choice of 7..13 is kept by the tuned handle only,
-                              other handles take the fastest of 1..6) */
+                              has one, else as 7) */
 } phia_opts;
 
 /* Annealing schedule.  No values are given in the paper; every field is explicit. */

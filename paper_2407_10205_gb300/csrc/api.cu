@@ -103,6 +103,8 @@ struct phia_s {
     int8_t *d_Jk = nullptr;
     float *d_Jf = nullptr;
     int32_t *d_hk = nullptr;
+    float *d_hf = nullptr;              // h as FP32, padded with zeros to a multiple of 16 (dense instances)
+    int32_t *d_hmax = nullptr;          // max |h|
     int32_t *d_rowptr = nullptr, *d_col = nullptr;
     int8_t *d_val = nullptr;
     // per-replica state
@@ -276,6 +278,9 @@ RunArgs base_args(phia_t *p, int R) {
     a.Jk = p->d_Jk;
     a.Jf = p->d_Jf;
     a.hk = p->d_hk;
+    a.hf = p->d_hf;
+    a.h_max = p->d_hmax;
+    a.max_abs_k = p->max_abs_k;
     a.row_ptr = p->d_rowptr; a.col = p->d_col; a.val = p->d_val;
     a.R = R;
     a.q = ldexpf(1.0f, -p->frac_bits);
@@ -388,6 +393,9 @@ int finish_create(phia_t *p, const int32_t *h_k, const phia_opts *opts,
                   cudaMemcpyKind h_kind = cudaMemcpyHostToDevice) {
     CU(pool_alloc((void **)&p->d_hk, (size_t)p->N * 4, p->device, p->stream));
     CU(cudaMemcpyAsync(p->d_hk, h_k, (size_t)p->N * 4, h_kind, p->stream));
+    CU(pool_alloc((void **)&p->d_hf, (size_t)round_up(p->N, 16) * 4, p->device, p->stream));
+    CU(pool_alloc((void **)&p->d_hmax, 4, p->device, p->stream));
+    CU(launch_pad_field(p->d_hk, p->N, p->d_hf, p->d_hmax, p->stream));
     CU(pool_alloc((void **)&p->d_min_hit, 8, p->device, p->stream));
     CU(pool_alloc((void **)&p->d_start_ns, 8, p->device, p->stream));
     CU(cudaMemsetAsync(p->d_start_ns, 0, 8, p->stream));
@@ -1029,7 +1037,7 @@ void phia_destroy(phia_t *p) {
     cudaSetDevice(p->device);
     cudaStreamSynchronize(p->stream);
     free_replicas(p);
-    for (void *b : {(void *)p->d_Jk, (void *)p->d_Jf, (void *)p->d_hk, (void *)p->d_Jop, (void *)p->d_min_hit,
+    for (void *b : {(void *)p->d_Jk, (void *)p->d_Jf, (void *)p->d_hk, (void *)p->d_hf, (void *)p->d_hmax, (void *)p->d_Jop, (void *)p->d_min_hit,
                     (void *)p->d_iters, (void *)p->d_err, (void *)p->d_ctl, (void *)p->d_start_ns})
         pool_free(b, p->stream);
     cudaFree(p->d_rowptr); cudaFree(p->d_col); cudaFree(p->d_val);

@@ -1195,15 +1195,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 bool make_map(CUtensorMap *m, const void *base, int op, uint64_t inner_elems, uint64_t rows, uint64_t row_bytes,
               uint32_t box_rows) {
-    auto enc = encode_fn();
-    if (!enc) return false;
-    const CUtensorMapDataType dt = op == kOpE4M3 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    const cuuint64_t dims[2] = {inner_elems, rows};
-    const cuuint64_t strides[1] = {row_bytes};
-    const cuuint32_t box[2] = {(cuuint32_t)(kBKB / (op == kOpE4M3 ? 1 : 2)), box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(m, dt, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return tc_operand_map(m, base, op, inner_elems, rows, row_bytes, box_rows);
 }
 
 template <int OP, int BN, int CL, bool RING>
@@ -1455,6 +1447,19 @@ cudaError_t run_variant(const LargeBuffers &B, const RunArgs &a, cudaStream_t st
 
 }  // namespace
 
+bool tc_operand_map(void *map, const void *base, int op, uint64_t inner_elems, uint64_t rows, uint64_t row_bytes,
+                    uint32_t box_rows) {
+    auto enc = encode_fn();
+    if (!enc) return false;
+    const CUtensorMapDataType dt = op == kOpE4M3 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    const cuuint64_t dims[2] = {inner_elems, rows};
+    const cuuint64_t strides[1] = {row_bytes};
+    const cuuint32_t box[2] = {(cuuint32_t)(kBKB / (op == kOpE4M3 ? 1 : 2)), box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    return enc(static_cast<CUtensorMap *>(map), dt, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cudaStream_t st, int *launches) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1472,7 +1477,22 @@ cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cud
     // memory for three accumulators; where the mainloops set the pace they cut the bytes
     // per tile at the same tiles per CTA (N = 4000, 1200 replicas: 26.2 against 30.8 us
     // with 224-wide tiles, as the estimate has it).
-    const int lv = a.large_variant;
+    int lv = a.large_variant;
+    if ((lv == 0 || lv == 7) && B.ready && B.sbits && !a.field_mode) {
+        // Automatic, and variant 7: the kernel whose estimated iteration time is least -- the
+        // overlapped kernel with narrow tiles (k_tc_narrow.cu) or the one here (its estimate as below, with 1 us more of gap where a CTA has one tile, as
+        // measured at the sizes where the three meet).
+        double wide = 1e30;
+        for (int bn : {256, 224, 160, 128}) {
+            const double w = (double)(((int64_t)(B.Mpad / kBM) * ((a.R + bn - 1) / bn) + sms - 1) / sms);
+            const double E = 0.045 * bn, M = (double)B.Kbytes * (128 + bn) / 90000.0;
+            wide = std::min(wide, std::max(std::max(w * E, w * M), E + 2.5 + M));
+        }
+        int width = 0;
+        const double narrow = narrow_estimate(a.N, a.R, B.Kbytes, sms, &width);
+        if (narrow < wide) return launch_tc_narrow(B, a, op, width, st, launches, sms);
+        lv = 7;
+    }
     if ((lv == 7 || lv >= 10) && B.ready && B.sbits && !a.field_mode) {
         const int mt = B.Mpad / kBM;
         const int want = lv == 10 ? 256 : lv == 11 ? 224 : lv == 12 ? 128 : lv == 13 ? 160 : 0;
