@@ -352,10 +352,29 @@ bool takes_warp(const phia_t *p, const RunArgs &a) {
     return tc_small_tile_replicas(a.R, 0) < 16;
 }
 
+// Automatic handles of 129 .. 384 spins: whether this run takes the cluster kernel (which has no
+// early stop) instead of the warp-level one or the resident tcgen05 one.  By their estimated
+// times per iteration; measured (us) N = 256 x 256 1.08 against 1.18 (tcgen05) and 1.77 (warp),
+// 300 x 256 1.49 against 1.72, 384 x 256 1.50 against 1.89, 384 x 1024 3.05 against 1.89.
+bool takes_cluster(const phia_t *p, const RunArgs &a) {
+    if (p->path != PHIA_PATH_TC || p->large || p->inc || !p->auto_tile || p->tuned || a.field_mode || a.accept_test == 1 ||
+        a.stop_at_target || p->N <= 128)
+        return false;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) return false;
+    const int per_cta = tc_small_tile_replicas(a.R, 0);
+    const int waves = (a.R + per_cta * sms - 1) / (per_cta * sms);
+    const double other = takes_warp(p, a) ? warp_small_estimate(p->N, a.R, sms)
+                                          : waves * ((p->N <= 256 ? 1.2 : 1.9) + (per_cta == 16 ? 0.5 : 0.0) +
+                                                     (p->op == kOpBF16 ? 0.35 : 0.0));
+    return cluster_small_estimate(p->N, a.R, p->op) < other;
+}
+
 cudaError_t launch_path(phia_t *p, const RunArgs &a, int *launches) {
-    const bool warp = takes_warp(p, a);
+    const bool cluster = takes_cluster(p, a), warp = !cluster && takes_warp(p, a);
     if (!a.field_mode)
-        p->last_kernel = p->path != PHIA_PATH_TC ? 0 : p->large ? 2 : warp ? 3 : p->inc ? 4 : 1;
+        p->last_kernel = p->path != PHIA_PATH_TC ? 0 : p->large || cluster ? 2 : warp ? 3 : p->inc ? 4 : 1;
+    if (cluster) return launch_cluster_small(a, p->op, p->stream, launches);
     if (p->path == PHIA_PATH_TC && p->large) {
         LargeBuffers B;
         B.Jop = p->d_Jop; B.S = p->d_S; B.Epart = p->d_Epart; B.flags = p->d_flags; B.ready = p->d_ready;

@@ -1480,7 +1480,8 @@ cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cud
     int lv = a.large_variant;
     if ((lv == 0 || lv == 7) && B.ready && B.sbits && !a.field_mode) {
         // Automatic, and variant 7: the kernel whose estimated iteration time is least -- the
-        // overlapped kernel with narrow tiles (k_tc_narrow.cu) or the one here (its estimate as below, with 1 us more of gap where a CTA has one tile, as
+        // cluster kernel (k_cluster.cu), the overlapped kernel with narrow tiles (k_tc_narrow.cu) or
+        // the one here (its estimate as below, with 1 us more of gap where a CTA has one tile, as
         // measured at the sizes where the three meet).
         double wide = 1e30;
         for (int bn : {256, 224, 160, 128}) {
@@ -1490,6 +1491,8 @@ cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cud
         }
         int width = 0;
         const double narrow = narrow_estimate(a.N, a.R, B.Kbytes, sms, &width);
+        if (!a.stall_producer && cluster_small_estimate(a.N, a.R, op) < std::min(narrow, wide))
+            return launch_cluster_small(a, op, st, launches);
         if (narrow < wide) return launch_tc_narrow(B, a, op, width, st, launches, sms);
         lv = 7;
     }

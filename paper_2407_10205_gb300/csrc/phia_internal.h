@@ -258,12 +258,20 @@ int set_last_error(int code, const char *msg);
 // instances with at most nmax spins.
 int warp_small_max_n();
 // Automatic handles take it up to here: with 17 warps the registers run short (N = 256: 1.3 to
-// 1.8 us an iteration, against 1.18 for the tcgen05 one).
+// 1.8 us an iteration, against 1.05 for the cluster kernel and 1.18 for the tcgen05 one).
 int warp_small_auto_n();
 cudaError_t launch_warp_small(const RunArgs &a, cudaStream_t st, int *launches);
 cudaError_t launch_warp_small_batch(const RunArgs &a, int nmax, cudaStream_t st);
 // Its estimated time per iteration (us).
 double warp_small_estimate(int N, int R, int sms);
+
+// The same over thread-block clusters, 128 spins a CTA, 8 replicas a cluster (no field mode and
+// no early stop): cluster_small_min_n() <= N <= cluster_small_max_n(op).
+int cluster_small_min_n();
+int cluster_small_max_n(int op);
+cudaError_t launch_cluster_small(const RunArgs &a, int op, cudaStream_t st, int *launches);
+// Its estimated time per iteration (us; 1e30 where it does not apply).
+double cluster_small_estimate(int N, int R, int op);
 
 // Incremental-field resident kernel for small dense instances (CUDA cores, exact
 // integer field updated by the columns whose spin changed sign; no field mode).
