@@ -67,7 +67,7 @@ extern "C" {
 #define PHIA_OP_AUTO 0     /* E4M3 when every |k| <= 16, else BF16 */
 #define PHIA_OP_E4M3 1     /* FP8 e4m3, exact for |k| <= 16 */
 #define PHIA_OP_BF16 2     /* BF16, exact for every int8 k */
-#define PHIA_PEAK_S8_MMA_SYNC 3   /* phia_mma_peak only: warp-level int8 mma.sync (the int8 kernel's route) */
+#define PHIA_PEAK_S8_MMA_SYNC 3   /* phia_mma_peak only: warp-level int8 mma.sync */
 
 typedef struct phia_opts {
     int32_t path;          /* PHIA_PATH_* */

@@ -40,17 +40,36 @@ int fail(int code, const char *fmt, ...) {
         if (e_ != cudaSuccess) return fail(PHIA_ECUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
     } while (0)
 
-__global__ void reset_records_kernel(int R, int W, int64_t *best_e, int64_t *best_step, int64_t *hit,
-                                     uint32_t *bits, uint64_t *hit_ns, uint64_t *start_ns) {
+// Counters of a run, at the head of a handle's record block: one copy brings them and the
+// per-replica records back.
+struct RunCounters {
+    int32_t err, pad;
+    unsigned long long iters, min_hit;
+    uint64_t start_ns;
+};
+
+// The state before a run: counters, acceptance counts and, when the records start afresh,
+// best / target records and best states.
+__global__ void reset_run_kernel(int R, int W, int reset, RunCounters *ctr, int64_t *best_e, int64_t *best_step, int64_t *hit,
+                                 uint64_t *hit_ns, uint32_t *bits, int64_t *prop, int64_t *acc) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < R) {
-        best_e[idx] = LLONG_MAX;
-        best_step[idx] = -1;
-        hit[idx] = -1;
-        hit_ns[idx] = 0;
+    if (idx == 0) {
+        ctr->err = 0;
+        ctr->iters = 0;
+        ctr->min_hit = ~0ull;
+        if (reset) ctr->start_ns = phia::globaltimer_ns();   // the run's start on the device clock
     }
-    if (idx < (int64_t)R * W) bits[idx] = 0u;
-    if (idx == 0) *start_ns = phia::globaltimer_ns();   // the run's start on the device clock
+    if (idx < R) {
+        prop[idx] = 0;
+        acc[idx] = 0;
+        if (reset) {
+            best_e[idx] = LLONG_MAX;
+            best_step[idx] = -1;
+            hit[idx] = -1;
+            hit_ns[idx] = 0;
+        }
+    }
+    if (reset && idx < (int64_t)R * W) bits[idx] = 0u;
 }
 
 // J = k q in FP32 for the FP32 path, from the device copy of k.
@@ -114,6 +133,9 @@ struct phia_s {
     float *d_x = nullptr, *d_v = nullptr;
     int8_t *d_s0 = nullptr, *d_s1 = nullptr;
     int64_t *d_eacc = nullptr;
+    // record block: RunCounters, then best energy, its iteration, first hit and %globaltimer of the
+    // hit per replica (R_cap entries each)
+    uint8_t *d_rec = nullptr;
     int64_t *d_best_e = nullptr, *d_best_step = nullptr, *d_hit = nullptr;
     uint32_t *d_bits = nullptr;
     int64_t *d_prop = nullptr, *d_acc = nullptr;   // acceptance test counts per replica (Table 3, state 4)
@@ -142,15 +164,17 @@ struct phia_s {
     int stall_producer = 0;             // testing aid: the per-iteration kernel's TMA producer issues nothing
 };
 
+// Device buffers of handles, batches and server requests come from one stream-ordered memory
+// pool per device.  Creating and destroying them in a loop, as a caller with a new instance per
+// request does, then costs neither cudaMalloc round trips nor the device-wide synchronisation
+// of cudaFree, which waits for the other requests' kernels; freed blocks beyond 1/16 of the
+// device's memory go back at the next synchronisation.
 namespace {
-
-// A handle's device buffers come from one stream-ordered memory pool per device that
-// keeps freed blocks (release threshold at its maximum).  Creating and destroying handles
-// in a loop, as a caller with a new instance per request does, then costs neither
-// cudaMalloc round trips nor the device-wide synchronisation of cudaFree; the pool keeps
-// its peak size reserved for the process.
 std::mutex g_pool_mu;
 std::map<int, cudaMemPool_t> g_pools;
+}  // namespace
+
+namespace phia {
 
 cudaError_t pool_alloc(void **ptr, size_t bytes, int device, cudaStream_t st) {
     cudaMemPool_t pool = nullptr;
@@ -163,9 +187,12 @@ cudaError_t pool_alloc(void **ptr, size_t bytes, int device, cudaStream_t st) {
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
             props.location.id = device;
-            cudaError_t e = cudaMemPoolCreate(&pool, &props);
+            cudaDeviceProp dp;
+            cudaError_t e = cudaGetDeviceProperties(&dp, device);
             if (e != cudaSuccess) return e;
-            uint64_t keep = UINT64_MAX;
+            e = cudaMemPoolCreate(&pool, &props);
+            if (e != cudaSuccess) return e;
+            uint64_t keep = dp.totalGlobalMem / 16;
             e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
             if (e != cudaSuccess) return e;
             g_pools[device] = pool;
@@ -180,13 +207,16 @@ void pool_free(void *ptr, cudaStream_t st) {
     if (ptr) cudaFreeAsync(ptr, st);
 }
 
+}  // namespace phia
+
+namespace {
+
 void free_replicas(phia_t *p) {
     for (void *b : {(void *)p->d_S, (void *)p->d_Epart, (void *)p->d_flags, (void *)p->d_ready, (void *)p->d_sbits,
                     (void *)p->d_X,
                     (void *)p->d_V,
                     (void *)p->d_x, (void *)p->d_v, (void *)p->d_s0, (void *)p->d_s1, (void *)p->d_eacc,
-                    (void *)p->d_best_e, (void *)p->d_best_step, (void *)p->d_hit, (void *)p->d_bits,
-                    (void *)p->d_hit_ns, (void *)p->d_prop, (void *)p->d_acc, (void *)p->d_xstart,
+                    (void *)p->d_rec, (void *)p->d_bits, (void *)p->d_prop, (void *)p->d_acc, (void *)p->d_xstart,
                     (void *)p->d_elast, (void *)p->d_estart, (void *)p->d_xxs, (void *)p->d_vvs, (void *)p->d_hass})
         pool_free(b, p->stream);
     p->d_prop = p->d_acc = nullptr; p->d_xstart = nullptr; p->d_elast = p->d_estart = nullptr;
@@ -194,7 +224,8 @@ void free_replicas(phia_t *p) {
     p->d_S = nullptr; p->d_Epart = nullptr; p->d_flags = nullptr; p->d_ready = nullptr; p->d_sbits = nullptr;
     p->d_X = p->d_V = nullptr;
     p->d_x = p->d_v = nullptr; p->d_s0 = p->d_s1 = nullptr; p->d_eacc = nullptr;
-    p->d_best_e = p->d_best_step = p->d_hit = nullptr; p->d_bits = nullptr; p->d_hit_ns = nullptr;
+    p->d_rec = nullptr; p->d_best_e = p->d_best_step = p->d_hit = nullptr; p->d_bits = nullptr; p->d_hit_ns = nullptr;
+    p->d_min_hit = p->d_iters = nullptr; p->d_err = nullptr; p->d_start_ns = nullptr;
     p->R_cap = 0;
 }
 
@@ -228,10 +259,7 @@ int ensure_replicas(phia_t *p, int R) {
         al((void **)&p->d_X, Rp * Mp * 4); al((void **)&p->d_V, Rp * Mp * 4);
     }
     al((void **)&p->d_eacc, (size_t)R * 8);
-    al((void **)&p->d_best_e, (size_t)R * 8);
-    al((void **)&p->d_best_step, (size_t)R * 8);
-    al((void **)&p->d_hit, (size_t)R * 8);
-    al((void **)&p->d_hit_ns, (size_t)R * 8);
+    al((void **)&p->d_rec, sizeof(RunCounters) + 4 * (size_t)R * 8);
     al((void **)&p->d_bits, (size_t)R * p->W * 4);
     if (!ok) {
         cudaGetLastError();
@@ -239,6 +267,16 @@ int ensure_replicas(phia_t *p, int R) {
         return fail(PHIA_ENOMEM, "device allocation for %d replicas failed", R);
     }
     p->cap_large = p->large;
+    RunCounters *ctr = reinterpret_cast<RunCounters *>(p->d_rec);
+    p->d_err = &ctr->err;
+    p->d_iters = &ctr->iters;
+    p->d_min_hit = &ctr->min_hit;
+    p->d_start_ns = &ctr->start_ns;
+    p->d_best_e = reinterpret_cast<int64_t *>(p->d_rec + sizeof(RunCounters));
+    p->d_best_step = p->d_best_e + R;
+    p->d_hit = p->d_best_step + R;
+    p->d_hit_ns = reinterpret_cast<uint64_t *>(p->d_hit + R);
+    CU(cudaMemsetAsync(p->d_rec, 0, sizeof(RunCounters), p->stream));
     CU(cudaMemsetAsync(p->d_eacc, 0, (size_t)R * 8, p->stream));
     if (p->large) {
         const size_t Rp = (size_t)large_rpad_handle(R);
@@ -250,11 +288,11 @@ int ensure_replicas(phia_t *p, int R) {
     return PHIA_OK;
 }
 
-int reset_records(phia_t *p, int R) {
-    const int64_t n = std::max<int64_t>(R, (int64_t)R * p->W);
-    reset_records_kernel<<<(unsigned)((n + 255) / 256), 256, 0, p->stream>>>(R, p->W, p->d_best_e, p->d_best_step,
-                                                                             p->d_hit, p->d_bits, p->d_hit_ns,
-                                                                             p->d_start_ns);
+int reset_run(phia_t *p, int R, bool reset) {
+    const int64_t n = std::max<int64_t>(R, reset ? (int64_t)R * p->W : 0);
+    reset_run_kernel<<<(unsigned)((n + 255) / 256), 256, 0, p->stream>>>(
+        R, p->W, reset ? 1 : 0, reinterpret_cast<RunCounters *>(p->d_rec), p->d_best_e, p->d_best_step, p->d_hit,
+        p->d_hit_ns, p->d_bits, p->d_prop, p->d_acc);
     CU(cudaGetLastError());
     return PHIA_OK;
 }
@@ -415,12 +453,6 @@ int finish_create(phia_t *p, const int32_t *h_k, const phia_opts *opts,
     CU(pool_alloc((void **)&p->d_hf, (size_t)round_up(p->N, 16) * 4, p->device, p->stream));
     CU(pool_alloc((void **)&p->d_hmax, 4, p->device, p->stream));
     CU(launch_pad_field(p->d_hk, p->N, p->d_hf, p->d_hmax, p->stream));
-    CU(pool_alloc((void **)&p->d_min_hit, 8, p->device, p->stream));
-    CU(pool_alloc((void **)&p->d_start_ns, 8, p->device, p->stream));
-    CU(cudaMemsetAsync(p->d_start_ns, 0, 8, p->stream));
-    CU(pool_alloc((void **)&p->d_iters, 8, p->device, p->stream));
-    CU(pool_alloc((void **)&p->d_err, 4, p->device, p->stream));
-    CU(cudaMemsetAsync(p->d_err, 0, 4, p->stream));
     CU(pool_alloc((void **)&p->d_ctl, sizeof(IterCtl), p->device, p->stream));
     p->graphs = step_graphs_new();
     CU(cudaEventCreate(&p->ev0));
@@ -732,15 +764,8 @@ static int run_impl(phia_t *p, const phia_schedule *sched, int32_t R, int64_t t0
     }
     rc = ensure_replicas(p, R);
     if (rc) return rc;
-    if (reset) {
-        rc = reset_records(p, R);
-        if (rc) return rc;
-    }
-    CU(cudaMemsetAsync(p->d_min_hit, 0xFF, 8, p->stream));
-    CU(cudaMemsetAsync(p->d_iters, 0, 8, p->stream));
-    CU(cudaMemsetAsync(p->d_err, 0, 4, p->stream));
-    CU(cudaMemsetAsync(p->d_prop, 0, (size_t)R * 8, p->stream));
-    CU(cudaMemsetAsync(p->d_acc, 0, (size_t)R * 8, p->stream));
+    rc = reset_run(p, R, reset != 0);
+    if (rc) return rc;
     RunArgs a = base_args(p, R);
     a.accept_test = sched->accept_test;
     a.proposed = p->d_prop;
@@ -752,7 +777,7 @@ static int run_impl(phia_t *p, const phia_schedule *sched, int32_t R, int64_t t0
     a.seed = seed;
     a.x_in = x_in; a.v_in = v_in; a.x_out = x_out; a.v_out = v_out;
     a.has_target = sched->has_target; a.stop_at_target = sched->stop_at_target; a.target = sched->target_k;
-    int launches = reset ? 1 : 0;
+    int launches = 1;
     CU(cudaEventRecord(p->ev0, p->stream));
     cudaError_t e = launch_path(p, a, &launches);
     if (e != cudaSuccess) return fail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
@@ -899,34 +924,44 @@ int phia_sync(phia_t *p) {
     return PHIA_OK;
 }
 
-static int fetch_records(phia_t *p, std::vector<int64_t> &be, std::vector<int64_t> &bs, std::vector<int64_t> &hs) {
+// The last run's counters and records (R = R_last entries each), in one copy.
+struct HostRecords {
+    std::vector<uint8_t> raw;
+    RunCounters ctr;
+    int R = 0;
+    const int64_t *be = nullptr, *bs = nullptr, *hs = nullptr;
+    const uint64_t *hit_ns = nullptr;
+};
+
+static int fetch_records(phia_t *p, HostRecords &h) {
     if (!p->ran) return fail(PHIA_ESTATE, "no run on this handle yet");
     CU(cudaSetDevice(p->device));
+    const size_t cap = (size_t)p->R_cap;
+    h.raw.resize(sizeof(RunCounters) + 4 * cap * 8);
+    CU(cudaMemcpyAsync(h.raw.data(), p->d_rec, h.raw.size(), cudaMemcpyDeviceToHost, p->stream));
     CU(cudaStreamSynchronize(p->stream));
-    int32_t err = 0;
-    CU(cudaMemcpy(&err, p->d_err, 4, cudaMemcpyDeviceToHost));
-    if (err) return fail(PHIA_ETIMEOUT, "a bounded device wait expired during the run");
-    const int R = p->R_last;
-    be.resize(R); bs.resize(R); hs.resize(R);
-    CU(cudaMemcpy(be.data(), p->d_best_e, (size_t)R * 8, cudaMemcpyDeviceToHost));
-    CU(cudaMemcpy(bs.data(), p->d_best_step, (size_t)R * 8, cudaMemcpyDeviceToHost));
-    CU(cudaMemcpy(hs.data(), p->d_hit, (size_t)R * 8, cudaMemcpyDeviceToHost));
+    memcpy(&h.ctr, h.raw.data(), sizeof h.ctr);
+    if (h.ctr.err) return fail(PHIA_ETIMEOUT, "a bounded device wait expired during the run");
+    h.R = p->R_last;
+    h.be = reinterpret_cast<const int64_t *>(h.raw.data() + sizeof(RunCounters));
+    h.bs = h.be + cap;
+    h.hs = h.bs + cap;
+    h.hit_ns = reinterpret_cast<const uint64_t *>(h.hs + cap);
     return PHIA_OK;
 }
 
 // Result replica: with stop-at-target and a hit, the earliest hit (ties: lowest index);
 // otherwise the lowest energy (ties: earliest step, then lowest index).
-static int pick_result(phia_t *p, const std::vector<int64_t> &be, const std::vector<int64_t> &bs,
-                       const std::vector<int64_t> &hs) {
+static int pick_result(const phia_t *p, const HostRecords &h) {
     int best = -1;
     if (p->last_stop) {
-        for (int r = 0; r < (int)hs.size(); ++r)
-            if (hs[r] >= 0 && (best < 0 || hs[r] < hs[best])) best = r;
+        for (int r = 0; r < h.R; ++r)
+            if (h.hs[r] >= 0 && (best < 0 || h.hs[r] < h.hs[best])) best = r;
         if (best >= 0) return best;
     }
-    for (int r = 0; r < (int)be.size(); ++r) {
-        if (bs[r] < 0) continue;
-        if (best < 0 || be[r] < be[best] || (be[r] == be[best] && bs[r] < bs[best])) best = r;
+    for (int r = 0; r < h.R; ++r) {
+        if (h.bs[r] < 0) continue;
+        if (best < 0 || h.be[r] < h.be[best] || (h.be[r] == h.be[best] && h.bs[r] < h.bs[best])) best = r;
     }
     return best;
 }
@@ -934,12 +969,12 @@ static int pick_result(phia_t *p, const std::vector<int64_t> &be, const std::vec
 int phia_best(phia_t *p, int64_t *energy_k, int8_t *spins) {
     if (!p) return fail(PHIA_EINVAL, "handle is NULL");
     if (p->batch) return batch_best(p->batch, 0, energy_k, spins);
-    std::vector<int64_t> be, bs, hs;
-    int rc = fetch_records(p, be, bs, hs);
+    HostRecords h;
+    int rc = fetch_records(p, h);
     if (rc) return rc;
-    const int r = pick_result(p, be, bs, hs);
+    const int r = pick_result(p, h);
     if (r < 0) return fail(PHIA_ESTATE, "no replica recorded a state");
-    if (energy_k) *energy_k = be[r];
+    if (energy_k) *energy_k = h.be[r];
     if (spins) {
         std::vector<uint32_t> w(p->W);
         CU(cudaMemcpy(w.data(), p->d_bits + (size_t)r * p->W, (size_t)p->W * 4, cudaMemcpyDeviceToHost));
@@ -962,12 +997,8 @@ int phia_gahmc(phia_t *p, const phia_gahmc_schedule *sched, int32_t R, int64_t K
     CU(cudaSetDevice(p->device));
     int rc = ensure_replicas(p, R);
     if (rc) return rc;
-    rc = reset_records(p, R);
+    rc = reset_run(p, R, true);
     if (rc) return rc;
-    CU(cudaMemsetAsync(p->d_iters, 0, 8, p->stream));
-    CU(cudaMemsetAsync(p->d_err, 0, 4, p->stream));
-    CU(cudaMemsetAsync(p->d_prop, 0, (size_t)R * 8, p->stream));
-    CU(cudaMemsetAsync(p->d_acc, 0, (size_t)R * 8, p->stream));
     RunArgs a = base_args(p, R);
     a.beta0 = sched->beta0; a.beta1 = sched->beta1;
     a.seed = seed;
@@ -989,8 +1020,8 @@ int phia_gahmc(phia_t *p, const phia_gahmc_schedule *sched, int32_t R, int64_t K
 int phia_acceptance(phia_t *p, int32_t R, int64_t *proposed, int64_t *accepted) {
     if (!p) return fail(PHIA_EINVAL, "handle is NULL");
     if (p->batch) return fail(PHIA_ENOTSUP, "the acceptance test does not run on the CSR path");
-    std::vector<int64_t> be, bs, hs;
-    int rc = fetch_records(p, be, bs, hs);
+    HostRecords h;
+    int rc = fetch_records(p, h);
     if (rc) return rc;
     if (R != p->R_last) return fail(PHIA_EINVAL, "replicas (%d) differs from the last run (%d)", R, p->R_last);
     if (proposed) CU(cudaMemcpy(proposed, p->d_prop, (size_t)R * 8, cudaMemcpyDeviceToHost));
@@ -1002,13 +1033,13 @@ int phia_replica_results(phia_t *p, int32_t R, int64_t *best_energy_k, int64_t *
                          uint32_t *best_bits) {
     if (!p) return fail(PHIA_EINVAL, "handle is NULL");
     if (p->batch) return batch_replica_results(p->batch, 0, R, best_energy_k, best_step, hit_step, best_bits);
-    std::vector<int64_t> be, bs, hs;
-    int rc = fetch_records(p, be, bs, hs);
+    HostRecords h;
+    int rc = fetch_records(p, h);
     if (rc) return rc;
     if (R != p->R_last) return fail(PHIA_EINVAL, "replicas (%d) differs from the last run (%d)", R, p->R_last);
-    if (best_energy_k) memcpy(best_energy_k, be.data(), (size_t)R * 8);
-    if (best_step) memcpy(best_step, bs.data(), (size_t)R * 8);
-    if (hit_step) memcpy(hit_step, hs.data(), (size_t)R * 8);
+    if (best_energy_k) memcpy(best_energy_k, h.be, (size_t)R * 8);
+    if (best_step) memcpy(best_step, h.bs, (size_t)R * 8);
+    if (hit_step) memcpy(hit_step, h.hs, (size_t)R * 8);
     if (best_bits) CU(cudaMemcpy(best_bits, p->d_bits, (size_t)R * p->W * 4, cudaMemcpyDeviceToHost));
     return PHIA_OK;
 }
@@ -1016,30 +1047,26 @@ int phia_replica_results(phia_t *p, int32_t R, int64_t *best_energy_k, int64_t *
 int phia_stats_get(phia_t *p, phia_stats *out) {
     if (!p || !out) return fail(PHIA_EINVAL, "NULL argument");
     if (p->batch) return batch_stats(p->batch, 0, out);
-    std::vector<int64_t> be, bs, hs;
-    int rc = fetch_records(p, be, bs, hs);
+    HostRecords h;
+    int rc = fetch_records(p, h);
     if (rc) return rc;
     memset(out, 0, sizeof *out);
-    unsigned long long iters = 0;
-    CU(cudaMemcpy(&iters, p->d_iters, 8, cudaMemcpyDeviceToHost));
     float ms = 0.f;
     CU(cudaEventElapsedTime(&ms, p->ev0, p->ev1));
     out->replicas = p->R_last;
     out->steps = p->last_steps;
-    out->spin_updates = (int64_t)iters * p->N;
-    const int r = pick_result(p, be, bs, hs);
+    out->spin_updates = (int64_t)h.ctr.iters * p->N;
+    const int r = pick_result(p, h);
     out->best_replica = r;
-    out->best_energy_k = r >= 0 ? be[r] : 0;
-    out->best_step = r >= 0 ? bs[r] : -1;
+    out->best_energy_k = r >= 0 ? h.be[r] : 0;
+    out->best_step = r >= 0 ? h.bs[r] : -1;
     out->hit_step = -1;
     out->hit_replica = -1;
-    for (int k = 0; k < (int)hs.size(); ++k)
-        if (hs[k] >= 0 && (out->hit_step < 0 || hs[k] < out->hit_step)) { out->hit_step = hs[k]; out->hit_replica = k; }
+    for (int k = 0; k < h.R; ++k)
+        if (h.hs[k] >= 0 && (out->hit_step < 0 || h.hs[k] < out->hit_step)) { out->hit_step = h.hs[k]; out->hit_replica = k; }
     out->hit_ns = -1;
     if (out->hit_replica >= 0) {
-        uint64_t t_hit = 0, t_start = 0;
-        CU(cudaMemcpy(&t_hit, p->d_hit_ns + out->hit_replica, 8, cudaMemcpyDeviceToHost));
-        CU(cudaMemcpy(&t_start, p->d_start_ns, 8, cudaMemcpyDeviceToHost));
+        const uint64_t t_hit = h.hit_ns[out->hit_replica], t_start = h.ctr.start_ns;
         if (t_hit >= t_start && t_start != 0) out->hit_ns = (int64_t)(t_hit - t_start);
     }
     out->device_ms = ms;
@@ -1056,8 +1083,7 @@ void phia_destroy(phia_t *p) {
     cudaSetDevice(p->device);
     cudaStreamSynchronize(p->stream);
     free_replicas(p);
-    for (void *b : {(void *)p->d_Jk, (void *)p->d_Jf, (void *)p->d_hk, (void *)p->d_hf, (void *)p->d_hmax, (void *)p->d_Jop, (void *)p->d_min_hit,
-                    (void *)p->d_iters, (void *)p->d_err, (void *)p->d_ctl, (void *)p->d_start_ns})
+    for (void *b : {(void *)p->d_Jk, (void *)p->d_Jf, (void *)p->d_hk, (void *)p->d_hf, (void *)p->d_hmax, (void *)p->d_Jop, (void *)p->d_ctl})
         pool_free(b, p->stream);
     cudaFree(p->d_rowptr); cudaFree(p->d_col); cudaFree(p->d_val);
     step_graphs_free(p->graphs);

@@ -75,6 +75,7 @@ struct phia_batch_s {
     StepGraphCache *graphs = nullptr;       // its step launches as replayable graphs
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     bool ran = false;
+    bool waits_checked = false;         // the last run's error flag has been read (and is clear)
     int64_t last_steps = 0;
     int last_launches = 0;
     int last_stop = 0;
@@ -111,9 +112,9 @@ __global__ void batch_reset_records(int64_t n, int64_t nbits, int64_t *best_e, i
 }
 
 void free_state(phia_batch_s *b) {
-    cudaFree(b->d_X); cudaFree(b->d_V); cudaFree(b->d_S); cudaFree(b->d_Esum); cudaFree(b->d_flags);
-    cudaFree(b->d_best_e); cudaFree(b->d_best_step); cudaFree(b->d_hit); cudaFree(b->d_bits);
-    cudaFree(b->d_hit_ns);
+    for (void *p : {(void *)b->d_X, (void *)b->d_V, (void *)b->d_S, (void *)b->d_Esum, (void *)b->d_flags,
+                    (void *)b->d_best_e, (void *)b->d_bits, (void *)b->d_hit_ns})
+        pool_free(p, b->stream);
     b->d_X = b->d_V = nullptr; b->d_S = nullptr; b->d_Esum = nullptr; b->d_flags = nullptr;
     b->d_best_e = b->d_best_step = b->d_hit = nullptr; b->d_bits = nullptr; b->d_hit_ns = nullptr;
     b->Rcap = 0;
@@ -189,16 +190,16 @@ int ensure_state(phia_batch_s *b, int R) {
     const int64_t reps = (int64_t)R * b->count;
     bool ok = true;
     auto al = [&](void **p, size_t n) {
-        if (ok && cudaMalloc(p, std::max<size_t>(n, 16)) != cudaSuccess) ok = false;
+        if (ok && pool_alloc(p, n, b->device, b->stream) != cudaSuccess) ok = false;
     };
     al((void **)&b->d_X, (size_t)rows * R * 4);
     al((void **)&b->d_V, (size_t)rows * R * 4);
     al((void **)&b->d_S, (size_t)4 * rows * (R / 32) * 4);
     al((void **)&b->d_Esum, (size_t)2 * reps * 8);
     al((void **)&b->d_flags, (size_t)2 * reps);
-    al((void **)&b->d_best_e, (size_t)reps * 8);
-    al((void **)&b->d_best_step, (size_t)reps * 8);
-    al((void **)&b->d_hit, (size_t)reps * 8);
+    al((void **)&b->d_best_e, (size_t)3 * reps * 8);   // best energy, its iteration, first hit
+    b->d_best_step = b->d_best_e + reps;
+    b->d_hit = b->d_best_step + reps;
     al((void **)&b->d_hit_ns, (size_t)reps * 8);
     al((void **)&b->d_bits, (size_t)bits * 4);
     if (!ok) {
@@ -448,10 +449,12 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
     b->device = o.device;
     b->stream = (cudaStream_t)o.stream;
     bool ok = true;
+    auto al = [&](void **dst, size_t bytes) {
+        if (ok && pool_alloc(dst, bytes, b->device, b->stream) != cudaSuccess) ok = false;
+    };
     auto up = [&](void **dst, const void *src, size_t bytes) {
-        if (!ok) return;
-        if (cudaMalloc(dst, std::max<size_t>(bytes, 16)) != cudaSuccess) { ok = false; return; }
-        if (bytes && cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+        al(dst, bytes);
+        if (ok && bytes && cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, b->stream) != cudaSuccess) ok = false;
     };
     up((void **)&b->d_slice, slice.data(), slice.size() * 4);
     b->col16 = b->max_np <= 16384;
@@ -467,17 +470,16 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
     up((void **)&b->d_blocks, b->blocks.data(), b->blocks.size() * sizeof(CsrBlock));
     up((void **)&b->d_targets, b->targets.data(), b->targets.size() * sizeof(long long));
     up((void **)&b->d_dJ, dj.data(), dj.size());
-    if (ok && cudaMalloc((void **)&b->d_inst, sizeof(CsrInst) * std::max<size_t>(b->inst.size(), 1)) != cudaSuccess)
-        ok = false;
-    if (ok && cudaMalloc((void **)&b->d_sets, sizeof(CsrSet) * std::max<size_t>(b->inst.size(), 1)) != cudaSuccess)
-        ok = false;
-    if (ok && cudaMalloc((void **)&b->d_min_hit, 8) != cudaSuccess) ok = false;
-    if (ok && cudaMalloc((void **)&b->d_start_ns, 8) != cudaSuccess) ok = false;
-    if (ok && cudaMemset(b->d_start_ns, 0, 8) != cudaSuccess) ok = false;
-    if (ok && cudaMalloc((void **)&b->d_iters, 8) != cudaSuccess) ok = false;
-    if (ok && cudaMalloc((void **)&b->d_err, 4) != cudaSuccess) ok = false;
-    if (ok && cudaMalloc((void **)&b->d_ctl, sizeof(IterCtl)) != cudaSuccess) ok = false;
-    if (ok && cudaMalloc((void **)&b->d_sync, 4 * sizeof(unsigned)) != cudaSuccess) ok = false;
+    al((void **)&b->d_inst, sizeof(CsrInst) * b->inst.size());
+    al((void **)&b->d_sets, sizeof(CsrSet) * b->inst.size());
+    al((void **)&b->d_min_hit, 8);
+    al((void **)&b->d_start_ns, 8);
+    al((void **)&b->d_iters, 8);
+    al((void **)&b->d_err, 4);
+    al((void **)&b->d_ctl, sizeof(IterCtl));
+    al((void **)&b->d_sync, 4 * sizeof(unsigned));
+    if (ok && cudaMemsetAsync(b->d_start_ns, 0, 8, b->stream) != cudaSuccess) ok = false;
+    if (ok && cudaStreamSynchronize(b->stream) != cudaSuccess) ok = false;    // the host arrays end here
     if (ok) b->graphs = step_graphs_new();
     if (ok && (cudaEventCreate(&b->ev0) != cudaSuccess || cudaEventCreate(&b->ev1) != cudaSuccess)) ok = false;
     if (!ok) {
@@ -532,6 +534,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     BCU(cudaMemsetAsync(b->d_min_hit, 0xFF, 8, b->stream));
     BCU(cudaMemsetAsync(b->d_iters, 0, 8, b->stream));
     BCU(cudaMemsetAsync(b->d_err, 0, 4, b->stream));
+    b->waits_checked = false;
     CsrArgs C;
     memset(&C, 0, sizeof C);
     RunArgs &a = C.a;
@@ -620,9 +623,9 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
             if (b->small_host.size() > beg) groups.push_back(SmallGroup{beg, b->small_host.size(), nmax});
         }
         if (b->small_host.size() > b->small_cap) {
-            cudaFree(b->d_small);
+            pool_free(b->d_small, b->stream);
             b->d_small = nullptr;
-            if (cudaMalloc((void **)&b->d_small, b->small_host.size() * sizeof(SmallCta)) != cudaSuccess)
+            if (pool_alloc((void **)&b->d_small, b->small_host.size() * sizeof(SmallCta), b->device, b->stream) != cudaSuccess)
                 return bfail(PHIA_ENOMEM, "CTA table allocation failed");
             b->small_cap = b->small_host.size();
         }
@@ -669,15 +672,19 @@ int batch_records(phia_batch_s *b, int inst, std::vector<int64_t> &be, std::vect
     if (inst < 0 || inst >= b->count) return bfail(PHIA_EINVAL, "instance %d out of range", inst);
     BCU(cudaSetDevice(b->device));
     BCU(cudaStreamSynchronize(b->stream));
-    int32_t err = 0;
-    BCU(cudaMemcpy(&err, b->d_err, 4, cudaMemcpyDeviceToHost));
-    if (err) return bfail(PHIA_ETIMEOUT, "a bounded device wait expired during the run");
-    const int n = b->R_real;
-    const size_t off = (size_t)inst * b->R;
-    be.resize(n); bs.resize(n); hs.resize(n);
-    BCU(cudaMemcpy(be.data(), b->d_best_e + off, (size_t)n * 8, cudaMemcpyDeviceToHost));
-    BCU(cudaMemcpy(bs.data(), b->d_best_step + off, (size_t)n * 8, cudaMemcpyDeviceToHost));
-    BCU(cudaMemcpy(hs.data(), b->d_hit + off, (size_t)n * 8, cudaMemcpyDeviceToHost));
+    if (!b->waits_checked) {        // the finished run's error flag, once
+        int32_t err = 0;
+        BCU(cudaMemcpy(&err, b->d_err, 4, cudaMemcpyDeviceToHost));
+        if (err) return bfail(PHIA_ETIMEOUT, "a bounded device wait expired during the run");
+        b->waits_checked = true;
+    }
+    const size_t n = (size_t)b->R_real, off = (size_t)inst * b->R;
+    std::vector<int64_t> raw(3 * n);            // the three records of the instance in one copy
+    BCU(cudaMemcpy2D(raw.data(), n * 8, b->d_best_e + off, (size_t)(b->d_best_step - b->d_best_e) * 8, n * 8, 3,
+                     cudaMemcpyDeviceToHost));
+    be.assign(raw.begin(), raw.begin() + n);
+    bs.assign(raw.begin() + n, raw.begin() + 2 * n);
+    hs.assign(raw.begin() + 2 * n, raw.end());
     return PHIA_OK;
 }
 
@@ -846,11 +853,11 @@ void phia_batch_destroy(phia_batch_t *b) {
     cudaSetDevice(b->device);
     cudaStreamSynchronize(b->stream);
     free_state(b);
-    cudaFree(b->d_inst); cudaFree(b->d_blocks); cudaFree(b->d_slice); cudaFree(b->d_col); cudaFree(b->d_val);
-    cudaFree(b->d_sets); cudaFree(b->d_hk2); cudaFree(b->d_rowof); cudaFree(b->d_posof);
-    cudaFree(b->d_hk); cudaFree(b->d_targets); cudaFree(b->d_min_hit); cudaFree(b->d_start_ns); cudaFree(b->d_iters); cudaFree(b->d_err);
-    cudaFree(b->d_dJ); cudaFree(b->d_small); cudaFree(b->d_sync);
-    cudaFree(b->d_ctl);
+    for (void *p : {(void *)b->d_inst, (void *)b->d_blocks, (void *)b->d_slice, b->d_col, (void *)b->d_val,
+                    (void *)b->d_sets, (void *)b->d_hk2, (void *)b->d_rowof, (void *)b->d_posof, (void *)b->d_hk,
+                    (void *)b->d_targets, (void *)b->d_min_hit, (void *)b->d_start_ns, (void *)b->d_iters,
+                    (void *)b->d_err, (void *)b->d_dJ, (void *)b->d_small, (void *)b->d_sync, (void *)b->d_ctl})
+        pool_free(p, b->stream);
     step_graphs_free(b->graphs);
     if (b->ev0) cudaEventDestroy(b->ev0);
     if (b->ev1) cudaEventDestroy(b->ev1);

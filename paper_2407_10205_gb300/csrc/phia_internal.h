@@ -250,6 +250,9 @@ int batch_best(phia_batch_s *b, int inst, int64_t *energy_k, int8_t *spins);
 int batch_replica_results(phia_batch_s *b, int inst, int32_t R, int64_t *be, int64_t *bs, int64_t *hs, uint32_t *bits);
 int batch_stats(phia_batch_s *b, int inst, phia_stats *out);
 
+// Device memory from the library's pool, ordered on a stream.
+cudaError_t pool_alloc(void **ptr, size_t bytes, int device, cudaStream_t st);
+void pool_free(void *ptr, cudaStream_t st);
 // Thread-local error message of the C ABI.
 int set_last_error(int code, const char *msg);
 

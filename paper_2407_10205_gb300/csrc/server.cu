@@ -122,8 +122,10 @@ void finish(phia_server_s *S, Request &r, int code) {
         phia_destroy(r.h_dev);
         r.h_dev = nullptr;
     }
-    cudaFree(r.x);
-    cudaFree(r.v);
+    if (r.slot >= 0) {
+        pool_free(r.x, S->streams[r.slot]);
+        pool_free(r.v, S->streams[r.slot]);
+    }
     r.x = r.v = nullptr;
     if (r.ev) cudaEventDestroy(r.ev);
     r.ev = nullptr;
@@ -181,7 +183,9 @@ int admit(phia_server_s *S, Request &r, int slot) {
     }
     if (rc) return rc;
     const size_t bytes = (size_t)r.replicas * r.N * 4;
-    if (cudaMalloc(&r.x, bytes) != cudaSuccess || cudaMalloc(&r.v, bytes) != cudaSuccess) return PHIA_ENOMEM;
+    if (pool_alloc((void **)&r.x, bytes, S->opts.device, S->streams[slot]) != cudaSuccess ||
+        pool_alloc((void **)&r.v, bytes, S->opts.device, S->streams[slot]) != cudaSuccess)
+        return PHIA_ENOMEM;
     if (cudaEventCreateWithFlags(&r.ev, cudaEventDisableTiming) != cudaSuccess) return PHIA_ECUDA;
     rc = phia_init_state(r.h_dev, r.replicas, r.seed, r.x, r.v);
     if (rc) return rc;
@@ -379,8 +383,10 @@ void phia_server_destroy(phia_server_t *S) {
         Request &r = kv.second;
         if (r.ev) cudaEventSynchronize(r.ev);
         if (r.h_dev) phia_destroy(r.h_dev);
-        cudaFree(r.x);
-        cudaFree(r.v);
+        if (r.slot >= 0) {
+            pool_free(r.x, S->streams[r.slot]);
+            pool_free(r.v, S->streams[r.slot]);
+        }
         if (r.ev) cudaEventDestroy(r.ev);
     }
     for (cudaStream_t s : S->streams) cudaStreamDestroy(s);
