@@ -102,6 +102,11 @@ __device__ __forceinline__ float momentum_quad(float v, float x, float I, float 
     return __fmaf_rn(eps, __fmaf_rn(f, I, -x), v);
 }
 
+// Programmatic dependent launch: lets the next launch's blocks start once all of this one's
+// have; and the wait of such a block for the end of the launch before it.
+__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // All ones when s = sgn x is -1 (x < 0 or NaN), 0 when it is +1 (x >= 0, both zeros).
 __device__ __forceinline__ uint32_t minus_mask(float x) {
     uint32_t m;
@@ -371,11 +376,6 @@ __device__ __forceinline__ void cp_async_4(void *dst, const void *src, bool vali
 __device__ __forceinline__ uint64_t l2_evict_last_policy() {
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-__device__ __forceinline__ uint64_t l2_evict_normal_policy() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
 // 16-byte global store (16-byte aligned) under an L2 policy from createpolicy.

@@ -49,7 +49,7 @@ std::vector<uint8_t> make_key(const void *func, dim3 grid, dim3 block, size_t sm
 }
 
 cudaError_t build(const void *func, dim3 grid, dim3 block, size_t smem, void **args, int64_t len, unsigned cluster,
-                  cudaGraphExec_t *out) {
+                  bool overlap, cudaGraphExec_t *out) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaGraphCreate(&g, 0);
     if (e != cudaSuccess) return e;
@@ -63,7 +63,13 @@ cudaError_t build(const void *func, dim3 grid, dim3 block, size_t smem, void **a
     cudaGraphNode_t prev = nullptr;
     for (int64_t i = 0; i < len && e == cudaSuccess; ++i) {
         cudaGraphNode_t node;
-        e = cudaGraphAddKernelNode(&node, g, prev ? &prev : nullptr, prev ? 1 : 0, &kp);
+        e = cudaGraphAddKernelNode(&node, g, prev && !overlap ? &prev : nullptr, prev && !overlap ? 1 : 0, &kp);
+        if (e == cudaSuccess && prev && overlap) {
+            cudaGraphEdgeData edge{};
+            edge.from_port = cudaGraphKernelNodePortProgrammatic;
+            edge.type = cudaGraphDependencyTypeProgrammatic;
+            e = cudaGraphAddDependencies(g, &prev, &node, &edge, 1);
+        }
         if (e == cudaSuccess && cluster > 1) {
             cudaKernelNodeAttrValue v{};
             v.clusterDim.x = cluster;
@@ -81,25 +87,33 @@ cudaError_t build(const void *func, dim3 grid, dim3 block, size_t smem, void **a
 }  // namespace
 
 cudaError_t launch_one(const void *func, dim3 grid, dim3 block, size_t smem, void **args, unsigned cluster,
-                       cudaStream_t st) {
-    if (cluster <= 1) return cudaLaunchKernel(func, grid, block, args, smem, st);
+                       bool overlap, cudaStream_t st) {
+    if (cluster <= 1 && !overlap) return cudaLaunchKernel(func, grid, block, args, smem, st);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cluster;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    if (cluster > 1) {
+        cudaLaunchAttribute &x = at[cfg.numAttrs++];
+        x.id = cudaLaunchAttributeClusterDimension;
+        x.val.clusterDim.x = cluster;
+        x.val.clusterDim.y = 1;
+        x.val.clusterDim.z = 1;
+    }
+    if (overlap) {
+        cudaLaunchAttribute &x = at[cfg.numAttrs++];
+        x.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        x.val.programmaticStreamSerializationAllowed = 1;
+    }
     return cudaLaunchKernelExC(&cfg, func, args);
 }
 
 cudaError_t launch_steps(StepGraphCache *cache, const void *func, dim3 grid, dim3 block, size_t smem, void **args,
-                         const void *key, size_t key_bytes, int64_t steps, cudaStream_t st, unsigned cluster) {
+                         const void *key, size_t key_bytes, int64_t steps, cudaStream_t st, unsigned cluster,
+                         bool overlap) {
     int64_t done = 0;
     if (cache && steps >= 2) {
         const int64_t len = steps < kGraphLen ? steps : kGraphLen;
@@ -120,7 +134,7 @@ cudaError_t launch_steps(StepGraphCache *cache, const void *func, dim3 grid, dim
             }
         }
         if (build_now) {
-            cudaError_t e = build(func, grid, block, smem, args, len, cluster, &exec);
+            cudaError_t e = build(func, grid, block, smem, args, len, cluster, overlap, &exec);
             if (e != cudaSuccess) return e;
             if (cache->entries.size() >= kMaxGraphs) {
                 cudaGraphExecDestroy(cache->entries.front().exec);
@@ -133,8 +147,8 @@ cudaError_t launch_steps(StepGraphCache *cache, const void *func, dim3 grid, dim
             if (e != cudaSuccess) return e;
         }
     }
-    for (; done < steps; ++done) {
-        cudaError_t e = launch_one(func, grid, block, smem, args, cluster, st);
+    for (const int64_t first = done; done < steps; ++done) {
+        cudaError_t e = launch_one(func, grid, block, smem, args, cluster, overlap && done > first, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

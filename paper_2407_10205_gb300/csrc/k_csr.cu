@@ -26,7 +26,8 @@
 // replicas to a lane: every neighbour cost the warp a load of 32 bytes, its address and its
 // share of the byte permutes for 8 replicas a lane instead of 32.  Per iteration (us), that
 // form and this one: 48 Erdos-Renyi instances of 100 .. 3000 spins x 256 replicas 166 / 139, 12
-// of them x 256 44 / 26, one of 5000 spins x 256 27 / 15, where the longest slice sets the time.
+// of them x 256 44 / 26, one of 5000 spins x 256 27 / 15, where the longest slice sets the time; with the update in a
+// loop and launches that overlap (below) 12 of it, and 6.9 instead of 10 for one of 105 spins.
 //
 // The instances go through their iterations in sets whose state fits in L2 together: a set runs
 // all of its iterations before the next begins (the instances are independent), so x and v are
@@ -55,14 +56,15 @@ __device__ __forceinline__ void settle_csr(const CsrArgs &C, const CsrInst &in, 
     *slot = 0ull;
     const long long E = -twice / 2;
     int imp = 0;
-    const bool frozen = a.stop_at_target && a.hit_step[rec] >= 0;
-    if (!frozen && E < a.best_e[rec]) {
+    const long long best = (long long)__ldcg(a.best_e + rec), hit = (long long)__ldcg(a.hit_step + rec);
+    const bool frozen = a.stop_at_target && hit >= 0;
+    if (!frozen && E < best) {
         a.best_e[rec] = E;
         a.best_step[rec] = tt;
         imp = 1;
     }
     const long long target = C.targets ? C.targets[b] : a.target;
-    if (a.has_target && a.hit_step[rec] < 0 && E <= target) {
+    if (a.has_target && hit < 0 && E <= target) {
         a.hit_step[rec] = tt;
         if (a.hit_ns) a.hit_ns[rec] = globaltimer_ns();
     }
@@ -113,6 +115,18 @@ struct Entry<false> {
     __device__ __forceinline__ uint32_t at(int n) const { return n == 0 ? c.x : n == 1 ? c.y : n == 2 ? c.z : c.w; }
 };
 
+// A lane's first entries of a slice: as many as gather_row keeps in flight.
+template <bool C16>
+struct Ahead {
+    static constexpr int D = C16 ? 3 : 1;
+    Entry<C16> nx[D];
+    __device__ __forceinline__ void load(const CsrArgs &C, int e, int e_end, int lane) {
+#pragma unroll
+        for (int u = 0; u < D; ++u)
+            if (e + u < e_end) nx[u].load(C, e + u, lane);
+    }
+};
+
 // acc[r] of the lane's row over its couplings: entries [e, e_end) of the slice, 4 neighbours
 // each; the next entries load meanwhile (three ahead with 16-bit offsets, whose registers allow
 // it: an entry's L2 latency is several times its arithmetic).  SCALED: acc_r carries the factor
@@ -120,12 +134,9 @@ struct Entry<false> {
 // take the bit down to place 0 instead, as the factor could leave 32 bits.
 template <bool SMEM, bool C16, bool SCALED>
 __device__ __forceinline__ void gather_row(const CsrArgs &C, const char *spins, int e, int e_end, int lane,
-                                           int32_t (&acc)[32]) {
-    constexpr int D = C16 ? 3 : 1;
-    Entry<C16> nx[D];
-#pragma unroll
-    for (int u = 0; u < D; ++u)
-        if (e + u < e_end) nx[u].load(C, e + u, lane);
+                                           Ahead<C16> &ahead, int32_t (&acc)[32]) {
+    constexpr int D = Ahead<C16>::D;
+    Entry<C16>(&nx)[D] = ahead.nx;
 #pragma unroll 1
     for (; e < e_end; e += D) {
 #pragma unroll
@@ -150,10 +161,41 @@ __device__ __forceinline__ void gather_row(const CsrArgs &C, const char *spins, 
     }
 }
 
+// A block of a step launch with its place in the count of blocks that have read the iteration:
+// the last one, whose count says that all have, advances it for the next launch.
+__device__ __forceinline__ void step_done(IterCtl *c, unsigned ticket) {
+    if (ticket != gridDim.x * gridDim.y - 1) return;
+    c->done = 0;
+    c->t = __ldcg(&c->t) + 1;
+}
+
+// Sums over a warp's rows of 8 replicas' terms: replica lane % 8 in every lane.  Three halving
+// exchanges, then two whole ones (8 warp sums would take 8 cycles each).
+__device__ __forceinline__ int32_t sum_rows8(const int32_t (&e)[8], int lane) {
+    const bool h4 = lane & 4, h2 = lane & 2, h1 = lane & 1;
+    int32_t a[4], b[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = (h4 ? e[4 + k] : e[k]) + __shfl_xor_sync(0xffffffffu, h4 ? e[k] : e[4 + k], 4);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) b[k] = (h2 ? a[2 + k] : a[k]) + __shfl_xor_sync(0xffffffffu, h2 ? a[k] : a[2 + k], 2);
+    int32_t s = (h1 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h1 ? b[0] : b[1], 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 8);
+    s += __shfl_xor_sync(0xffffffffu, s, 16);
+    return s;
+}
+
+// Momentum draws d = t1 of replicas r0 .. r0 + 7 of a spin (out of line: once per trajectory).
+__device__ __noinline__ void refresh8(float *v, uint64_t seed, uint32_t inst, uint32_t r0, uint32_t i, uint32_t t1) {
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) v[k] = draw_v(seed, inst, r0 + k, i, t1);
+}
+
 // One work unit of iteration t: C.slices slices of an instance (block `bi` of the list) x
 // C.gblock groups of 32 replicas (the y-th such set).  Uses the block's shared memory; every
-// thread of the block calls it.
-template <bool SMEM, bool C16>
+// thread of the block calls it.  STEP: the unit of a step launch, which may start before the
+// launch for t - 1 has ended: what no iteration changes (the block, its instance, the first
+// entries) loads first, then it waits for that launch and reads its iteration.
+template <bool SMEM, bool C16, bool STEP>
 __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_t t, int64_t t_first, int64_t t_end,
                                          char *smem) {
     const RunArgs &a = C.a;
@@ -167,6 +209,34 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
     const bool active = g < groups;
     const int nsl = in.Np / 32;
     const int s_end = min(nsl, blk.s0 + C.slices);
+    const int s_first = active ? blk.s0 + sp : s_end;              // this warp's first slice
+    int e0 = 0, e1 = 0;
+    Ahead<C16> ahead;
+    if (s_first < s_end) {
+        e0 = C.slice[in.slice_off + s_first];
+        e1 = C.slice[in.slice_off + s_first + 1];
+        ahead.load(C, e0, e1, lane);
+    }
+    if constexpr (STEP) {
+        t_first = __ldcg(&C.ctl->t_first);
+        t_end = __ldcg(&C.ctl->t_end);
+        grid_dependency_wait();
+        t = __ldcg(&C.ctl->t);
+    }
+
+    // x and v of a slice's first 8 replicas load while the rest goes on, the others 8 replicas ahead
+    // of their use.
+    const size_t qs = (size_t)in.Np * 4;               // floats between quads of replicas
+    float4 xq[2], vq[2];
+    auto load_quads = [&](int s) {
+        const size_t o = in.x_off + ((size_t)g * 8 * in.Np + s * 32 + lane) * 4;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            xq[k] = __ldcg(reinterpret_cast<const float4 *>(C.X + o + k * qs));
+            vq[k] = __ldcg(reinterpret_cast<const float4 *>(C.V + o + k * qs));
+        }
+    };
+    if (s_first < s_end) load_quads(s_first);
 
     // The spins of this iteration of the block's groups into shared memory.
     const uint32_t *Sg = spin_buf(C, in, t);
@@ -176,8 +246,8 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
         for (int e = tid * 4; e < words; e += kBlk * 4) cp_async_16(smem + (size_t)e * 4, src + e);
         cp_async_commit();
     }
-    // (a) records of iteration t-1 (the first block of each instance).
-    if (blk.s0 == 0 && t - 1 >= t_first) {
+    // (a) records of iteration t-1 (the last block of each instance, whose rows are the shortest).
+    if (blk.s0 + C.slices >= nsl && t - 1 >= t_first) {
         for (int e = tid; e < G * 32; e += kBlk)
             if (y * G * 32 + e < C.R) settle_csr(C, in, b, y * G * 32 + e, t - 1);
     }
@@ -200,10 +270,11 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
             }
         }
     }
-    if constexpr (SMEM) {
-        cp_async_wait<0>();
-        __syncthreads();
-    }
+    if constexpr (SMEM) cp_async_wait<0>();
+    if constexpr (SMEM || STEP) __syncthreads();
+    unsigned ticket = 0;          // every thread of the block has read the iteration
+    if constexpr (STEP)
+        if (tid == 0) ticket = atomicAdd(&C.ctl->done, 1u);
     // (c) field and update.
     if (active) {
         const char *spins = SMEM ? smem + (size_t)gi * in.Np * 4 : reinterpret_cast<const char *>(Sg + (size_t)g * in.Np);
@@ -213,103 +284,115 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
         const bool more = t + 1 < t_end;
         const bool refresh_next = more && refresh_at(t + 1, a.refresh);
         long long esum = 0;                            // replica `lane` of the group
-        for (int s = blk.s0 + sp; s < s_end; s += spar) {
+        for (int s = s_first; s < s_end; s += spar) {
             const int p = s * 32 + lane;
             float *X = C.X + in.x_off + ((size_t)g * 8 * in.Np + p) * 4;
             float *V = C.V + in.x_off + ((size_t)g * 8 * in.Np + p) * 4;
-            const size_t qs = (size_t)in.Np * 4;       // floats between quads of replicas
-            // x and v of the group's first 8 replicas load while the gather runs, the others two quads
-            // ahead of their use.
-            float4 xq[2], vq[2];
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                xq[k] = *reinterpret_cast<const float4 *>(X + k * qs);
-                vq[k] = *reinterpret_cast<const float4 *>(V + k * qs);
+            if (s != s_first) {
+                load_quads(s);
+                e0 = C.slice[in.slice_off + s];
+                e1 = C.slice[in.slice_off + s + 1];
+                ahead.load(C, e0, e1, lane);
             }
             int32_t acc[32];
 #pragma unroll
             for (int r = 0; r < 32; ++r) acc[r] = 0;
-            const int e0 = C.slice[in.slice_off + s], e1 = C.slice[in.slice_off + s + 1];
-            if (in.wide) gather_row<SMEM, C16, false>(C, spins, e0, e1, lane, acc);
-            else gather_row<SMEM, C16, true>(C, spins, e0, e1, lane, acc);
+            if (in.wide) gather_row<SMEM, C16, false>(C, spins, e0, e1, lane, ahead, acc);
+            else gather_row<SMEM, C16, true>(C, spins, e0, e1, lane, ahead, acc);
             const int2 hh = __ldg(reinterpret_cast<const int2 *>(C.hk) + in.pos_off + p);    // h, h - ksum
             const int row = refresh_next ? C.row_of[in.pos_off + p] : 0;
             uint32_t bits = 0;
+            // 8 replicas at a time, their accumulators moved down to the front: one copy of the code
+            // instead of four, as a straight line over all 32 replicas (with the draws of a refresh in it)
+            // is fetched anew for every slice: its update took 8000 to 10000 cycles, most of them
+            // waiting for instructions.
+#pragma unroll 1
+            for (int o = 0; o < 4; ++o) {
+                float xs[8] = {xq[0].x, xq[0].y, xq[0].z, xq[0].w, xq[1].x, xq[1].y, xq[1].z, xq[1].w}, If[8];
+                float vn[8] = {vq[0].x, vq[0].y, vq[0].z, vq[0].w, vq[1].x, vq[1].y, vq[1].z, vq[1].w};
+                float *Xo = X + 2 * o * qs, *Vo = V + 2 * o * qs;
+                if (o < 3) {
 #pragma unroll
-            for (int qd = 0; qd < 8; ++qd) {
-                const float4 x4 = xq[qd & 1], v4 = vq[qd & 1];
-                if (qd < 6) {
-                    xq[qd & 1] = *reinterpret_cast<const float4 *>(X + (qd + 2) * qs);
-                    vq[qd & 1] = *reinterpret_cast<const float4 *>(V + (qd + 2) * qs);
+                    for (int k = 0; k < 2; ++k) {
+                        xq[k] = __ldcg(reinterpret_cast<const float4 *>(Xo + (2 + k) * qs));
+                        vq[k] = __ldcg(reinterpret_cast<const float4 *>(Vo + (2 + k) * qs));
+                    }
                 }
-                int32_t e4[4];
-                float xs[4] = {x4.x, x4.y, x4.z, x4.w}, If[4];
-                float vn[4] = {v4.x, v4.y, v4.z, v4.w};
+                int32_t e8[8];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int r = qd * 4 + k, bit = r & 7;
-                    const int32_t twice = (in.wide || bit == 0) ? acc[r] << 1 : acc[r] >> (bit - 1);
+                for (int k = 0; k < 8; ++k) {
+                    const int32_t twice = (in.wide || k == 0) ? acc[k] << 1 : acc[k] >> (k - 1);
                     const int32_t I = twice + hh.y;                                   // Eq. 6, exact
                     const int32_t m = (int32_t)minus_mask(xs[k]);
-                    const int32_t e = ((I + hh.x) ^ m) - m;                           // s (I + h)
-                    if (in.wide) {      // sums of such terms may leave 32 bits: halves apart, at once
-                        const long long es = (long long)__reduce_add_sync(0xffffffffu, e & 0xffff) +
-                                             ((long long)__reduce_add_sync(0xffffffffu, e >> 16) << 16);
-                        if (lane == r) esum += es;
-                    } else {
-                        e4[k] = e;
-                    }
+                    e8[k] = ((I + hh.x) ^ m) - m;                                     // s (I + h)
                     If[k] = (float)I;
                 }
-                if (!in.wide) {
-                    // Sums over the rows of 4 replicas: two halving exchanges leave replica lane % 4 in
-                    // a lane, three more sum it over the warp (32 warp sums would take 8 cycles each).
-                    const bool h2 = lane & 2, h1 = lane & 1;
-                    const int32_t a0 = (h2 ? e4[2] : e4[0]) + __shfl_xor_sync(0xffffffffu, h2 ? e4[0] : e4[2], 2);
-                    const int32_t a1 = (h2 ? e4[3] : e4[1]) + __shfl_xor_sync(0xffffffffu, h2 ? e4[1] : e4[3], 2);
-                    int32_t es = (h1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, h1 ? a0 : a1, 1);
+                long long es;
+                if (in.wide) {          // sums of such terms may leave 32 bits: halves apart
+                    int32_t lo[8], hi[8];
 #pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) es += __shfl_xor_sync(0xffffffffu, es, o);
-                    if ((lane >> 2) == qd) esum += es;
+                    for (int k = 0; k < 8; ++k) {
+                        lo[k] = e8[k] & 0xffff;
+                        hi[k] = e8[k] >> 16;
+                    }
+                    es = (long long)sum_rows8(lo, lane) + ((long long)sum_rows8(hi, lane) << 16);
+                } else {
+                    es = sum_rows8(e8, lane);
                 }
+                if ((lane >> 3) == o) esum += es;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
+                for (int k = 0; k < 8; ++k) {
                     const float f = a.deriv == 1 ? factor_quad(xs[k], bgq, gamma) : factor_exact(xs[k], bgq4, gamma);
                     vn[k] = momentum_of(vn[k], xs[k], If[k], f, eps);
                 }
                 if (refresh_next && row >= 0) {
+                    float w[8];
+                    refresh8(w, a.seed, in.inst_id, (uint32_t)(g * 32 + 8 * o), (uint32_t)row, (uint32_t)(t + 1));
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        vn[k] = draw_v(a.seed, in.inst_id, (uint32_t)(g * 32 + qd * 4 + k), (uint32_t)row, (uint32_t)(t + 1));
+                    for (int k = 0; k < 8; ++k) vn[k] = w[k];
                 }
                 if (more) {
+                    uint32_t plus = 0;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
+                    for (int k = 0; k < 8; ++k) {
                         xs[k] = __fmaf_rn(eps, vn[k], xs[k]);
-                        bits |= ~minus_mask(xs[k]) & (1u << (qd * 4 + k));
+                        plus |= ~minus_mask(xs[k]) & (1u << k);
                     }
-                    *reinterpret_cast<float4 *>(X + qd * qs) = make_float4(xs[0], xs[1], xs[2], xs[3]);
+                    bits |= plus << (8 * o);
+                    *reinterpret_cast<float4 *>(Xo) = make_float4(xs[0], xs[1], xs[2], xs[3]);
+                    *reinterpret_cast<float4 *>(Xo + qs) = make_float4(xs[4], xs[5], xs[6], xs[7]);
                 }
-                *reinterpret_cast<float4 *>(V + qd * qs) = make_float4(vn[0], vn[1], vn[2], vn[3]);
+                *reinterpret_cast<float4 *>(Vo) = make_float4(vn[0], vn[1], vn[2], vn[3]);
+                *reinterpret_cast<float4 *>(Vo + qs) = make_float4(vn[4], vn[5], vn[6], vn[7]);
+#pragma unroll
+                for (int r = 0; r < 24; ++r) acc[r] = acc[r + 8];
             }
             if (more) Snext[p] = bits;
         }
         atomicAdd(reinterpret_cast<unsigned long long *>(C.Esum) + (size_t)(t & 1) * C.total_reps + in.rec_off + g * 32 + lane,
                   (unsigned long long)esum);
     }
-    if constexpr (SMEM) __syncthreads();   // the shared spins are free for the next unit
+    if constexpr (SMEM && !STEP) __syncthreads();   // the shared spins are free for the next unit
+    if constexpr (STEP)
+        if (tid == 0) step_done(C.ctl, ticket);
 }
 
 // One launch per iteration of a set of instances: a block per work unit (the grid is that of
-// the largest set); the iteration and the set come from C.ctl.
+// the largest set); the iteration and the set come from C.ctl.  A launch lets the next one's
+// blocks start as soon as its own have all started (they wait for its end before they read what
+// it writes), so the boundary costs neither a launch nor the loads of what is the same in every
+// iteration.
 template <bool SMEM, bool C16>
 __global__ void __launch_bounds__(kBlk, 2) csr_step(const CsrArgs C) {
     extern __shared__ __align__(16) char smem[];
-    const int64_t t = C.ctl->t, t_first = C.ctl->t_first, t_end = C.ctl->t_end;
-    const CsrSet set = C.sets[C.ctl->set];
-    if ((int)blockIdx.x < set.len[C.list]) csr_unit<SMEM, C16>(C, set.off[C.list] + blockIdx.x, blockIdx.y, t, t_first, t_end, smem);
-    __syncthreads();
-    if (threadIdx.x == 0) iter_ctl_finish(C.ctl);
+    grid_dependents_launch();
+    const CsrSet set = C.sets[__ldcg(&C.ctl->set)];
+    if ((int)blockIdx.x < set.len[C.list]) {
+        csr_unit<SMEM, C16, true>(C, set.off[C.list] + blockIdx.x, blockIdx.y, 0, 0, 0, smem);
+    } else {
+        grid_dependency_wait();
+        if (threadIdx.x == 0) step_done(C.ctl, atomicAdd(&C.ctl->done, 1u));
+    }
 }
 
 // Grid-wide barrier of a cooperative launch (every block resident): bar[0] counts the
@@ -358,7 +441,7 @@ __global__ void __launch_bounds__(kBlk, 2) csr_persistent(const CsrArgs C, unsig
                 const int u = unit;
                 __syncthreads();
                 if (u >= units) break;
-                csr_unit<SMEM, C16>(C, set.off[C.list] + u % nb, u / nb, t, t_first, t_end, smem);
+                csr_unit<SMEM, C16, false>(C, set.off[C.list] + u % nb, u / nb, t, t_first, t_end, smem);
             }
             if (!grid_barrier(bar, kWaitTimeoutNs)) {
                 if (threadIdx.x == 0) atomicExch(C.a.err, 1);
@@ -564,7 +647,7 @@ cudaError_t launch_iterations(const CsrArgs &C, size_t smem, StepGraphCache *gra
             ++*launches;
         }
         e = launch_steps(graphs, reinterpret_cast<const void *>(k), dim3(max_blocks, ny), dim3(kBlk), smem, args, &Cs,
-                         sizeof Cs, C.a.nsteps, st);
+                         sizeof Cs, C.a.nsteps, st, 1, true);
         if (e != cudaSuccess) return e;
         *launches += (int)C.a.nsteps;
     }

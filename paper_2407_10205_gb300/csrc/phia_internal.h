@@ -115,9 +115,12 @@ void step_graphs_free(StepGraphCache *c);
 // chunks replay one cached graph of up to 100 launches, the rest launch directly.  With
 // no cache every launch is direct.  The cache key is the kernel, its launch shape and
 // the argument bytes `key` (`key_bytes` of them).  cluster > 1: thread-block clusters of
-// that many CTAs along x.
+// that many CTAs along x.  overlap: the kernel waits by itself (griddepcontrol) for the launch
+// before it, so that a launch may start while the one before it runs; the first launch of a graph
+// or of a row of direct launches starts after all work before it.
 cudaError_t launch_steps(StepGraphCache *cache, const void *func, dim3 grid, dim3 block, size_t smem, void **args,
-                         const void *key, size_t key_bytes, int64_t steps, cudaStream_t st, unsigned cluster = 1);
+                         const void *key, size_t key_bytes, int64_t steps, cudaStream_t st, unsigned cluster = 1,
+                         bool overlap = false);
 constexpr int kOpE4M3 = 1;
 constexpr int kOpBF16 = 2;
 
