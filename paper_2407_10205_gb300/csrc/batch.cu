@@ -34,6 +34,9 @@ struct phia_batch_s {
     // small dense members: a resident kernel over a table of CTAs
     std::vector<int> dense_pub;         // public indices
     std::vector<int64_t> dense_joff;    // offset of each member's J in d_dJ
+    // sparse members that are small enough for a resident kernel as well (all of the batch's, else
+    // none): offset of each one's dense J in d_dJ
+    std::vector<int64_t> cand_joff;
     int8_t *d_dJ = nullptr;
     SmallCta *d_small = nullptr;
     size_t small_cap = 0;
@@ -225,6 +228,7 @@ struct PackedInst {
     std::vector<uint32_t> val;
     int wide = 0;
     int small_op = 0;       // small dense member: its tensor-core operand (no slices built)
+    std::vector<int8_t> dense;   // J of a member with slices that a resident kernel could run too
 };
 
 void pack_error(PackedInst &out, int code, const char *fmt, ...) {
@@ -277,6 +281,18 @@ void pack_slices(int n, const int32_t *rp, const int32_t *col, const int8_t *val
     }
     // |I + h| <= bound: 128 rows' terms and a sum scaled by 2^7 stay in 32 bits up to 2^23.
     out.wide = bound > ((int64_t)1 << 23);
+    if (n > cluster_batch_max_n()) return;
+    out.dense.assign((size_t)n * n, 0);
+    for (int i = 0; i < n; ++i)
+        for (int32_t c = rp[i]; c < rp[i + 1]; ++c) {
+            int8_t &k = out.dense[(size_t)i * n + col[c]];
+            const int sum = (int)k + val[c];                // entries of one coupling add up
+            if (std::abs(sum) > 127) {
+                out.dense.clear();
+                return;
+            }
+            k = (int8_t)sum;
+        }
 }
 
 void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
@@ -373,6 +389,7 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         for (std::thread &t : workers) t.join();
     }
     size_t tot_sl = 0, tot_ent = 0, tot_pos = 0, tot_inv = 0, tot_h = 0, tot_dj = 0;
+    bool all_cand = true;
     for (int k = 0; k < count; ++k) {
         if (packed[(size_t)k].code != PHIA_OK)
             return cleanup(bfail(packed[(size_t)k].code, "%s", packed[(size_t)k].msg.c_str()));
@@ -380,7 +397,8 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         tot_ent += packed[(size_t)k].val.size();
         tot_pos += packed[(size_t)k].row_of.size();
         tot_inv += packed[(size_t)k].pos_of.size();
-        if (packed[(size_t)k].small_op) {
+        all_cand &= packed[(size_t)k].small_op || !packed[(size_t)k].dense.empty();
+        if (packed[(size_t)k].small_op || !packed[(size_t)k].dense.empty()) {
             tot_h += (size_t)d[k].N;
             tot_dj += (size_t)d[k].N * d[k].N;
         }
@@ -410,6 +428,11 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
             continue;
         }
         b->csr_pub.push_back(k);
+        if (all_cand) {
+            b->cand_joff.push_back((int64_t)dj.size());
+            dj.insert(dj.end(), pk.dense.begin(), pk.dense.end());
+            hk.insert(hk.end(), x.h_k, x.h_k + n);
+        }
         CsrInst in{};
         in.N = n;
         in.Np = round_up(n, 32);
@@ -556,12 +579,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     a.min_hit = b->d_min_hit; a.replica_iters = b->d_iters; a.err = b->d_err;
     C.inst = b->d_inst; C.count = ncsr;
     C.blocks = b->d_blocks;
-    if (ncsr > 0 && b->sets_R != R) {
-        rc = make_sets(b, R);
-        if (rc) return rc;
-    }
     C.sets = b->d_sets;
-    C.nsets = (int32_t)b->sets.size();
     C.max_np = b->max_np;
     C.slice = b->d_slice; C.col = b->d_col; C.col16 = b->col16 ? 1 : 0; C.val = b->d_val; C.hk = b->d_hk2;
     C.row_of = b->d_rowof; C.pos_of = b->d_posof;
@@ -586,28 +604,46 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     C.R = R; C.R_real = R_real;
     C.max_words = b->max_words;
     C.total_slices = b->total_slices;
-    // Small dense members: a table of CTAs (8 replicas each) per size class, every instance's
-    // own couplings, field, scale, Philox id, target and records.  Up to 256 spins they run on
-    // the warp-level kernel (classes of at most 64, 128 and 256 spins, as its register use
-    // grows with the size it is built for), above on the resident tcgen05 kernel.
+    // Members on the resident kernels: a table of CTAs or clusters (8 replicas each) per size
+    // class, every instance's own couplings, field, scale, Philox id, target and records.  Dense
+    // members: up to 256 spins on the warp-level kernel (classes of at most 64, 128 and 256 spins,
+    // as its register use grows with the size it is built for), above on the resident tcgen05
+    // kernel.  Sparse members go to the warp-level kernel or, above 256 spins, to the cluster kernel
+    // where their estimated iterations take less together than the gather's, which no instance takes
+    // below 7 us (launch, records, the copy of the spins and a slice come one after the other).
+    enum { kWarp, kTcgen05, kCluster };
     struct SmallGroup {
         size_t begin, end;       // in small_host
-        int nmax;
+        int nmax, kernel;
     };
     std::vector<SmallGroup> groups;
-    if (!b->dense_pub.empty()) {
+    bool gathers = ncsr > 0;
+    if (ncsr > 0 && !b->cand_joff.empty() && !field_mode && (b->count == 1 || (!x_in && !x_out))) {
+        int sms = 0;
+        BCU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
+        double us = 0.0;
+        for (const CsrInst &in : b->inst)
+            us += in.N <= warp_small_max_n() ? warp_small_estimate(in.N, R_real, sms) : cluster_small_estimate(in.N, R_real, kOpBF16);
+        gathers = us > 5.0;
+    }
+    const bool resident = ncsr > 0 && !gathers;
+    if (!b->dense_pub.empty() || resident) {
         b->small_host.clear();
-        const int bounds[5] = {0, 64, 128, warp_small_max_n(), INT_MAX};
-        for (int cls = 0; cls < 4; ++cls) {
+        struct Class {
+            int above, nmax, kernel;
+        };
+        const Class classes[] = {{0, 64, kWarp},       {64, 128, kWarp},     {128, 256, kWarp},
+                                 {256, 384, kTcgen05}, {256, 384, kCluster}, {384, 512, kCluster}};
+        for (const Class &cls : classes) {
             const size_t beg = b->small_host.size();
             int nmax = 0;
-            for (size_t m = 0; m < b->dense_pub.size(); ++m) {
-                const int k = b->dense_pub[m], n = b->N[(size_t)k];
-                if (n <= bounds[cls] || n > bounds[cls + 1]) continue;
+            auto add = [&](int k, int64_t joff) {
+                const int n = b->N[(size_t)k];
+                if (n <= cls.above || n > cls.nmax) return;
                 nmax = std::max(nmax, n);
                 for (int r0 = 0; r0 < R_real; r0 += 8) {
                     SmallCta c{};
-                    c.Jk = b->d_dJ + b->dense_joff[m];
+                    c.Jk = b->d_dJ + joff;
                     c.hk = b->d_hk + b->h_off[(size_t)k];
                     c.N = n;
                     c.W = (int32_t)words_of(n);
@@ -619,8 +655,12 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
                     c.target = target_of(k);
                     b->small_host.push_back(c);
                 }
-            }
-            if (b->small_host.size() > beg) groups.push_back(SmallGroup{beg, b->small_host.size(), nmax});
+            };
+            if (cls.kernel != kCluster)
+                for (size_t m = 0; m < b->dense_pub.size(); ++m) add(b->dense_pub[m], b->dense_joff[m]);
+            if (cls.kernel != kTcgen05 && resident)
+                for (size_t m = 0; m < b->csr_pub.size(); ++m) add(b->csr_pub[m], b->cand_joff[m]);
+            if (b->small_host.size() > beg) groups.push_back(SmallGroup{beg, b->small_host.size(), nmax, cls.kernel});
         }
         if (b->small_host.size() > b->small_cap) {
             pool_free(b->d_small, b->stream);
@@ -636,7 +676,12 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     C.ctl = b->d_ctl;
     C.sync = b->d_sync;
     C.persistent = (b->csr_mode == 1 && !field_mode) ? 1 : 0;
-    if (ncsr > 0) {
+    if (gathers) {
+        if (b->sets_R != R) {
+            rc = make_sets(b, R);
+            if (rc) return rc;
+        }
+        C.nsets = (int32_t)b->sets.size();
         cudaError_t e = launch_csr(C, b->set_max, b->graphs, b->stream, &launches);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
     }
@@ -649,8 +694,10 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         ad.small_cta = b->d_small + grp.begin;
         ad.small_ctas = (int32_t)(grp.end - grp.begin);
         ad.has_target = b->any_target || sched->has_target;
-        cudaError_t e = grp.nmax <= warp_small_max_n() ? launch_warp_small_batch(ad, grp.nmax, b->stream)
-                                                       : launch_tc_small_batch(ad, grp.nmax, b->stream);
+        ad.x_in = x_in; ad.v_in = v_in; ad.x_out = x_out; ad.v_out = v_out;
+        cudaError_t e = grp.kernel == kWarp      ? launch_warp_small_batch(ad, grp.nmax, b->stream)
+                        : grp.kernel == kTcgen05 ? launch_tc_small_batch(ad, grp.nmax, b->stream)
+                                                 : launch_cluster_batch(ad, grp.nmax, b->stream);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
         ++launches;
     }

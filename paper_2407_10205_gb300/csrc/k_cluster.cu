@@ -68,8 +68,9 @@ __device__ __forceinline__ void st_async_u64(uint32_t addr, uint2 v, uint32_t mb
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr), "l"(w), "r"(mbar)
                  : "memory");
 }
-// KS: MMA K-steps of 32 bytes (every spin of the instance); CW: warps per CTA.
-template <int KS, int OP, int CW>
+// KS: MMA K-steps of 32 bytes (every spin of the instance); CW: warps per CTA; BATCHED: the cluster's
+// instance is its entry of a batch's table (a.small_cta).
+template <int KS, int OP, int CW, bool BATCHED>
 __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs a, int cl) {
     using Sh = ClusterShared<KS>;
     extern __shared__ __align__(16) uint8_t smem[];
@@ -77,9 +78,12 @@ __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs
     volatile int32_t *tout = &sm->timed_out;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, q = lane & 3;
-    const int N = a.N, nit = (int)a.nsteps;
+    SmallCta ic;
+    if constexpr (BATCHED) ic = a.small_cta[blockIdx.x / cl];
+    else ic = SmallCta{a.Jk, a.hk, a.N, a.W, a.inst, a.q, (int32_t)(blockIdx.x / cl) * 8, 0, 0, a.target};
+    const int N = ic.N, nit = (int)a.nsteps;
     const int rank = (int)cluster_ctarank();
-    const int rbase = (int)(blockIdx.x / cl) * 8;
+    const int rbase = ic.rbase;
     const int nwarps = (N + 15) / 16;                 // warps of the cluster that own spins
     const uint64_t kWaitNs = a.wait_ns > 0 ? (uint64_t)a.wait_ns : kWaitTimeoutNs;
     const uint32_t bytes = (uint32_t)(nwarps * 32) * (OP == kOpE4M3 ? 4u : 8u);   // an iteration's spins
@@ -107,13 +111,13 @@ __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs
     if (gw < nwarps) {
         const int i[2] = {16 * gw + g, 16 * gw + g + 8};
         uint32_t af[KS][4];
-        load_fragments<OP, KS>(af, a.Jk, N, i, q);
+        load_fragments<OP, KS>(af, ic.Jk, N, i, q);
         Elems s;
         float hf[2];
         int32_t h2c[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int32_t h = i[u] < N ? a.hk[i[u]] : 0;
+            const int32_t h = i[u] < N ? ic.hk[i[u]] : 0;
             hf[u] = (float)h;
             h2c[u] = 2 * h - (int32_t)kMagicBits;
         }
@@ -131,10 +135,9 @@ __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs
             }
         };
         const int r0 = rbase + 2 * q;
-        const SmallCta ic{a.Jk, a.hk, a.N, a.W, a.inst, a.q, rbase, 0, 0, a.target};
         initial_state(s, a, ic, r0, i);
         send_spins(0);
-        const float inv_tm1 = inv_tm1_of(a.T_total), gq = a.gamma * a.q, eps = a.eps, gamma = a.gamma;
+        const float inv_tm1 = inv_tm1_of(a.T_total), gq = a.gamma * ic.q, eps = a.eps, gamma = a.gamma;
         const int refresh = a.refresh, deriv = a.deriv, t0 = (int)a.t0;
         int rc = refresh > 0 ? (t0 + 1) % refresh : 1;
         // Energy terms of iteration it (d: its field, m: its spins) to rank 0.
@@ -150,7 +153,7 @@ __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs
         Record rec;
         rec.live = false;
         const bool records = rank == 0 && warp < 8;
-        if (records) rec.load(a, 0, rbase + warp);
+        if (records) rec.load(a, ic.rec_off, rbase + warp);
         const uint32_t imp0 = smem_u32(&sm->improved[0][0]), ibar0 = smem_u32(&sm->ibar[0]);
         // Rank 0: record of iteration it, replica `warp`, and word of it to every CTA.
         auto settle = [&](int it) -> bool {
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs
             const long long twice = (long long)__reduce_add_sync(0xffffffffu, (e0 & 0xffff) + (e1 & 0xffff)) +
                                     ((long long)__reduce_add_sync(0xffffffffu, (e0 >> 16) + (e1 >> 16)) << 16);
             bool first_hit;
-            const bool imp = rec.settle(a, a.target, t0 + it, twice, first_hit);
+            const bool imp = rec.settle(a, ic.target, t0 + it, twice, first_hit);
             if (lane < cl)
                 st_async_u32(map_rank(imp0 + (uint32_t)((it & 3) * 8 + warp) * 4, (uint32_t)lane), imp,
                              map_rank(ibar0 + 8 * (it & 3), (uint32_t)lane));
@@ -202,7 +205,7 @@ __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs
                 }
                 momentum_step(s, d, f, hf, eps);
                 if (it + 1 < nit) {
-                    if (refresh > 0 && rc == 0) refresh_step(s, a.seed, a.inst, (uint32_t)r0, i, (uint32_t)(t0 + it + 1));
+                    if (refresh > 0 && rc == 0) refresh_step(s, a.seed, ic.inst, (uint32_t)r0, i, (uint32_t)(t0 + it + 1));
                     position_step(s, eps);
                     send_spins((it + 1) & 1);
                 }
@@ -220,12 +223,12 @@ __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs
             hist[0] = now;
         }
         if (ok) {
-            best.store(a.best_bits, rbase, a.R, a.W, gw, N, lane);
+            best.store(a.best_bits + ic.bits_off, rbase, a.R, ic.W, gw, N, lane);
             if (a.x_out) export_state(s, a, N, r0, i);
         } else {
             *tout = 1;
         }
-        if (records && lane == 0) rec.store(a, 0, rbase + warp);
+        if (records && lane == 0) rec.store(a, ic.rec_off, rbase + warp);
         if (gw == 0 && lane == 0)
             atomicAdd(a.replica_iters, (unsigned long long)((long long)min(8, a.R - rbase) * nit));
     }
@@ -234,45 +237,46 @@ __global__ void __launch_bounds__(32 * CW, 1) cluster_small_kernel(const RunArgs
     cluster_sync_all();          // no CTA leaves while another may still write into it
 }
 
-template <int KS, int OP, int CW>
-cudaError_t config(int N, int R, cudaStream_t st, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at) {
+// Launch of a run (a) on `clusters` clusters, or with a null the number of clusters that the GPU
+// holds at once.
+template <int KS, int OP, int CW, bool BATCHED>
+cudaError_t launch_cfg(const RunArgs *a, int N, int clusters, cudaStream_t st, int *resident) {
     constexpr size_t smem = sizeof(ClusterShared<KS>);
     const int cl = (N + 16 * CW - 1) / (16 * CW);
-    cudaError_t e = cudaFuncSetAttribute(cluster_small_kernel<KS, OP, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cfg.gridDim = dim3((unsigned)cl * (unsigned)((R + 7) / 8));
+    auto k = cluster_small_kernel<KS, OP, CW, BATCHED>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    cfg.gridDim = dim3((unsigned)cl * (unsigned)clusters);
     cfg.blockDim = dim3(32 * CW);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)cl;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
     cfg.numAttrs = 1;
-    return e;
-}
-
-// Launch of a run (a), or with a null the number of clusters that the GPU holds at once.
-template <int KS, int OP, int CW>
-cudaError_t launch_cfg(const RunArgs *a, int N, int R, cudaStream_t st, int *resident) {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
-    cudaError_t e = config<KS, OP, CW>(N, R, st, cfg, at[0]);
-    if (e != cudaSuccess) return e;
-    if (!a) return cudaOccupancyMaxActiveClusters(resident, reinterpret_cast<const void *>(cluster_small_kernel<KS, OP, CW>), &cfg);
-    e = cudaLaunchKernelEx(&cfg, cluster_small_kernel<KS, OP, CW>, *a, (int)at[0].val.clusterDim.x);
+    if (!a) return cudaOccupancyMaxActiveClusters(resident, reinterpret_cast<const void *>(k), &cfg);
+    e = cudaLaunchKernelEx(&cfg, k, *a, cl);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // bf16 fragments up to 512 spins (the warp-level e4m3 MMA runs as conversions and two FP16 MMAs),
 // e4m3 ones above, where bf16 would not fit the registers.  8 warps per CTA, 12 between 257 and
 // 384 spins (two CTAs instead of three).
-cudaError_t dispatch(const RunArgs *a, int N, int R, cudaStream_t st, int *resident) {
-    if (N <= 256) return launch_cfg<16, kOpBF16, 8>(a, N, R, st, resident);
-    if (N <= 384) return launch_cfg<24, kOpBF16, 12>(a, N, R, st, resident);
-    if (N <= 512) return launch_cfg<32, kOpBF16, 8>(a, N, R, st, resident);
-    if (N <= 768) return launch_cfg<24, kOpE4M3, 8>(a, N, R, st, resident);
-    return launch_cfg<32, kOpE4M3, 8>(a, N, R, st, resident);
+template <bool BATCHED>
+cudaError_t dispatch(const RunArgs *a, int N, int clusters, cudaStream_t st, int *resident) {
+    if constexpr (!BATCHED)
+        if (N <= 256) return launch_cfg<16, kOpBF16, 8, false>(a, N, clusters, st, resident);
+    if (N <= 384) return launch_cfg<24, kOpBF16, 12, BATCHED>(a, N, clusters, st, resident);
+    if (N <= 512) return launch_cfg<32, kOpBF16, 8, BATCHED>(a, N, clusters, st, resident);
+    if constexpr (!BATCHED) {
+        if (N <= 768) return launch_cfg<24, kOpE4M3, 8, false>(a, N, clusters, st, resident);
+        return launch_cfg<32, kOpE4M3, 8, false>(a, N, clusters, st, resident);
+    }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -283,7 +287,7 @@ int cluster_small_max_n(int op) { return op == kOpE4M3 ? 1024 : 512; }
 double cluster_small_estimate(int N, int R, int op) {
     if (N < cluster_small_min_n() || N > cluster_small_max_n(op)) return 1e30;
     int resident = 0;
-    if (dispatch(nullptr, N, R, nullptr, &resident) != cudaSuccess || resident < 1) {
+    if (dispatch<false>(nullptr, N, 1, nullptr, &resident) != cudaSuccess || resident < 1) {
         cudaGetLastError();
         return 1e30;
     }
@@ -294,7 +298,15 @@ double cluster_small_estimate(int N, int R, int op) {
 cudaError_t launch_cluster_small(const RunArgs &a, int op, cudaStream_t st, int *launches) {
     if (a.N < cluster_small_min_n() || a.N > cluster_small_max_n(op)) return cudaErrorInvalidValue;
     if (launches) *launches += 1;
-    return dispatch(&a, a.N, a.R, st, nullptr);
+    return dispatch<false>(&a, a.N, (a.R + 7) / 8, st, nullptr);
+}
+
+int cluster_batch_max_n() { return 512; }
+
+cudaError_t launch_cluster_batch(const RunArgs &a, int nmax, cudaStream_t st) {
+    if (a.small_ctas < 1) return cudaSuccess;
+    if (nmax > cluster_batch_max_n()) return cudaErrorInvalidValue;
+    return dispatch<true>(&a, nmax, a.small_ctas, st, nullptr);
 }
 
 }  // namespace phia

@@ -278,6 +278,10 @@ int cluster_small_max_n(int op);
 cudaError_t launch_cluster_small(const RunArgs &a, int op, cudaStream_t st, int *launches);
 // Its estimated time per iteration (us; 1e30 where it does not apply).
 double cluster_small_estimate(int N, int R, int op);
+// And over a table of clusters (a.small_cta) of instances of 257 .. nmax spins, or of 385 .. nmax
+// where nmax > 384 (every CTA of a cluster has to own spins); nmax <= cluster_batch_max_n().
+int cluster_batch_max_n();
+cudaError_t launch_cluster_batch(const RunArgs &a, int nmax, cudaStream_t st);
 
 // Incremental-field resident kernel for small dense instances (CUDA cores, exact
 // integer field updated by the columns whose spin changed sign; no field mode).

@@ -10,6 +10,11 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
+def _mask(n, keep):
+    m = np.triu(np.random.default_rng(n).random((n, n)) < keep, 1)
+    return m | m.T
+
+
 def _to_csr(d):
     rows, cols = np.nonzero(d.k)
     rp = np.zeros(d.n + 1, dtype=np.int32)
@@ -28,10 +33,10 @@ def test_slices_equal_the_dense_kernel(gpu_lib, N, R, kmax, hmax, keep, csr_mode
     phia = gpu_lib
     T = 60
     d = ins.dense_int(N, kmax, hmax, seed=N + R)
-    m = np.triu(np.random.default_rng(N).random((N, N)) < keep, 1)
-    d = ins.Dense((d.k * (m | m.T)).astype(np.int8), d.kh)
+    d = ins.Dense((d.k * _mask(N, keep)).astype(np.int8), d.kh)
     sched = phia.schedule(0.01, 0.2, 0.1, 2.0, refresh=17)
-    with phia.Batch([_to_csr(d)], csr_mode=csr_mode) as B:
+    # beside a member too large for the resident kernels, so that the gather runs
+    with phia.Batch([_to_csr(d), ins.erdos_renyi(600, 0.02, 127, 31, 4, seed=1)], csr_mode=csr_mode) as B:
         B.anneal(sched, R, T, seed=3)
         a = B.replica_results(0, R)
     with phia.Annealer(d.k, d.kh, path=phia.PATH_TC, tc_kernel=phia.KERNEL_PER_STEP, large_variant=1) as A:
@@ -78,3 +83,39 @@ def test_several_sets_equal_each_instance_alone(gpu_lib):
                 alone = A.replica_results(0, R)
             for u, w in zip(mix[k], alone):
                 assert np.array_equal(u, w)
+
+
+# Edges of the resident kernels' sizes: 16-spin warps, the classes of 64, 128 and 256 spins, clusters
+# of 2 and 4 CTAs, and the first size that gathers; replicas in one wave and in many.
+@pytest.mark.parametrize("N,R", [(1, 3), (16, 40), (64, 8), (65, 33), (128, 300), (129, 17), (256, 256), (257, 9),
+                                 (384, 70), (385, 5), (512, 256), (513, 40), (300, 3000)])
+def test_small_sparse_handles_equal_the_gather(gpu_lib, N, R):
+    """Small sparse instances run on a resident kernel where that is estimated faster: records
+    (frozen at a replica's own hit where the run stops at a target) and states of runs in pieces
+    are those of the gather."""
+    phia = gpu_lib
+    T = 50
+    c = _to_csr(ins.Dense((ins.dense_int(N, 127, 9, seed=N).k * _mask(N, 0.1)).astype(np.int8),
+                          ins.dense_int(N, 7, 90, seed=N).kh))
+    big = ins.erdos_renyi(600, 0.02, 127, 31, 4, seed=1)
+    for target, stop in ((None, False), (-40 * N, True)):
+        sched = phia.schedule(0.01, 0.1, 0.1, 2.0, refresh=13, target=target, stop_at_target=stop)
+        with phia.Batch([c, big]) as B:
+            B.anneal(sched, R, T, seed=5)
+            a = B.replica_results(0, R)
+        with phia.Annealer(h_k=c.kh, csr=(c.row_ptr, c.col, c.val), path=phia.PATH_CSR) as A:
+            x = torch.empty((R, N), device="cuda"); v = torch.empty((R, N), device="cuda")
+            phia.init_state(A.h, R, 5, x, v)
+            for t0, n in ((0, 1), (1, 2), (3, T - 3)):
+                phia.run(A.h, sched, R, t0, n, T, 5, x, v, reset_best=(t0 == 0))
+            b = phia.replica_results(A.h, R, N)
+            torch.cuda.synchronize()
+            assert phia.stats_get(A.h).path == phia.PATH_CSR
+        for u, w in zip(a, b):
+            assert np.array_equal(u, w)
+    with phia.Annealer(c.to_dense().k, c.kh, path=phia.PATH_TC, tc_kernel=phia.KERNEL_PER_STEP, large_variant=1) as D:
+        xd = torch.empty((R, N), device="cuda"); vd = torch.empty((R, N), device="cuda")
+        phia.init_state(D.h, R, 5, xd, vd)
+        phia.run(D.h, phia.schedule(0.01, 0.1, 0.1, 2.0, refresh=13), R, 0, T, T, 5, xd, vd)
+        torch.cuda.synchronize()
+        assert torch.equal(x, xd) and torch.equal(v, vd)
