@@ -36,6 +36,7 @@
 // Records are lagged: the launch for iteration t settles t - 1 (the instance's first unit)
 // and copies the best spins of t - 2 for the replicas that improved then.
 #include <algorithm>
+#include <type_traits>
 
 #include "device_common.cuh"
 #include "phia_internal.h"
@@ -194,8 +195,9 @@ __device__ __noinline__ void refresh8(float *v, uint64_t seed, uint32_t inst, ui
 // C.gblock groups of 32 replicas (the y-th such set).  Uses the block's shared memory; every
 // thread of the block calls it.  STEP: the unit of a step launch, which may start before the
 // launch for t - 1 has ended: what no iteration changes (the block, its instance, the first
-// entries) loads first, then it waits for that launch and reads its iteration.
-template <bool SMEM, bool C16, bool STEP>
+// entries) loads first, then it waits for that launch and reads its iteration.  SMEM: the spins are
+// gathered from shared memory; STAGED: x and v of a slice pass through it.
+template <bool SMEM, bool C16, bool STAGED, bool STEP>
 __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_t t, int64_t t_first, int64_t t_end,
                                          char *smem) {
     const RunArgs &a = C.a;
@@ -224,20 +226,6 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
         t = __ldcg(&C.ctl->t);
     }
 
-    // x and v of a slice's first 8 replicas load while the rest goes on, the others 8 replicas ahead
-    // of their use.
-    const size_t qs = (size_t)in.Np * 4;               // floats between quads of replicas
-    float4 xq[2], vq[2];
-    auto load_quads = [&](int s) {
-        const size_t o = in.x_off + ((size_t)g * 8 * in.Np + s * 32 + lane) * 4;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            xq[k] = __ldcg(reinterpret_cast<const float4 *>(C.X + o + k * qs));
-            vq[k] = __ldcg(reinterpret_cast<const float4 *>(C.V + o + k * qs));
-        }
-    };
-    if (s_first < s_end) load_quads(s_first);
-
     // The spins of this iteration of the block's groups into shared memory.
     const uint32_t *Sg = spin_buf(C, in, t);
     if constexpr (SMEM) {
@@ -246,6 +234,30 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
         for (int e = tid * 4; e < words; e += kBlk * 4) cp_async_16(smem + (size_t)e * 4, src + e);
         cp_async_commit();
     }
+    // x and v of a slice load while the gather runs: all of it into the warp's part of shared memory
+    // (a lane's own values, which nobody else reads), or the first 8 replicas into registers and
+    // the others 8 replicas ahead of their use, which then waits for L2.
+    const size_t qs = (size_t)in.Np * 4;               // floats between quads of replicas
+    float4 *const stage = reinterpret_cast<float4 *>(smem + C.stage_off) + warp * (16 * 32) + lane;
+    float4 xq[2], vq[2];
+    auto fetch_state = [&](int s) {
+        const size_t o = in.x_off + ((size_t)g * 8 * in.Np + s * 32 + lane) * 4;
+        if constexpr (STAGED) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                cp_async_16(stage + 64 * k, C.X + o + k * qs);
+                cp_async_16(stage + 64 * k + 32, C.V + o + k * qs);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                xq[k] = __ldcg(reinterpret_cast<const float4 *>(C.X + o + k * qs));
+                vq[k] = __ldcg(reinterpret_cast<const float4 *>(C.V + o + k * qs));
+            }
+        }
+    };
+    if (s_first < s_end) fetch_state(s_first);
+    if constexpr (STAGED) cp_async_commit();
     // (a) records of iteration t-1 (the last block of each instance, whose rows are the shortest).
     if (blk.s0 + C.slices >= nsl && t - 1 >= t_first) {
         for (int e = tid; e < G * 32; e += kBlk)
@@ -270,7 +282,7 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
             }
         }
     }
-    if constexpr (SMEM) cp_async_wait<0>();
+    if constexpr (SMEM) cp_async_wait<STAGED ? 1 : 0>();
     if constexpr (SMEM || STEP) __syncthreads();
     unsigned ticket = 0;          // every thread of the block has read the iteration
     if constexpr (STEP)
@@ -289,7 +301,8 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
             float *X = C.X + in.x_off + ((size_t)g * 8 * in.Np + p) * 4;
             float *V = C.V + in.x_off + ((size_t)g * 8 * in.Np + p) * 4;
             if (s != s_first) {
-                load_quads(s);
+                fetch_state(s);
+                if constexpr (STAGED) cp_async_commit();
                 e0 = C.slice[in.slice_off + s];
                 e1 = C.slice[in.slice_off + s + 1];
                 ahead.load(C, e0, e1, lane);
@@ -302,16 +315,24 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
             const int2 hh = __ldg(reinterpret_cast<const int2 *>(C.hk) + in.pos_off + p);    // h, h - ksum
             const int row = refresh_next ? C.row_of[in.pos_off + p] : 0;
             uint32_t bits = 0;
+            if constexpr (STAGED) cp_async_wait<0>();
             // 8 replicas at a time, their accumulators moved down to the front: one copy of the code
             // instead of four, as a straight line over all 32 replicas (with the draws of a refresh in it)
             // is fetched anew for every slice: its update took 8000 to 10000 cycles, most of them
             // waiting for instructions.
 #pragma unroll 1
             for (int o = 0; o < 4; ++o) {
+                float *Xo = X + 2 * o * qs, *Vo = V + 2 * o * qs;
+                if constexpr (STAGED) {
+                    const float4 *so = stage + 128 * o;
+                    xq[0] = so[0];
+                    vq[0] = so[32];
+                    xq[1] = so[64];
+                    vq[1] = so[96];
+                }
                 float xs[8] = {xq[0].x, xq[0].y, xq[0].z, xq[0].w, xq[1].x, xq[1].y, xq[1].z, xq[1].w}, If[8];
                 float vn[8] = {vq[0].x, vq[0].y, vq[0].z, vq[0].w, vq[1].x, vq[1].y, vq[1].z, vq[1].w};
-                float *Xo = X + 2 * o * qs, *Vo = V + 2 * o * qs;
-                if (o < 3) {
+                if (!STAGED && o < 3) {
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
                         xq[k] = __ldcg(reinterpret_cast<const float4 *>(Xo + (2 + k) * qs));
@@ -382,13 +403,13 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
 // blocks start as soon as its own have all started (they wait for its end before they read what
 // it writes), so the boundary costs neither a launch nor the loads of what is the same in every
 // iteration.
-template <bool SMEM, bool C16>
+template <bool SMEM, bool C16, bool STAGED>
 __global__ void __launch_bounds__(kBlk, 2) csr_step(const CsrArgs C) {
     extern __shared__ __align__(16) char smem[];
     grid_dependents_launch();
     const CsrSet set = C.sets[__ldcg(&C.ctl->set)];
     if ((int)blockIdx.x < set.len[C.list]) {
-        csr_unit<SMEM, C16, true>(C, set.off[C.list] + blockIdx.x, blockIdx.y, 0, 0, 0, smem);
+        csr_unit<SMEM, C16, STAGED, true>(C, set.off[C.list] + blockIdx.x, blockIdx.y, 0, 0, 0, smem);
     } else {
         grid_dependency_wait();
         if (threadIdx.x == 0) step_done(C.ctl, atomicAdd(&C.ctl->done, 1u));
@@ -424,7 +445,7 @@ __device__ bool grid_barrier(unsigned *bar, uint64_t timeout_ns) {
 // takes work units from a counter (units of uneven cost balance themselves), then the grid
 // meets at a barrier.  ctr[k & 1] hands out the units of the launch's k-th iteration; block 0
 // clears it after that iteration's barrier, before it is used again.
-template <bool SMEM, bool C16>
+template <bool SMEM, bool C16, bool STAGED>
 __global__ void __launch_bounds__(kBlk, 2) csr_persistent(const CsrArgs C, unsigned *bar, unsigned *ctr) {
     extern __shared__ __align__(16) char smem[];
     __shared__ int unit;
@@ -441,7 +462,7 @@ __global__ void __launch_bounds__(kBlk, 2) csr_persistent(const CsrArgs C, unsig
                 const int u = unit;
                 __syncthreads();
                 if (u >= units) break;
-                csr_unit<SMEM, C16, false>(C, set.off[C.list] + u % nb, u / nb, t, t_first, t_end, smem);
+                csr_unit<SMEM, C16, STAGED, false>(C, set.off[C.list] + u % nb, u / nb, t, t_first, t_end, smem);
             }
             if (!grid_barrier(bar, kWaitTimeoutNs)) {
                 if (threadIdx.x == 0) atomicExch(C.a.err, 1);
@@ -608,7 +629,7 @@ __global__ void csr_count(const CsrArgs C) {
         atomicAdd(C.a.replica_iters, (unsigned long long)((long long)C.total_reps * C.a.nsteps));
 }
 
-template <bool SMEM, bool C16>
+template <bool SMEM, bool C16, bool STAGED>
 cudaError_t launch_iterations(const CsrArgs &C, size_t smem, StepGraphCache *graphs, cudaStream_t st, int sms,
                               int max_blocks, int *launches) {
     const int ny = (C.R / 32 + C.gblock - 1) / C.gblock;
@@ -617,7 +638,7 @@ cudaError_t launch_iterations(const CsrArgs &C, size_t smem, StepGraphCache *gra
     Cs.x_out = Cs.v_out = nullptr;
     if (C.persistent) {
         // Every iteration in one cooperative launch: as many blocks as can be resident.
-        auto k = csr_persistent<SMEM, C16>;
+        auto k = csr_persistent<SMEM, C16, STAGED>;
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int per_sm = 0;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kBlk, smem);
@@ -637,7 +658,7 @@ cudaError_t launch_iterations(const CsrArgs &C, size_t smem, StepGraphCache *gra
     // arguments leave out what only the prologue and the export read.
     Cs.a.t0 = 0;
     Cs.a.nsteps = 0;
-    auto k = csr_step<SMEM, C16>;
+    auto k = csr_step<SMEM, C16, STAGED>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void *args[1] = {&Cs};
@@ -674,27 +695,43 @@ cudaError_t launch_csr(const CsrArgs &Cin, const int32_t *max_len, StepGraphCach
     const unsigned conv = (unsigned)(C.total_slices * groups);
     csr_prologue<<<conv, kBlk, 0, st>>>(C);
     ++n;
-    // Groups per block: up to 8 share one reading of the couplings (through L1) and of the
-    // shared memory that two blocks an SM have; spins of an instance too large for it are read
-    // from L2.  Slices per block: 4, fewer while the units do not fill the GPU twice over (a
-    // set's time is that of its heaviest blocks).
+    // Groups per block: up to 8 share one reading of the couplings (through L1), as many as leave
+    // two blocks an SM their shared memory, with x and v staged in it (48 instances of 100 .. 3000
+    // spins x 256 replicas 122 us an iteration against 140 from registers, one of 10000 19.5 against
+    // 21.8).  A single group's spins that leave no room for both keep the two blocks and load x and
+    // v into registers (20000 spins 36 against 43); larger ones are staged by one block an SM
+    // (30000: 61 against 65), and spins too large for that are read from L2 (50000: 91 against 128
+    // with them in shared memory and nothing staged; staged as well 60000 takes 116 against 112).
+    constexpr size_t kStage = (size_t)kWarps * 16 * 32 * sizeof(float4);      // x and v of a slice per warp
+    constexpr size_t kTwo = 113 * 1024, kOne = 226 * 1024;                     // two blocks an SM, one
     int G = 1;
     while (G < 8 && G < groups) G *= 2;
-    constexpr size_t kTwo = 113 * 1024, kOne = 226 * 1024;
-    while (G > 1 && (size_t)G * C.max_np * 4 > kTwo) G /= 2;
-    const size_t bytes = (size_t)G * C.max_np * 4;
-    const bool in_smem = bytes <= kOne;
-    if (!in_smem)
+    while (G > 1 && (size_t)G * C.max_np * 4 + kStage > kTwo) G /= 2;
+    size_t bytes = (size_t)G * C.max_np * 4;
+    const bool in_smem = bytes <= kTwo || bytes + kStage <= kOne;
+    const bool staged = in_smem && (bytes + kStage <= kTwo || bytes > kTwo);
+    if (!in_smem) {
         for (G = 1; G < 8 && G < groups;) G *= 2;
+        bytes = 0;
+    }
+    C.stage_off = (int32_t)bytes;
+    if (staged) bytes += kStage;
     C.gblock = G;
     const int spar = kWarps / G, ny = (groups + G - 1) / G;
+    // Slices per block: 4, or as many as it has lanes for, fewer while the units do not fill the GPU
+    // twice over (a set's time is that of its heaviest blocks).
     int li = spar >= 8 ? 3 : 2;                 // block lists of 1, 2, 4, 8 slices
     while ((1 << li) > spar && (int64_t)max_len[li] * ny < 4 * (int64_t)sms) --li;
     C.slices = 1 << li;
     C.list = li;
-    if (in_smem && C.col16) e = launch_iterations<true, true>(C, bytes, graphs, st, sms, max_len[li], &n);
-    else if (in_smem) e = launch_iterations<true, false>(C, bytes, graphs, st, sms, max_len[li], &n);
-    else e = launch_iterations<false, false>(C, 0, graphs, st, sms, max_len[li], &n);
+    auto go = [&](auto smem, auto c16, auto stg) {
+        return launch_iterations<smem.value, c16.value, stg.value>(C, bytes, graphs, st, sms, max_len[li], &n);
+    };
+    constexpr std::true_type yes{};
+    constexpr std::false_type no{};
+    if (!in_smem) e = go(no, no, no);
+    else if (C.col16) e = staged ? go(yes, yes, yes) : go(yes, yes, no);
+    else e = staged ? go(yes, no, yes) : go(yes, no, no);
     if (e != cudaSuccess) return e;
     const int64_t t_last = C.a.t0 + C.a.nsteps - 1;
     csr_settle_all<<<C.count, 256, 0, st>>>(C, t_last);

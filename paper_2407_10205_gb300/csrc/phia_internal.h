@@ -208,6 +208,7 @@ struct CsrArgs {
     int32_t list;           // the list in use
     int32_t slices;         // slices per block of that list
     int32_t gblock;         // groups of 32 replicas per block
+    int32_t stage_off;      // the warps' x and v in a block's shared memory
     int32_t max_np;         // largest Np
     const int32_t *slice;   // first entry of each slice (an entry: 4 neighbours of 32 rows)
     const void *col;        // [entries][32][4] byte offsets of the neighbours' positions, uint16 or uint32

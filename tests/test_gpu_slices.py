@@ -46,9 +46,10 @@ def test_slices_equal_the_dense_kernel(gpu_lib, N, R, kmax, hmax, keep, csr_mode
         assert np.array_equal(u, w)
 
 
-@pytest.mark.parametrize("N", [16384, 16390])
+@pytest.mark.parametrize("N", [12300, 12600, 16384, 16390, 30000, 42000])
 def test_both_offset_widths(gpu_lib, N):
-    """16-bit neighbour offsets up to 16384 positions, 32-bit ones above: fields and energies."""
+    """16-bit neighbour offsets up to 16384 positions, 32-bit ones above, with x and v staged in
+    shared memory or not, the spins in shared memory or not: fields and energies."""
     phia = gpu_lib
     c = ins.erdos_renyi(N, 6.0 / N, 127, 31, 4, seed=N)
     P = o.Instance(c.kh, row_ptr=c.row_ptr, col=c.col, val=c.val, frac_bits=4)
