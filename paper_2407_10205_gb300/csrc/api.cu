@@ -122,8 +122,6 @@ struct phia_s {
     int8_t *d_Jk = nullptr;
     float *d_Jf = nullptr;
     int32_t *d_hk = nullptr;
-    float *d_hf = nullptr;              // h as FP32, padded with zeros to a multiple of 16 (dense instances)
-    int32_t *d_hmax = nullptr;          // max |h|
     int32_t *d_rowptr = nullptr, *d_col = nullptr;
     int8_t *d_val = nullptr;
     // per-replica state
@@ -316,8 +314,6 @@ RunArgs base_args(phia_t *p, int R) {
     a.Jk = p->d_Jk;
     a.Jf = p->d_Jf;
     a.hk = p->d_hk;
-    a.hf = p->d_hf;
-    a.h_max = p->d_hmax;
     a.max_abs_k = p->max_abs_k;
     a.row_ptr = p->d_rowptr; a.col = p->d_col; a.val = p->d_val;
     a.R = R;
@@ -450,9 +446,6 @@ int finish_create(phia_t *p, const int32_t *h_k, const phia_opts *opts,
                   cudaMemcpyKind h_kind = cudaMemcpyHostToDevice) {
     CU(pool_alloc((void **)&p->d_hk, (size_t)p->N * 4, p->device, p->stream));
     CU(cudaMemcpyAsync(p->d_hk, h_k, (size_t)p->N * 4, h_kind, p->stream));
-    CU(pool_alloc((void **)&p->d_hf, (size_t)round_up(p->N, 16) * 4, p->device, p->stream));
-    CU(pool_alloc((void **)&p->d_hmax, 4, p->device, p->stream));
-    CU(launch_pad_field(p->d_hk, p->N, p->d_hf, p->d_hmax, p->stream));
     CU(pool_alloc((void **)&p->d_ctl, sizeof(IterCtl), p->device, p->stream));
     p->graphs = step_graphs_new();
     CU(cudaEventCreate(&p->ev0));
@@ -1083,7 +1076,7 @@ void phia_destroy(phia_t *p) {
     cudaSetDevice(p->device);
     cudaStreamSynchronize(p->stream);
     free_replicas(p);
-    for (void *b : {(void *)p->d_Jk, (void *)p->d_Jf, (void *)p->d_hk, (void *)p->d_hf, (void *)p->d_hmax, (void *)p->d_Jop, (void *)p->d_ctl})
+    for (void *b : {(void *)p->d_Jk, (void *)p->d_Jf, (void *)p->d_hk, (void *)p->d_Jop, (void *)p->d_ctl})
         pool_free(b, p->stream);
     cudaFree(p->d_rowptr); cudaFree(p->d_col); cudaFree(p->d_val);
     step_graphs_free(p->graphs);

@@ -58,29 +58,7 @@ __global__ void check_dense_kernel(const int8_t *J, const int32_t *h, int N, uns
         if (h[i] >= (1 << 24) || h[i] <= -(1 << 24)) atomicMin(&res[2], (unsigned long long)i);
 }
 
-// One block: h as FP32 (|h| < 2^24, exact), zeros up to the next multiple of 16, max |h|.
-__global__ void pad_field_kernel(const int32_t *hk, int N, float *hf, int32_t *h_max) {
-    __shared__ unsigned int mx;
-    if (threadIdx.x == 0) mx = 0;
-    __syncthreads();
-    unsigned int m = 0;
-    for (int i = threadIdx.x; i < (N + 15) / 16 * 16; i += blockDim.x) {
-        const int32_t h = i < N ? hk[i] : 0;
-        hf[i] = (float)h;
-        m = max(m, (unsigned int)abs(h));
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(&mx, m);
-    __syncthreads();
-    if (threadIdx.x == 0) *h_max = (int32_t)mx;
-}
-
 }  // namespace
-
-cudaError_t launch_pad_field(const int32_t *hk, int N, float *hf, int32_t *h_max, cudaStream_t st) {
-    pad_field_kernel<<<1, 1024, 0, st>>>(hk, N, hf, h_max);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_check_dense(const int8_t *J, const int32_t *h, int N, unsigned long long *res, unsigned blocks,
                                cudaStream_t st) {

@@ -66,6 +66,7 @@ struct NarrowShared {
     uint64_t accf;                // the accumulator holds an iteration's fields
     uint64_t tiledone;            // the epilogue warps finished an iteration
     uint64_t drain;               // every MMA issued has completed
+    alignas(16) float h[64];      // field of the tile's spins, 0 past N
     uint32_t tmem_base;
     int32_t timed_out;
     int64_t rec_settled;          // last iteration the records warp settled
@@ -225,7 +226,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int N = a.N;
     const uint64_t kWaitNs = a.wait_ns > 0 ? (uint64_t)a.wait_ns : kWaitTimeoutNs;
     // A chunk's 16 energy terms s (I + h) add up exactly in FP32 while |I + h| <= 2^20.
-    const bool exact_sums = (int64_t)a.max_abs_k * (N - 1) + 2 * (int64_t)*a.h_max <= (int64_t)1 << 20;
+    const int32_t h_mine = tid < BN && m * BN + tid < N ? a.hk[m * BN + tid] : 0;
+    const bool h_small = (int64_t)a.max_abs_k * (N - 1) + 2 * (int64_t)abs(h_mine) <= (int64_t)1 << 20;
+    if (tid < BN) sh->h[tid] = (float)h_mine;
     uint32_t *ready = L.ready, *settled = L.ready + L.rtiles;
 
     if (warp == 0) {
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         fence_mbarrier_init();
     }
     tc_fence_before();
-    __syncthreads();
+    const bool exact_sums = __syncthreads_and(h_small) != 0;
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
 
@@ -394,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 float h[kChunk], f[kChunk];
 #pragma unroll
                 for (int k = 0; k < kChunk / 4; ++k) {
-                    const float4 h4 = __ldg(reinterpret_cast<const float4 *>(a.hf + i0 + 4 * k));
+                    const float4 h4 = *reinterpret_cast<const float4 *>(&sh->h[cg * kColsPerWarp + c * kChunk + 4 * k]);
                     h[4 * k] = h4.x; h[4 * k + 1] = h4.y; h[4 * k + 2] = h4.z; h[4 * k + 3] = h4.w;
                 }
                 if (a.deriv == 1) {
@@ -407,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tmem_ld_wait_x16(acc);
                 // Field I = J s + h (Eq. 6): acc and h are exact integers, their FP32 sum rounds the
                 // exact field.  Energy terms s (I + h) (Eq. 2 through Eq. 6) of the replica: where a
-                // chunk's add up exactly in FP32 (the handle knows max |k|, max |h| and N) they are
+                // chunk's add up exactly in FP32 (the tile's max |h|, max |k| and N say so) they are
                 // converted once, otherwise each by itself.  Spins past N have zero couplings, h = 0
                 // and x = v = 0.
                 float I[kChunk];

@@ -29,8 +29,6 @@ struct RunArgs {
     int32_t frac_bits;
     const int8_t *Jk;      // dense k, [N][N] int8 (exact storage)
     const int32_t *hk;     // [N]
-    const float *hf;       // hk as FP32 (exact), zero-padded to a multiple of 16 entries (dense handles)
-    const int32_t *h_max;  // max |hk| (dense handles)
     int32_t max_abs_k;     // max |k| (dense handles)
     const float *Jf;       // FP32 copy of J = k q (FP32 path)
     const int32_t *row_ptr; const int32_t *col; const int8_t *val;  // CSR
@@ -157,8 +155,6 @@ double narrow_estimate(int N, int R, int Kbytes, int sms, int *width);
 // 2-D tensor map of an operand array (128-byte swizzle, box of one swizzle row x box_rows).
 bool tc_operand_map(void *map, const void *base, int op, uint64_t inner_elems, uint64_t rows, uint64_t row_bytes,
                     uint32_t box_rows);
-// hk as FP32, zero-padded to a multiple of 16, and max |hk| into *h_max.
-cudaError_t launch_pad_field(const int32_t *hk, int N, float *hf, int32_t *h_max, cudaStream_t st);
 cudaError_t launch_convert_operand(const int8_t *Jk, int N, void *Jop, int Mpad, int Kbytes, int op, cudaStream_t st);
 // Device checks of a dense instance into res[4] (initialised by the caller to
 // {ULLONG_MAX, ULLONG_MAX, ULLONG_MAX, 0}): res[0] lowest i*N+j with k_ij != k_ji (i < j),
