@@ -22,8 +22,8 @@
 // out sets the run's error flag and the warp winds down.
 //
 // bf16 fragments up to 512 spins; above, e4m3 ones, as bf16 rows of J no longer fit in registers.
-// Per iteration (us): N = 512 x 256 replicas 1.24 against 10.85 with one launch per iteration,
-// 333 x 500 1.54, 600 x 64 1.78, 1000 x 64 2.44.  (With plain remote stores, a fence and an
+// Per iteration (us): N = 512 x 256 replicas 1.15 against 10.9 with one launch per iteration,
+// 600 x 128 1.68 against 11.2, 1000 x 64 2.35 against 11.7; 333 x 500 1.54.  (With plain remote stores, a fence and an
 // arrival on every CTA's mbarrier in the place of st.async, N = 512 took 1.8.)
 #include <algorithm>
 #include <climits>

@@ -24,16 +24,17 @@
 // 32 dot products, 32 masks, 8 byte permutes, 4 shared loads) and of the update, with the x, v
 // stream (16 bytes per spin update) behind them.  The earlier form took a row to a warp and 8
 // replicas to a lane: every neighbour cost the warp a load of 32 bytes, its address and its
-// share of the byte permutes for 8 replicas a lane instead of 32.  Per iteration (us), that
-// form and this one: 48 Erdos-Renyi instances of 100 .. 3000 spins x 256 replicas 166 / 139, 12
-// of them x 256 44 / 26, one of 5000 spins x 256 27 / 15, where the longest slice sets the time; with the update in a
-// loop and launches that overlap (below) 12 of it, and 6.9 instead of 10 for one of 105 spins.
+// share of the byte permutes for 8 replicas a lane instead of 32.  Per iteration (us, 256 replicas),
+// that form and this one: one Erdos-Renyi instance of 625 spins 20.9 / 7.6, of 1760 36.0 / 12.4, of
+// 5000 27.1 / 10.7, where latencies in a row set the time; 12 instances of 100 .. 3000 spins
+// 56.9 / 32.8, 48 of them 180 / 122.5, 256 of them 654 / 568.
 //
 // The instances go through their iterations in sets whose state fits in L2 together: a set runs
 // all of its iterations before the next begins (the instances are independent), so x and v are
-// read from L2 instead of the memory they would fall out to between two iterations of a batch.
+// read from L2 instead of the memory they would fall out to between two iterations of a batch
+// (48 instances 117 us an iteration against 135 in one set, 256 of them 636 against 653).
 //
-// Records are lagged: the launch for iteration t settles t - 1 (the instance's first unit)
+// Records are lagged: the launch for iteration t settles t - 1 (the instance's last unit)
 // and copies the best spins of t - 2 for the replicas that improved then.
 #include <algorithm>
 #include <type_traits>
@@ -47,6 +48,12 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kBlk = 32 * kWarps;
+
+// The word of position p and group g in a spin buffer: [group][Np], so that a group's spins are
+// copied as one piece, or (C.by_pos) [Np][group], so that a neighbour's groups share a sector.
+__device__ __forceinline__ size_t spin_word(const CsrArgs &C, const CsrInst &in, int g, int p) {
+    return C.by_pos ? (size_t)p * (C.R / 32) + g : (size_t)g * in.Np + p;
+}
 
 __device__ __forceinline__ void settle_csr(const CsrArgs &C, const CsrInst &in, int b, int r, int64_t tt) {
     const RunArgs &a = C.a;
@@ -128,14 +135,27 @@ struct Ahead {
     }
 };
 
+// 4 neighbours of a lane's row: acc[r] += sum k [s = +1] over them.  SCALED: acc_r carries the
+// factor 2^(r % 8) of its bit's place (one instruction less per replica); rows of over 2^16
+// couplings take the bit down to place 0 instead, as the factor could leave 32 bits.
+template <bool SCALED>
+__device__ __forceinline__ void add_neighbours(const uint32_t (&w)[4], uint32_t k, int32_t (&acc)[32]) {
+    uint32_t B[4];
+    transpose4(w, B);
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+        const int bit = r & 7;
+        if constexpr (SCALED) acc[r] = dp4a_us(B[r >> 3] & (0x01010101u << bit), k, acc[r]);
+        else acc[r] = dp4a_us((B[r >> 3] >> bit) & 0x01010101u, k, acc[r]);
+    }
+}
+
 // acc[r] of the lane's row over its couplings: entries [e, e_end) of the slice, 4 neighbours
 // each; the next entries load meanwhile (three ahead with 16-bit offsets, whose registers allow
-// it: an entry's L2 latency is several times its arithmetic).  SCALED: acc_r carries the factor
-// 2^(r % 8) of its bit's place (one instruction less per replica); rows of over 2^16 couplings
-// take the bit down to place 0 instead, as the factor could leave 32 bits.
-template <bool SMEM, bool C16, bool SCALED>
-__device__ __forceinline__ void gather_row(const CsrArgs &C, const char *spins, int e, int e_end, int lane,
-                                           Ahead<C16> &ahead, int32_t (&acc)[32]) {
+// it: an entry's L2 latency is several times its arithmetic).  Spins in shared memory.
+template <bool C16, bool SCALED>
+__device__ __forceinline__ void gather_smem(const CsrArgs &C, const char *spins, int e, int e_end, int lane,
+                                            Ahead<C16> &ahead, int32_t (&acc)[32]) {
     constexpr int D = Ahead<C16>::D;
     Entry<C16>(&nx)[D] = ahead.nx;
 #pragma unroll 1
@@ -145,20 +165,41 @@ __device__ __forceinline__ void gather_row(const CsrArgs &C, const char *spins, 
             if (u > 0 && e + u >= e_end) break;
             const Entry<C16> en = nx[u];
             if (e + u + D < e_end) nx[u].load(C, e + u + D, lane);
-            uint32_t w[4], B[4];
+            uint32_t w[4];
 #pragma unroll
-            for (int n = 0; n < 4; ++n) {
-                if constexpr (SMEM) w[n] = *reinterpret_cast<const uint32_t *>(spins + en.at(n));
-                else w[n] = __ldcg(reinterpret_cast<const uint32_t *>(spins + en.at(n)));
-            }
-            transpose4(w, B);
-#pragma unroll
-            for (int r = 0; r < 32; ++r) {
-                const int bit = r & 7;
-                if constexpr (SCALED) acc[r] = dp4a_us(B[r >> 3] & (0x01010101u << bit), en.k, acc[r]);
-                else acc[r] = dp4a_us((B[r >> 3] >> bit) & 0x01010101u, en.k, acc[r]);
-            }
+            for (int n = 0; n < 4; ++n) w[n] = *reinterpret_cast<const uint32_t *>(spins + en.at(n));
+            add_neighbours<SCALED>(w, en.k, acc);
         }
+    }
+}
+
+// The same from global memory, spins by position (`groups` words each): the block's warps take
+// the groups of a slice side by side, so that one of them brings a neighbour's sector to L1.  The
+// next entry's words load while this one's are added.
+// CACHED: through L1, which a launch finds empty; iterations within one launch read L2.
+template <bool C16, bool SCALED, bool CACHED>
+__device__ __forceinline__ void gather_global(const CsrArgs &C, const char *spins, uint32_t groups, int e, int e_end,
+                                              int lane, Ahead<C16> &ahead, int32_t (&acc)[32]) {
+    Entry<C16> nx = ahead.nx[0];
+    uint32_t w[4] = {0u, 0u, 0u, 0u}, k = nx.k;
+    auto words = [&]() {
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const uint32_t *p = reinterpret_cast<const uint32_t *>(spins + (size_t)nx.at(n) * groups);
+            w[n] = CACHED ? *p : __ldcg(p);
+        }
+    };
+    if (e < e_end) words();
+    if (e + 1 < e_end) nx.load(C, e + 1, lane);
+#pragma unroll 1
+    for (; e < e_end; ++e) {
+        const uint32_t c[4] = {w[0], w[1], w[2], w[3]}, ck = k;
+        if (e + 1 < e_end) {
+            words();
+            k = nx.k;
+            if (e + 2 < e_end) nx.load(C, e + 2, lane);
+        }
+        add_neighbours<SCALED>(c, ck, acc);
     }
 }
 
@@ -269,11 +310,11 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
         const bool imp = __ldcg(C.flags + (size_t)((t - 2) & 1) * C.total_reps + in.rec_off + g * 32 + lane) != 0;
         const uint32_t mask = __ballot_sync(0xffffffffu, imp);
         if (mask) {
-            const uint32_t *Sb = spin_buf(C, in, t - 2) + (size_t)g * in.Np;
+            const uint32_t *Sb = spin_buf(C, in, t - 2);
             const int W = (in.N + 31) / 32;
             for (int w = blk.s0 + sp; w < s_end; w += spar) {
                 const int i = w * 32 + lane;
-                const uint32_t word = i < in.N ? __ldcg(Sb + C.pos_of[in.inv_off + i]) : 0u;
+                const uint32_t word = i < in.N ? __ldcg(Sb + spin_word(C, in, g, C.pos_of[in.inv_off + i])) : 0u;
                 for (uint32_t m = mask; m; m &= m - 1) {
                     const int r = __ffs(m) - 1;
                     const uint32_t bits = __ballot_sync(0xffffffffu, (word >> r) & 1u);
@@ -289,8 +330,8 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
         if (tid == 0) ticket = atomicAdd(&C.ctl->done, 1u);
     // (c) field and update.
     if (active) {
-        const char *spins = SMEM ? smem + (size_t)gi * in.Np * 4 : reinterpret_cast<const char *>(Sg + (size_t)g * in.Np);
-        uint32_t *Snext = spin_buf(C, in, t + 1) + (size_t)g * in.Np;
+        const char *spins = SMEM ? smem + (size_t)gi * in.Np * 4 : reinterpret_cast<const char *>(Sg + g);
+        uint32_t *Snext = spin_buf(C, in, t + 1);
         const float bgq = beta_at(t, inv_tm1_of(a.T_total), a.beta0, a.beta1) * (a.gamma * in.q);
         const float eps = a.eps, gamma = a.gamma, bgq4 = 4.0f * bgq;
         const bool more = t + 1 < t_end;
@@ -310,8 +351,13 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
             int32_t acc[32];
 #pragma unroll
             for (int r = 0; r < 32; ++r) acc[r] = 0;
-            if (in.wide) gather_row<SMEM, C16, false>(C, spins, e0, e1, lane, ahead, acc);
-            else gather_row<SMEM, C16, true>(C, spins, e0, e1, lane, ahead, acc);
+            if constexpr (SMEM) {
+                if (in.wide) gather_smem<C16, false>(C, spins, e0, e1, lane, ahead, acc);
+                else gather_smem<C16, true>(C, spins, e0, e1, lane, ahead, acc);
+            } else {
+                if (in.wide) gather_global<C16, false, STEP>(C, spins, groups, e0, e1, lane, ahead, acc);
+                else gather_global<C16, true, STEP>(C, spins, groups, e0, e1, lane, ahead, acc);
+            }
             const int2 hh = __ldg(reinterpret_cast<const int2 *>(C.hk) + in.pos_off + p);    // h, h - ksum
             const int row = refresh_next ? C.row_of[in.pos_off + p] : 0;
             uint32_t bits = 0;
@@ -388,7 +434,7 @@ __device__ __forceinline__ void csr_unit(const CsrArgs &C, int bi, int y, int64_
 #pragma unroll
                 for (int r = 0; r < 24; ++r) acc[r] = acc[r + 8];
             }
-            if (more) Snext[p] = bits;
+            if (more) Snext[spin_word(C, in, g, p)] = bits;
         }
         atomicAdd(reinterpret_cast<unsigned long long *>(C.Esum) + (size_t)(t & 1) * C.total_reps + in.rec_off + g * 32 + lane,
                   (unsigned long long)esum);
@@ -532,7 +578,7 @@ __global__ void __launch_bounds__(kBlk) csr_prologue(const CsrArgs C) {
     if (qd == 0) {
 #pragma unroll
         for (int w = 1; w < 8; ++w) bits |= part[w][lane];
-        spin_buf(C, in, a.t0)[(size_t)g * in.Np + p] = bits;
+        spin_buf(C, in, a.t0)[spin_word(C, in, g, p)] = bits;
     }
 }
 
@@ -575,7 +621,7 @@ __global__ void __launch_bounds__(kBlk) csr_copy_all(const CsrArgs C, int64_t t_
         const uint32_t mask = __ballot_sync(
             0xffffffffu, C.flags[(size_t)(tt & 1) * C.total_reps + in.rec_off + g * 32 + lane] != 0);
         if (!mask) continue;
-        const uint32_t word = i < in.N ? spin_buf(C, in, tt)[(size_t)g * in.Np + C.pos_of[in.inv_off + i]] : 0u;
+        const uint32_t word = i < in.N ? spin_buf(C, in, tt)[spin_word(C, in, g, C.pos_of[in.inv_off + i])] : 0u;
         for (uint32_t m = mask; m; m &= m - 1) {
             const int r = __ffs(m) - 1;
             const uint32_t bits = __ballot_sync(0xffffffffu, (word >> r) & 1u);
@@ -693,27 +739,25 @@ cudaError_t launch_csr(const CsrArgs &Cin, const int32_t *max_len, StepGraphCach
     }
     const int groups = C.R / 32;
     const unsigned conv = (unsigned)(C.total_slices * groups);
-    csr_prologue<<<conv, kBlk, 0, st>>>(C);
-    ++n;
     // Groups per block: up to 8 share one reading of the couplings (through L1), as many as leave
     // two blocks an SM their shared memory, with x and v staged in it (48 instances of 100 .. 3000
     // spins x 256 replicas 122 us an iteration against 140 from registers, one of 10000 19.5 against
     // 21.8).  A single group's spins that leave no room for both keep the two blocks and load x and
-    // v into registers (20000 spins 36 against 43); larger ones are staged by one block an SM
-    // (30000: 61 against 65), and spins too large for that are read from L2 (50000: 91 against 128
-    // with them in shared memory and nothing staged; staged as well 60000 takes 116 against 112).
+    // v into registers (20000 spins x 256 36 us against 43 with one block, x 1024 117 against 153
+    // with the spins gathered from global memory).  Larger ones are gathered from global memory, by
+    // position (30000 x 256 48 against 62 from one block's shared memory).
     constexpr size_t kStage = (size_t)kWarps * 16 * 32 * sizeof(float4);      // x and v of a slice per warp
-    constexpr size_t kTwo = 113 * 1024, kOne = 226 * 1024;                     // two blocks an SM, one
+    constexpr size_t kTwo = 113 * 1024;                                        // two blocks an SM
     int G = 1;
     while (G < 8 && G < groups) G *= 2;
     while (G > 1 && (size_t)G * C.max_np * 4 + kStage > kTwo) G /= 2;
     size_t bytes = (size_t)G * C.max_np * 4;
-    const bool in_smem = bytes <= kTwo || bytes + kStage <= kOne;
-    const bool staged = in_smem && (bytes + kStage <= kTwo || bytes > kTwo);
+    const bool in_smem = bytes <= kTwo, staged = bytes + kStage <= kTwo;
     if (!in_smem) {
         for (G = 1; G < 8 && G < groups;) G *= 2;
         bytes = 0;
     }
+    C.by_pos = in_smem ? 0 : 1;
     C.stage_off = (int32_t)bytes;
     if (staged) bytes += kStage;
     C.gblock = G;
@@ -724,14 +768,16 @@ cudaError_t launch_csr(const CsrArgs &Cin, const int32_t *max_len, StepGraphCach
     while ((1 << li) > spar && (int64_t)max_len[li] * ny < 4 * (int64_t)sms) --li;
     C.slices = 1 << li;
     C.list = li;
+    csr_prologue<<<conv, kBlk, 0, st>>>(C);
+    ++n;
     auto go = [&](auto smem, auto c16, auto stg) {
         return launch_iterations<smem.value, c16.value, stg.value>(C, bytes, graphs, st, sms, max_len[li], &n);
     };
     constexpr std::true_type yes{};
     constexpr std::false_type no{};
-    if (!in_smem) e = go(no, no, no);
-    else if (C.col16) e = staged ? go(yes, yes, yes) : go(yes, yes, no);
-    else e = staged ? go(yes, no, yes) : go(yes, no, no);
+    if (!in_smem) e = go(no, no, no);                  // more than 16384 positions
+    else if (staged) e = go(yes, yes, yes);            // at most 12544
+    else e = C.col16 ? go(yes, yes, no) : go(yes, no, no);
     if (e != cudaSuccess) return e;
     const int64_t t_last = C.a.t0 + C.a.nsteps - 1;
     csr_settle_all<<<C.count, 256, 0, st>>>(C, t_last);

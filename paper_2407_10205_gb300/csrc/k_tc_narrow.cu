@@ -21,7 +21,7 @@
 // couplings of the first stages, which do not depend on the iteration, are copied before the
 // wait), and the epilogue is 16 or 32 elements a thread.  The wide tiles of k_tc_large.cu (128 x
 // 128 .. 256) leave most SMs idle here and carry x and v through global memory: per
-// iteration 11.8 us at N = 700 x 1000 replicas against 6.0 here, 14.5 against 8.9 at 1001 x
+// iteration 11.8 us at N = 700 x 1000 replicas against 5.3 here, 14.5 against 8.2 at 1001 x
 // 600 (bf16).  With more tiles than SMs the wide ones win (N = 2000 x 4096: 23.4 us against
 // 25.8 for this form with wide tiles), so it is not built for that.
 //

@@ -31,9 +31,10 @@
 // records spread over the compute warps instead, N = 200 took 1.25 us an iteration against
 // 0.77: a replica's record is some 50 instructions.)
 //
-// Per iteration, 256 replicas, against the tcgen05 resident kernel (us): N = 16 0.39 / 0.85,
-// 64 0.40 / 0.83, 128 0.54 / 0.86, 200 0.82 / 1.12, 230 0.85 / 1.18; at N = 256 the registers of
-// 17 warps run short and it loses.
+// Per iteration, 256 replicas, this kernel and the tcgen05 resident one (us): N = 16 0.31 / 0.85,
+// 64 0.34 / 0.83, 128 0.50 / 0.86, 200 0.80 / 1.12, 230 0.82 / 1.18; at N = 256 the registers of
+// 17 warps run short and it loses.  (Factors and energies between the MMAs instead of after them:
+// N = 64 0.44 against 0.33, 200 0.88 against 0.79; the MMAs are the longer chain.)
 #include <algorithm>
 #include <climits>
 

@@ -182,7 +182,7 @@ struct CsrInst {
     int64_t inv_off;        // into pos_of, per spin
     int64_t x_off;          // into X, V ([R/32][8][Np][4] per instance)
     int64_t xin_off;        // into caller arrays ([R][N] per instance)
-    int64_t s_off;          // into each spin buffer, in uint32 words ([R/32][Np] per instance)
+    int64_t s_off;          // into each spin buffer, in uint32 words (see CsrArgs.by_pos)
     int64_t rec_off;        // into per-replica records (R per instance)
     int64_t bits_off;       // into best_bits (R * ceil(N/32) per instance)
 };
@@ -205,6 +205,7 @@ struct CsrArgs {
     int32_t slices;         // slices per block of that list
     int32_t gblock;         // groups of 32 replicas per block
     int32_t stage_off;      // the warps' x and v in a block's shared memory
+    int32_t by_pos;         // 1: spin buffers are [Np][R/32], 0: [R/32][Np]
     int32_t max_np;         // largest Np
     const int32_t *slice;   // first entry of each slice (an entry: 4 neighbours of 32 rows)
     const void *col;        // [entries][32][4] byte offsets of the neighbours' positions, uint16 or uint32
