@@ -106,7 +106,7 @@ KERNEL_TRAFFIC_BYTES = {
     "tc_flow_run": (2_078_996_000 + 4_795_566_000) // 100,   # N = 2000, 4096 replicas: a 100-iteration launch,
                                                              # per iteration (a launch runs all of them)
     "tc_large_step": None,                                   # not re-captured since its last change
-    "csr_step": 975_512_832 + 774_093_056,                   # 256 ER instances, 256 replicas (one iteration)
+    "csr_step": None,                                        # not re-captured since its last change
     "tc_small_kernel": 140_544,                              # N = 200, 1024 replicas (a launch is the whole run)
 }
 
@@ -345,7 +345,7 @@ def _peaks():
 def mma_probe(phia):
     """Dense rates measured on this GPU by the library's own probe (phia_mma_peak): tcgen05
     M = 128, N = 256 MMAs from shared memory on every SM, e4m3 and bf16 (TFLOP/s); and the
-    warp-level int8 mma.sync route of the int8 resident kernel (integer TOP/s)."""
+    warp-level int8 mma.sync route (integer TOP/s)."""
     out = {}
     for name, op in (("e4m3", phia.OP_E4M3), ("bf16", phia.OP_BF16), ("s8_mma_sync", phia.PEAK_S8_MMA_SYNC)):
         try:
@@ -372,7 +372,7 @@ def _roofline(w, kernel_ms, stats, peaks, src, probe=None, large_variant=0):
     peak = 2.0 * bf16_peak if e4m3 else bf16_peak
     achieved = 2.0 * N * su / (kernel_ms * 1e-3) / 1e12
     kname = {1: "tc_small_kernel", 2: "tc_flow_run" if large_variant >= 7 else "tc_large_step",
-             3: "imma_small_kernel", 4: "inc_small_kernel"}.get(stats.tc_kernel, "?")
+             3: "warp_small_kernel", 4: "inc_small_kernel"}.get(stats.tc_kernel, "?")
     out = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
            "traffic": KERNEL_TRAFFIC_BYTES.get(kname), "kernel": kname,
            "flops_per_spin_update": 2 * N,
@@ -860,7 +860,7 @@ def measure_dense(args, w, rank=0, world=1, local=0, with_cpu=True, dist=None):
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "fp32", "data": "synthetic",
         "config": {"workload": w["name"], "N": N, "replicas": R, "iterations": T, "path": "tc",
-                   "tc_kernel": {1: "resident tcgen05", 2: "per-iteration tcgen05", 3: "resident int8 mma.sync",
+                   "tc_kernel": {1: "resident tcgen05", 2: "per-iteration tcgen05", 3: "resident warp-level",
                                  4: "resident incremental field"}.get(st.tc_kernel, str(st.tc_kernel)),
                    "autotune": {"tc_kernel": tune.tc_kernel, "tile_replicas": tune.tile_replicas,
                                 "coupling_mem": tune.coupling_mem, "candidates": tune.candidates,
@@ -950,7 +950,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--tile-replicas", type=int, default=0, help="tensor-core replicas per CTA (0 = auto)")
     ap.add_argument("--coupling-mem", type=int, default=0, help="tensor-core: 1 = J in shared, 2 = in tensor memory")
-    ap.add_argument("--tc-kernel", type=int, default=0, help="tensor-core kernel: 1 tcgen05 resident, 2 per-iteration, 3 int8 mma.sync")
+    ap.add_argument("--tc-kernel", type=int, default=0, help="tensor-core kernel: 1 tcgen05 resident, 2 per-iteration, 3 resident warp-level")
     ap.add_argument("--max-inflight", type=int, default=0, help="serving: request slots (0 = the workload's)")
     ap.add_argument("--chunk-iters", type=int, default=0, help="serving: iterations per chunk (0 = the workload's)")
     ap.add_argument("--no-comparator", action="store_true", help="serving: skip the FP32 comparator runs")

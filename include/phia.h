@@ -367,7 +367,9 @@ int phia_run_noalloc(const int8_t *J_k, const int32_t *h_k, int32_t N, int32_t f
  * Many independent instances of uneven N annealed together.  Dense descriptors with
  * N <= 256 run on the resident warp-level kernel, those with N <= 384 and every |k| <= 16 on
  * the resident tcgen05 kernel, over a table of CTAs (8 replicas each): every such instance,
- * all iterations, one launch per size class.  The other instances run on the sparse path
+ * all iterations, one launch per size class.  A batch whose other members are all of at most 512
+ * spins runs those on resident kernels too where that is estimated faster (the results are the
+ * same, each replica's record frozen at its own hit).  The other instances run on the sparse path
  * (larger dense descriptors converted to CSR), in sets whose state fits in L2 together, by
  * default with one launch per iteration and set (replayed as CUDA graphs);
  * phia_opts.tc_kernel = 1 at creation gives one persistent cooperative launch for every
