@@ -185,12 +185,12 @@ cudaError_t pool_alloc(void **ptr, size_t bytes, int device, cudaStream_t st) {
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
             props.location.id = device;
-            cudaDeviceProp dp;
-            cudaError_t e = cudaGetDeviceProperties(&dp, device);
+            size_t free_bytes = 0, total_bytes = 0;
+            cudaError_t e = cudaMemGetInfo(&free_bytes, &total_bytes);
             if (e != cudaSuccess) return e;
             e = cudaMemPoolCreate(&pool, &props);
             if (e != cudaSuccess) return e;
-            uint64_t keep = dp.totalGlobalMem / 16;
+            uint64_t keep = total_bytes / 16;
             e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
             if (e != cudaSuccess) return e;
             g_pools[device] = pool;

@@ -243,7 +243,8 @@ void pack_error(PackedInst &out, int code, const char *fmt, ...) {
 
 // The slices of a checked instance: rows sorted by their number of couplings (descending,
 // ties in row order), 32 to a slice, every row padded to the slice's longest with k = 0.
-void pack_slices(int n, const int32_t *rp, const int32_t *col, const int8_t *val, const int32_t *h, PackedInst &out) {
+void pack_slices(int n, const int32_t *rp, const int32_t *col, const int8_t *val, const int32_t *h, int threads,
+                 PackedInst &out) {
     const int np = round_up(n, 32), ns = np / 32;
     std::vector<int32_t> order((size_t)n);
     for (int i = 0; i < n; ++i) order[(size_t)i] = i;
@@ -262,25 +263,41 @@ void pack_slices(int n, const int32_t *rp, const int32_t *col, const int8_t *val
     out.col.assign((size_t)out.slice[(size_t)ns] * 128, 0);
     out.val.assign((size_t)out.slice[(size_t)ns] * 32, 0u);
     out.hk2.assign((size_t)np * 2, 0);
-    int64_t bound = 0;
-    for (int p = 0; p < n; ++p) {
-        const int i = order[(size_t)p], lane = p & 31;
-        const size_t e0 = (size_t)out.slice[(size_t)p / 32];
-        int64_t mag = 2 * std::abs((int64_t)h[i]);
-        int32_t ksum = 0;
-        for (int32_t c = rp[i]; c < rp[i + 1]; ++c) {
-            const size_t m = (size_t)(c - rp[i]), e = e0 + m / 4;
-            out.col[(e * 32 + (size_t)lane) * 4 + m % 4] = out.pos_of[(size_t)col[c]] * 4;
-            out.val[e * 32 + (size_t)lane] |= (uint32_t)(uint8_t)val[c] << (8 * (m % 4));
-            ksum += val[c];
-            mag += std::abs((int)val[c]);
+    // Whole slices to a host thread: an instance of 1e6 couplings takes several ms on one.
+    std::atomic<int64_t> bound{0};
+    auto fill = [&](int s0, int s1) {
+        int64_t most = 0;
+        for (int p = s0 * 32; p < std::min(n, s1 * 32); ++p) {
+            const int i = order[(size_t)p], lane = p & 31;
+            const size_t e0 = (size_t)out.slice[(size_t)p / 32];
+            int64_t mag = 2 * std::abs((int64_t)h[i]);
+            int32_t ksum = 0;
+            for (int32_t c = rp[i]; c < rp[i + 1]; ++c) {
+                const size_t m = (size_t)(c - rp[i]), e = e0 + m / 4;
+                out.col[(e * 32 + (size_t)lane) * 4 + m % 4] = out.pos_of[(size_t)col[c]] * 4;
+                out.val[e * 32 + (size_t)lane] |= (uint32_t)(uint8_t)val[c] << (8 * (m % 4));
+                ksum += val[c];
+                mag += std::abs((int)val[c]);
+            }
+            out.hk2[(size_t)p * 2] = h[i];
+            out.hk2[(size_t)p * 2 + 1] = h[i] - ksum;
+            most = std::max(most, mag);
         }
-        out.hk2[(size_t)p * 2] = h[i];
-        out.hk2[(size_t)p * 2 + 1] = h[i] - ksum;
-        bound = std::max(bound, mag);
+        for (int64_t b = bound.load(); b < most && !bound.compare_exchange_weak(b, most);) {}
+    };
+    const int nt = std::min<int>({threads, ns, rp[n] / 65536 + 1});
+    std::vector<std::thread> workers;
+    int done = 0;                                  // slices given out, by entries
+    for (int k = 1; k <= nt; ++k) {
+        int next = done;
+        while (next < ns && (k == nt || (int64_t)out.slice[(size_t)next] * nt < (int64_t)out.slice[(size_t)ns] * k)) ++next;
+        if (k < nt) workers.emplace_back(fill, done, next);
+        else fill(done, next);
+        done = next;
     }
+    for (std::thread &w : workers) w.join();
     // |I + h| <= bound: 128 rows' terms and a sum scaled by 2^7 stay in 32 bits up to 2^23.
-    out.wide = bound > ((int64_t)1 << 23);
+    out.wide = bound.load() > ((int64_t)1 << 23);
     if (n > cluster_batch_max_n()) return;
     out.dense.assign((size_t)n * n, 0);
     for (int i = 0; i < n; ++i)
@@ -295,7 +312,7 @@ void pack_slices(int n, const int32_t *rp, const int32_t *col, const int8_t *val
         }
 }
 
-void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
+void pack_instance(const phia_instance_desc &x, int k, int threads, PackedInst &out) {
     const int n = x.N;
     if (n < 1) return pack_error(out, PHIA_EINVAL, "instance %d: N must be >= 1", k);
     if (x.frac_bits < 0 || x.frac_bits > 30) return pack_error(out, PHIA_EINVAL, "instance %d: bad frac_bits", k);
@@ -335,7 +352,7 @@ void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
             }
             rp[i + 1] = (int32_t)col.size();
         }
-        return pack_slices(n, rp.data(), col.data(), val.data(), x.h_k, out);
+        return pack_slices(n, rp.data(), col.data(), val.data(), x.h_k, threads, out);
     }
     if (!x.row_ptr || !x.col || !x.val_k) return pack_error(out, PHIA_EINVAL, "instance %d: CSR arrays missing", k);
     if (x.row_ptr[0] != 0) return pack_error(out, PHIA_EINVAL, "instance %d: row_ptr[0] != 0", k);
@@ -357,7 +374,7 @@ void pack_instance(const phia_instance_desc &x, int k, PackedInst &out) {
                 return pack_error(out, PHIA_EINVAL, "instance %d: CSR is not symmetric at (%d, %d)", k, i, j);
         }
     }
-    pack_slices(n, x.row_ptr, x.col, x.val_k, x.h_k, out);
+    pack_slices(n, x.row_ptr, x.col, x.val_k, x.h_k, threads, out);
 }
 
 int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d, const phia_opts *opts) {
@@ -379,10 +396,11 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
     std::vector<PackedInst> packed((size_t)count);
     {
         std::atomic<int> next{0};
+        const int cores = std::max(1, (int)std::thread::hardware_concurrency());
+        const int nthreads = std::min<int>(count, cores);
         auto work = [&]() {
-            for (int k; (k = next.fetch_add(1)) < count;) pack_instance(d[k], k, packed[(size_t)k]);
+            for (int k; (k = next.fetch_add(1)) < count;) pack_instance(d[k], k, cores / nthreads, packed[(size_t)k]);
         };
-        const int nthreads = std::max(1, std::min<int>(count, (int)std::thread::hardware_concurrency()));
         std::vector<std::thread> workers;
         for (int t = 1; t < nthreads; ++t) workers.emplace_back(work);
         work();
@@ -407,7 +425,11 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
     std::vector<int32_t> slice, col, hk2, row_of, pos_of, hk;
     std::vector<uint32_t> val;
     std::vector<int8_t> dj;
-    slice.reserve(tot_sl); col.reserve(4 * tot_ent); val.reserve(tot_ent); hk2.reserve(2 * tot_pos);
+    if (count > 1) {
+        col.reserve(4 * tot_ent);
+        val.reserve(tot_ent);
+    }
+    slice.reserve(tot_sl); hk2.reserve(2 * tot_pos);
     row_of.reserve(tot_pos); pos_of.reserve(tot_inv); hk.reserve(tot_h); dj.reserve(tot_dj);
     for (int k = 0; k < count; ++k) {
         const phia_instance_desc &x = d[k];
@@ -445,8 +467,13 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         in.inv_off = (int64_t)pos_of.size();
         const int32_t ent0 = (int32_t)(val.size() / 32);
         for (int32_t e : pk.slice) slice.push_back(ent0 + e);
-        col.insert(col.end(), pk.col.begin(), pk.col.end());
-        val.insert(val.end(), pk.val.begin(), pk.val.end());
+        if (count == 1) {
+            col = std::move(pk.col);
+            val = std::move(pk.val);
+        } else {
+            col.insert(col.end(), pk.col.begin(), pk.col.end());
+            val.insert(val.end(), pk.val.begin(), pk.val.end());
+        }
         hk2.insert(hk2.end(), pk.hk2.begin(), pk.hk2.end());
         row_of.insert(row_of.end(), pk.row_of.begin(), pk.row_of.end());
         pos_of.insert(pos_of.end(), pk.pos_of.begin(), pk.pos_of.end());
