@@ -165,8 +165,8 @@ struct phia_s {
 // Device buffers of handles, batches and server requests come from one stream-ordered memory
 // pool per device.  Creating and destroying them in a loop, as a caller with a new instance per
 // request does, then costs neither cudaMalloc round trips nor the device-wide synchronisation
-// of cudaFree, which waits for the other requests' kernels; freed blocks beyond 1/16 of the
-// device's memory go back at the next synchronisation.
+// of cudaFree, which waits for the other requests' kernels; freed blocks beyond 16 GiB
+// go back at the next synchronisation.
 namespace {
 std::mutex g_pool_mu;
 std::map<int, cudaMemPool_t> g_pools;
@@ -185,12 +185,9 @@ cudaError_t pool_alloc(void **ptr, size_t bytes, int device, cudaStream_t st) {
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
             props.location.id = device;
-            size_t free_bytes = 0, total_bytes = 0;
-            cudaError_t e = cudaMemGetInfo(&free_bytes, &total_bytes);
+            cudaError_t e = cudaMemPoolCreate(&pool, &props);
             if (e != cudaSuccess) return e;
-            e = cudaMemPoolCreate(&pool, &props);
-            if (e != cudaSuccess) return e;
-            uint64_t keep = total_bytes / 16;
+            uint64_t keep = (uint64_t)16 << 30;
             e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
             if (e != cudaSuccess) return e;
             g_pools[device] = pool;
