@@ -43,7 +43,7 @@ struct phia_batch_s {
     std::vector<SmallCta> small_host;
     std::vector<int64_t> bits_pub;      // per public instance: offset of its best states
     std::vector<long long> targets;     // per instance, LLONG_MIN = none
-    std::vector<CsrBlock> blocks;       // the block lists for 1, 2, 4 and 8 slices a block
+    std::vector<CsrBlock> blocks;       // the block lists for 1, 2, 4 and 8 slices a block, in instance order
     std::vector<int32_t> first_block[4];   // per CSR member (and one past): its first block in each list
     std::vector<CsrSet> sets;           // instances whose state fits in L2 together, for sets_R replicas
     int sets_R = 0;
@@ -148,7 +148,9 @@ void layout(phia_batch_s *b, int R) {
 }
 
 // Sets of consecutive CSR members for R replicas: as few as keep a set's x and v within 0.4 of L2,
-// of about equal size.
+// of about equal size.  The device gets a copy of the block lists with each set's blocks sorted: the
+// host's stay in instance order, which first_block counts on when another replica count cuts the
+// members into other sets.
 int make_sets(phia_batch_s *b, int R) {
     int l2 = 0;
     BCU(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, b->device));
@@ -157,8 +159,10 @@ int make_sets(phia_batch_s *b, int R) {
     for (const CsrInst &in : b->inst) total += (int64_t)in.Np * R * 8;
     const int64_t budget = std::max<int64_t>(1, (int64_t)(0.4 * l2));
     const int64_t share = total / std::max<int64_t>(1, (total + budget - 1) / budget) + 1;
+    b->sets_R = 0;
     b->sets.clear();
     std::fill(b->set_max, b->set_max + 4, 0);
+    std::vector<CsrBlock> blocks = b->blocks;
     int64_t seen = 0;
     for (int c0 = 0, c = 0; c < n; ++c) {
         seen += (int64_t)b->inst[(size_t)c].Np * R * 8;
@@ -171,12 +175,12 @@ int make_sets(phia_batch_s *b, int R) {
         }
         // the heaviest blocks first
         for (int l = 0; l < 4; ++l)
-            std::stable_sort(b->blocks.begin() + s.off[l], b->blocks.begin() + s.off[l] + s.len[l],
+            std::stable_sort(blocks.begin() + s.off[l], blocks.begin() + s.off[l] + s.len[l],
                              [&](const CsrBlock &x, const CsrBlock &y) { return x.work > y.work; });
         b->sets.push_back(s);
         c0 = c + 1;
     }
-    BCU(cudaMemcpyAsync(b->d_blocks, b->blocks.data(), b->blocks.size() * sizeof(CsrBlock), cudaMemcpyHostToDevice, b->stream));
+    BCU(cudaMemcpyAsync(b->d_blocks, blocks.data(), blocks.size() * sizeof(CsrBlock), cudaMemcpyHostToDevice, b->stream));
     BCU(cudaMemcpyAsync(b->d_sets, b->sets.data(), b->sets.size() * sizeof(CsrSet), cudaMemcpyHostToDevice, b->stream));
     BCU(cudaStreamSynchronize(b->stream));
     b->sets_R = R;

@@ -1,0 +1,37 @@
+"""GPU tests of one batch used several times: what a run leaves behind (the cut into sets, tables,
+times) must not reach the next one."""
+import numpy as np
+import pytest
+
+from paper_2407_10205_gb300 import instances as ins
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _records(B, count, R):
+    return [B.replica_results(k, R) for k in range(count)]
+
+
+@pytest.mark.parametrize("mode", [1, 2])
+def test_replica_counts_may_change_between_runs(gpu_lib, mode):
+    """8 bytes of state per spin and replica: 64 replicas are one set of instances, 1024 and 2048
+    several, cut at other places.  Sizes and densities go up and down, so that the heaviest blocks of
+    a set come from all of its members."""
+    phia = gpu_lib
+    g = np.random.default_rng(7)
+    insts = [ins.erdos_renyi(int(n), float(d), 127, 31, 4, seed=k)
+             for k, (n, d) in enumerate(zip(g.integers(200, 2500, 14), g.uniform(0.004, 0.05, 14)))]
+    sched = phia.schedule(0.01, 0.2, 0.1, 2.0, refresh=5)
+    counts, T = (64, 2048, 64, 1024), 12
+    fresh = {}
+    for R in set(counts):
+        with phia.Batch(insts, csr_mode=mode) as B:
+            B.anneal(sched, R, T, seed=9)
+            fresh[R] = _records(B, len(insts), R)
+    with phia.Batch(insts, csr_mode=mode) as B:
+        for R in counts:
+            B.anneal(sched, R, T, seed=9)
+            for a, b in zip(_records(B, len(insts), R), fresh[R]):
+                for u, w in zip(a, b):
+                    assert np.array_equal(u, w)
