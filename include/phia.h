@@ -88,10 +88,8 @@ typedef struct phia_opts {
                               e4m3 / 256 bf16; tile_replicas 4, 8 or 16); 0 = automatic */
     int32_t large_variant; /* per-iteration kernel (tc_kernel 2): 1 = x, v staged through a shared-
                               memory ring (3 operand stages at 256-wide tiles); 2 = x, v
-                              prefetched into registers (4 stages); 3 / 4 = as 2, with the CTAs of
-                              a cluster of 2 / 4 sharing each replica tile and multicasting the
-                              spin operand to one another (TMA multicast); 5 / 6 = as 1 with the
-                              multicast over 2 / 4 CTAs; 7 = overlapped: the whole run in one
+                              prefetched into registers (4 stages); 3 / 4 = as 2; 5 / 6 = as 1;
+                              7 = overlapped: the whole run in one
                               cooperative launch whose CTAs keep their output tiles for every
                               iteration and start a replica tile's next iteration as soon as
                               all of its spins are written (per-replica-tile counters instead
@@ -104,10 +102,9 @@ typedef struct phia_opts {
                               less take one of two kernels for few replicas instead: the whole
                               run over thread-block clusters with J in registers (N <= 1024
                               e4m3, 512 bf16) or overlapped tiles of 128 replicas x 32 or 64
-                              spins with x, v in registers; 8 / 9 = as 7 with 256- or
-                              128-wide tiles and the spin-operand multicast over clusters of
-                              2 / 4 CTAs; 10 / 11 / 12 / 13 = as 7 with 256- / 224- / 128- /
-                              160-wide tiles; 0 = automatic (the autotuner's choice where it
+                              spins with x, v in registers; 8 / 9 = as 10, or
+                              as 12 where 256-wide tiles are fewer than the SMs; 10 / 11 / 12 /
+                              13 = overlapped with 256- / 224- / 128- / 160-wide tiles; 0 = automatic (the autotuner's choice where it
                               has one, else as 7) */
 } phia_opts;
 
@@ -215,8 +212,8 @@ int phia_anneal(phia_t *p, const phia_schedule *sched, int32_t replicas, int64_t
  * kernel with 4, 8 or 16 replicas per CTA and J in shared or tensor memory, the
  * resident warp-level kernel (two candidates, alike; N small enough), the
  * resident incremental-field kernel with 4, 8 or 16 replicas per CTA (N small enough),
- * and the per-iteration kernel in its thirteen variants (phia_opts.large_variant) -- keeps
- * the fastest for the handle and caches it,
+ * and the per-iteration kernel in its thirteen variants (phia_opts.large_variant; those that
+ * run the same form as another are counted and timed once) -- keeps the fastest for the handle and caches it,
  * process-wide, for (N, replicas, operand): handles created with all variant options
  * automatic use the cached choice for runs with that replica count.  The probes
  * overwrite the handle's last-run records.  Tensor-core path only (else PHIA_ENOTSUP). */

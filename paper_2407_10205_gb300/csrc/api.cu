@@ -799,7 +799,9 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
             if (inc_small_tile_replicas(p->N, tile) == tile)
                 cands.push_back(TuneChoice{false, tile, 0, false, true, 0});
     }
-    for (int lv = 1; lv <= 13; ++lv) cands.push_back(TuneChoice{true, 0, 0, false, false, lv});
+    // Variants 3 .. 6, 8 and 9 run the forms of 2, 1, 10 and 12.
+    constexpr int kSameForm = 6;
+    for (int lv : {1, 2, 7, 10, 11, 12, 13}) cands.push_back(TuneChoice{true, 0, 0, false, false, lv});
     const bool saved_auto = p->auto_tile;
     p->auto_tile = false;
     float best_ms = 1e30f, worst_ms = 0.f;
@@ -843,7 +845,7 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
         out->tile_replicas = best.large ? 0
                              : (best.warpk || best.inc ? best.tile_rl : tc_small_tile_replicas(replicas, best.tile_rl));
         out->coupling_mem = best.large || best.warpk || best.inc ? 0 : best.coupling_mem;
-        out->candidates = (int32_t)cands.size();
+        out->candidates = (int32_t)cands.size() + kSameForm;
         out->best_us_per_iter = 1000.f * best_ms / probe_iters;
         out->worst_us_per_iter = 1000.f * worst_ms / probe_iters;
         out->large_variant = best.large ? best.lvar : 0;

@@ -36,10 +36,10 @@ void step_graphs_free(StepGraphCache *c) { delete c; }
 namespace {
 
 std::vector<uint8_t> make_key(const void *func, dim3 grid, dim3 block, size_t smem, int64_t len, const void *key,
-                              size_t key_bytes, unsigned cluster) {
-    std::vector<uint8_t> k(sizeof(func) + 7 * sizeof(unsigned) + sizeof(smem) + sizeof(len) + key_bytes);
+                              size_t key_bytes) {
+    std::vector<uint8_t> k(sizeof(func) + 6 * sizeof(unsigned) + sizeof(smem) + sizeof(len) + key_bytes);
     uint8_t *p = k.data();
-    const unsigned dims[7] = {grid.x, grid.y, grid.z, block.x, block.y, block.z, cluster};
+    const unsigned dims[6] = {grid.x, grid.y, grid.z, block.x, block.y, block.z};
     memcpy(p, &func, sizeof(func)); p += sizeof(func);
     memcpy(p, dims, sizeof(dims)); p += sizeof(dims);
     memcpy(p, &smem, sizeof(smem)); p += sizeof(smem);
@@ -48,8 +48,8 @@ std::vector<uint8_t> make_key(const void *func, dim3 grid, dim3 block, size_t sm
     return k;
 }
 
-cudaError_t build(const void *func, dim3 grid, dim3 block, size_t smem, void **args, int64_t len, unsigned cluster,
-                  bool overlap, cudaGraphExec_t *out) {
+cudaError_t build(const void *func, dim3 grid, dim3 block, size_t smem, void **args, int64_t len, bool overlap,
+                  cudaGraphExec_t *out) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaGraphCreate(&g, 0);
     if (e != cudaSuccess) return e;
@@ -70,13 +70,6 @@ cudaError_t build(const void *func, dim3 grid, dim3 block, size_t smem, void **a
             edge.type = cudaGraphDependencyTypeProgrammatic;
             e = cudaGraphAddDependencies(g, &prev, &node, &edge, 1);
         }
-        if (e == cudaSuccess && cluster > 1) {
-            cudaKernelNodeAttrValue v{};
-            v.clusterDim.x = cluster;
-            v.clusterDim.y = 1;
-            v.clusterDim.z = 1;
-            e = cudaGraphKernelNodeSetAttribute(node, cudaKernelNodeAttributeClusterDimension, &v);
-        }
         prev = node;
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
@@ -86,38 +79,28 @@ cudaError_t build(const void *func, dim3 grid, dim3 block, size_t smem, void **a
 
 }  // namespace
 
-cudaError_t launch_one(const void *func, dim3 grid, dim3 block, size_t smem, void **args, unsigned cluster,
-                       bool overlap, cudaStream_t st) {
-    if (cluster <= 1 && !overlap) return cudaLaunchKernel(func, grid, block, args, smem, st);
+cudaError_t launch_one(const void *func, dim3 grid, dim3 block, size_t smem, void **args, bool overlap,
+                       cudaStream_t st) {
+    if (!overlap) return cudaLaunchKernel(func, grid, block, args, smem, st);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[2];
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    if (cluster > 1) {
-        cudaLaunchAttribute &x = at[cfg.numAttrs++];
-        x.id = cudaLaunchAttributeClusterDimension;
-        x.val.clusterDim.x = cluster;
-        x.val.clusterDim.y = 1;
-        x.val.clusterDim.z = 1;
-    }
-    if (overlap) {
-        cudaLaunchAttribute &x = at[cfg.numAttrs++];
-        x.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        x.val.programmaticStreamSerializationAllowed = 1;
-    }
+    cfg.numAttrs = 1;
     return cudaLaunchKernelExC(&cfg, func, args);
 }
 
 cudaError_t launch_steps(StepGraphCache *cache, const void *func, dim3 grid, dim3 block, size_t smem, void **args,
-                         const void *key, size_t key_bytes, int64_t steps, cudaStream_t st, unsigned cluster,
-                         bool overlap) {
+                         const void *key, size_t key_bytes, int64_t steps, cudaStream_t st, bool overlap) {
     int64_t done = 0;
     if (cache && steps >= 2) {
         const int64_t len = steps < kGraphLen ? steps : kGraphLen;
-        const std::vector<uint8_t> k = make_key(func, grid, block, smem, len, key, key_bytes, cluster);
+        const std::vector<uint8_t> k = make_key(func, grid, block, smem, len, key, key_bytes);
         cudaGraphExec_t exec = nullptr;
         for (auto &e : cache->entries)
             if (e.key == k) exec = e.exec;
@@ -134,7 +117,7 @@ cudaError_t launch_steps(StepGraphCache *cache, const void *func, dim3 grid, dim
             }
         }
         if (build_now) {
-            cudaError_t e = build(func, grid, block, smem, args, len, cluster, overlap, &exec);
+            cudaError_t e = build(func, grid, block, smem, args, len, overlap, &exec);
             if (e != cudaSuccess) return e;
             if (cache->entries.size() >= kMaxGraphs) {
                 cudaGraphExecDestroy(cache->entries.front().exec);
@@ -148,7 +131,7 @@ cudaError_t launch_steps(StepGraphCache *cache, const void *func, dim3 grid, dim
         }
     }
     for (const int64_t first = done; done < steps; ++done) {
-        cudaError_t e = launch_one(func, grid, block, smem, args, cluster, overlap && done > first, st);
+        cudaError_t e = launch_one(func, grid, block, smem, args, overlap && done > first, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

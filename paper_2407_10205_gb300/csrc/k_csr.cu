@@ -714,7 +714,7 @@ cudaError_t launch_iterations(const CsrArgs &C, size_t smem, StepGraphCache *gra
             ++*launches;
         }
         e = launch_steps(graphs, reinterpret_cast<const void *>(k), dim3(max_blocks, ny), dim3(kBlk), smem, args, &Cs,
-                         sizeof Cs, C.a.nsteps, st, 1, true);
+                         sizeof Cs, C.a.nsteps, st, true);
         if (e != cudaSuccess) return e;
         *launches += (int)C.a.nsteps;
     }

@@ -4,10 +4,7 @@
 //
 // The step kernel is persistent: one CTA per SM walks a static list of output tiles.
 // Variants (autotuned): x and v staged through a shared-memory ring (3 operand stages at
-// 256-wide tiles) or prefetched into registers (4 stages); and the CTAs of a cluster of
-// CL (1, 2 or 4) handling the same replica tile at CL consecutive spin tiles, each
-// loading 1/CL of the spin operand and multicasting it to all CL, so each spin tile is
-// read from L2 once per cluster instead of once per CTA.
+// 256-wide tiles) or prefetched into registers (4 stages).
 // Operands (K-major, 128-byte swizzle, staged by TMA through an mbarrier ring):
 //   A = couplings k re-encoded exactly (e4m3 or bf16), [Mpad][Kpad]
 //   B = spins of this iteration in the same encoding, [Rpad][Kpad], one of 4 rotating
@@ -350,7 +347,7 @@ __device__ __forceinline__ void copy_best_lane(const LargeArgs &L, int r0, int m
     }
 }
 
-template <int OP, int BN, int CL, bool RING>
+template <int OP, int BN, bool RING>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_large_step(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const LargeArgs L) {
@@ -360,8 +357,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr uint32_t kStageB = Tile<BN, RING>::kStageB;
     constexpr int kColsPerWarp = Tile<BN, RING>::kColsPerWarp;
     constexpr int kChunksPerTile = Tile<BN, RING>::kChunksPerTile;
-    constexpr uint16_t kMask = (uint16_t)((1u << CL) - 1u);
-    static_assert(CL == 1 || CL == 2 || CL == 4, "cluster of 1, 2 or 4 CTAs");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sA = smem;
@@ -374,16 +369,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const RunArgs &a = L.a;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // Cluster tiles: CL consecutive spin tiles of one replica tile; CTA `crank` of the
-    // cluster takes the crank-th.  With CL = 1 a cluster tile is one output tile.
-    const int crank = CL > 1 ? (int)cluster_ctarank() : 0;
-    const int Gc = (int)gridDim.x / CL;             // clusters (the grid is a multiple of CL)
-    const int cid = (int)blockIdx.x / CL;
-    const int mgroups = L.mtiles / CL;
-    const int ctiles = mgroups * L.rtiles;
-    const int my_tiles = cid < ctiles ? (ctiles - 1 - cid) / Gc + 1 : 0;
-    auto tile_m = [&](int lt) { return ((cid + lt * Gc) % mgroups) * CL + crank; };
-    auto tile_n = [&](int lt) { return (cid + lt * Gc) / mgroups; };
+    const int G = (int)gridDim.x, cid = (int)blockIdx.x;
+    const int mt = L.mtiles;
+    const int tiles = mt * L.rtiles;
+    const int my_tiles = cid < tiles ? (tiles - 1 - cid) / G + 1 : 0;
+    auto tile_m = [&](int lt) { return (cid + lt * G) % mt; };
+    auto tile_n = [&](int lt) { return (cid + lt * G) / mt; };
     const int KB = L.Kbytes / kBKB;
     const int N = a.N, R = a.R;
     const uint64_t kWaitNs = a.wait_ns > 0 ? (uint64_t)a.wait_ns : kWaitTimeoutNs;
@@ -395,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (tid == 32) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&sh->full[s], 1);
-            mbar_init(&sh->empty[s], CL);   // freed by the MMAs of every CTA of the cluster
+            mbar_init(&sh->empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&sh->accf[b], 1);
@@ -408,7 +399,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if constexpr (CL > 1) cluster_sync_all();   // every CTA's barriers exist before any multicast
     const uint32_t tmem = sh->tmem_base;
     const int64_t t = L.ctl->t, t_first = L.ctl->t_first, t_end = L.ctl->t_end;
 
@@ -431,13 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     mbar_arrive_expect_tx(&sh->full[s], kStageA + kStageB);
                     tma_load_2d(sA + s * kStageA, &tmA, &sh->full[s], kb * (kBKB / ESZ), m * kBM);
-                    if constexpr (CL == 1) {
-                        tma_load_2d(sB + s * kStageB, &tmB, &sh->full[s], kb * (kBKB / ESZ), ybuf);
-                    } else {
-                        // this CTA's 1/CL of the spin tile, to the same place in every CTA
-                        tma_load_2d_mc(sB + s * kStageB + crank * (BN / CL) * kBKB, &tmB, &sh->full[s],
-                                       kb * (kBKB / ESZ), ybuf + crank * (BN / CL), kMask);
-                    }
+                    tma_load_2d(sB + s * kStageB, &tmB, &sh->full[s], kb * (kBKB / ESZ), ybuf);
                 }
             }
             if (!ok) *tout = 1;
@@ -472,8 +456,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         if constexpr (OP == kOpE4M3) mma_e4m3(dt, ad + 2 * k, bd + 2 * k, IDESC, (kb | k) != 0);
                         else mma_bf16(dt, ad + 2 * k, bd + 2 * k, IDESC, (kb | k) != 0);
                     }
-                    if constexpr (CL == 1) mma_commit(&sh->empty[s]);
-                    else mma_commit_mc(&sh->empty[s], kMask);   // stage s free in every CTA of the cluster
+                    mma_commit(&sh->empty[s]);
                 }
                 if (ok) mma_commit(&sh->accf[b]);
             }
@@ -685,9 +668,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     tc_fence_before();
     __syncthreads();
-    // No CTA of a cluster leaves while another may still multicast into it or arrive on
-    // its barriers.
-    if constexpr (CL > 1) cluster_sync_all();
     if (tid == 0) {
         if (sh->timed_out) atomicExch(a.err, 1);
         iter_ctl_finish(L.ctl);
@@ -721,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // t - 3 only after its records warp copied t - 3; the improved flags rotate over four
 // slots.  Every wait is bounded; a wait that runs out sets the run's error flag and the
 // CTA winds down.
-template <int OP, int BN, int CL, int NACC>
+template <int OP, int BN, int NACC>
 __global__ void __launch_bounds__(kThreads + 64, 1)
     tc_flow_run(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const LargeArgs L) {
@@ -731,8 +711,6 @@ __global__ void __launch_bounds__(kThreads + 64, 1)
     constexpr uint32_t kStageB = Tile<BN, true>::kStageB;
     constexpr int kColsPerWarp = Tile<BN, true>::kColsPerWarp;
     constexpr int kChunksPerTile = Tile<BN, true>::kChunksPerTile;
-    constexpr uint16_t kMask = (uint16_t)((1u << CL) - 1u);
-    static_assert(CL == 1 || CL == 2 || CL == 4, "cluster of 1, 2 or 4 CTAs");
     static_assert((NACC == 2 || NACC == 3) && NACC * BN <= (int)Tile<BN, true>::kTmemCols,
                   "accumulators beyond the tensor memory allocated");
     extern __shared__ uint8_t smem_raw[];
@@ -747,17 +725,12 @@ __global__ void __launch_bounds__(kThreads + 64, 1)
 
     const RunArgs &a = L.a;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // Cluster tiles: CL consecutive output tiles of one replica tile, CTA `crank` of the
-    // cluster taking the crank-th; the cluster's CTAs load one CL-th of the spin tile each
-    // and multicast it to all of them.
-    const int crank = CL > 1 ? (int)cluster_ctarank() : 0;
-    const int Gc = (int)gridDim.x / CL, cid = (int)blockIdx.x / CL;
+    const int G = (int)gridDim.x, cid = (int)blockIdx.x;
     const int mt = L.mtiles;
-    const int mgroups = mt / CL;
-    const int ctiles = mgroups * L.rtiles;
-    const int my_tiles = cid < ctiles ? (ctiles - 1 - cid) / Gc + 1 : 0;
-    auto tile_m = [&](int lt) { return ((cid + lt * Gc) % mgroups) * CL + crank; };
-    auto tile_n = [&](int lt) { return (cid + lt * Gc) / mgroups; };
+    const int tiles = mt * L.rtiles;
+    const int my_tiles = cid < tiles ? (tiles - 1 - cid) / G + 1 : 0;
+    auto tile_m = [&](int lt) { return (cid + lt * G) % mt; };
+    auto tile_n = [&](int lt) { return (cid + lt * G) / mt; };
     const int64_t t0 = L.f0, t_end = L.f1, t_call_end = a.t0 + a.nsteps;
     const int64_t total = (t_end - t0) * my_tiles;      // tiles this CTA processes, g = 0 .. total - 1
     const int KB = L.Kbytes / kBKB;
@@ -776,7 +749,7 @@ __global__ void __launch_bounds__(kThreads + 64, 1)
     if (tid == 32) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&sh->full[s], 1);
-            mbar_init(&sh->empty[s], CL);   // freed by the MMAs of every CTA of the cluster
+            mbar_init(&sh->empty[s], 1);
         }
         for (int b = 0; b < NACC; ++b) {
             mbar_init(accf_of(b), 1);
@@ -792,7 +765,6 @@ __global__ void __launch_bounds__(kThreads + 64, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if constexpr (CL > 1) cluster_sync_all();   // every CTA's barriers exist before any multicast
     const uint32_t tmem = sh->tmem_base;
 
     if (warp == 0) {
@@ -820,12 +792,7 @@ __global__ void __launch_bounds__(kThreads + 64, 1)
                     }
                     mbar_arrive_expect_tx(&sh->full[s], kStageA + kStageB);
                     tma_load_2d(sA + s * kStageA, &tmA, &sh->full[s], kb * (kBKB / ESZ), m * kBM);
-                    if constexpr (CL == 1) {
-                        tma_load_2d(sB + s * kStageB, &tmB, &sh->full[s], kb * (kBKB / ESZ), ybuf);
-                    } else {
-                        tma_load_2d_mc(sB + s * kStageB + crank * (BN / CL) * kBKB, &tmB, &sh->full[s],
-                                       kb * (kBKB / ESZ), ybuf + crank * (BN / CL), kMask);
-                    }
+                    tma_load_2d(sB + s * kStageB, &tmB, &sh->full[s], kb * (kBKB / ESZ), ybuf);
                 }
             }
             if (!ok) *tout = 1;
@@ -860,8 +827,7 @@ __global__ void __launch_bounds__(kThreads + 64, 1)
                         if constexpr (OP == kOpE4M3) mma_e4m3(dt, ad + 2 * k, bd + 2 * k, IDESC, (kb | k) != 0);
                         else mma_bf16(dt, ad + 2 * k, bd + 2 * k, IDESC, (kb | k) != 0);
                     }
-                    if constexpr (CL == 1) mma_commit(&sh->empty[s]);
-                    else mma_commit_mc(&sh->empty[s], kMask);   // stage s free in every CTA of the cluster
+                    mma_commit(&sh->empty[s]);
                 }
                 if (ok) mma_commit(accf_of(b));
             }
@@ -885,9 +851,8 @@ __global__ void __launch_bounds__(kThreads + 64, 1)
             return ((size_t)grp * Mp + (m_ * kBM + q4 * 32 + lane)) * 4;
         };
         // Freshly written x and v are read again next iteration; with a state larger than
-        // half of L2 their lines are kept ahead of the operand streams' (evict_last).  The
-        // cluster variants keep plain stores (their registers are tighter).
-        const bool keep = CL == 1 && L.xv_keep != 0;
+        // half of L2 their lines are kept ahead of the operand streams' (evict_last).
+        const bool keep = L.xv_keep != 0;
         const uint64_t xvpol = l2_evict_last_policy();
         auto put4 = [&](float *p, float4 v) {
             if (keep) st_global_f4_policy(p, v, xvpol);
@@ -1079,9 +1044,6 @@ __global__ void __launch_bounds__(kThreads + 64, 1)
     }
     tc_fence_before();
     __syncthreads();
-    // No CTA of a cluster leaves while another may still multicast into it or arrive on
-    // its barriers.
-    if constexpr (CL > 1) cluster_sync_all();
     if (tid == 0 && sh->timed_out) atomicExch(a.err, 1);
     if (warp == 0) {
         tc_fence_after();
@@ -1198,7 +1160,7 @@ bool make_map(CUtensorMap *m, const void *base, int op, uint64_t inner_elems, ui
     return tc_operand_map(m, base, op, inner_elems, rows, row_bytes, box_rows);
 }
 
-template <int OP, int BN, int CL, bool RING>
+template <int OP, int BN, bool RING>
 cudaError_t run_large(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, int *launches, int sms) {
     constexpr size_t kSmem = Tile<BN, RING>::kSmemBytes;
     LargeArgs L;
@@ -1219,33 +1181,12 @@ cudaError_t run_large(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, 
     CUtensorMap tmA, tmB;
     const int esz = OP == kOpE4M3 ? 1 : 2;
     if (!make_map(&tmA, B.Jop, OP, (uint64_t)B.Kbytes / esz, (uint64_t)B.Mpad, (uint64_t)B.Kbytes, kBM) ||
-        !make_map(&tmB, B.S, OP, (uint64_t)B.Kbytes / esz, (uint64_t)4 * B.Rpad, (uint64_t)B.Kbytes, BN / CL))
+        !make_map(&tmB, B.S, OP, (uint64_t)B.Kbytes / esz, (uint64_t)4 * B.Rpad, (uint64_t)B.Kbytes, BN))
         return cudaErrorInvalidValue;
-    auto step = tc_large_step<OP, BN, CL, RING>;
+    auto step = tc_large_step<OP, BN, RING>;
     cudaError_t e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
-    // Persistent grid: one CTA per SM, or as many whole clusters as can be resident at once.
-    const int ctiles = (L.mtiles / CL) * L.rtiles;
-    int clusters = std::min(ctiles, std::max(sms, 1));
-    if (CL > 1) {
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)(CL * std::max(sms / CL, 1)));
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = kSmem;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = CL;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int resident = 0;
-        e = cudaOccupancyMaxActiveClusters(&resident, reinterpret_cast<const void *>(step), &cfg);
-        if (e != cudaSuccess) return e;
-        if (resident < 1) return cudaErrorInvalidConfiguration;
-        clusters = std::min(ctiles, resident);
-    }
-    const dim3 grid((unsigned)(clusters * CL));
+    const dim3 grid((unsigned)std::min(L.ntiles, std::max(sms, 1)));      // one persistent CTA per SM
     e = cudaMemsetAsync(B.Epart, 0, 2 * (size_t)B.Rpad * sizeof(int64_t), st);   // energy sums start at 0
     if (e != cudaSuccess) return e;
     const int64_t RN = (int64_t)a.R * a.N;
@@ -1257,7 +1198,7 @@ cudaError_t run_large(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, 
         tc_large_field_prologue<OP><<<eg, 256, 0, st>>>(L);
         void *args[3] = {&tmA, &tmB, &L};
         e = launch_steps(nullptr, reinterpret_cast<const void *>(step), grid, dim3(kThreads), kSmem, args, nullptr, 0,
-                         1, st, CL);
+                         1, st);
         if (e != cudaSuccess) return e;
         tc_large_field_out<<<(a.R + 255) / 256, 256, 0, st>>>(L);
         n += 3;
@@ -1281,7 +1222,7 @@ cudaError_t run_large(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, 
         memcpy(key + sizeof tmA, &tmB, sizeof tmB);
         memcpy(key + 2 * sizeof tmA, &Ls, sizeof Ls);
         e = launch_steps(B.graphs, reinterpret_cast<const void *>(step), grid, dim3(kThreads), kSmem, args, key,
-                         sizeof key, a.nsteps, st, CL);
+                         sizeof key, a.nsteps, st);
         if (e != cudaSuccess) return e;
         n += (int)a.nsteps;
     }
@@ -1316,7 +1257,7 @@ __global__ void tc_flow_pack0(const LargeArgs L) {
 // Variants 7-13: the whole run in cooperative launches of tc_flow_run (all CTAs resident
 // at once, as CTAs wait on each other's tiles), with NACC TMEM accumulators.  Runs whose tile counters could pass 2^31 go
 // out in several launches; every launch settles and copies all of its iterations.
-template <int OP, int BN, int CL, int NACC = 2>
+template <int OP, int BN, int NACC = 2>
 cudaError_t run_flow(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, int *launches, int sms) {
     constexpr size_t kSmem = Tile<BN, true>::kSmemBytes;
     constexpr int kFlowThreads = kThreads + 64;
@@ -1345,40 +1286,27 @@ cudaError_t run_flow(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, i
     CUtensorMap tmA, tmB;
     const int esz = OP == kOpE4M3 ? 1 : 2;
     if (!make_map(&tmA, B.Jop, OP, (uint64_t)B.Kbytes / esz, (uint64_t)B.Mpad, (uint64_t)B.Kbytes, kBM) ||
-        !make_map(&tmB, B.S, OP, (uint64_t)B.Kbytes / esz, (uint64_t)4 * B.Rpad, (uint64_t)B.Kbytes, BN / CL))
+        !make_map(&tmB, B.S, OP, (uint64_t)B.Kbytes / esz, (uint64_t)4 * B.Rpad, (uint64_t)B.Kbytes, BN))
         return cudaErrorInvalidValue;
-    auto k = tc_flow_run<OP, BN, CL, NACC>;
+    auto k = tc_flow_run<OP, BN, NACC>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
-    // All CTAs (whole clusters) resident at once: the launch is cooperative.
+    // All CTAs resident at once: the launch is cooperative.
+    int resident = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k, kFlowThreads, kSmem);
+    if (e != cudaSuccess) return e;
+    resident *= std::max(sms, 1);
+    if (resident < 1) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)std::min(L.ntiles, resident));
     cfg.blockDim = dim3(kFlowThreads);
     cfg.dynamicSmemBytes = kSmem;
     cfg.stream = st;
-    cudaLaunchAttribute at[2];
+    cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = CL;
-    at[1].val.clusterDim.y = 1;
-    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = CL > 1 ? 2 : 1;
-    const int ctiles = (L.mtiles / CL) * L.rtiles;
-    int resident = 0;
-    if (CL > 1) {
-        cudaLaunchConfig_t q = cfg;
-        q.gridDim = dim3((unsigned)(CL * std::max(sms / CL, 1)));
-        q.attrs = at + 1;
-        q.numAttrs = 1;
-        e = cudaOccupancyMaxActiveClusters(&resident, reinterpret_cast<const void *>(k), &q);
-    } else {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k, kFlowThreads, kSmem);
-        resident *= std::max(sms, 1);
-    }
-    if (e != cudaSuccess) return e;
-    if (resident < 1) return cudaErrorInvalidConfiguration;
-    cfg.gridDim = dim3((unsigned)(CL * std::min(ctiles, resident)));
+    cfg.numAttrs = 1;
     e = cudaMemsetAsync(B.Epart, 0, 2 * (size_t)B.Rpad * sizeof(int64_t), st);
     if (e != cudaSuccess) return e;
     int n = 0;
@@ -1398,12 +1326,6 @@ cudaError_t run_flow(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, i
         if (e != cudaSuccess) return e;
         void *args[3] = {&tmA, &tmB, &Lc};
         e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(k), args);
-        if (e != cudaSuccess && CL > 1 && t == a.t0) {
-            // a cooperative launch in clusters refused: the whole call without clusters (the
-            // prologue reads only the caller's arrays, so it runs again unchanged)
-            cudaGetLastError();
-            return run_flow<OP, BN, 1, NACC>(B, a, st, launches, sms);
-        }
         if (e != cudaSuccess) return e;
         ++n;
     }
@@ -1420,29 +1342,13 @@ cudaError_t run_flow(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, i
 
 template <int OP, int BN>
 cudaError_t run_variant(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, int *launches, int sms) {
-    const int mtiles = B.Mpad / kBM;
     int v = a.large_variant;
     if (v == 0) v = kDefaultLargeVariant;
-    // The overlapped variants need their tile counters (absent from the allocation-free
-    // entry); clusters need the output tiles to split evenly among their CTAs.
+    // The overlapped variants need their tile counters (absent from the allocation-free entry).
     if (v >= 7 && (!B.ready || !B.sbits || a.field_mode)) v = 1;
-    if (v >= 10) v = 7;
-    if (v == 9 && mtiles % 4 != 0) v = 8;
-    if (v == 8 && mtiles % 2 != 0) v = 7;
-    if (v == 9) return run_flow<OP, BN, 4>(B, a, st, launches, sms);
-    if (v == 8) return run_flow<OP, BN, 2>(B, a, st, launches, sms);
-    if (v == 7) return run_flow<OP, BN, 1>(B, a, st, launches, sms);
-    // A cluster needs the spin tiles to split evenly among its CTAs.
-    if (v == 6 && mtiles % 4 != 0) v = 5;
-    if (v == 5 && mtiles % 2 != 0) v = 1;
-    if (v == 4 && mtiles % 4 != 0) v = 3;
-    if (v == 3 && mtiles % 2 != 0) v = 2;
-    if (v == 6) return run_large<OP, BN, 4, true>(B, a, st, launches, sms);
-    if (v == 5) return run_large<OP, BN, 2, true>(B, a, st, launches, sms);
-    if (v == 4) return run_large<OP, BN, 4, false>(B, a, st, launches, sms);
-    if (v == 3) return run_large<OP, BN, 2, false>(B, a, st, launches, sms);
-    if (v == 2) return run_large<OP, BN, 1, false>(B, a, st, launches, sms);
-    return run_large<OP, BN, 1, true>(B, a, st, launches, sms);
+    if (v >= 7) return run_flow<OP, BN>(B, a, st, launches, sms);
+    if (v >= 2 && v <= 4) return run_large<OP, BN, false>(B, a, st, launches, sms);
+    return run_large<OP, BN, true>(B, a, st, launches, sms);
 }
 
 }  // namespace
@@ -1516,15 +1422,15 @@ cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cud
         }
         if (!best_bn) best_bn = 256;   // a fixed width the padding cannot hold: the standard one
         if (op == kOpE4M3) {
-            if (best_bn == 224) return run_flow<kOpE4M3, 224, 1>(B, a, st, launches, sms);
-            if (best_bn == 160) return run_flow<kOpE4M3, 160, 1, 3>(B, a, st, launches, sms);
-            if (best_bn == 128) return run_flow<kOpE4M3, 128, 1>(B, a, st, launches, sms);
-            return run_flow<kOpE4M3, 256, 1>(B, a, st, launches, sms);
+            if (best_bn == 224) return run_flow<kOpE4M3, 224>(B, a, st, launches, sms);
+            if (best_bn == 160) return run_flow<kOpE4M3, 160, 3>(B, a, st, launches, sms);
+            if (best_bn == 128) return run_flow<kOpE4M3, 128>(B, a, st, launches, sms);
+            return run_flow<kOpE4M3, 256>(B, a, st, launches, sms);
         }
-        if (best_bn == 224) return run_flow<kOpBF16, 224, 1>(B, a, st, launches, sms);
-        if (best_bn == 160) return run_flow<kOpBF16, 160, 1, 3>(B, a, st, launches, sms);
-        if (best_bn == 128) return run_flow<kOpBF16, 128, 1>(B, a, st, launches, sms);
-        return run_flow<kOpBF16, 256, 1>(B, a, st, launches, sms);
+        if (best_bn == 224) return run_flow<kOpBF16, 224>(B, a, st, launches, sms);
+        if (best_bn == 160) return run_flow<kOpBF16, 160, 3>(B, a, st, launches, sms);
+        if (best_bn == 128) return run_flow<kOpBF16, 128>(B, a, st, launches, sms);
+        return run_flow<kOpBF16, 256>(B, a, st, launches, sms);
     }
     // 256-replica tiles when they still give every SM one, else 128-replica tiles.
     const bool wide = (int64_t)(B.Mpad / kBM) * ((a.R + 255) / 256) >= sms;
