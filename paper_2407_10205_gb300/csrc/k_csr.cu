@@ -48,6 +48,7 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kBlk = 32 * kWarps;
+constexpr size_t kTwo = 113 * 1024;            // shared memory of one of two blocks on an SM
 
 // The word of position p and group g in a spin buffer: [group][Np], so that a group's spins are
 // copied as one piece, or (C.by_pos) [Np][group], so that a neighbour's groups share a sector.
@@ -685,7 +686,7 @@ cudaError_t launch_iterations(const CsrArgs &C, size_t smem, StepGraphCache *gra
     if (C.persistent) {
         // Every iteration in one cooperative launch: as many blocks as can be resident.
         auto k = csr_persistent<SMEM, C16, STAGED>;
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTwo);
         int per_sm = 0;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kBlk, smem);
         if (e != cudaSuccess) return e;
@@ -705,7 +706,7 @@ cudaError_t launch_iterations(const CsrArgs &C, size_t smem, StepGraphCache *gra
     Cs.a.t0 = 0;
     Cs.a.nsteps = 0;
     auto k = csr_step<SMEM, C16, STAGED>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTwo);
     if (e != cudaSuccess) return e;
     void *args[1] = {&Cs};
     for (int set = 0; set < C.nsets; ++set) {
@@ -747,7 +748,6 @@ cudaError_t launch_csr(const CsrArgs &Cin, const int32_t *max_len, StepGraphCach
     // with the spins gathered from global memory).  Larger ones are gathered from global memory, by
     // position (30000 x 256 48 against 62 from one block's shared memory).
     constexpr size_t kStage = (size_t)kWarps * 16 * 32 * sizeof(float4);      // x and v of a slice per warp
-    constexpr size_t kTwo = 113 * 1024;                                        // two blocks an SM
     int G = 1;
     while (G < 8 && G < groups) G *= 2;
     while (G > 1 && (size_t)G * C.max_np * 4 + kStage > kTwo) G /= 2;

@@ -266,7 +266,7 @@ cudaError_t launch_gahmc(const RunArgs &a, float travel, int64_t K, int64_t *cou
     g.counts = counts; g.events = events; g.events_cap = events_cap;
     g.replica_iters = a.replica_iters;
     const size_t smem = (size_t)kGWarps * ((gahmc_warp_bytes(a.N) + 15) & ~(size_t)15);
-    cudaError_t e = cudaFuncSetAttribute(gahmc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(gahmc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxCtaSmem);
     if (e != cudaSuccess) return e;
     gahmc_kernel<<<(a.R + kGWarps - 1) / kGWarps, 32 * kGWarps, smem, st>>>(g);
     return cudaGetLastError();

@@ -306,7 +306,7 @@ cudaError_t launch_g(const RunArgs &a, cudaStream_t st) {
     constexpr int RL = RPT * G;
     const int smem = inc_smem_bytes(a.N, RL);
     auto kern = inc_small_kernel<RPT, G>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxCtaSmem);
     if (e != cudaSuccess) return e;
     const int WG = (a.N + 31) / 32;
     const int grid = (a.R + RL - 1) / RL;

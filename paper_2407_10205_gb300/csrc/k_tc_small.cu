@@ -617,7 +617,7 @@ cudaError_t launch_cfg(const RunArgs &a, int Kpad, cudaStream_t st) {
     // The derivative mode is a template parameter: the update loop stays straight-line.
     auto kern = a.deriv == 1 ? tc_small_kernel<MT, OP, CH, RPT, AT, 1, METRO>
                              : tc_small_kernel<MT, OP, CH, RPT, AT, 0, METRO>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxCtaSmem);
     if (e != cudaSuccess) return e;
     const int grid = (a.R + RL - 1) / RL;
     kern<<<grid, 128 * MT * CH + 64 * MT, smem, st>>>(a, Kpad);
@@ -672,7 +672,7 @@ cudaError_t launch_tc_small_batch(const RunArgs &a, int nmax, cudaStream_t st) {
     const size_t smem = (size_t)(3 * 128 + kNB) * Kpad + sizeof(SmallShared) + 16;
     auto kern = a.deriv == 1 ? tc_small_kernel<3, kOpE4M3, 2, 4, false, 1, false, true>
                              : tc_small_kernel<3, kOpE4M3, 2, 4, false, 0, false, true>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxCtaSmem);
     if (e != cudaSuccess) return e;
     kern<<<a.small_ctas, 128 * 3 * 2 + 64 * 3, smem, st>>>(a, Kpad);
     return cudaGetLastError();

@@ -69,6 +69,11 @@ struct RunArgs {
     int32_t small_ctas;                  // its length
 };
 
+// What a CTA may have.  A kernel's limit of dynamic shared memory belongs to the function on its
+// device: every thread's launches share it.  So it is always set to a value that holds for every
+// size, never to the launch's own, which could lower it under another thread's launch.
+constexpr size_t kMaxCtaSmem = 227 * 1024;
+
 constexpr uint64_t kWaitTimeoutNs = 2000000000ull;  // 2 s bound on every device-side wait
 
 // Iteration control of a per-iteration path, in device memory.  The run's prologue
