@@ -219,18 +219,20 @@ void worker_loop(phia_server_s *S) {
                 if (rc) finish(S, r, rc);
             }
         }
-        // admit queued requests in arrival order while a slot and memory are free
-        while (!S->queue.empty()) {
+        // admit the next queued request, in arrival order, if a slot and memory are free: one a pass, as
+        // its checks and uploads take milliseconds in which no running request gets its next chunk
+        if (!S->queue.empty()) {
             const int64_t id = S->queue.front();
             Request &r = S->reqs[id];
             auto it = std::find(S->slot_req.begin(), S->slot_req.end(), (int64_t)-1);
-            if (it == S->slot_req.end()) break;
-            if (S->used_bytes + r.bytes > S->opts.hbm_budget_bytes && S->used_bytes > 0) break;
-            S->queue.pop_front();
-            S->used_bytes += r.bytes;
-            const int rc = admit(S, r, (int)(it - S->slot_req.begin()));
-            if (rc) finish(S, r, rc);
-            progress = true;
+            if (it != S->slot_req.end() &&
+                (S->used_bytes + r.bytes <= S->opts.hbm_budget_bytes || S->used_bytes == 0)) {
+                S->queue.pop_front();
+                S->used_bytes += r.bytes;
+                const int rc = admit(S, r, (int)(it - S->slot_req.begin()));
+                if (rc) finish(S, r, rc);
+                progress = true;
+            }
         }
         S->cv.notify_all();
         if (!progress) {
