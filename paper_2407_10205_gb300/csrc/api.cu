@@ -159,6 +159,7 @@ struct phia_s {
     bool accept_moved = false;          // an automatic handle runs the acceptance test on the resident kernel
     TuneChoice before_accept{};         // ... and the choice that it had before
     int64_t wait_ns = 0;                // testing aid (phia_debug_wait): device wait bound, 0 = default
+    bool in_turns = false;              // its runs share the device with others (server requests)
     int stall_producer = 0;             // testing aid: the per-iteration kernel's TMA producer issues nothing
 };
 
@@ -173,6 +174,8 @@ std::map<int, cudaMemPool_t> g_pools;
 }  // namespace
 
 namespace phia {
+
+void set_in_turns(phia_s *p, bool in_turns) { p->in_turns = in_turns; }
 
 cudaError_t pool_alloc(void **ptr, size_t bytes, int device, cudaStream_t st) {
     cudaMemPool_t pool = nullptr;
@@ -324,6 +327,7 @@ RunArgs base_args(phia_t *p, int R) {
     a.coupling_mem = p->coupling_mem;
     a.wait_ns = p->wait_ns;
     a.stall_producer = p->stall_producer;
+    a.in_turns = p->in_turns ? 1 : 0;
     a.large_variant = p->large_variant ? p->large_variant : p->tuned_variant;
     return a;
 }

@@ -1341,8 +1341,7 @@ cudaError_t run_flow(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, i
 }
 
 template <int OP, int BN>
-cudaError_t run_variant(const LargeBuffers &B, const RunArgs &a, cudaStream_t st, int *launches, int sms) {
-    int v = a.large_variant;
+cudaError_t run_variant(const LargeBuffers &B, const RunArgs &a, int v, cudaStream_t st, int *launches, int sms) {
     if (v == 0) v = kDefaultLargeVariant;
     // The overlapped variants need their tile counters (absent from the allocation-free entry).
     if (v >= 7 && (!B.ready || !B.sbits || a.field_mode)) v = 1;
@@ -1399,8 +1398,15 @@ cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cud
         const double narrow = narrow_estimate(a.N, a.R, B.Kbytes, sms, &width);
         if (!a.stall_producer && cluster_small_estimate(a.N, a.R, op) < std::min(narrow, wide))
             return launch_cluster_small(a, op, st, launches);
-        if (narrow < wide) return launch_tc_narrow(B, a, op, width, st, launches, sms);
-        lv = 7;
+        // A run beside others holds at most half of the SMs; a larger one takes its turns launch by
+        // launch.  In one cooperative launch it would hold them for all of its iterations (22 us each at
+        // N = 6000 x 256), and each iteration of a sparse run beside it would wait for its end.
+        const int64_t tiles = narrow < wide ? (int64_t)((a.N + width - 1) / width) * ((a.R + 127) / 128) : sms;
+        if (a.in_turns && 2 * tiles > sms) lv = 1;
+        else if (narrow < wide) return launch_tc_narrow(B, a, op, width, st, launches, sms);
+        else lv = 7;
+    } else if (a.in_turns && lv >= 7) {
+        lv = 1;
     }
     if ((lv == 7 || lv >= 10) && B.ready && B.sbits && !a.field_mode) {
         const int mt = B.Mpad / kBM;
@@ -1432,11 +1438,12 @@ cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cud
         if (best_bn == 128) return run_flow<kOpBF16, 128>(B, a, st, launches, sms);
         return run_flow<kOpBF16, 256>(B, a, st, launches, sms);
     }
-    // 256-replica tiles when they still give every SM one, else 128-replica tiles.
+    // One launch per iteration; 256-replica tiles when they still give every SM one, else 128-replica
+    // tiles.
     const bool wide = (int64_t)(B.Mpad / kBM) * ((a.R + 255) / 256) >= sms;
     if (op == kOpE4M3)
-        return wide ? run_variant<kOpE4M3, 256>(B, a, st, launches, sms) : run_variant<kOpE4M3, 128>(B, a, st, launches, sms);
-    return wide ? run_variant<kOpBF16, 256>(B, a, st, launches, sms) : run_variant<kOpBF16, 128>(B, a, st, launches, sms);
+        return wide ? run_variant<kOpE4M3, 256>(B, a, lv, st, launches, sms) : run_variant<kOpE4M3, 128>(B, a, lv, st, launches, sms);
+    return wide ? run_variant<kOpBF16, 256>(B, a, lv, st, launches, sms) : run_variant<kOpBF16, 128>(B, a, lv, st, launches, sms);
 }
 
 }  // namespace phia

@@ -63,6 +63,8 @@ struct RunArgs {
     int32_t stall_producer;              // per-iteration kernel, testing: the TMA producer issues nothing
     int32_t large_variant;               // per-iteration kernel: 0 auto, 1, 5, 6 x/v ring, 2-4 x/v in
                                          // registers, 7-13 overlapped (phia_opts.large_variant)
+    int32_t in_turns;                    // per-iteration kernel: other work runs beside this run, so no launch
+                                         // whose CTAs hold the SMs and wait on each other
     int32_t accept_test;                 // Table 3 state 4: 1 = Metropolis test on H at trajectory ends
     int64_t *proposed, *accepted;        // [R] per-replica counts of the test (accept_test = 1)
     const SmallCta *small_cta;           // batched small dense runs: one entry per CTA
@@ -239,6 +241,7 @@ struct CsrArgs {
 cudaError_t launch_csr(const CsrArgs &C, const int32_t *max_len, StepGraphCache *graphs, cudaStream_t st, int *launches);
 
 }  // namespace phia
+struct phia_s;
 struct phia_batch_s;
 struct phia_instance_desc;
 struct phia_opts;
@@ -256,6 +259,8 @@ int batch_stats(phia_batch_s *b, int inst, phia_stats *out);
 // Device memory from the library's pool, ordered on a stream.
 cudaError_t pool_alloc(void **ptr, size_t bytes, int device, cudaStream_t st);
 void pool_free(void *ptr, cudaStream_t st);
+// Whether a dense handle's next runs share the device with other runs (RunArgs.in_turns).
+void set_in_turns(phia_s *p, bool in_turns);
 // Thread-local error message of the C ABI.
 int set_last_error(int code, const char *msg);
 
