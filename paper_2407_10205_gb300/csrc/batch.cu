@@ -58,6 +58,16 @@ struct phia_batch_s {
     int32_t *d_slice = nullptr, *d_hk2 = nullptr, *d_rowof = nullptr, *d_posof = nullptr;
     uint32_t *d_val = nullptr;
     int32_t *d_hk = nullptr;            // fields of the small dense members
+    // the CSR members once more with a row to a warp (k_csr_rows.cu), where some replica count may take it
+    std::vector<CsrRowsInst> rows_inst;
+    int32_t rows_blocks = 0;
+    int64_t total_rows = 0;
+    double degree = 0.0;                // couplings a row, with those that pad the slices
+    int longest = 0;                    // couplings of the longest row
+    CsrRowsInst *d_rows_inst = nullptr;
+    CsrRowsBlock *d_rows_blocks = nullptr;
+    int32_t *d_rows_ptr = nullptr, *d_rows_col = nullptr, *d_rows_h = nullptr;
+    int8_t *d_rows_val = nullptr;
     long long *d_targets = nullptr;
     bool any_target = false;
     // replica state (R padded to a multiple of 32)
@@ -125,6 +135,38 @@ void free_state(phia_batch_s *b) {
 
 int64_t words_of(int n) { return (n + 31) / 32; }
 
+// Picoseconds per update (spin, replica as run, iteration) of the two sparse forms once an instance
+// fills the GPU, fitted to 20000 .. 60000 spins x 256 .. 1024 replicas of degree 6 .. 60: k_csr.cu
+// with its spins in shared memory (up to 28928 positions) or by position, and k_csr_rows.cu.
+double lanes_ps(const phia_batch_s *b) {
+    return b->max_np <= 28928 ? 4.55 + 0.023 * b->degree : 4.1 + 0.105 * b->degree;
+}
+double rows_ps(const phia_batch_s *b) { return 3.5 + 0.052 * b->degree; }
+
+// A row of thousands of couplings among short ones: one warp's way along it, 0.036 us a coupling, can
+// be the whole iteration.
+bool has_hub(const phia_batch_s *b) { return b->longest >= 2048 && b->longest >= 8.0 * b->degree; }
+
+// Whether a replica count exists for which k_csr_rows.cu is the faster form.  Up to 12544 positions
+// k_csr.cu has x and v in shared memory too and is never slower (10000 x 1024, degree 6: 40 us
+// against 42).
+bool rows_form_possible(const phia_batch_s *b) {
+    return has_hub(b) || (b->max_np > 12544 && rows_ps(b) < lanes_ps(b));
+}
+
+// Whether a run of `replicas` takes it.  It pads them to 256 instead of 32, and below 5e6 updates an
+// iteration latencies set the time (13000 x 256 of degree 6: 18.3 us against 17.7).  Where a hub sets
+// it (stars: a ring and one row coupled to all), k_csr.cu keeps up with 16-bit offsets and few
+// replicas (10000 x 256 366 us against 368) and not past them (10000 x 1024 657 us against 400, 20000 x
+// 64 878 against 724, 30000 x 64 1870 against 1094).
+bool rows_form(const phia_batch_s *b, int replicas) {
+    if (!b->d_rows_inst) return false;
+    const double updates = (double)b->total_rows * round_up(replicas, 256);
+    const double lanes_us = 1e-6 * (double)b->total_rows * round_up(replicas, 32) * lanes_ps(b);
+    if (has_hub(b) && 0.036 * b->longest > lanes_us) return b->max_np > 16384 || replicas > 256;
+    return updates >= 5e6 && 1e-6 * updates * rows_ps(b) < lanes_us;
+}
+
 // Per-replica offsets for R replicas per instance: records and best states by public
 // index (instance k's records start at k R), CSR state over the CSR members only.
 void layout(phia_batch_s *b, int R) {
@@ -144,6 +186,14 @@ void layout(phia_batch_s *b, int R) {
         x += (int64_t)in.Np * R;
         xin += (int64_t)in.N * b->R_real;
         s += (int64_t)in.Np * (R / 32);
+        if (c < b->rows_inst.size()) {
+            CsrRowsInst &ri = b->rows_inst[c];
+            ri.x_off = ri.row_base * R;
+            ri.xin_off = in.xin_off;
+            ri.s_off = ri.row_base * (R / 32);
+            ri.rec_off = in.rec_off;
+            ri.bits_off = in.bits_off;
+        }
     }
 }
 
@@ -316,6 +366,29 @@ void pack_slices(int n, const int32_t *rp, const int32_t *col, const int8_t *val
         }
 }
 
+// The rows of a checked instance in their own order, every one padded to a multiple of 8 entries with
+// k = 0, after those of the instances before.
+void append_rows(const phia_instance_desc &x, std::vector<int32_t> &ptr, std::vector<int32_t> &col, std::vector<int8_t> &val) {
+    const size_t base = col.size();
+    ptr.push_back(0);
+    for (int i = 0; i < x.N; ++i) {
+        if (x.J_k) {
+            const int8_t *row = x.J_k + (size_t)i * x.N;
+            for (int j = 0; j < x.N; ++j)
+                if (row[j] != 0) {
+                    col.push_back(j);
+                    val.push_back(row[j]);
+                }
+        } else {
+            col.insert(col.end(), x.col + x.row_ptr[i], x.col + x.row_ptr[i + 1]);
+            val.insert(val.end(), x.val_k + x.row_ptr[i], x.val_k + x.row_ptr[i + 1]);
+        }
+        col.resize(base + (col.size() - base + 7) / 8 * 8, 0);
+        val.resize(col.size(), 0);
+        ptr.push_back((int32_t)(col.size() - base));
+    }
+}
+
 void pack_instance(const phia_instance_desc &x, int k, int threads, PackedInst &out) {
     const int n = x.N;
     if (n < 1) return pack_error(out, PHIA_EINVAL, "instance %d: N must be >= 1", k);
@@ -470,6 +543,7 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         in.pos_off = (int64_t)row_of.size();
         in.inv_off = (int64_t)pos_of.size();
         const int32_t ent0 = (int32_t)(val.size() / 32);
+        const int longest = 4 * pk.slice[1];           // rows are sorted by length
         for (int32_t e : pk.slice) slice.push_back(ent0 + e);
         if (count == 1) {
             col = std::move(pk.col);
@@ -484,7 +558,36 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         pk = PackedInst();
         b->max_np = std::max(b->max_np, in.Np);
         b->total_slices += in.Np / 32;
+        b->total_rows += n;
+        b->longest = std::max(b->longest, longest);
         b->inst.push_back(in);
+    }
+    std::vector<int32_t> rows_ptr, rows_col, rows_h;
+    std::vector<int8_t> rows_val;
+    std::vector<CsrRowsBlock> rows_blocks;
+    b->degree = b->total_rows ? 4.0 * (double)(slice.empty() ? 0 : slice.back()) * 32.0 / (double)b->total_rows : 0.0;
+    if (rows_form_possible(b)) {
+        const size_t most = (size_t)(b->degree * (double)b->total_rows) + 8 * (size_t)b->total_rows;
+        rows_col.reserve(most);
+        rows_val.reserve(most);
+        int64_t row_base = 0;
+        for (size_t c = 0; c < b->inst.size(); ++c) {
+            const phia_instance_desc &x = d[b->csr_pub[c]];
+            CsrRowsInst ri{};
+            ri.N = x.N;
+            ri.inst_id = x.instance_id;
+            ri.q = b->inst[c].q;
+            ri.rp_off = (int64_t)rows_ptr.size();
+            ri.nz_off = (int64_t)rows_col.size();
+            ri.h_off = (int64_t)rows_h.size();
+            ri.row_base = row_base;
+            row_base += x.N;
+            append_rows(x, rows_ptr, rows_col, rows_val);
+            rows_h.insert(rows_h.end(), x.h_k, x.h_k + x.N);
+            for (int i0 = 0; i0 < x.N; i0 += 64) rows_blocks.push_back(CsrRowsBlock{(int32_t)c, i0});
+            b->rows_inst.push_back(ri);
+        }
+        b->rows_blocks = (int32_t)rows_blocks.size();
     }
     for (int l = 0; l < 4; ++l)
         for (size_t c = 0; c <= b->inst.size(); ++c) {
@@ -524,6 +627,14 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
     up((void **)&b->d_blocks, b->blocks.data(), b->blocks.size() * sizeof(CsrBlock));
     up((void **)&b->d_targets, b->targets.data(), b->targets.size() * sizeof(long long));
     up((void **)&b->d_dJ, dj.data(), dj.size());
+    if (!b->rows_inst.empty()) {
+        up((void **)&b->d_rows_ptr, rows_ptr.data(), rows_ptr.size() * 4);
+        up((void **)&b->d_rows_col, rows_col.data(), rows_col.size() * 4);
+        up((void **)&b->d_rows_val, rows_val.data(), rows_val.size());
+        up((void **)&b->d_rows_h, rows_h.data(), rows_h.size() * 4);
+        up((void **)&b->d_rows_blocks, rows_blocks.data(), rows_blocks.size() * sizeof(CsrRowsBlock));
+        al((void **)&b->d_rows_inst, sizeof(CsrRowsInst) * b->rows_inst.size());
+    }
     al((void **)&b->d_inst, sizeof(CsrInst) * b->inst.size());
     al((void **)&b->d_sets, sizeof(CsrSet) * b->inst.size());
     al((void **)&b->d_min_hit, 8);
@@ -560,7 +671,8 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         if (total > ((int64_t)1 << 31)) return bfail(PHIA_ERANGE, "total_steps must be < 2^31");
     }
     if (R_real < 1) return bfail(PHIA_EINVAL, "replicas must be >= 1");
-    const int R = round_up(R_real, 32);
+    const bool by_rows = !field_mode && rows_form(b, R_real);
+    const int R = round_up(R_real, by_rows ? 256 : 32);
     BCU(cudaSetDevice(b->device));
     if (!field_mode && !reset && (!b->ran || b->R_real != R_real))
         return bfail(PHIA_ESTATE, "reset_best = 0 needs a previous run with the same replica count");
@@ -574,6 +686,8 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         return bfail(PHIA_ENOTSUP, "runs from a given state take CSR instances");
     if (ncsr > 0)
         BCU(cudaMemcpyAsync(b->d_inst, b->inst.data(), sizeof(CsrInst) * ncsr, cudaMemcpyHostToDevice, b->stream));
+    if (by_rows)
+        BCU(cudaMemcpyAsync(b->d_rows_inst, b->rows_inst.data(), sizeof(CsrRowsInst) * ncsr, cudaMemcpyHostToDevice, b->stream));
     const int64_t reps = (int64_t)R * b->count;
     int64_t nbits = 0;
     for (int k = 0; k < b->count; ++k) nbits += (int64_t)R * words_of(b->N[k]);
@@ -707,7 +821,26 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     C.ctl = b->d_ctl;
     C.sync = b->d_sync;
     C.persistent = (b->csr_mode == 1 && !field_mode) ? 1 : 0;
-    if (gathers) {
+    if (by_rows) {
+        CsrRowsArgs W;
+        memset(&W, 0, sizeof W);
+        W.a = C.a;
+        W.inst = b->d_rows_inst; W.count = ncsr;
+        W.blocks = b->d_rows_blocks; W.nblocks = b->rows_blocks;
+        W.row_ptr = b->d_rows_ptr; W.col = b->d_rows_col; W.val = b->d_rows_val; W.hk = b->d_rows_h;
+        W.X = C.X; W.V = C.V;
+        W.x_in = x_in; W.v_in = v_in; W.x_out = x_out; W.v_out = v_out;
+        W.S = C.S; W.total_swords = b->total_rows * (R / 32);
+        W.Esum = C.Esum; W.flags = C.flags; W.total_reps = reps;
+        W.best_bits = C.best_bits;
+        W.targets = C.targets;
+        W.R = R; W.R_real = R_real;
+        W.max_words = C.max_words;
+        W.total_rows = b->total_rows;
+        W.ctl = C.ctl; W.persistent = C.persistent; W.sync = C.sync;
+        cudaError_t e = launch_csr_rows(W, b->graphs, b->stream, &launches);
+        if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
+    } else if (gathers) {
         if (b->sets_R != R) {
             rc = make_sets(b, R);
             if (rc) return rc;
@@ -934,7 +1067,8 @@ void phia_batch_destroy(phia_batch_t *b) {
     for (void *p : {(void *)b->d_inst, (void *)b->d_blocks, (void *)b->d_slice, b->d_col, (void *)b->d_val,
                     (void *)b->d_sets, (void *)b->d_hk2, (void *)b->d_rowof, (void *)b->d_posof, (void *)b->d_hk,
                     (void *)b->d_targets, (void *)b->d_min_hit, (void *)b->d_start_ns, (void *)b->d_iters,
-                    (void *)b->d_err, (void *)b->d_dJ, (void *)b->d_small, (void *)b->d_sync, (void *)b->d_ctl})
+                    (void *)b->d_rows_inst, (void *)b->d_rows_blocks, (void *)b->d_rows_ptr, (void *)b->d_rows_col,
+                    (void *)b->d_rows_val, (void *)b->d_rows_h, (void *)b->d_err, (void *)b->d_dJ, (void *)b->d_small, (void *)b->d_sync, (void *)b->d_ctl})
         pool_free(p, b->stream);
     step_graphs_free(b->graphs);
     if (b->ev0) cudaEventDestroy(b->ev0);

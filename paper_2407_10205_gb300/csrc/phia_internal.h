@@ -240,6 +240,54 @@ struct CsrArgs {
 // max_len: the most blocks that a set has in each list.
 cudaError_t launch_csr(const CsrArgs &C, const int32_t *max_len, StepGraphCache *graphs, cudaStream_t st, int *launches);
 
+// The sparse path for large instances of few couplings a row, a row to a warp (see k_csr_rows.cu).
+struct CsrRowsInst {
+    int32_t N;
+    uint32_t inst_id;       // fourth Philox counter word
+    float q;                // 2^-frac_bits
+    int32_t pad;
+    int64_t rp_off;         // into row_ptr (N + 1 entries, values relative to nz_off)
+    int64_t nz_off;         // into col / val (rows padded to multiples of 8 entries with k = 0)
+    int64_t h_off;          // into hk
+    int64_t row_base;       // global index of row 0 (rows are stored instance after instance)
+    int64_t x_off;          // into X, V ([N][R] per instance)
+    int64_t xin_off;        // into caller arrays ([R][N] per instance)
+    int64_t s_off;          // into each spin buffer, in uint32 words ([N][R/32] per instance)
+    int64_t rec_off;        // into per-replica records (R per instance)
+    int64_t bits_off;       // into best_bits (R * ceil(N/32) per instance)
+};
+struct CsrRowsBlock {
+    int32_t inst;
+    int32_t i0;             // first of up to 64 rows
+};
+struct CsrRowsArgs {
+    RunArgs a;              // run parameters; record pointers indexed by rec_off + r
+    const CsrRowsInst *inst;
+    int32_t count;
+    const CsrRowsBlock *blocks;
+    int32_t nblocks;
+    const int32_t *row_ptr; const int32_t *col; const int8_t *val; const int32_t *hk;
+    float *X, *V;
+    const float *x_in, *v_in;
+    float *x_out, *v_out;
+    uint32_t *S;            // 4 rotating spin buffers of total_swords words each
+    int64_t total_swords;
+    int64_t *Esum;          // [2][total_reps]
+    int8_t *flags;          // [2][total_reps]
+    int64_t total_reps;
+    uint32_t *best_bits;
+    const long long *targets;   // per instance, or null (then a.target)
+    int32_t R;              // replicas per instance as run (multiple of 256)
+    int32_t R_real;         // replicas the caller asked for (<= R); the rest pad the groups
+    int32_t max_words;      // max ceil(N/32)
+    int64_t total_rows;
+    IterCtl *ctl;           // iteration control
+    int32_t persistent;     // 1: every iteration in one cooperative launch (grid barrier per iteration)
+    int32_t pad1;
+    unsigned *sync;         // 4 words of device memory for that launch's barrier and work counters
+};
+cudaError_t launch_csr_rows(const CsrRowsArgs &C, StepGraphCache *graphs, cudaStream_t st, int *launches);
+
 }  // namespace phia
 struct phia_s;
 struct phia_batch_s;
