@@ -156,6 +156,7 @@ struct phia_s {
     int large_variant = 0;              // per-iteration kernel variant requested (0 = automatic)
     int tuned_variant = 0;              // the autotuner's choice for it
     bool tuned = false;                 // the kernel is the autotuner's choice for this replica count
+    TuneChoice created{};               // the choice of an automatic handle without the autotuner's
     bool accept_moved = false;          // an automatic handle runs the acceptance test on the resident kernel
     TuneChoice before_accept{};         // ... and the choice that it had before
     int64_t wait_ns = 0;                // testing aid (phia_debug_wait): device wait bound, 0 = default
@@ -352,8 +353,21 @@ int ensure_operand(phia_t *p) {
     return PHIA_OK;
 }
 
+TuneChoice choice_of(const phia_t *p) {
+    return TuneChoice{p->large, p->tile_rl, p->coupling_mem, p->warpk, p->inc, p->tuned_variant};
+}
+void set_choice(phia_t *p, const TuneChoice &c) {
+    p->large = c.large;
+    p->tile_rl = c.tile_rl;
+    p->coupling_mem = c.coupling_mem;
+    p->warpk = c.warpk;
+    p->inc = c.inc;
+    p->tuned_variant = c.lvar;
+}
+
 // A handle whose kernel variant is automatic takes the cached autotune choice for its
-// (N, replicas, operand), if any.
+// (N, replicas, operand), or without one the choice that it was created with: another
+// replica count's does not stay.
 int apply_tuned(phia_t *p, int R) {
     if (!p->auto_tile || p->path != PHIA_PATH_TC) return PHIA_OK;
     TuneChoice c;
@@ -361,19 +375,13 @@ int apply_tuned(phia_t *p, int R) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tune.find(TuneKey{p->N, R, p->op});
         p->tuned = it != g_tune.end();
-        if (!p->tuned) return PHIA_OK;
-        c = it->second;
+        c = p->tuned ? it->second : p->created;
     }
     if (c.large) {
         int rc = ensure_operand(p);
         if (rc) return rc;
     }
-    p->large = c.large;
-    p->warpk = c.warpk;
-    p->inc = c.inc;
-    p->tile_rl = c.tile_rl;
-    p->coupling_mem = c.coupling_mem;
-    p->tuned_variant = c.lvar;
+    set_choice(p, c);
     return PHIA_OK;
 }
 
@@ -629,6 +637,7 @@ int create_dense(phia_t **out, const int8_t *J_k, const int32_t *h_k, int32_t N,
         p->warpk = o.tc_kernel == 3 || (p->auto_tile && N <= warp_small_auto_n());
         p->inc = o.tc_kernel == 4;
     }
+    p->created = choice_of(p);
     const size_t NN = (size_t)N * N;
     auto cleanup = [&](int code) { phia_destroy(p); return code; };
     if (pool_alloc((void **)&p->d_Jk, NN, p->device, p->stream) != cudaSuccess)

@@ -1,0 +1,31 @@
+"""GPU tests of what a handle's kernel choice is after the calls that change it: a tuned replica
+count, an acceptance run."""
+import numpy as np
+import pytest
+
+from paper_2407_10205_gb300 import instances as ins
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _kernel_of(phia, h, sched, R, T=20):
+    phia.anneal(h, sched, R, T, 5)
+    st = phia.stats_get(h)
+    return st.tc_kernel, st.kernel_launches
+
+
+@pytest.mark.parametrize("N", [150, 230, 1100, 1536, 2000])
+def test_a_tuned_replica_count_leaves_others_alone(gpu_lib, N):
+    """Tuned for 8192 replicas, a handle runs 64 as a fresh one does (its kernel shows in the code and the
+    number of launches: 2 for the kernels that run from one launch, one more for each conversion)."""
+    phia = gpu_lib
+    d = ins.dense_int(N, 7, 7, N)
+    sched = phia.schedule(0.01, 0.1, 0.1, 2.0, refresh=50)
+    with phia.Annealer(d.k, d.kh, path=phia.PATH_TC, instance_id=3) as B:
+        fresh = _kernel_of(phia, B.h, sched, 64)
+    with phia.Annealer(d.k, d.kh, path=phia.PATH_TC, instance_id=3) as A:
+        phia.autotune(A.h, sched, 8192, probe_iters=10)
+        tuned = _kernel_of(phia, A.h, sched, 8192)
+        assert _kernel_of(phia, A.h, sched, 64) == fresh
+        assert _kernel_of(phia, A.h, sched, 8192) == tuned
