@@ -723,6 +723,13 @@ int phia_create_csr(phia_t **out, const int32_t *row_ptr, const int32_t *col, co
     return PHIA_OK;
 }
 
+// Back to the kernel of ordinary runs after one with the acceptance test.
+static void after_accept(phia_t *p) {
+    if (!p->accept_moved) return;
+    p->accept_moved = false;
+    set_choice(p, p->before_accept);
+}
+
 static int run_impl(phia_t *p, const phia_schedule *sched, int32_t R, int64_t t0, int64_t steps, int64_t total,
                     uint64_t seed, const float *x_in, float *x_out, const float *v_in, float *v_out, int reset) {
     if (!p) return fail(PHIA_EINVAL, "handle is NULL");
@@ -734,8 +741,7 @@ static int run_impl(phia_t *p, const phia_schedule *sched, int32_t R, int64_t t0
     if (sched->accept_test == 1 && p->path == PHIA_PATH_TC) {
         // The acceptance test runs in the resident tcgen05 kernel with J in shared memory.
         if (p->auto_tile && p->N <= tc_small_max_n(p->op)) {
-            if (!p->accept_moved)
-                p->before_accept = TuneChoice{p->large, p->tile_rl, p->coupling_mem, p->warpk, p->inc, p->tuned_variant};
+            if (!p->accept_moved) p->before_accept = choice_of(p);
             p->accept_moved = true;
             p->large = p->warpk = p->inc = false;
             p->coupling_mem = 1;
@@ -745,16 +751,7 @@ static int run_impl(phia_t *p, const phia_schedule *sched, int32_t R, int64_t t0
                         tc_small_max_n(p->op));
         }
     }
-    if (sched->accept_test == 0 && p->accept_moved) {   // back to the kernel of ordinary runs
-        const TuneChoice &c = p->before_accept;
-        p->accept_moved = false;
-        p->large = c.large;
-        p->warpk = c.warpk;
-        p->inc = c.inc;
-        p->tile_rl = c.tile_rl;
-        p->coupling_mem = c.coupling_mem;
-        p->tuned_variant = c.lvar;
-    }
+    if (sched->accept_test == 0) after_accept(p);
     if (steps < 1) return fail(PHIA_EINVAL, "steps must be >= 1");
     if (t0 < 0 || total < t0 + steps) return fail(PHIA_EINVAL, "need 0 <= t0 and t0 + steps <= total_steps");
     if (total > (int64_t)1 << 31) return fail(PHIA_ERANGE, "total_steps must be < 2^31 (Philox counter word)");
@@ -815,6 +812,9 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
     // Variants 3 .. 6, 8 and 9 run the forms of 2, 1, 10 and 12.
     constexpr int kSameForm = 6;
     for (int lv : {1, 2, 7, 10, 11, 12, 13}) cands.push_back(TuneChoice{true, 0, 0, false, false, lv});
+    // The probes run the candidates: not the kernel of before an acceptance run, which the first of them
+    // would go back to, with the candidate's choice overwritten.
+    after_accept(p);
     const bool saved_auto = p->auto_tile;
     p->auto_tile = false;
     float best_ms = 1e30f, worst_ms = 0.f;
@@ -824,12 +824,7 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
             int rc = ensure_operand(p);
             if (rc) { p->auto_tile = saved_auto; return rc; }
         }
-        p->large = c.large;
-        p->warpk = c.warpk;
-        p->inc = c.inc;
-        p->tile_rl = c.tile_rl;
-        p->coupling_mem = c.coupling_mem;
-        p->tuned_variant = c.lvar;
+        set_choice(p, c);
         float ms = 0.f;
         for (int rep = 0; rep < 2; ++rep) {   // the first run warms up
             int rc = run_impl(p, sched, replicas, 0, probe_iters, probe_iters, 1, nullptr, nullptr, nullptr, nullptr, 1);
@@ -840,12 +835,7 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
         if (ms < best_ms) { best_ms = ms; best = c; }
         worst_ms = std::max(worst_ms, ms);
     }
-    p->large = best.large;
-    p->warpk = best.warpk;
-    p->inc = best.inc;
-    p->tile_rl = best.tile_rl;
-    p->coupling_mem = best.coupling_mem;
-    p->tuned_variant = best.lvar;
+    set_choice(p, best);
     p->tuned = true;
     p->auto_tile = saved_auto;
     {

@@ -29,3 +29,24 @@ def test_a_tuned_replica_count_leaves_others_alone(gpu_lib, N):
         tuned = _kernel_of(phia, A.h, sched, 8192)
         assert _kernel_of(phia, A.h, sched, 64) == fresh
         assert _kernel_of(phia, A.h, sched, 8192) == tuned
+
+
+@pytest.mark.parametrize("N", [16, 40, 64, 90, 128])
+def test_autotune_after_an_acceptance_run_times_its_candidates(gpu_lib, N):
+    """The tuner's time is that of the kernel it chose.  Sizes where the warp-level kernel takes half the
+    time of the first candidate, which the tuner credited with it."""
+    phia = gpu_lib
+    R, T = 256, 2000
+    d = ins.dense_int(N, 7, 7, N)
+    plain = phia.schedule(0.01, 0.1, 0.1, 2.0, refresh=50)
+    with phia.Annealer(d.k, d.kh, path=phia.PATH_TC) as A:
+        phia.anneal(A.h, phia.schedule(0.01, 0.1, 0.1, 2.0, refresh=50, accept_test=1), R, 50, 5)
+        res = phia.autotune(A.h, plain, R, probe_iters=T)
+        best = min(_device_us(phia, A.h, plain, R, T) for _ in range(3))
+        assert phia.stats_get(A.h).tc_kernel == res.tc_kernel
+        assert best < 1.3 * res.best_us_per_iter
+
+
+def _device_us(phia, h, sched, R, T):
+    phia.anneal(h, sched, R, T, 5)
+    return 1000.0 * phia.stats_get(h).device_ms / T
