@@ -126,7 +126,6 @@ struct phia_s {
     int8_t *d_val = nullptr;
     // per-replica state
     int R_cap = 0, R_last = 0;
-    bool cap_large = false;             // replica buffers allocated for the per-iteration kernel
     bool auto_tile = true;              // kernel variant chosen automatically (autotune cache)
     float *d_x = nullptr, *d_v = nullptr;
     int8_t *d_s0 = nullptr, *d_s1 = nullptr;
@@ -210,26 +209,58 @@ void pool_free(void *ptr, cudaStream_t st) {
 
 namespace {
 
-void free_replicas(phia_t *p) {
+void free_large(phia_t *p) {
     for (void *b : {(void *)p->d_S, (void *)p->d_Epart, (void *)p->d_flags, (void *)p->d_ready, (void *)p->d_sbits,
-                    (void *)p->d_X,
-                    (void *)p->d_V,
-                    (void *)p->d_x, (void *)p->d_v, (void *)p->d_s0, (void *)p->d_s1, (void *)p->d_eacc,
+                    (void *)p->d_X, (void *)p->d_V})
+        pool_free(b, p->stream);
+    p->d_S = nullptr; p->d_Epart = nullptr; p->d_flags = nullptr; p->d_ready = nullptr; p->d_sbits = nullptr;
+    p->d_X = p->d_V = nullptr;
+}
+
+void free_replicas(phia_t *p) {
+    free_large(p);
+    for (void *b : {(void *)p->d_x, (void *)p->d_v, (void *)p->d_s0, (void *)p->d_s1, (void *)p->d_eacc,
                     (void *)p->d_rec, (void *)p->d_bits, (void *)p->d_prop, (void *)p->d_acc, (void *)p->d_xstart,
                     (void *)p->d_elast, (void *)p->d_estart, (void *)p->d_xxs, (void *)p->d_vvs, (void *)p->d_hass})
         pool_free(b, p->stream);
     p->d_prop = p->d_acc = nullptr; p->d_xstart = nullptr; p->d_elast = p->d_estart = nullptr;
     p->d_xxs = p->d_vvs = nullptr; p->d_hass = nullptr;
-    p->d_S = nullptr; p->d_Epart = nullptr; p->d_flags = nullptr; p->d_ready = nullptr; p->d_sbits = nullptr;
-    p->d_X = p->d_V = nullptr;
     p->d_x = p->d_v = nullptr; p->d_s0 = p->d_s1 = nullptr; p->d_eacc = nullptr;
     p->d_rec = nullptr; p->d_best_e = p->d_best_step = p->d_hit = nullptr; p->d_bits = nullptr; p->d_hit_ns = nullptr;
     p->d_min_hit = p->d_iters = nullptr; p->d_err = nullptr; p->d_start_ns = nullptr;
     p->R_cap = 0;
 }
 
+// What the per-iteration kernel needs of a handle's replicas, for R_cap of them, when the handle first
+// takes it.  The records stay as they are: a run that goes on after an acceptance run may change
+// from the resident kernel to this one.
+int ensure_large(phia_t *p) {
+    if (!p->large || p->d_S) return PHIA_OK;
+    const size_t Rp = (size_t)large_rpad_handle(p->R_cap), Mp = (size_t)round_up(p->N, 128);
+    bool ok = true;
+    auto al = [&](void **ptr, size_t bytes) {
+        if (ok && pool_alloc(ptr, bytes, p->device, p->stream) != cudaSuccess) ok = false;
+    };
+    al((void **)&p->d_S, 4 * Rp * p->Kbytes);
+    al((void **)&p->d_Epart, 2 * Rp * 8);
+    al((void **)&p->d_flags, 4 * Rp);
+    al((void **)&p->d_ready, 2 * (Rp / 128) * sizeof(uint32_t));
+    al((void **)&p->d_sbits, 4 * Rp * (Mp / 32) * sizeof(uint32_t));
+    al((void **)&p->d_X, Rp * Mp * 4);          // x, v in the interleaved [Rp/4][Mp][4] layout
+    al((void **)&p->d_V, Rp * Mp * 4);
+    if (!ok) {
+        cudaGetLastError();
+        free_large(p);
+        return fail(PHIA_ENOMEM, "device allocation for %d replicas failed", p->R_cap);
+    }
+    CU(cudaMemsetAsync(p->d_S, 0, 4 * Rp * p->Kbytes, p->stream));   // K and replica padding stay 0
+    CU(cudaMemsetAsync(p->d_flags, 0, 4 * Rp, p->stream));
+    CU(cudaMemsetAsync(p->d_Epart, 0, 2 * Rp * 8, p->stream));
+    return PHIA_OK;
+}
+
 int ensure_replicas(phia_t *p, int R) {
-    if (R <= p->R_cap && p->cap_large == p->large) return PHIA_OK;
+    if (R <= p->R_cap) return ensure_large(p);
     CU(cudaStreamSynchronize(p->stream));
     free_replicas(p);
     const size_t RN = (size_t)R * p->N;
@@ -247,16 +278,6 @@ int ensure_replicas(phia_t *p, int R) {
     }
     al((void **)&p->d_prop, (size_t)R * 8);
     al((void **)&p->d_acc, (size_t)R * 8);
-    if (p->large) {
-        const size_t Rp = (size_t)large_rpad_handle(R);
-        al((void **)&p->d_S, 4 * Rp * p->Kbytes);
-        al((void **)&p->d_Epart, 2 * Rp * 8);
-        al((void **)&p->d_flags, 4 * Rp);
-        al((void **)&p->d_ready, 2 * (Rp / 128) * sizeof(uint32_t));
-        const size_t Mp = (size_t)round_up(p->N, 128);   // x, v in the interleaved [Rp/4][Mp][4] layout
-        al((void **)&p->d_sbits, 4 * Rp * (Mp / 32) * sizeof(uint32_t));
-        al((void **)&p->d_X, Rp * Mp * 4); al((void **)&p->d_V, Rp * Mp * 4);
-    }
     al((void **)&p->d_eacc, (size_t)R * 8);
     al((void **)&p->d_rec, sizeof(RunCounters) + 4 * (size_t)R * 8);
     al((void **)&p->d_bits, (size_t)R * p->W * 4);
@@ -265,7 +286,6 @@ int ensure_replicas(phia_t *p, int R) {
         free_replicas(p);
         return fail(PHIA_ENOMEM, "device allocation for %d replicas failed", R);
     }
-    p->cap_large = p->large;
     RunCounters *ctr = reinterpret_cast<RunCounters *>(p->d_rec);
     p->d_err = &ctr->err;
     p->d_iters = &ctr->iters;
@@ -277,14 +297,8 @@ int ensure_replicas(phia_t *p, int R) {
     p->d_hit_ns = reinterpret_cast<uint64_t *>(p->d_hit + R);
     CU(cudaMemsetAsync(p->d_rec, 0, sizeof(RunCounters), p->stream));
     CU(cudaMemsetAsync(p->d_eacc, 0, (size_t)R * 8, p->stream));
-    if (p->large) {
-        const size_t Rp = (size_t)large_rpad_handle(R);
-        CU(cudaMemsetAsync(p->d_S, 0, 4 * Rp * p->Kbytes, p->stream));   // K and replica padding stay 0
-        CU(cudaMemsetAsync(p->d_flags, 0, 4 * Rp, p->stream));
-        CU(cudaMemsetAsync(p->d_Epart, 0, 2 * Rp * 8, p->stream));
-    }
     p->R_cap = R;
-    return PHIA_OK;
+    return ensure_large(p);
 }
 
 int reset_run(phia_t *p, int R, bool reset) {

@@ -50,3 +50,28 @@ def test_autotune_after_an_acceptance_run_times_its_candidates(gpu_lib, N):
 def _device_us(phia, h, sched, R, T):
     phia.anneal(h, sched, R, T, 5)
     return 1000.0 * phia.stats_get(h).device_ms / T
+
+
+def test_a_run_goes_on_after_an_acceptance_run(gpu_lib):
+    """384 spins x 16384 replicas are tuned to a per-iteration kernel; a run with the acceptance test
+    takes the resident one.  The ordinary run that goes on from it keeps its records."""
+    phia = gpu_lib
+    N, R = 384, 16384
+    d = ins.dense_int(N, 7, 7, 2)
+    kw = dict(refresh=5)
+    test, plain = (phia.schedule(0.01, 0.1, 0.1, 2.0, accept_test=k, **kw) for k in (1, 0))
+    out = []
+    for fixed in (True, False):
+        o = dict(tc_kernel=phia.KERNEL_RESIDENT, coupling_mem=phia.MEM_SHARED) if fixed else {}
+        with phia.Annealer(d.k, d.kh, path=phia.PATH_TC, **o) as A:
+            if not fixed:
+                assert phia.autotune(A.h, plain, R, probe_iters=10).tc_kernel == 2
+            x, v = torch.empty((R, N), device="cuda"), torch.empty((R, N), device="cuda")
+            phia.init_state(A.h, R, 7, x, v)
+            phia.run(A.h, test, R, 0, 20, 30, 7, x, v)
+            # backwards, so that the second piece improves few replicas and the first's records count
+            phia.run(A.h, phia.schedule(0.0, 0.0, 0.1, 2.0, **kw), R, 20, 10, 30, 7, x, v, reset_best=False)
+            out.append(phia.replica_results(A.h, R, N))
+    assert (out[0][1] < 20).any()
+    for u, w in zip(*out):
+        assert np.array_equal(u, w)
