@@ -688,6 +688,20 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         BCU(cudaMemcpyAsync(b->d_inst, b->inst.data(), sizeof(CsrInst) * ncsr, cudaMemcpyHostToDevice, b->stream));
     if (by_rows)
         BCU(cudaMemcpyAsync(b->d_rows_inst, b->rows_inst.data(), sizeof(CsrRowsInst) * ncsr, cudaMemcpyHostToDevice, b->stream));
+    // Whether the sparse members gather, or run on the resident kernels (below).
+    bool gathers = ncsr > 0;
+    if (ncsr > 0 && !b->cand_joff.empty() && !field_mode && (b->count == 1 || (!x_in && !x_out))) {
+        int sms = 0;
+        BCU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
+        double us = 0.0;
+        for (const CsrInst &in : b->inst)
+            us += in.N <= warp_small_max_n() ? warp_small_estimate(in.N, R_real, sms) : cluster_small_estimate(in.N, R_real, kOpBF16);
+        gathers = us > 5.0;
+    }
+    if (gathers && !by_rows && !field_mode && b->sets_R != R) {      // host work: before the run's time begins
+        rc = make_sets(b, R);
+        if (rc) return rc;
+    }
     const int64_t reps = (int64_t)R * b->count;
     int64_t nbits = 0;
     for (int k = 0; k < b->count; ++k) nbits += (int64_t)R * words_of(b->N[k]);
@@ -762,15 +776,6 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         int nmax, kernel;
     };
     std::vector<SmallGroup> groups;
-    bool gathers = ncsr > 0;
-    if (ncsr > 0 && !b->cand_joff.empty() && !field_mode && (b->count == 1 || (!x_in && !x_out))) {
-        int sms = 0;
-        BCU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
-        double us = 0.0;
-        for (const CsrInst &in : b->inst)
-            us += in.N <= warp_small_max_n() ? warp_small_estimate(in.N, R_real, sms) : cluster_small_estimate(in.N, R_real, kOpBF16);
-        gathers = us > 5.0;
-    }
     const bool resident = ncsr > 0 && !gathers;
     if (!b->dense_pub.empty() || resident) {
         b->small_host.clear();
@@ -841,10 +846,6 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         cudaError_t e = launch_csr_rows(W, b->graphs, b->stream, &launches);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
     } else if (gathers) {
-        if (b->sets_R != R) {
-            rc = make_sets(b, R);
-            if (rc) return rc;
-        }
         C.nsets = (int32_t)b->sets.size();
         cudaError_t e = launch_csr(C, b->set_max, b->graphs, b->stream, &launches);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
