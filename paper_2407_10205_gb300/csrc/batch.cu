@@ -10,6 +10,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <string>
 #include <thread>
 #include <vector>
@@ -21,6 +22,50 @@
 #include "phia_internal.h"
 
 using namespace phia;
+
+namespace {
+
+// What the choice between the two sparse forms goes by, over all CSR members.
+struct SparseShape {
+    int max_np = 0;                     // most positions (spins rounded up to 32)
+    int64_t rows = 0;
+    double degree = 0.0;                // couplings a row, with those that pad the slices
+    int longest = 0;                    // couplings of the longest row
+};
+
+// Picoseconds per update (spin, replica as run, iteration) of the two sparse forms once an instance
+// fills the GPU, fitted to 20000 .. 60000 spins x 256 .. 1024 replicas of degree 6 .. 60: k_csr.cu
+// with its spins in shared memory (up to 28928 positions) or by position, and k_csr_rows.cu.
+double lanes_ps(const SparseShape &s) {
+    return s.max_np <= 28928 ? 4.55 + 0.023 * s.degree : 4.1 + 0.105 * s.degree;
+}
+double rows_ps(const SparseShape &s) { return 3.5 + 0.052 * s.degree; }
+
+// A row of thousands of couplings among short ones: one warp's way along it, 0.036 us a coupling, can
+// be the whole iteration.
+bool has_hub(const SparseShape &s) { return s.longest >= 2048 && s.longest >= 8.0 * s.degree; }
+
+// Whether a replica count exists for which k_csr_rows.cu is the faster form.  Up to 12544 positions
+// k_csr.cu has x and v in shared memory too and is never slower (10000 x 1024, degree 6: 40 us
+// against 42).
+bool rows_form_possible(const SparseShape &s) {
+    return has_hub(s) || (s.max_np > 12544 && rows_ps(s) < lanes_ps(s));
+}
+
+// Whether a run of `replicas` takes it.  It pads them to 256 instead of 32, and below 5e6 updates an
+// iteration latencies set the time (13000 x 256 of degree 6: 18.3 us against 17.7).  Where a hub sets
+// it (stars: a ring and one row coupled to all), k_csr.cu keeps up with 16-bit offsets and few
+// replicas (10000 x 256 366 us against 368) and not past them (10000 x 1024 657 us against 400, 20000 x
+// 64 878 against 724, 30000 x 64 1870 against 1094).
+bool rows_form(const SparseShape &s, int replicas) {
+    if (!rows_form_possible(s)) return false;
+    const double updates = (double)s.rows * round_up(replicas, 256);
+    const double lanes_us = 1e-6 * (double)s.rows * round_up(replicas, 32) * lanes_ps(s);
+    if (has_hub(s) && 0.036 * s.longest > lanes_us) return s.max_np > 16384 || replicas > 256;
+    return updates >= 5e6 && 1e-6 * updates * rows_ps(s) < lanes_us;
+}
+
+}  // namespace
 
 struct phia_batch_s {
     int device = 0;
@@ -50,7 +95,7 @@ struct phia_batch_s {
     int32_t set_max[4] = {0, 0, 0, 0};
     CsrSet *d_sets = nullptr;
     int64_t total_slices = 0;
-    int max_words = 0, max_np = 0;
+    int max_words = 0;
     CsrInst *d_inst = nullptr;
     CsrBlock *d_blocks = nullptr;
     void *d_col = nullptr;              // uint16 offsets (col16) or uint32
@@ -61,9 +106,7 @@ struct phia_batch_s {
     // the CSR members once more with a row to a warp (k_csr_rows.cu), where some replica count may take it
     std::vector<CsrRowsInst> rows_inst;
     int32_t rows_blocks = 0;
-    int64_t total_rows = 0;
-    double degree = 0.0;                // couplings a row, with those that pad the slices
-    int longest = 0;                    // couplings of the longest row
+    SparseShape shape;
     CsrRowsInst *d_rows_inst = nullptr;
     CsrRowsBlock *d_rows_blocks = nullptr;
     int32_t *d_rows_ptr = nullptr, *d_rows_col = nullptr, *d_rows_h = nullptr;
@@ -134,38 +177,6 @@ void free_state(phia_batch_s *b) {
 }
 
 int64_t words_of(int n) { return (n + 31) / 32; }
-
-// Picoseconds per update (spin, replica as run, iteration) of the two sparse forms once an instance
-// fills the GPU, fitted to 20000 .. 60000 spins x 256 .. 1024 replicas of degree 6 .. 60: k_csr.cu
-// with its spins in shared memory (up to 28928 positions) or by position, and k_csr_rows.cu.
-double lanes_ps(const phia_batch_s *b) {
-    return b->max_np <= 28928 ? 4.55 + 0.023 * b->degree : 4.1 + 0.105 * b->degree;
-}
-double rows_ps(const phia_batch_s *b) { return 3.5 + 0.052 * b->degree; }
-
-// A row of thousands of couplings among short ones: one warp's way along it, 0.036 us a coupling, can
-// be the whole iteration.
-bool has_hub(const phia_batch_s *b) { return b->longest >= 2048 && b->longest >= 8.0 * b->degree; }
-
-// Whether a replica count exists for which k_csr_rows.cu is the faster form.  Up to 12544 positions
-// k_csr.cu has x and v in shared memory too and is never slower (10000 x 1024, degree 6: 40 us
-// against 42).
-bool rows_form_possible(const phia_batch_s *b) {
-    return has_hub(b) || (b->max_np > 12544 && rows_ps(b) < lanes_ps(b));
-}
-
-// Whether a run of `replicas` takes it.  It pads them to 256 instead of 32, and below 5e6 updates an
-// iteration latencies set the time (13000 x 256 of degree 6: 18.3 us against 17.7).  Where a hub sets
-// it (stars: a ring and one row coupled to all), k_csr.cu keeps up with 16-bit offsets and few
-// replicas (10000 x 256 366 us against 368) and not past them (10000 x 1024 657 us against 400, 20000 x
-// 64 878 against 724, 30000 x 64 1870 against 1094).
-bool rows_form(const phia_batch_s *b, int replicas) {
-    if (!b->d_rows_inst) return false;
-    const double updates = (double)b->total_rows * round_up(replicas, 256);
-    const double lanes_us = 1e-6 * (double)b->total_rows * round_up(replicas, 32) * lanes_ps(b);
-    if (has_hub(b) && 0.036 * b->longest > lanes_us) return b->max_np > 16384 || replicas > 256;
-    return updates >= 5e6 && 1e-6 * updates * rows_ps(b) < lanes_us;
-}
 
 // Per-replica offsets for R replicas per instance: records and best states by public
 // index (instance k's records start at k R), CSR state over the CSR members only.
@@ -454,6 +465,26 @@ void pack_instance(const phia_instance_desc &x, int k, int threads, PackedInst &
     pack_slices(n, x.row_ptr, x.col, x.val_k, x.h_k, threads, out);
 }
 
+int64_t csr_device_bytes(int n, const int32_t *row_ptr, int replicas) {
+    const int np = round_up(n, 32);
+    std::vector<int32_t> len((size_t)np, 0);
+    int64_t padded8 = 0;
+    for (int i = 0; i < n; ++i) {
+        len[(size_t)i] = row_ptr[i + 1] - row_ptr[i];
+        padded8 += (len[(size_t)i] + 7) / 8 * 8;
+    }
+    std::sort(len.begin(), len.end(), std::greater<int32_t>());
+    int64_t entries = 0;
+    for (int p = 0; p < np; p += 32) entries += (len[(size_t)p] + 3) / 4;
+    const SparseShape s{np, n, 128.0 * (double)entries / n, len[0]};
+    const int64_t R = round_up(replicas, rows_form(s, replicas) ? 256 : 32);
+    int64_t b = entries * 32 * (np <= 16384 ? 12 : 20) + (int64_t)np * 20;           // slices, h, positions
+    if (rows_form_possible(s)) b += padded8 * 5 + (int64_t)n * 8;
+    if (n <= cluster_batch_max_n()) b += (int64_t)n * n;
+    b += (int64_t)np * R * 8 + 4 * (int64_t)np * (R / 32) * 4;                       // x, v, spins
+    return b + R * (16 + 2 + 24 + 8) + R * words_of(n) * 4;                          // sums, flags, records
+}
+
 int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d, const phia_opts *opts) {
     if (!out) return bfail(PHIA_EINVAL, "out is NULL");
     *out = nullptr;
@@ -556,18 +587,18 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         row_of.insert(row_of.end(), pk.row_of.begin(), pk.row_of.end());
         pos_of.insert(pos_of.end(), pk.pos_of.begin(), pk.pos_of.end());
         pk = PackedInst();
-        b->max_np = std::max(b->max_np, in.Np);
+        b->shape.max_np = std::max(b->shape.max_np, in.Np);
         b->total_slices += in.Np / 32;
-        b->total_rows += n;
-        b->longest = std::max(b->longest, longest);
+        b->shape.rows += n;
+        b->shape.longest = std::max(b->shape.longest, longest);
         b->inst.push_back(in);
     }
     std::vector<int32_t> rows_ptr, rows_col, rows_h;
     std::vector<int8_t> rows_val;
     std::vector<CsrRowsBlock> rows_blocks;
-    b->degree = b->total_rows ? 4.0 * (double)(slice.empty() ? 0 : slice.back()) * 32.0 / (double)b->total_rows : 0.0;
-    if (rows_form_possible(b)) {
-        const size_t most = (size_t)(b->degree * (double)b->total_rows) + 8 * (size_t)b->total_rows;
+    b->shape.degree = b->shape.rows ? 4.0 * (double)(slice.empty() ? 0 : slice.back()) * 32.0 / (double)b->shape.rows : 0.0;
+    if (rows_form_possible(b->shape)) {
+        const size_t most = (size_t)(b->shape.degree * (double)b->shape.rows) + 8 * (size_t)b->shape.rows;
         rows_col.reserve(most);
         rows_val.reserve(most);
         int64_t row_base = 0;
@@ -614,7 +645,7 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         if (ok && bytes && cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, b->stream) != cudaSuccess) ok = false;
     };
     up((void **)&b->d_slice, slice.data(), slice.size() * 4);
-    b->col16 = b->max_np <= 16384;
+    b->col16 = b->shape.max_np <= 16384;
     std::vector<uint16_t> col16;
     if (b->col16) col16.assign(col.begin(), col.end());
     if (b->col16) up(&b->d_col, col16.data(), col16.size() * 2);
@@ -671,7 +702,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         if (total > ((int64_t)1 << 31)) return bfail(PHIA_ERANGE, "total_steps must be < 2^31");
     }
     if (R_real < 1) return bfail(PHIA_EINVAL, "replicas must be >= 1");
-    const bool by_rows = !field_mode && rows_form(b, R_real);
+    const bool by_rows = !field_mode && b->d_rows_inst && rows_form(b->shape, R_real);
     const int R = round_up(R_real, by_rows ? 256 : 32);
     BCU(cudaSetDevice(b->device));
     if (!field_mode && !reset && (!b->ran || b->R_real != R_real))
@@ -739,7 +770,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     C.inst = b->d_inst; C.count = ncsr;
     C.blocks = b->d_blocks;
     C.sets = b->d_sets;
-    C.max_np = b->max_np;
+    C.max_np = b->shape.max_np;
     C.slice = b->d_slice; C.col = b->d_col; C.col16 = b->col16 ? 1 : 0; C.val = b->d_val; C.hk = b->d_hk2;
     C.row_of = b->d_rowof; C.pos_of = b->d_posof;
     C.X = b->d_X; C.V = b->d_V;
@@ -835,13 +866,13 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         W.row_ptr = b->d_rows_ptr; W.col = b->d_rows_col; W.val = b->d_rows_val; W.hk = b->d_rows_h;
         W.X = C.X; W.V = C.V;
         W.x_in = x_in; W.v_in = v_in; W.x_out = x_out; W.v_out = v_out;
-        W.S = C.S; W.total_swords = b->total_rows * (R / 32);
+        W.S = C.S; W.total_swords = b->shape.rows * (R / 32);
         W.Esum = C.Esum; W.flags = C.flags; W.total_reps = reps;
         W.best_bits = C.best_bits;
         W.targets = C.targets;
         W.R = R; W.R_real = R_real;
         W.max_words = C.max_words;
-        W.total_rows = b->total_rows;
+        W.total_rows = b->shape.rows;
         W.ctl = C.ctl; W.persistent = C.persistent; W.sync = C.sync;
         cudaError_t e = launch_csr_rows(W, b->graphs, b->stream, &launches);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));

@@ -300,6 +300,8 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
 int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64_t t0, int64_t steps, int64_t total,
               uint64_t seed, const float *x_in, float *x_out, const float *v_in, float *v_out, int reset,
               const int8_t *spins_in, int32_t *field_out, int64_t *energy_out);
+// Device bytes of a batch of one checked CSR instance with `replicas` replicas.
+int64_t csr_device_bytes(int n, const int32_t *row_ptr, int replicas);
 int batch_best(phia_batch_s *b, int inst, int64_t *energy_k, int8_t *spins);
 int batch_replica_results(phia_batch_s *b, int inst, int32_t R, int64_t *be, int64_t *bs, int64_t *hs, uint32_t *bits);
 int batch_stats(phia_batch_s *b, int inst, phia_stats *out);

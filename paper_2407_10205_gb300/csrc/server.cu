@@ -98,8 +98,7 @@ int64_t estimate_bytes(const Request &r, bool fp32) {
         const int64_t Kb = (N * 2 + 127) / 128 * 128, Mp = (N + 127) / 128 * 128;
         b += Mp * Kb + 4 * ((R + 127) / 128 * 128) * Kb + R * N * 8;   // operand, spin buffers, state
     } else {
-        b += (int64_t)r.col.size() * 5 + (N + 1) * 4;                 // CSR
-        b += Rp * N * 8 + 4 * N * (Rp / 32) * 4;                      // state, spin bits
+        b += csr_device_bytes(r.N, r.row_ptr.data(), (int)R);
     }
     return b + (1 << 20);
 }

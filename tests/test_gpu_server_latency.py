@@ -41,3 +41,21 @@ def test_large_dense_requests_in_turns_equal_the_same_alone(gpu_lib):
             alone = A.anneal(sched, 300, 160, 5 + k)
         assert st.state == 2 and st.energy_k == alone.energy_k
         assert (spins == alone.spins).all()
+
+
+def test_the_budget_counts_what_a_sparse_request_takes(gpu_lib):
+    """Slices pad the rows, and large instances keep their couplings twice (some 10 bytes each): a budget
+    that holds the rest of the request and 5 bytes a coupling is not enough."""
+    phia = gpu_lib
+    n, R = 40000, 256
+    c = ins.erdos_renyi(n, 100.0 / n, 127, 31, 4, 1)
+    rest = 2 * R * n * 4 + n * 8 * 256 + 4 * n * 8 * 4 + 256 * (24 + n // 8) + 8 * n + (1 << 20)
+    sched = phia.schedule(0.02, 0.5, 0.1, 2.0)
+    with phia.Server(max_inflight=1, hbm_budget_bytes=rest + 5 * c.nnz) as S:
+        with pytest.raises(phia.PhiaError) as e:
+            S.submit(c, sched, R, 10, seed=1)
+        assert e.value.code == phia.ENOMEM
+    with phia.Server(max_inflight=1, hbm_budget_bytes=rest + 12 * c.nnz) as S:
+        rid = S.submit(c, sched, R, 10, seed=1)
+        S.wait_all()
+        assert S.poll(rid)[0].state == 2
