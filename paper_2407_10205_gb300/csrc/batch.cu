@@ -19,6 +19,7 @@
 
 #include "../../include/phia.h"
 #include "device_common.cuh"
+#include "grow.h"
 #include "phia_internal.h"
 
 using namespace phia;
@@ -843,12 +844,12 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
                 for (size_t m = 0; m < b->csr_pub.size(); ++m) add(b->csr_pub[m], b->cand_joff[m]);
             if (b->small_host.size() > beg) groups.push_back(SmallGroup{beg, b->small_host.size(), nmax, cls.kernel});
         }
-        if (b->small_host.size() > b->small_cap) {
-            pool_free(b->d_small, b->stream);
-            b->d_small = nullptr;
-            if (pool_alloc((void **)&b->d_small, b->small_host.size() * sizeof(SmallCta), b->device, b->stream) != cudaSuccess)
-                return bfail(PHIA_ENOMEM, "CTA table allocation failed");
-            b->small_cap = b->small_host.size();
+        auto take = [&](SmallCta **q, size_t bytes) {
+            return pool_alloc((void **)q, bytes, b->device, b->stream) == cudaSuccess;
+        };
+        if (!grow_table(b->d_small, b->small_cap, b->small_host.size(), take, [&](SmallCta *q) { pool_free(q, b->stream); })) {
+            cudaGetLastError();
+            return bfail(PHIA_ENOMEM, "CTA table allocation failed");
         }
         BCU(cudaMemcpyAsync(b->d_small, b->small_host.data(), b->small_host.size() * sizeof(SmallCta),
                             cudaMemcpyHostToDevice, b->stream));
