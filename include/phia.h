@@ -210,10 +210,10 @@ int phia_anneal(phia_t *p, const phia_schedule *sched, int32_t replicas, int64_t
 /* Autotuner.  Times short probe runs (probe_iters iterations of `replicas` replicas) of
  * every tensor-core kernel variant that applies to this handle -- the resident tcgen05
  * kernel with 4, 8 or 16 replicas per CTA and J in shared or tensor memory, the
- * resident warp-level kernel (two candidates, alike; N small enough), the
+ * resident warp-level kernel (two settings of the same form; N small enough), the
  * resident incremental-field kernel with 4, 8 or 16 replicas per CTA (N small enough),
- * and the per-iteration kernel in its thirteen variants (phia_opts.large_variant; those that
- * run the same form as another are counted and timed once) -- keeps the fastest for the handle and caches it,
+ * and the per-iteration kernel in its thirteen variants (phia_opts.large_variant); settings that
+ * run the form of another are counted among the candidates and timed once -- keeps the fastest for the handle and caches it,
  * process-wide, for (N, replicas, operand): handles created with all variant options
  * automatic use the cached choice for runs with that replica count.  The probes
  * overwrite the handle's last-run records.  Tensor-core path only (else PHIA_ENOTSUP). */

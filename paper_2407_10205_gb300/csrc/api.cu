@@ -826,17 +826,19 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
         for (int tile : {4, 8, 16})
             for (int mem : {1, 2}) cands.push_back(TuneChoice{false, tile, mem, false, false, 0});
     }
+    // Settings that run the form of another are counted and timed once: the warp-level kernel has 8
+    // replicas per CTA whatever is asked for, and variants 3 .. 6, 8 and 9 of the per-iteration kernel
+    // run the forms of 2, 1, 10 and 12.
+    int same_form = 6;
     if (p->N <= warp_small_max_n()) {
         cands.push_back(TuneChoice{false, 8, 0, true, false, 0});
-        cands.push_back(TuneChoice{false, 16, 0, true, false, 0});
+        ++same_form;
     }
     if (p->N <= std::min(inc_small_max_n(), tc_small_max_n(p->op))) {
         for (int tile : {4, 8, 16})
             if (inc_small_tile_replicas(p->N, tile) == tile)
                 cands.push_back(TuneChoice{false, tile, 0, false, true, 0});
     }
-    // Variants 3 .. 6, 8 and 9 run the forms of 2, 1, 10 and 12.
-    constexpr int kSameForm = 6;
     for (int lv : {1, 2, 7, 10, 11, 12, 13}) cands.push_back(TuneChoice{true, 0, 0, false, false, lv});
     // The probes run the candidates: not the kernel of before an acceptance run, which the first of them
     // would go back to, with the candidate's choice overwritten.
@@ -874,7 +876,7 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
         out->tile_replicas = best.large ? 0
                              : (best.warpk || best.inc ? best.tile_rl : tc_small_tile_replicas(replicas, best.tile_rl));
         out->coupling_mem = best.large || best.warpk || best.inc ? 0 : best.coupling_mem;
-        out->candidates = (int32_t)cands.size() + kSameForm;
+        out->candidates = (int32_t)cands.size() + same_form;
         out->best_us_per_iter = 1000.f * best_ms / probe_iters;
         out->worst_us_per_iter = 1000.f * worst_ms / probe_iters;
         out->large_variant = best.large ? best.lvar : 0;

@@ -75,3 +75,17 @@ def test_a_run_goes_on_after_an_acceptance_run(gpu_lib):
     assert (out[0][1] < 20).any()
     for u, w in zip(*out):
         assert np.array_equal(u, w)
+
+
+def test_the_warp_kernels_tile_is_reported_as_it_is(gpu_lib):
+    """It runs 8 replicas per CTA, whatever is asked for."""
+    phia = gpu_lib
+    sched, seen = phia.schedule(0.01, 0.1, 0.1, 2.0, refresh=50), 0
+    for N in (8, 16, 24, 32, 48, 64):
+        d = ins.dense_int(N, 7, 7, N)
+        with phia.Annealer(d.k, d.kh, path=phia.PATH_TC, instance_id=9) as A:
+            res = phia.autotune(A.h, sched, 72, probe_iters=100)
+        if res.tc_kernel == 3:
+            seen += 1
+            assert res.tile_replicas == 8
+    assert seen
