@@ -356,7 +356,7 @@ def mma_probe(phia):
     return out
 
 
-def _roofline(w, kernel_ms, stats, peaks, src, probe=None, large_variant=0):
+def _roofline(w, kernel_ms, stats, peaks, src, probe=None):
     """Roofline of the dominant kernel of a dense workload.  The field (Eq. 6) is a dense
     contraction of 2 N flops per spin update (2 R N^2 per iteration): achieved = those
     flops / device time, against the e4m3 tensor peak taken as the measured bf16 burst
@@ -371,7 +371,8 @@ def _roofline(w, kernel_ms, stats, peaks, src, probe=None, large_variant=0):
     bf16_peak = float(peaks["bf16_tflops"])
     peak = 2.0 * bf16_peak if e4m3 else bf16_peak
     achieved = 2.0 * N * su / (kernel_ms * 1e-3) / 1e12
-    kname = {1: "tc_small_kernel", 2: "tc_flow_run" if large_variant >= 7 else "tc_large_step",
+    kname = {1: "tc_small_kernel",
+             2: {1: "tc_large_step", 2: "tc_flow_run", 3: "tc_narrow_run", 4: "cluster_small_kernel"}.get(stats.large_form, "?"),
              3: "warp_small_kernel", 4: "inc_small_kernel"}.get(stats.tc_kernel, "?")
     out = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
            "traffic": KERNEL_TRAFFIC_BYTES.get(kname), "kernel": kname,
@@ -383,7 +384,7 @@ def _roofline(w, kernel_ms, stats, peaks, src, probe=None, large_variant=0):
         if mp:
             out["probe_peak"] = mp
             out["frac_of_probe_peak"] = achieved / mp
-    if stats.tc_kernel == 2:
+    if stats.large_form in (1, 2):       # x and v go through memory every iteration
         # per iteration: one launch of tc_large_step; tc_flow_run runs all T in one launch,
         # so its per-launch figures are T times these over T times the time
         launch_ms = kernel_ms / T
@@ -821,8 +822,7 @@ def measure_dense(args, w, rank=0, world=1, local=0, with_cpu=True, dist=None):
     value = world * su_step / (ms_per_step * 1e-3)
 
     # e2e: public C ABI from host buffers, host<->device copies inside the timed region, on
-    # the kernel the autotuner chose (named explicitly: a new automatic handle would not take
-    # a cooperative variant)
+    # the kernel the autotuner chose (named explicitly)
     e2e_ms = []
     for k in range(max(2, min(args.steps, 3))):
         torch.cuda.synchronize()
@@ -872,7 +872,7 @@ def measure_dense(args, w, rank=0, world=1, local=0, with_cpu=True, dist=None):
                    "parallelism": f"replicas sharded over {world} GPU(s), no collective"},
         "e2e": {"value": su_step / (e2e_step * 1e-3), "unit": METRIC, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "ms_per_step": e2e_step},
-        "roofline": _roofline(w, kernel_ms, st, peaks, src, probe, tune.large_variant),
+        "roofline": _roofline(w, kernel_ms, st, peaks, src, probe),
         "gpu_launches": launches,
         "clocks": cs.summary(),
         "comparator": {"path": "fp32 per-instance, one launch per step", "value": cmp_value, "unit": METRIC,

@@ -161,7 +161,9 @@ typedef struct phia_stats {
     int32_t tc_kernel;     /* dense kernel used (1 resident tcgen05, 2 per iteration, overlapped or
                               over clusters, 3 resident warp-level, 4 resident incremental field),
                               0 for other paths */
-    int32_t reserved0;     /* 0 */
+    int32_t large_form;    /* where tc_kernel is 2, what ran: 1 one launch per iteration, 2 overlapped,
+                              3 overlapped with tiles of 32 or 64 spins, 4 over thread-block
+                              clusters; else 0 */
     int64_t hit_ns;        /* device time to target: %globaltimer nanoseconds from the start of
                               the run (its record reset, the first call of a resumed run) to
                               the recording of hit_step for hit_replica, or -1.  The resident

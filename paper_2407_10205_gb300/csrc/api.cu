@@ -105,6 +105,7 @@ struct phia_s {
     bool large = false;                 // tensor-core path through the per-iteration kernel
     bool warpk = false;                 // tensor-core path through the warp-level resident kernel
     int last_kernel = 0;                // stats.tc_kernel of the last run
+    int last_form = 0;                  // ... and large_form
     bool inc = false;                   // dense path through the incremental-field resident kernel
     void *d_Jop = nullptr;              // couplings in the operand encoding (per-iteration kernel)
     int Mpad = 0, Kbytes = 0;
@@ -443,6 +444,7 @@ cudaError_t launch_path(phia_t *p, const RunArgs &a, int *launches) {
     const bool cluster = takes_cluster(p, a), warp = !cluster && takes_warp(p, a);
     if (!a.field_mode)
         p->last_kernel = p->path != PHIA_PATH_TC ? 0 : p->large || cluster ? 2 : warp ? 3 : p->inc ? 4 : 1;
+    if (!a.field_mode) p->last_form = cluster ? 4 : 0;
     if (cluster) return launch_cluster_small(a, p->op, p->stream, launches);
     if (p->path == PHIA_PATH_TC && p->large) {
         LargeBuffers B;
@@ -450,7 +452,7 @@ cudaError_t launch_path(phia_t *p, const RunArgs &a, int *launches) {
         B.sbits = p->d_sbits;
         B.X = p->d_X; B.V = p->d_V; B.Kbytes = p->Kbytes; B.Mpad = p->Mpad; B.Rpad = large_rpad_handle(a.R);
         B.ctl = p->d_ctl; B.graphs = p->graphs;
-        return launch_tc_large(B, a, p->op, p->stream, launches);
+        return launch_tc_large(B, a, p->op, p->stream, launches, a.field_mode ? nullptr : &p->last_form);
     }
     // The warp-level and the incremental kernel have no field-only mode: the resident tcgen05
     // kernel covers the same sizes.
@@ -1028,6 +1030,7 @@ int phia_gahmc(phia_t *p, const phia_gahmc_schedule *sched, int32_t R, int64_t K
     a.x_in = x; a.v_in = v; a.x_out = x; a.v_out = v;
     a.has_target = sched->has_target; a.target = sched->target_k;
     CU(cudaEventRecord(p->ev0, p->stream));
+    p->last_form = 0;
     p->last_kernel = p->large ? 2 : p->inc ? 4 : p->warpk && !p->auto_tile ? 3 : 1;
     cudaError_t e = launch_gahmc(a, sched->travel, K, counts, events, events_cap, p->stream);
     if (e != cudaSuccess) return fail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
@@ -1097,6 +1100,7 @@ int phia_stats_get(phia_t *p, phia_stats *out) {
     out->operand = p->op == kOpE4M3 ? PHIA_OP_E4M3 : (p->op == kOpBF16 ? PHIA_OP_BF16 : 0);
     out->kernel_launches = p->last_launches;
     out->tc_kernel = p->last_kernel;
+    out->large_form = p->last_form;
     return PHIA_OK;
 }
 

@@ -1365,7 +1365,9 @@ bool tc_operand_map(void *map, const void *base, int op, uint64_t inner_elems, u
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cudaStream_t st, int *launches) {
+cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cudaStream_t st, int *launches, int *form) {
+    int other = 0;
+    int &ran = form ? *form : other;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1396,18 +1398,23 @@ cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cud
         }
         int width = 0;
         const double narrow = narrow_estimate(a.N, a.R, B.Kbytes, sms, &width);
-        if (!a.stall_producer && cluster_small_estimate(a.N, a.R, op) < std::min(narrow, wide))
+        if (!a.stall_producer && cluster_small_estimate(a.N, a.R, op) < std::min(narrow, wide)) {
+            ran = 4;
             return launch_cluster_small(a, op, st, launches);
+        }
         // A run beside others holds at most half of the SMs; a larger one takes its turns launch by
         // launch.  In one cooperative launch it would hold them for all of its iterations (22 us each at
         // N = 6000 x 256), and each iteration of a sparse run beside it would wait for its end.
         const int64_t tiles = narrow < wide ? (int64_t)((a.N + width - 1) / width) * ((a.R + 127) / 128) : sms;
         if (a.in_turns && 2 * tiles > sms) lv = 1;
-        else if (narrow < wide) return launch_tc_narrow(B, a, op, width, st, launches, sms);
-        else lv = 7;
+        else if (narrow < wide) {
+            ran = 3;
+            return launch_tc_narrow(B, a, op, width, st, launches, sms);
+        } else lv = 7;
     } else if (a.in_turns && lv >= 7) {
         lv = 1;
     }
+    ran = lv >= 7 && B.ready && B.sbits && !a.field_mode ? 2 : 1;
     if ((lv == 7 || lv >= 10) && B.ready && B.sbits && !a.field_mode) {
         const int mt = B.Mpad / kBM;
         const int want = lv == 10 ? 256 : lv == 11 ? 224 : lv == 12 ? 128 : lv == 13 ? 160 : 0;

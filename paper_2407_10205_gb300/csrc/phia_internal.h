@@ -149,7 +149,9 @@ struct LargeBuffers {
     uint32_t *sbits;      // [4][Rpad][Mpad/32] packed spins of the overlapped variant, or null
     int32_t Kbytes, Mpad, Rpad;
 };
-cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cudaStream_t st, int *launches);
+// *form: what ran (phia_stats.large_form).
+cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cudaStream_t st, int *launches,
+                            int *form = nullptr);
 // The overlapped kernel with narrow tiles (width 32 or 64 output spins; one cooperative launch
 // per call): needs B.ready and B.sbits.
 cudaError_t launch_tc_narrow(const LargeBuffers &B, const RunArgs &a, int op, int width, cudaStream_t st, int *launches,

@@ -53,7 +53,7 @@ class Stats(ctypes.Structure):
                 ("best_step", ctypes.c_int64), ("hit_step", ctypes.c_int64), ("hit_replica", ctypes.c_int64),
                 ("device_ms", ctypes.c_float), ("path", ctypes.c_int32), ("operand", ctypes.c_int32),
                 ("kernel_launches", ctypes.c_int32), ("tc_kernel", ctypes.c_int32),
-                ("reserved0", ctypes.c_int32), ("hit_ns", ctypes.c_int64)]
+                ("large_form", ctypes.c_int32), ("hit_ns", ctypes.c_int64)]
 
 
 class InstanceDesc(ctypes.Structure):

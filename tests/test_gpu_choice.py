@@ -89,3 +89,19 @@ def test_the_warp_kernels_tile_is_reported_as_it_is(gpu_lib):
             seen += 1
             assert res.tile_replicas == 8
     assert seen
+
+
+@pytest.mark.parametrize("N,R,variant,form", [(2000, 4096, 0, 2), (2000, 4096, 1, 1), (2000, 4096, 11, 2), (1500, 256, 7, 3),
+                                              (600, 64, 7, 4), (600, 64, 0, 4), (600, 64, 12, 2)])
+def test_stats_name_the_form_that_ran(gpu_lib, N, R, variant, form):
+    phia = gpu_lib
+    d = ins.sk_pm1(N, 1)
+    with phia.Annealer(d.k, d.kh, path=phia.PATH_TC, tc_kernel=phia.KERNEL_PER_STEP, large_variant=variant) as A:
+        phia.anneal(A.h, phia.schedule(0.01, 0.1, 0.1, 2.0), R, 4, 1)
+        st = phia.stats_get(A.h)
+        assert (st.tc_kernel, st.large_form) == (2, form)
+    d = ins.sk_pm1(300, 1)
+    with phia.Annealer(d.k, d.kh, path=phia.PATH_TC) as A:
+        phia.anneal(A.h, phia.schedule(0.01, 0.1, 0.1, 2.0), 64, 4, 1)
+        st = phia.stats_get(A.h)
+        assert (st.tc_kernel, st.large_form) in ((2, 4), (1, 0))
