@@ -437,7 +437,7 @@ bool takes_cluster(const phia_t *p, const RunArgs &a) {
     const double other = takes_warp(p, a) ? warp_small_estimate(p->N, a.R, sms)
                                           : waves * ((p->N <= 256 ? 1.2 : 1.9) + (per_cta == 16 ? 0.5 : 0.0) +
                                                      (p->op == kOpBF16 ? 0.35 : 0.0));
-    return cluster_small_estimate(p->N, a.R, p->op) < other;
+    return cluster_small_estimate(p->N, a.R, p->op, sms, other) < other;
 }
 
 cudaError_t launch_path(phia_t *p, const RunArgs &a, int *launches) {

@@ -727,7 +727,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         BCU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
         double us = 0.0;
         for (const CsrInst &in : b->inst)
-            us += in.N <= warp_small_max_n() ? warp_small_estimate(in.N, R_real, sms) : cluster_small_estimate(in.N, R_real, kOpBF16);
+            us += in.N <= warp_small_max_n() ? warp_small_estimate(in.N, R_real, sms) : cluster_small_estimate(in.N, R_real, kOpBF16, sms, 5.0);
         gathers = us > 5.0;
     }
     if (gathers && !by_rows && !field_mode && b->sets_R != R) {      // host work: before the run's time begins

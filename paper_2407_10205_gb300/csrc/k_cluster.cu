@@ -298,15 +298,21 @@ cudaError_t dispatch(const RunArgs *a, int N, int clusters, cudaStream_t st, int
 int cluster_small_min_n() { return 128; }          // rank 0 settles a replica per warp
 int cluster_small_max_n(int op) { return op == kOpE4M3 ? 1024 : 512; }
 
-double cluster_small_estimate(int N, int R, int op) {
+double cluster_small_estimate(int N, int R, int op, int sms, double limit) {
     if (N < cluster_small_min_n() || N > cluster_small_max_n(op)) return 1e30;
+    const double wave = N <= 512 ? 0.8 + 0.0009 * N : 0.8 + 0.0016 * N;
+    // The number of clusters that the GPU holds is asked of the kernel, which loads its code once per
+    // process (a first run at N = 600 x 2000 replicas 1.0 ms without it, 2.1 with it): not where CTAs on all
+    // SMs, one on each (168 registers a thread and more), would not be fast enough.
+    const int cl = (N + 127) / 128, most = std::max(1, N > 256 && N <= 384 ? sms / 2 : sms / cl);
+    if (((R + 7) / 8 + most - 1) / most * wave >= limit) return 1e30;
     int resident = 0;
     if (dispatch<false>(nullptr, N, 1, nullptr, &resident) != cudaSuccess || resident < 1) {
         cudaGetLastError();
         return 1e30;
     }
     const int waves = ((R + 7) / 8 + resident - 1) / resident;
-    return waves * (N <= 512 ? 0.8 + 0.0009 * N : 0.8 + 0.0016 * N);
+    return waves * wave;
 }
 
 cudaError_t launch_cluster_small(const RunArgs &a, int op, cudaStream_t st, int *launches) {

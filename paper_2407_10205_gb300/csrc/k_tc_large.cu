@@ -1398,7 +1398,7 @@ cudaError_t launch_tc_large(const LargeBuffers &B, const RunArgs &a, int op, cud
         }
         int width = 0;
         const double narrow = narrow_estimate(a.N, a.R, B.Kbytes, sms, &width);
-        if (!a.stall_producer && cluster_small_estimate(a.N, a.R, op) < std::min(narrow, wide)) {
+        if (!a.stall_producer && cluster_small_estimate(a.N, a.R, op, sms, std::min(narrow, wide)) < std::min(narrow, wide)) {
             ran = 4;
             return launch_cluster_small(a, op, st, launches);
         }

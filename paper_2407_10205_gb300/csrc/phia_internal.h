@@ -333,8 +333,8 @@ double warp_small_estimate(int N, int R, int sms);
 int cluster_small_min_n();
 int cluster_small_max_n(int op);
 cudaError_t launch_cluster_small(const RunArgs &a, int op, cudaStream_t st, int *launches);
-// Its estimated time per iteration (us; 1e30 where it does not apply).
-double cluster_small_estimate(int N, int R, int op);
+// Its estimated time per iteration (us; 1e30 where it does not apply, or cannot be below `limit`).
+double cluster_small_estimate(int N, int R, int op, int sms, double limit);
 // And over a table of clusters (a.small_cta) of instances of 257 .. nmax spins, or of 385 .. nmax
 // where nmax > 384 (every CTA of a cluster has to own spins); nmax <= cluster_batch_max_n().
 int cluster_batch_max_n();
