@@ -11,7 +11,9 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <new>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -285,6 +287,17 @@ int ensure_state(phia_batch_s *b, int R) {
 
 namespace phia {
 
+// Starts fn on a thread of `workers` (which has room for it); false where the system has none left.
+template <typename F>
+bool start_thread(std::vector<std::thread> &workers, F fn) {
+    try {
+        workers.emplace_back(fn);
+        return true;
+    } catch (const std::system_error &) {
+        return false;
+    }
+}
+
 // One instance of a batch, checked and converted to slices of 32 rows (relative to the
 // instance), before concatenation; code/msg hold its first error.
 struct PackedInst {
@@ -353,12 +366,12 @@ void pack_slices(int n, const int32_t *rp, const int32_t *col, const int8_t *val
     };
     const int nt = std::min<int>({threads, ns, rp[n] / 65536 + 1});
     std::vector<std::thread> workers;
+    workers.reserve((size_t)nt);
     int done = 0;                                  // slices given out, by entries
     for (int k = 1; k <= nt; ++k) {
         int next = done;
         while (next < ns && (k == nt || (int64_t)out.slice[(size_t)next] * nt < (int64_t)out.slice[(size_t)ns] * k)) ++next;
-        if (k < nt) workers.emplace_back(fill, done, next);
-        else fill(done, next);
+        if (k == nt || !start_thread(workers, [&fill, done, next] { fill(done, next); })) fill(done, next);
         done = next;
     }
     for (std::thread &w : workers) w.join();
@@ -486,18 +499,21 @@ int64_t csr_device_bytes(int n, const int32_t *row_ptr, int replicas) {
     return b + R * (16 + 2 + 24 + 8) + R * words_of(n) * 4;                          // sums, flags, records
 }
 
-int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d, const phia_opts *opts) {
-    if (!out) return bfail(PHIA_EINVAL, "out is NULL");
-    *out = nullptr;
+// batch_create; b: the batch as far as it got, for the caller to destroy after an exception.
+int create_batch(phia_batch_s *&b, phia_batch_s **out, int32_t count, const phia_instance_desc *d, const phia_opts *opts) {
     if (count < 1 || !d) return bfail(PHIA_EINVAL, "need count >= 1 and descriptors");
     phia_opts o{};
     if (opts) o = *opts;
     if (o.path != PHIA_PATH_AUTO && o.path != PHIA_PATH_CSR)
         return bfail(PHIA_ENOTSUP, "batches run on the CSR path");
     if (o.tc_kernel < 0 || o.tc_kernel > 2) return bfail(PHIA_EINVAL, "batches: tc_kernel must be 0, 1 or 2");
-    phia_batch_s *b = new phia_batch_s();
+    b = new phia_batch_s();
     b->csr_mode = o.tc_kernel == 1 ? 1 : 2;
-    auto cleanup = [&](int code) { phia_batch_destroy(b); return code; };
+    auto cleanup = [&](int code) {
+        phia_batch_destroy(b);
+        b = nullptr;
+        return code;
+    };
     b->count = count;
     // Instances are checked and converted independently, on every host core (a batch of
     // 256 instances with 2.8e7 couplings took 1.3 s on one core); the first failing
@@ -508,10 +524,19 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
         const int cores = std::max(1, (int)std::thread::hardware_concurrency());
         const int nthreads = std::min<int>(count, cores);
         auto work = [&]() {
-            for (int k; (k = next.fetch_add(1)) < count;) pack_instance(d[k], k, cores / nthreads, packed[(size_t)k]);
+            for (int k; (k = next.fetch_add(1)) < count;) {
+                try {
+                    pack_instance(d[k], k, cores / nthreads, packed[(size_t)k]);
+                } catch (const std::bad_alloc &) {
+                    packed[(size_t)k] = PackedInst();
+                    packed[(size_t)k].code = PHIA_ENOMEM;
+                    packed[(size_t)k].msg = "no host memory";
+                }
+            }
         };
         std::vector<std::thread> workers;
-        for (int t = 1; t < nthreads; ++t) workers.emplace_back(work);
+        workers.reserve((size_t)nthreads);
+        for (int t = 1; t < nthreads && start_thread(workers, work); ++t) {}
         work();
         for (std::thread &t : workers) t.join();
     }
@@ -687,9 +712,21 @@ int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d,
     return PHIA_OK;
 }
 
+int batch_create(phia_batch_s **out, int32_t count, const phia_instance_desc *d, const phia_opts *opts) {
+    if (!out) return bfail(PHIA_EINVAL, "out is NULL");
+    *out = nullptr;
+    phia_batch_s *b = nullptr;
+    try {
+        return create_batch(b, out, count, d, opts);
+    } catch (const std::bad_alloc &) {
+        phia_batch_destroy(b);
+        return bfail(PHIA_ENOMEM, "no host memory for the batch");
+    }
+}
+
 int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64_t t0, int64_t steps, int64_t total,
               uint64_t seed, const float *x_in, float *x_out, const float *v_in, float *v_out, int reset,
-              const int8_t *spins_in, int32_t *field_out, int64_t *energy_out) {
+              const int8_t *spins_in, int32_t *field_out, int64_t *energy_out) try {
     if (!b) return bfail(PHIA_EINVAL, "batch is NULL");
     const bool field_mode = spins_in != nullptr;
     if (!field_mode) {
@@ -907,6 +944,8 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         b->last_stop = sched->stop_at_target;
     }
     return PHIA_OK;
+} catch (const std::bad_alloc &) {
+    return bfail(PHIA_ENOMEM, "no host memory for the run");
 }
 
 // Per-replica records of one instance (first R_real replicas).
