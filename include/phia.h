@@ -61,7 +61,7 @@ extern "C" {
 #define PHIA_PATH_AUTO 0   /* dense -> PHIA_PATH_TC, CSR -> PHIA_PATH_CSR */
 #define PHIA_PATH_TC 1     /* tcgen05 tensor-core MMA, FP32 accumulation of integer products */
 #define PHIA_PATH_FP32 2   /* plain FP32 CUDA-core mat-vec, one launch per step (comparator) */
-#define PHIA_PATH_CSR 3    /* warp-per-row CSR gather over bit-packed spins */
+#define PHIA_PATH_CSR 3    /* sparse instances: gather over bit-packed spins, small ones resident */
 
 /* Tensor-core operand encoding of the int8 couplings (exact re-encodings of k). */
 #define PHIA_OP_AUTO 0     /* E4M3 when every |k| <= 16, else BF16 */
@@ -79,8 +79,9 @@ typedef struct phia_opts {
     int32_t coupling_mem;  /* tensor-core path, where J stays during a run: 1 = shared memory,
                               2 = tensor memory; 0 = automatic */
     int32_t tc_kernel;     /* tensor-core path: 1 = resident tcgen05 kernel (all iterations in one
-                              launch, J on chip; N <= 384 e4m3 / 256 bf16), 2 = one launch per
-                              iteration (J streamed by TMA; any N), 3 = resident warp-level
+                              launch, J on chip; N <= 384 e4m3 / 256 bf16), 2 = the kernels for
+                              any N (J streamed by TMA): which of them large_variant says, one
+                              launch per iteration with 1 .. 6, else by estimate, 3 = resident warp-level
                               kernel (mma.sync with bf16 operands, J in registers; N <= 256;
                               8 replicas per CTA whatever tile_replicas says), 4 = resident incremental-field kernel
                               (CUDA cores: the exact integer field is updated by the columns of
@@ -104,8 +105,9 @@ typedef struct phia_opts {
                               e4m3, 512 bf16) or overlapped tiles of 128 replicas x 32 or 64
                               spins with x, v in registers; 8 / 9 = as 10, or
                               as 12 where 256-wide tiles are fewer than the SMs; 10 / 11 / 12 /
-                              13 = overlapped with 256- / 224- / 128- / 160-wide tiles; 0 = automatic (the autotuner's choice where it
-                              has one, else as 7) */
+                              13 = overlapped with 256- / 224- / 128- / 160-wide tiles; 0 = automatic
+                              (the autotuner's choice where it has one, else as 7; a server's
+                              requests as 1 where others run and 7 would hold most SMs) */
 } phia_opts;
 
 /* Annealing schedule.  No values are given in the paper; every field is explicit. */
@@ -155,7 +157,8 @@ typedef struct phia_stats {
     int64_t hit_step;      /* earliest iteration with E <= target over replicas, or -1 */
     int64_t hit_replica;   /* lowest replica index hitting at hit_step, or -1 */
     float device_ms;       /* device time of the last run, CUDA events on the handle's stream */
-    int32_t path;          /* path actually used (PHIA_PATH_TC / _FP32 / _CSR) */
+    int32_t path;          /* path used: PHIA_PATH_TC, _FP32, or _CSR for sparse instances,
+                              whichever kernel ran them */
     int32_t operand;       /* operand actually used (PHIA_OP_E4M3 / _BF16), 0 for other paths */
     int32_t kernel_launches; /* kernels launched by the last run */
     int32_t tc_kernel;     /* dense kernel used (1 resident tcgen05, 2 per iteration, overlapped or
@@ -193,8 +196,10 @@ int phia_create_from_device(phia_t **out, const int8_t *J_k, const int32_t *h_k,
 
 /* Create a sparse instance in CSR form (host arrays): row_ptr[N+1], col[nnz]
  * (0 <= col < N, no self loops), val_k[nnz] int8; the pattern and values must be
- * symmetric.  Stored zeros are allowed.  Runs on the CSR path (a batch of one); its
- * replicas run in groups of 32, other counts padded with unreported replicas.  One
+ * symmetric.  Stored zeros are allowed.  Runs on the CSR path (a batch of one): up to 512
+ * spins on a resident kernel where that is estimated faster, else as a gather whose
+ * replicas run in groups of 32 (of 256 for large instances of few couplings a row), other
+ * counts padded with unreported replicas.  The gather takes one
  * launch per iteration (opts->tc_kernel = 1: one persistent launch for the run instead;
  * that cooperative launch assumes no other persistent launch runs on the device at the
  * same time, and reports PHIA_ETIMEOUT rather than waiting without end if one does). */
@@ -369,8 +374,8 @@ int phia_run_noalloc(const int8_t *J_k, const int32_t *h_k, int32_t N, int32_t f
  * all iterations, one launch per size class.  A batch whose other members are all of at most 512
  * spins runs those on resident kernels too where that is estimated faster (the results are the
  * same, each replica's record frozen at its own hit).  The other instances run on the sparse path
- * (larger dense descriptors converted to CSR), in sets whose state fits in L2 together, by
- * default with one launch per iteration and set (replayed as CUDA graphs);
+ * (larger dense descriptors converted to CSR), in sets whose state fits in L2 together (large
+ * instances of few couplings a row in a form without sets), by default with one launch per iteration and set (replayed as CUDA graphs);
  * phia_opts.tc_kernel = 1 at creation gives one persistent cooperative launch for every
  * iteration of every instance instead (blocks take work units from a counter, the grid meets
  * at a bounded barrier between iterations), and phia_batch_autotune picks the faster.  Each instance keeps its own
@@ -399,8 +404,8 @@ int phia_batch_create(phia_batch_t **out, int32_t count, const phia_instance_des
                       const phia_opts *opts);
 
 /* Anneal `replicas` replicas of every instance for `steps` iterations (as phia_anneal
- * per instance).  The sparse path runs replicas in groups of 32; other counts are
- * padded with extra replicas that are run but never reported.  Asynchronous. */
+ * per instance).  The sparse path runs replicas in groups of 32 (large instances of few
+ * couplings a row: of 256 where that is faster); other counts are padded with extra replicas that are run but never reported.  Asynchronous. */
 int phia_batch_anneal(phia_batch_t *b, const phia_schedule *sched, int32_t replicas, int64_t steps,
                       uint64_t seed);
 

@@ -1,9 +1,11 @@
 // batch.cu -- batched multi-instance runs (phia_batch_* of the C ABI): instance validation
 // and packing, per-replica state of every instance.  Small dense instances (N <= 384 with
-// every |k| <= 16, N <= 256 otherwise) run on the resident tcgen05 kernel with a table of
-// CTAs, all their iterations in one launch per (operand, spin tiles) group; the rest run
-// on the CSR path (dense ones converted to CSR): 64-row blocks, one launch per iteration
-// or one persistent launch over all iterations.
+// every |k| <= 16, N <= 256 otherwise) run on resident kernels over a table of CTAs, all their
+// iterations in one launch per size class; the rest run on the sparse path (dense ones
+// converted): slices of 32 rows in sets of instances (k_csr.cu), or for large instances of few
+// couplings a row the form with a row to a warp (k_csr_rows.cu), with one launch per iteration
+// or one persistent launch over all iterations.  Batches of small sparse instances alone run on
+// the resident kernels too.
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -1058,7 +1060,7 @@ int batch_stats(phia_batch_s *b, int inst, phia_stats *out) {
         if (t_hit >= t_start && t_start != 0) out->hit_ns = (int64_t)(t_hit - t_start);
     }
     out->device_ms = ms;
-    out->path = b->inst.empty() ? PHIA_PATH_TC : PHIA_PATH_CSR;   // the sparse path whenever it runs
+    out->path = b->inst.empty() ? PHIA_PATH_TC : PHIA_PATH_CSR;   // sparse members, whichever kernel ran them
     out->kernel_launches = b->last_launches;
     (void)iters;
     return PHIA_OK;

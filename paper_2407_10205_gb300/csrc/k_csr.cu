@@ -25,14 +25,16 @@
 // stream (16 bytes per spin update) behind them.  The earlier form took a row to a warp and 8
 // replicas to a lane: every neighbour cost the warp a load of 32 bytes, its address and its
 // share of the byte permutes for 8 replicas a lane instead of 32.  Per iteration (us, 256 replicas),
-// that form and this one: one Erdos-Renyi instance of 625 spins 20.9 / 7.6, of 1760 36.0 / 12.4, of
-// 5000 27.1 / 10.7, where latencies in a row set the time; 12 instances of 100 .. 3000 spins
-// 56.9 / 32.8, 48 of them 180 / 122.5, 256 of them 654 / 568.
+// that form and this one: one Erdos-Renyi instance of 625 spins 20.9 / 7.0, of 1760 36.0 / 11.5, of
+// 5000 27.1 / 10.5, where latencies in a row set the time; 12 instances of 100 .. 3000 spins
+// 56.9 / 31.1, 48 of them 180 / 113, 256 of them 654 / 521.  For large instances of few couplings a
+// row that form is the faster one and stays (k_csr_rows.cu).
 //
 // The instances go through their iterations in sets whose state fits in L2 together: a set runs
 // all of its iterations before the next begins (the instances are independent), so x and v are
 // read from L2 instead of the memory they would fall out to between two iterations of a batch
-// (48 instances 117 us an iteration against 135 in one set, 256 of them 636 against 653).
+// (measured before x and v were staged in shared memory: 48 instances 117 us an iteration against
+// 135 in one set, 256 of them 636 against 653).
 //
 // Records are lagged: the launch for iteration t settles t - 1 (the instance's last unit)
 // and copies the best spins of t - 2 for the replicas that improved then.
@@ -739,7 +741,8 @@ cudaError_t launch_csr(const CsrArgs &Cin, const int32_t *max_len, StepGraphCach
     const int groups = C.R / 32;
     const unsigned conv = (unsigned)(C.total_slices * groups);
     // Groups per block: up to 8 share one reading of the couplings (through L1), as many as leave
-    // two blocks an SM their shared memory, with x and v staged in it (48 instances of 100 .. 3000
+    // two blocks an SM their shared memory (the figures here before copy_best took its present form),
+    // with x and v staged in it (48 instances of 100 .. 3000
     // spins x 256 replicas 122 us an iteration against 140 from registers, one of 10000 19.5 against
     // 21.8).  A single group's spins that leave no room for both keep the two blocks and load x and
     // v into registers (20000 spins x 256 36 us against 43 with one block, x 1024 117 against 153

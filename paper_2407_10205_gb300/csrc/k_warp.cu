@@ -204,8 +204,8 @@ cudaError_t launch_n(const RunArgs &a, int n, unsigned ctas, cudaStream_t st) {
         if (kw <= 1) return launch_cfg<1, false>(a, ctas, st);
         if (kw <= 2) return launch_cfg<2, false>(a, ctas, st);
         // Two CTAs of 9 warps on an SM leave a thread 96 registers, which cost an iteration 0.1 us:
-        // only where there are more CTAs than SMs (N = 128: 0.54 against 0.65 us up to 1216
-        // replicas, 1.04 against 0.82 at 2048).
+        // only where there are more CTAs than SMs (N = 128: 0.49 against 0.65 us up to 1216
+        // replicas, 1.04 against 0.79 at 2048).
         int dev = 0, sms = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -6,9 +6,9 @@
 
 namespace phia {
 
-// One CTA's instance in a batched run of small dense instances (the resident tcgen05
-// kernel with an instance table): where its couplings and field are, its size, Philox
-// instance id and fixed-point scale, its first replica, and where its records start.
+// The instance of one CTA (cluster) of a resident kernel that runs many instances from a table:
+// where its couplings and field are, its size, Philox instance id and fixed-point scale, its
+// first replica, and where its records start.
 struct SmallCta {
     const int8_t *Jk;       // [N][N]
     const int32_t *hk;      // [N]
@@ -67,7 +67,7 @@ struct RunArgs {
                                          // whose CTAs hold the SMs and wait on each other
     int32_t accept_test;                 // Table 3 state 4: 1 = Metropolis test on H at trajectory ends
     int64_t *proposed, *accepted;        // [R] per-replica counts of the test (accept_test = 1)
-    const SmallCta *small_cta;           // batched small dense runs: one entry per CTA
+    const SmallCta *small_cta;           // runs of many small instances: one entry per CTA or cluster
     int32_t small_ctas;                  // its length
 };
 

@@ -196,7 +196,8 @@ def schedule(beta0, beta1, eps, gamma, refresh=0, target=None, stop_at_target=Fa
 
 
 MEM_AUTO, MEM_SHARED, MEM_TENSOR = 0, 1, 2
-KERNEL_AUTO, KERNEL_RESIDENT, KERNEL_PER_STEP, KERNEL_IMMA, KERNEL_INCREMENTAL = 0, 1, 2, 3, 4
+KERNEL_AUTO, KERNEL_RESIDENT, KERNEL_PER_STEP, KERNEL_WARP, KERNEL_INCREMENTAL = 0, 1, 2, 3, 4
+KERNEL_IMMA = KERNEL_WARP   # an earlier name, of the int8 kernel that the warp-level one took the place of
 
 
 def opts(path=PATH_AUTO, operand=OP_AUTO, device=0, instance_id=0, stream=None, tile_replicas=0,
@@ -405,7 +406,7 @@ class Annealer:
 
 
 class Batch:
-    """Many instances annealed together on the sparse path (phia_batch_*).
+    """Many instances annealed together (phia_batch_*): sparse ones, and dense ones among them.
 
     ``instances``: objects with ``kh``, ``frac_bits`` and either ``k`` (dense) or
     ``row_ptr``/``col``/``val`` (CSR), e.g. from ``instances.py``.  ``targets``: optional
