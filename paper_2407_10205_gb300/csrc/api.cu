@@ -127,6 +127,7 @@ struct phia_s {
     int8_t *d_val = nullptr;
     // per-replica state
     int R_cap = 0, R_last = 0;
+    int L_cap = 0;                      // replicas that the per-iteration kernel's buffers are for
     bool auto_tile = true;              // kernel variant chosen automatically (autotune cache)
     float *d_x = nullptr, *d_v = nullptr;
     int8_t *d_s0 = nullptr, *d_s1 = nullptr;
@@ -216,6 +217,7 @@ void free_large(phia_t *p) {
         pool_free(b, p->stream);
     p->d_S = nullptr; p->d_Epart = nullptr; p->d_flags = nullptr; p->d_ready = nullptr; p->d_sbits = nullptr;
     p->d_X = p->d_V = nullptr;
+    p->L_cap = 0;
 }
 
 void free_replicas(phia_t *p) {
@@ -232,12 +234,13 @@ void free_replicas(phia_t *p) {
     p->R_cap = 0;
 }
 
-// What the per-iteration kernel needs of a handle's replicas, for R_cap of them, when the handle first
-// takes it.  The records stay as they are: a run that goes on after an acceptance run may change
-// from the resident kernel to this one.
-int ensure_large(phia_t *p) {
-    if (!p->large || p->d_S) return PHIA_OK;
-    const size_t Rp = (size_t)large_rpad_handle(p->R_cap), Mp = (size_t)round_up(p->N, 128);
+// What the per-iteration kernel needs of a handle's replicas.  The records stay as they are: a run that
+// goes on after an acceptance run may change from the resident kernel to this one.
+int ensure_large(phia_t *p, int R) {
+    if (!p->large || R <= p->L_cap) return PHIA_OK;
+    CU(cudaStreamSynchronize(p->stream));
+    free_large(p);
+    const size_t Rp = (size_t)large_rpad_handle(R), Mp = (size_t)round_up(p->N, 128);
     bool ok = true;
     auto al = [&](void **ptr, size_t bytes) {
         if (ok && pool_alloc(ptr, bytes, p->device, p->stream) != cudaSuccess) ok = false;
@@ -252,11 +255,12 @@ int ensure_large(phia_t *p) {
     if (!ok) {
         cudaGetLastError();
         free_large(p);
-        return fail(PHIA_ENOMEM, "device allocation for %d replicas failed", p->R_cap);
+        return fail(PHIA_ENOMEM, "device allocation for %d replicas failed", R);
     }
     CU(cudaMemsetAsync(p->d_S, 0, 4 * Rp * p->Kbytes, p->stream));   // K and replica padding stay 0
     CU(cudaMemsetAsync(p->d_flags, 0, 4 * Rp, p->stream));
     CU(cudaMemsetAsync(p->d_Epart, 0, 2 * Rp * 8, p->stream));
+    p->L_cap = R;
     return PHIA_OK;
 }
 
@@ -271,7 +275,7 @@ void place_records(phia_t *p, int R) {
 }
 
 int ensure_replicas(phia_t *p, int R) {
-    if (R <= p->R_cap) return ensure_large(p);
+    if (R <= p->R_cap) return ensure_large(p, R);
     CU(cudaStreamSynchronize(p->stream));
     free_replicas(p);
     p->ran = false;            // its records are gone
@@ -307,7 +311,7 @@ int ensure_replicas(phia_t *p, int R) {
     CU(cudaMemsetAsync(p->d_rec, 0, sizeof(RunCounters), p->stream));
     CU(cudaMemsetAsync(p->d_eacc, 0, (size_t)R * 8, p->stream));
     p->R_cap = R;
-    return ensure_large(p);
+    return ensure_large(p, R);
 }
 
 int reset_run(phia_t *p, int R, bool reset) {
