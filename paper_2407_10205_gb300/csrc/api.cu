@@ -850,21 +850,31 @@ int phia_autotune(phia_t *p, const phia_schedule *sched, int32_t replicas, int32
     // would go back to, with the candidate's choice overwritten.
     after_accept(p);
     const bool saved_auto = p->auto_tile;
+    const TuneChoice before = choice_of(p);
     p->auto_tile = false;
     float best_ms = 1e30f, worst_ms = 0.f;
     TuneChoice best = cands[0];
-    for (const TuneChoice &c : cands) {
+    auto probe = [&](const TuneChoice &c, float *ms) -> int {
         if (c.large) {
             int rc = ensure_operand(p);
-            if (rc) { p->auto_tile = saved_auto; return rc; }
+            if (rc) return rc;
         }
         set_choice(p, c);
-        float ms = 0.f;
         for (int rep = 0; rep < 2; ++rep) {   // the first run warms up
             int rc = run_impl(p, sched, replicas, 0, probe_iters, probe_iters, 1, nullptr, nullptr, nullptr, nullptr, 1);
-            if (rc) { p->auto_tile = saved_auto; return rc; }
+            if (rc) return rc;
             CU(cudaEventSynchronize(p->ev1));
-            CU(cudaEventElapsedTime(&ms, p->ev0, p->ev1));
+            CU(cudaEventElapsedTime(ms, p->ev0, p->ev1));
+        }
+        return PHIA_OK;
+    };
+    for (const TuneChoice &c : cands) {
+        float ms = 0.f;
+        const int rc = probe(c, &ms);
+        if (rc) {                             // the handle stays as it was
+            set_choice(p, before);
+            p->auto_tile = saved_auto;
+            return rc;
         }
         if (ms < best_ms) { best_ms = ms; best = c; }
         worst_ms = std::max(worst_ms, ms);

@@ -50,3 +50,19 @@ def test_device_time_leaves_out_the_host_work_of_a_first_run(gpu_lib):
                 B.anneal(sched, 32, 2, seed=9)
                 out.append(B.stats().device_ms)
     assert min(first[1:]) < 1.5 * min(second) + 0.1
+
+
+def test_small_sparse_and_dense_members_together(gpu_lib):
+    """All members on resident kernels, of every size class: the records of each alone."""
+    phia = gpu_lib
+    insts = [ins.dense_int(60, 7, 7, 1), ins.erdos_renyi(100, 0.1, 127, 31, 4, 2), ins.dense_int(300, 7, 7, 3),
+             ins.erdos_renyi(400, 0.05, 127, 31, 4, 4), ins.erdos_renyi(200, 0.05, 127, 31, 4, 5), ins.dense_int(130, 7, 7, 6)]
+    sched, R, T = phia.schedule(0.01, 0.2, 0.1, 2.0, refresh=7), 45, 60
+    with phia.Batch(insts, instance_ids=range(6)) as B:
+        B.anneal(sched, R, T, seed=9)
+        mix = _records(B, 6, R)
+    for k, c in enumerate(insts):
+        with phia.Batch([c], instance_ids=[k]) as A:
+            A.anneal(sched, R, T, seed=9)
+            for u, w in zip(mix[k], A.replica_results(0, R)):
+                assert np.array_equal(u, w)

@@ -105,3 +105,14 @@ def test_stats_name_the_form_that_ran(gpu_lib, N, R, variant, form):
         phia.anneal(A.h, phia.schedule(0.01, 0.1, 0.1, 2.0), 64, 4, 1)
         st = phia.stats_get(A.h)
         assert (st.tc_kernel, st.large_form) in ((2, 4), (1, 0))
+
+
+def test_an_autotune_that_fails_leaves_the_handle_as_it_was(gpu_lib):
+    phia = gpu_lib
+    d = ins.dense_int(100, 7, 7, 1)
+    good, bad = phia.schedule(0.01, 0.1, 0.1, 2.0), phia.schedule(0.01, 0.1, 0.0, 2.0)
+    with phia.Annealer(d.k, d.kh, path=phia.PATH_TC, tc_kernel=phia.KERNEL_PER_STEP, large_variant=1) as A:
+        with pytest.raises(phia.PhiaError) as e:
+            phia.autotune(A.h, bad, 32, probe_iters=10)
+        assert e.value.code == phia.EINVAL
+        assert _kernel_of(phia, A.h, good, 32)[0] == 2
