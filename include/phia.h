@@ -369,8 +369,8 @@ int phia_run_noalloc(const int8_t *J_k, const int32_t *h_k, int32_t N, int32_t f
 
 /* ---------------------------------------------------------------- batches
  * Many independent instances of uneven N annealed together.  Dense descriptors with
- * N <= 256 run on the resident warp-level kernel, those with N <= 384 and every |k| <= 16 on
- * the resident tcgen05 kernel, over a table of CTAs (8 replicas each): every such instance,
+ * N <= 240 run on the resident warp-level kernel, those with N <= 256, or N <= 384 and every
+ * |k| <= 16, on the resident tcgen05 kernel, over a table of CTAs (8 replicas each): every such instance,
  * all iterations, one launch per size class.  A batch whose other members are all of at most 512
  * spins runs those on resident kernels too where that is estimated faster (the results are the
  * same, each replica's record frozen at its own hit).  The other instances run on the sparse path

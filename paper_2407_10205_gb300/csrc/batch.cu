@@ -84,6 +84,7 @@ struct phia_batch_s {
     // small dense members: a resident kernel over a table of CTAs
     std::vector<int> dense_pub;         // public indices
     std::vector<int64_t> dense_joff;    // offset of each member's J in d_dJ
+    std::vector<int> dense_op;          // kOpE4M3 / kOpBF16
     // sparse members that are small enough for a resident kernel as well (all of the batch's, else
     // none): offset of each one's dense J in d_dJ
     std::vector<int64_t> cand_joff;
@@ -581,6 +582,7 @@ int create_batch(phia_batch_s *&b, phia_batch_s **out, int32_t count, const phia
         if (pk.small_op) {
             b->dense_pub.push_back(k);
             b->dense_joff.push_back((int64_t)dj.size());
+            b->dense_op.push_back(pk.small_op);
             dj.insert(dj.end(), x.J_k, x.J_k + (size_t)n * n);
             hk.insert(hk.end(), x.h_k, x.h_k + n);
             continue;
@@ -766,7 +768,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         BCU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
         double us = 0.0;
         for (const CsrInst &in : b->inst)
-            us += in.N <= warp_small_max_n() ? warp_small_estimate(in.N, R_real, sms) : cluster_small_estimate(in.N, R_real, kOpBF16, sms, 5.0);
+            us += in.N <= warp_small_auto_n() ? warp_small_estimate(in.N, R_real, sms) : cluster_small_estimate(in.N, R_real, kOpBF16, sms, 5.0);
         gathers = us > 5.0;
     }
     if (gathers && !by_rows && !field_mode && b->sets_R != R) {      // host work: before the run's time begins
@@ -835,26 +837,33 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
     C.max_words = b->max_words;
     C.total_slices = b->total_slices;
     // Members on the resident kernels: a table of CTAs or clusters (8 replicas each) per size
-    // class, every instance's own couplings, field, scale, Philox id, target and records.  Dense
-    // members: up to 256 spins on the warp-level kernel (classes of at most 64, 128 and 256 spins,
-    // as its register use grows with the size it is built for), above on the resident tcgen05
-    // kernel.  Sparse members go to the warp-level kernel or, above 256 spins, to the cluster kernel
-    // where their estimated iterations take less together than the gather's, which no instance takes
-    // below 7 us (launch, records, the copy of the spins and a slice come one after the other).
+    // class, every instance's own couplings, field, scale, Philox id, target and records.  Up to 240
+    // spins the warp-level kernel (classes, as its register use grows with the size it is built
+    // for; 32 dense members of 200 spins x 512 replicas: 18.8 us an iteration on the tcgen05 one); dense members
+    // above on the resident tcgen05 kernel (256 spins x 512: 20.0 us against 22.4 on the warp-level one),
+    // sparse ones on the cluster kernel.  Sparse members run here where their estimated iterations
+    // take less together than the gather's, which no instance takes below 7 us (launch, records, the
+    // copy of the spins and a slice come one after the other).
     enum { kWarp, kTcgen05, kCluster };
     struct SmallGroup {
         size_t begin, end;       // in small_host
-        int nmax, kernel;
+        int nmax, kernel, op;
     };
     std::vector<SmallGroup> groups;
     const bool resident = ncsr > 0 && !gathers;
     if (!b->dense_pub.empty() || resident) {
         b->small_host.clear();
         struct Class {
-            int above, nmax, kernel;
+            int above, nmax, kernel, op;     // op: of the dense members that kTcgen05 takes
         };
-        const Class classes[] = {{0, 64, kWarp},       {64, 128, kWarp},     {128, 256, kWarp},
-                                 {256, 384, kTcgen05}, {256, 384, kCluster}, {384, 512, kCluster}};
+        const Class classes[] = {{0, 64, kWarp, 0},
+                                 {64, 128, kWarp, 0},
+                                 {128, 240, kWarp, 0},
+                                 {240, 256, kTcgen05, kOpE4M3},
+                                 {240, 256, kTcgen05, kOpBF16},
+                                 {256, 384, kTcgen05, kOpE4M3},
+                                 {240, 384, kCluster, 0},
+                                 {384, 512, kCluster, 0}};
         for (const Class &cls : classes) {
             const size_t beg = b->small_host.size();
             int nmax = 0;
@@ -878,10 +887,11 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
                 }
             };
             if (cls.kernel != kCluster)
-                for (size_t m = 0; m < b->dense_pub.size(); ++m) add(b->dense_pub[m], b->dense_joff[m]);
+                for (size_t m = 0; m < b->dense_pub.size(); ++m)
+                    if (cls.kernel == kWarp || b->dense_op[m] == cls.op) add(b->dense_pub[m], b->dense_joff[m]);
             if (cls.kernel != kTcgen05 && resident)
                 for (size_t m = 0; m < b->csr_pub.size(); ++m) add(b->csr_pub[m], b->cand_joff[m]);
-            if (b->small_host.size() > beg) groups.push_back(SmallGroup{beg, b->small_host.size(), nmax, cls.kernel});
+            if (b->small_host.size() > beg) groups.push_back(SmallGroup{beg, b->small_host.size(), nmax, cls.kernel, cls.op});
         }
         auto take = [&](SmallCta **q, size_t bytes) {
             return pool_alloc((void **)q, bytes, b->device, b->stream) == cudaSuccess;
@@ -932,7 +942,7 @@ int batch_run(phia_batch_s *b, const phia_schedule *sched, int32_t R_real, int64
         ad.has_target = b->any_target || sched->has_target;
         ad.x_in = x_in; ad.v_in = v_in; ad.x_out = x_out; ad.v_out = v_out;
         cudaError_t e = grp.kernel == kWarp      ? launch_warp_small_batch(ad, grp.nmax, b->stream)
-                        : grp.kernel == kTcgen05 ? launch_tc_small_batch(ad, grp.nmax, b->stream)
+                        : grp.kernel == kTcgen05 ? launch_tc_small_batch(ad, grp.op, grp.nmax, b->stream)
                                                  : launch_cluster_batch(ad, grp.nmax, b->stream);
         if (e != cudaSuccess) return bfail(PHIA_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
         ++launches;

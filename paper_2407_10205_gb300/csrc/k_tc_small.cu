@@ -662,20 +662,30 @@ cudaError_t launch_mt(const RunArgs &a, int Kpad, cudaStream_t st) {
 
 int tc_small_max_n(int op) { return op == kOpE4M3 ? 384 : 256; }
 
-cudaError_t launch_tc_small_batch(const RunArgs &a, int nmax, cudaStream_t st) {
-    // Members of 257 .. 384 spins (e4m3, three 128-spin tiles).  K is padded for the largest
-    // (nmax), so that one shared-memory layout serves all of them (the couplings and spins
-    // past an instance's N are zero).
-    if (a.small_ctas < 1) return cudaSuccess;
-    if (nmax > tc_small_max_n(kOpE4M3)) return cudaErrorInvalidValue;
-    const int Kpad = (nmax + 31) / 32 * 32;
-    const size_t smem = (size_t)(3 * 128 + kNB) * Kpad + sizeof(SmallShared) + 16;
-    auto kern = a.deriv == 1 ? tc_small_kernel<3, kOpE4M3, 2, 4, false, 1, false, true>
-                             : tc_small_kernel<3, kOpE4M3, 2, 4, false, 0, false, true>;
+namespace {
+
+template <int MT, int OP>
+cudaError_t launch_batch_mt(const RunArgs &a, int nmax, cudaStream_t st) {
+    // K is padded for the largest member (nmax), so that one shared-memory layout serves all of
+    // them (the couplings and spins past an instance's N are zero).
+    constexpr int ESZ = OP == kOpE4M3 ? 1 : 2;
+    const int Kpad = OP == kOpE4M3 ? (nmax + 31) / 32 * 32 : (nmax + 15) / 16 * 16;
+    const size_t smem = (size_t)(MT * 128 + kNB) * Kpad * ESZ + sizeof(SmallShared) + 16;
+    auto kern = a.deriv == 1 ? tc_small_kernel<MT, OP, 2, 4, false, 1, false, true>
+                             : tc_small_kernel<MT, OP, 2, 4, false, 0, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxCtaSmem);
     if (e != cudaSuccess) return e;
-    kern<<<a.small_ctas, 128 * 3 * 2 + 64 * 3, smem, st>>>(a, Kpad);
+    kern<<<a.small_ctas, 128 * MT * 2 + 64 * MT, smem, st>>>(a, Kpad);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_tc_small_batch(const RunArgs &a, int op, int nmax, cudaStream_t st) {
+    if (a.small_ctas < 1) return cudaSuccess;
+    if (nmax > tc_small_max_n(op)) return cudaErrorInvalidValue;
+    if (nmax <= 256) return op == kOpE4M3 ? launch_batch_mt<2, kOpE4M3>(a, nmax, st) : launch_batch_mt<2, kOpBF16>(a, nmax, st);
+    return launch_batch_mt<3, kOpE4M3>(a, nmax, st);
 }
 
 cudaError_t launch_tc_small(const RunArgs &a, int op, cudaStream_t st, int *launches) {

@@ -212,13 +212,15 @@ cudaError_t launch_n(const RunArgs &a, int n, unsigned ctas, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         if (kw > 6 && kw <= 8 && (int)ctas <= sms) return launch_cfg<8, false, 1>(a, ctas, st);
         if (kw > 4 && kw <= 6) return launch_cfg<6, false>(a, ctas, st);
-        if (kw > 8 && kw <= 10) return launch_cfg<10, false>(a, ctas, st);
-        if (kw > 10 && kw <= 13) return launch_cfg<13, false>(a, ctas, st);
-        if (kw > 13 && kw <= 15) return launch_cfg<15, false>(a, ctas, st);
+        if (kw == 16) return launch_cfg<16, false>(a, ctas, st);
     }
     if (kw <= 4) return launch_cfg<4, BATCHED>(a, ctas, st);
     if (kw <= 8) return launch_cfg<8, BATCHED>(a, ctas, st);
-    return launch_cfg<16, BATCHED>(a, ctas, st);
+    // By the size of its largest member in a batch too: built for 16 warps, whose registers run short, 32
+    // members of 150 spins x 512 replicas took 19.8 us an iteration.
+    if (kw <= 10) return launch_cfg<10, BATCHED>(a, ctas, st);
+    if (kw <= 13) return launch_cfg<13, BATCHED>(a, ctas, st);
+    return launch_cfg<15, BATCHED>(a, ctas, st);
 }
 
 }  // namespace
@@ -241,7 +243,7 @@ cudaError_t launch_warp_small(const RunArgs &a, cudaStream_t st, int *launches) 
 
 cudaError_t launch_warp_small_batch(const RunArgs &a, int nmax, cudaStream_t st) {
     if (a.small_ctas < 1) return cudaSuccess;
-    if (nmax > warp_small_max_n()) return cudaErrorInvalidValue;
+    if (nmax > warp_small_auto_n()) return cudaErrorInvalidValue;
     return launch_n<true>(a, nmax, (unsigned)a.small_ctas, st);
 }
 

@@ -131,9 +131,9 @@ int tc_small_max_n(int op);
 int tc_small_tile_replicas(int R, int requested);
 cudaError_t launch_tc_small(const RunArgs &a, int op, cudaStream_t st, int *launches);
 // The same kernel over a table of CTAs (a.small_cta, a.small_ctas entries, 8 live replicas
-// each) of e4m3 instances of 257 .. nmax spins: all iterations of every instance in one
-// launch; no early stop at a target.
-cudaError_t launch_tc_small_batch(const RunArgs &a, int nmax, cudaStream_t st);
+// each) of instances of one operand and 129 .. nmax spins, or 257 .. nmax where nmax > 256: all
+// iterations of every instance in one launch; no early stop at a target.
+cudaError_t launch_tc_small_batch(const RunArgs &a, int op, int nmax, cudaStream_t st);
 
 // tcgen05 per-iteration kernel for dense instances of any size (TMA-staged J and spins).
 struct LargeBuffers {
@@ -318,7 +318,7 @@ int set_last_error(int code, const char *msg);
 
 // Warp-level tensor-core resident kernel (mma.sync bf16, J in registers) for small dense
 // instances, 8 replicas per CTA (no field mode), and over a table of CTAs (a.small_cta) of
-// instances with at most nmax spins.
+// instances with at most nmax <= warp_small_auto_n() spins.
 int warp_small_max_n();
 // Automatic handles take it up to here: with 17 warps the registers run short (N = 256: 1.3 to
 // 1.8 us an iteration, against 1.05 for the cluster kernel and 1.18 for the tcgen05 one).
@@ -335,7 +335,7 @@ int cluster_small_max_n(int op);
 cudaError_t launch_cluster_small(const RunArgs &a, int op, cudaStream_t st, int *launches);
 // Its estimated time per iteration (us; 1e30 where it does not apply, or cannot be below `limit`).
 double cluster_small_estimate(int N, int R, int op, int sms, double limit);
-// And over a table of clusters (a.small_cta) of instances of 257 .. nmax spins, or of 385 .. nmax
+// And over a table of clusters (a.small_cta) of instances of 193 .. nmax spins, or of 385 .. nmax
 // where nmax > 384 (every CTA of a cluster has to own spins); nmax <= cluster_batch_max_n().
 int cluster_batch_max_n();
 cudaError_t launch_cluster_batch(const RunArgs &a, int nmax, cudaStream_t st);

@@ -66,3 +66,25 @@ def test_small_sparse_and_dense_members_together(gpu_lib):
             A.anneal(sched, R, T, seed=9)
             for u, w in zip(mix[k], A.replica_results(0, R)):
                 assert np.array_equal(u, w)
+
+
+@pytest.mark.parametrize("top", [160, 161, 208, 209, 240, 256])
+def test_members_of_129_to_256_spins(gpu_lib, top):
+    """The kernels that a batch's launch is built for by its largest member (10, 13 or 15 warps), and the
+    tcgen05 and cluster kernels above 240 spins, for both operands: the records of each alone."""
+    phia = gpu_lib
+    insts = [ins.dense_int(129, 7, 7, 1), ins.dense_int(top, 7, 7, 2), ins.dense_int(top, 100, 7, 3),
+             ins.erdos_renyi(top, 0.1, 127, 31, 4, 4), ins.dense_int(max(129, top - 15), 100, 7, 5)]
+    R, T = 45, 40
+    for deriv in (0, 1):
+        sched = phia.schedule(0.01, 0.2, 0.1, 2.0, refresh=7, deriv=deriv)
+        with phia.Batch(insts, instance_ids=range(5)) as B:
+            B.anneal(sched, R, T, seed=9)
+            mix = _records(B, 5, R)
+        for k, c in enumerate(insts):
+            d = c if hasattr(c, "k") else c.to_dense()
+            with phia.Annealer(d.k, d.kh, d.frac_bits, path=phia.PATH_TC, instance_id=k, tc_kernel=phia.KERNEL_PER_STEP,
+                               large_variant=1) as A:
+                phia.anneal(A.h, sched, R, T, 9)
+                for u, w in zip(mix[k], phia.replica_results(A.h, R, d.n)):
+                    assert np.array_equal(u, w)
