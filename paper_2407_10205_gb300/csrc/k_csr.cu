@@ -652,10 +652,13 @@ __global__ void csr_field_only(const CsrArgs C) {
         if (C.col16) e16.load(C, e, lane);
         else e32.load(C, e, lane);
         const uint32_t kk = C.col16 ? e16.k : e32.k;
-        for (int n = 0; n < 4; ++n) {
-            const int kv = (int8_t)(kk >> (8 * n));
-            if (kv) I += kv * s[C.row_of[in.pos_off + (C.col16 ? e16.at(n) : e32.at(n)) / 4]];
-        }
+        // no look at the couplings first: the four ways from position to spin to sign run side by side
+        // (entries that pad a row are position 0 with k = 0)
+        int j[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) j[n] = C.row_of[in.pos_off + (C.col16 ? e16.at(n) : e32.at(n)) / 4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) I += (int8_t)(kk >> (8 * n)) * s[j[n]];
     }
     if (a.field_out) a.field_out[in.xin_off + (size_t)r * in.N + row] = I;
     atomicAdd(reinterpret_cast<unsigned long long *>(C.Esum) + in.rec_off + r,
